@@ -61,6 +61,21 @@ def test_route_batched(n, batch):
     assert np.array_equal(gpu_route(perm, n), oracle.route(perm, n))
 
 
+@pytest.mark.parametrize("n,batch", [(1, 2049), (2, 1031), (3, 131), (4, 67), (5, 33), (6, 17), (6, 10007), (7, 2401), (8, 5),
+                                     (8, 601), (9, 1201), (10, 149), (10, 593), (11, 297), (12, 149), (13, 149), (14, 149)])
+def test_route_blocks_that_share_a_cta(n, batch):
+    """Small permutations share a CTA (of 2^10 to 2^13 outputs, with few or many threads, by how many
+    there are), the last of which is padded; the permutations also start off a 16-byte boundary."""
+    perm = inputs.random_perm_batch(n, batch, seed0=13 * n)
+    want = oracle.route(perm, n)
+    assert np.array_equal(gpu_route(perm, n), want)
+    moved = dev(np.concatenate([np.zeros(1, dtype=np.uint32), perm.ravel()]))[1:]
+    bits = torch.full((binding.benes_switch_words(n, batch),), -1, dtype=torch.int32, device="cuda")
+    binding.benes_route(moved, n, batch, bits)
+    torch.cuda.synchronize()
+    assert np.array_equal(host(bits, np.uint32).reshape(want.shape), want)
+
+
 @pytest.mark.parametrize("n", [4, 9, 10, 13, 15, 16, 18, 20])
 @pytest.mark.parametrize("kind", ["identity", "shift1", "bitrev", "transpose", "sattolo"])
 def test_route_structured(n, kind):
