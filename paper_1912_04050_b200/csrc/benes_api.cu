@@ -188,11 +188,14 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
                  const Options &opt, const HostPipe *hp = nullptr) {
     const size_t T = batch << n;
     const size_t kFusedSplitWave = size_t(sm_count());   // CTAs of the fused kernel that run together (one per SM)
-    void *Sbuf[2];                     // two generations of switch records (wide: 16 B per switch)
+    // two generations of records: 8 bytes per switch, then, for wide levels, the plain P
+    void *Sbuf[2];
+    uint32_t *Pbuf[2];
     uint32_t *Qbuf[2];
     size_t off = 0;
     Sbuf[0] = ws + off; off += align_up(T * 8);
     Sbuf[1] = ws + off; off += align_up(T * 8);
+    for (int i = 0; i < 2; ++i) Pbuf[i] = reinterpret_cast<uint32_t *>(static_cast<char *>(Sbuf[i]) + T * 4);
     Qbuf[0] = reinterpret_cast<uint32_t *>(ws + off); off += align_up(T * 4);
     Qbuf[1] = reinterpret_cast<uint32_t *>(ws + off); off += align_up(T * 4);
     unsigned long long *Wd = reinterpret_cast<unsigned long long *>(ws + off); off += align_up(T * 8);
@@ -204,6 +207,15 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     // closer rulers (shorter walks) pay there although the lists get longer.
     const int kappa = (opt.kappa > 3 && T <= (size_t(1) << 22)) ? 3 : opt.kappa;
     const uint32_t cap = uint32_t(opt.walk_cap);
+    // (level 0: P is the caller's permutation, which nobody writes; the kernels load 16 bytes at a time)
+    if (reinterpret_cast<uintptr_t>(perm) % 16) {
+        BENES_CUDA_TRY(cudaMemcpyAsync(Pbuf[0], perm, T * 4, cudaMemcpyDeviceToDevice, s));
+        perm = Pbuf[0];
+    }
+    auto records = [&](int level, int buf) {
+        const bool packed = rec_is_packed(n - level, kappa);
+        return LevelRecords{kappa ? Sbuf[buf] : nullptr, packed ? nullptr : level ? Pbuf[buf] : const_cast<uint32_t *>(perm), packed};
+    };
     SampledScratch sc;
     int rc;
     if (kappa) {
@@ -220,21 +232,20 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
         const bool bucketed = opt.inverse_partitioned && T >= (size_t(1) << kInversePartitionMinLog2) &&
                               (T & ((size_t(1) << 18) - 1)) == 0;
         const int pieces = hp ? hp->pieces : 0;
-        const bool pk = rec_is_packed(n, kappa);
+        const LevelRecords S0 = records(0, 0);
         if (bucketed && pieces > 1) {
             if ((rc = launch_inverse_clear(fill, T, s))) return rc;
             const size_t per = T / size_t(pieces);
             for (int i = 0; i < pieces; ++i) {
                 BENES_CUDA_TRY(cudaStreamWaitEvent(s, hp->piece_ready[i], 0));
-                if ((rc = launch_inverse_partition_piece(perm, Sbuf[0], pk, Wd, fill, T, per * size_t(i),
-                                                         per, n, s)))
+                if ((rc = launch_inverse_partition_piece(perm, S0, Wd, fill, T, per * size_t(i), per, n, kappa, s)))
                     return rc;
             }
             rc = launch_inverse_scatter(Wd, Qbuf[0], T, n, s);
         } else {
             for (int i = 0; i < pieces; ++i) BENES_CUDA_TRY(cudaStreamWaitEvent(s, hp->piece_ready[i], 0));
-            rc = bucketed ? launch_inverse_partitioned(perm, Sbuf[0], pk, Qbuf[0], Wd, fill, T, n, s)
-                          : launch_inverse(perm, Sbuf[0], pk, Qbuf[0], T, n, s);
+            rc = bucketed ? launch_inverse_partitioned(perm, S0, Qbuf[0], Wd, fill, T, n, kappa, s)
+                          : launch_inverse(perm, S0, Qbuf[0], T, n, kappa, s);
         }
         if (rc) return rc;
     }
@@ -246,26 +257,24 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     for (int level = 0; n - level > fused_m; ++level) {
         const int m = n - level;
         const int out_stage = 2 * n - 2 - level;
-        void *S = Sbuf[cur];
+        const LevelRecords S = records(level, cur), Sn = records(level + 1, cur ^ 1);
         uint32_t *Q = Qbuf[cur];
-        const bool pk = rec_is_packed(m, kappa), pk_next = rec_is_packed(m - 1, kappa);
         uint32_t *gate = nullptr;
         if (kappa) {
             // ruler-sampled labelling; raises `gate` if a walk had to give up
             gate = gates + level;
-            if ((rc = sampled_label(S, pk, Q, Sbuf[cur ^ 1], pk_next, sc, T, m, kappa, uint32_t(level), cap,
-                                    opt.walk_pairs, L, out_stage, gate, s)))
+            if ((rc = sampled_label(S, Q, Sn, sc, T, m, kappa, uint32_t(level), cap, opt.walk_pairs, L, out_stage, gate, s)))
                 return rc;
         }
         // pointer jumping over all outputs: the whole labelling when sampling is
         // off, otherwise gated (returns at once unless this level's walks gave up)
         {
             ProfileScope ps(kFullLabel, s);
-            if ((rc = launch_full_label(S, pk, Q, Wd, T, m, L, out_stage, gate, s))) return rc;
+            if ((rc = launch_full_label(S, Q, Wd, T, m, L, out_stage, gate, s))) return rc;
         }
         {
             ProfileScope ps(kSplit, s);
-            if ((rc = launch_split(S, pk, Q, Sbuf[cur ^ 1], pk_next, Qbuf[cur ^ 1], T, m, L, level, out_stage, gate, s)))
+            if ((rc = launch_split(S, Q, Sn, Qbuf[cur ^ 1], T, m, kappa, L, level, out_stage, gate, s)))
                 return rc;
         }
         cur ^= 1;
@@ -277,7 +286,9 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
             if ((rc = copy_stage_rows(*hp, bits, n, batch, out_stage, 1, hp->d2h))) return rc;
         }
     }
-    const int records = rec_is_packed(fused_m, kappa) ? 2 : 1;
+    const LevelRecords tail = records(n - fused_m, cur);
+    const void *tail_p = tail.packed ? tail.S : tail.P;
+    const int tail_format = tail.packed ? 1 : 0;
     const size_t blocks = T >> fused_m;
     // the stages of the in-CTA levels are one run of rows in the middle
     const int first = n - fused_m, rows = 2 * fused_m - 1;
@@ -288,12 +299,12 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
         const size_t b1 = ((waves + 1) / 2) * kFusedSplitWave;
         {
             ProfileScope ps(kFused, s);
-            if ((rc = launch_fused(Sbuf[cur], records, T, fused_m, bits, n, s, 0, b1))) return rc;
+            if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, 0, b1))) return rc;
         }
         BENES_CUDA_TRY(cudaEventRecord(hp->stage_ready[kMaxLevels - 2], s));
         {
             ProfileScope ps(kFused, s);
-            if ((rc = launch_fused(Sbuf[cur], records, T, fused_m, bits, n, s, b1, blocks - b1))) return rc;
+            if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, b1, blocks - b1))) return rc;
         }
         // a block of 2^m outputs owns 2^(m-6) words of every stage
         const size_t w = stage_words(n) * 4, col1 = (b1 << (fused_m - 6)) * 4;
@@ -309,7 +320,7 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     }
     {
         ProfileScope ps(kFused, s);
-        if ((rc = launch_fused(Sbuf[cur], records, T, fused_m, bits, n, s))) return rc;
+        if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s))) return rc;
     }
     if (hp && hp->bits_host) {
         if ((rc = copy_stage_rows(*hp, bits, n, batch, first, rows, s))) return rc;

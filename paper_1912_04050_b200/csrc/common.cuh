@@ -155,36 +155,47 @@ struct BitsLayout {
 };
 
 // ---- layout of a level in HBM ------------------------------------------------
-// A level of the per-level path keeps its sub-permutations as one record per
-// output switch t of the flat array, and the inverses Q as a plain uint32
-// array (read at random, never claimed).  Two record formats:
+// A level of the per-level path keeps its sub-permutations (P, block-local values) and the claims
+// of the walks per output switch t of the flat array, and the inverses Q as a plain uint32 array
+// (read at random, never claimed).  Two formats of the first part:
 //
-//   wide   (16 B)  { P[2t], P[2t+1], owner, 0 }, P block-local; owner is
-//                  kUnowned until a walk of the sampled labelling claims the
-//                  switch with a compare-and-swap.  It sits in the record so
-//                  that claiming hits the sector the walker has just fetched.
+//   wide   P is a plain uint32 array (level 0: the caller's permutation itself), and S holds an
+//          8-byte claim record per switch: { P[2t], P[2t+1] } until a walk of the sampled labelling
+//          claims the switch, kClaimed | owner afterwards.  One 64-bit exchange returns the two P
+//          values and claims the switch.  What a claim costs is the random sector it dirties
+//          (2^25 of them: 1.30 ms in a 512 MiB table, 1.07 in 256, 0.62 in 128, 0.25 in 64 and
+//          less), so the records are as small as they can be and what the later kernels
+//          need in order stays apart from them.  The ruler switches are claimed from the start.
 //   packed (8 B)   P[2t] | P[2t+1] << m | owner << 2m for blocks of 2^m outputs,
 //                  owner local to the block, all ones = unowned.  One 64-bit
 //                  atomic AND both returns the two P values and claims the
-//                  switch, i.e. one memory operation instead of two.  Used
-//                  when the owner fits with room for the all-ones value:
-//                  2m + (m - kappa + 1) < 64.
+//                  switch, and there is no second copy of P.  Used when the owner fits
+//                  with room for the all-ones value: 2m + (m - kappa + 1) < 64.
 //
 // Owner = (ruler output that claimed the switch) << 1 | side of arrival.
+constexpr unsigned long long kClaimed = 1ull << 63;
 __host__ __device__ inline bool rec_is_packed(int m, int kappa) {
     return kappa != 0 && 3 * m - kappa + 1 < 64;
 }
 
+// The ruler switch of a group of 2^kappa switches (kmask = 2^kappa - 1); salt = level.
+__device__ __forceinline__ uint32_t ruler_slot(uint32_t group, uint32_t salt, uint32_t kmask) {
+    uint32_t h = group * 0x9E3779B1u + salt;
+    h ^= h >> 15;
+    h *= 0x85EBCA6Bu;
+    h ^= h >> 13;
+    return h & kmask;
+}
+
 template <bool PACKED>
-__device__ __forceinline__ void rec_read(const void *S, size_t t, int m, uint32_t &p0, uint32_t &p1) {
+__device__ __forceinline__ void rec_read(const void *S, const uint32_t *P, size_t t, int m, uint32_t &p0, uint32_t &p1) {
+    const uint32_t mask = (1u << m) - 1u;
     if (PACKED) {
         const unsigned long long w = __ldcs(static_cast<const unsigned long long *>(S) + t);
-        const uint32_t mask = (1u << m) - 1u;
         p0 = uint32_t(w) & mask;
         p1 = uint32_t(w >> m) & mask;
     } else {
-        const uint4 r = __ldcs(static_cast<const uint4 *>(S) + t);
-        const uint32_t mask = (1u << m) - 1u;
+        const uint2 r = __ldcs(reinterpret_cast<const uint2 *>(P) + t);
         p0 = BENES_GUARD(r.x, mask);
         p1 = BENES_GUARD(r.y, mask);
     }
@@ -192,12 +203,12 @@ __device__ __forceinline__ void rec_read(const void *S, size_t t, int m, uint32_
 
 // one P value, P[j], read at random
 template <bool PACKED>
-__device__ __forceinline__ uint32_t rec_p(const void *S, uint32_t j, int m) {
+__device__ __forceinline__ uint32_t rec_p(const void *S, const uint32_t *P, uint32_t j, int m) {
     if (PACKED) {
         const unsigned long long w = __ldg(static_cast<const unsigned long long *>(S) + (j >> 1));
         return uint32_t(w >> ((j & 1u) ? m : 0)) & ((1u << m) - 1u);
     }
-    return BENES_GUARD(static_cast<const uint32_t *>(S)[(size_t(j >> 1) << 2) | (j & 1u)], (1u << m) - 1u);
+    return BENES_GUARD(P[j], (1u << m) - 1u);
 }
 
 // A thread of the streaming kernels owns the two neighbouring switches 2i and
@@ -215,14 +226,36 @@ __device__ __forceinline__ void store_stage_bits64(uint32_t *row_words, uint32_t
     if (lane < 2) row_words[lane] = lane ? w1 : w0;
 }
 
-// an unowned record of a level with blocks of 2^m outputs
+// the packed record of a switch nobody owns, in a level with blocks of 2^m outputs
+__device__ __forceinline__ unsigned long long packed_record(int m, uint32_t p0, uint32_t p1) {
+    return (unsigned long long)p0 | ((unsigned long long)p1 << m) | (~0ull << (2 * m));
+}
+// the claim record of switch t of a level whose rulers are drawn with `salt`
+__device__ __forceinline__ unsigned long long claim_record(uint32_t t, uint32_t p0, uint32_t p1, int kappa, uint32_t salt) {
+    const uint32_t group = t >> kappa, kmask = (1u << kappa) - 1u;
+    return (t & kmask) == ruler_slot(group, salt, kmask) ? (kClaimed | (unsigned long long)(group << 2))
+                                                         : ((unsigned long long)p0 | ((unsigned long long)p1 << 32));
+}
+// Two neighbouring switches t, t + 1 (t even) of a level: 16-byte stores.  A wide level gets its P
+// here too, unless P is null (level 0), and its claim records, unless S is null (no sampling).
 template <bool PACKED>
-__device__ __forceinline__ void rec_write(void *S, size_t t, int m, uint32_t p0, uint32_t p1) {
-    if (PACKED)
-        static_cast<unsigned long long *>(S)[t] =
-            (unsigned long long)p0 | ((unsigned long long)p1 << m) | (~0ull << (2 * m));
-    else
-        static_cast<uint4 *>(S)[t] = make_uint4(p0, p1, kUnowned, 0u);
+__device__ __forceinline__ void rec_write2(void *S, uint32_t *P, size_t t, int m, uint4 p, int kappa, uint32_t salt) {
+    if (PACKED) {
+        static_cast<ulonglong2 *>(S)[t >> 1] = make_ulonglong2(packed_record(m, p.x, p.y), packed_record(m, p.z, p.w));
+    } else {
+        if (P) reinterpret_cast<uint4 *>(P)[t >> 1] = p;
+        if (S) static_cast<ulonglong2 *>(S)[t >> 1] = make_ulonglong2(claim_record(uint32_t(t), p.x, p.y, kappa, salt),
+                                                                      claim_record(uint32_t(t) + 1u, p.z, p.w, kappa, salt));
+    }
+}
+template <bool PACKED>
+__device__ __forceinline__ void rec_write(void *S, uint32_t *P, size_t t, int m, uint32_t p0, uint32_t p1, int kappa, uint32_t salt) {
+    if (PACKED) {
+        static_cast<unsigned long long *>(S)[t] = packed_record(m, p0, p1);
+    } else {
+        if (P) reinterpret_cast<uint2 *>(P)[t] = make_uint2(p0, p1);
+        if (S) static_cast<unsigned long long *>(S)[t] = claim_record(uint32_t(t), p0, p1, kappa, salt);
+    }
 }
 
 __device__ __forceinline__ unsigned long long make_word(uint32_t nxt, uint32_t mn) {
@@ -238,31 +271,38 @@ inline uint32_t stream_rounds(size_t items, int threads) {
 
 // ---- per-level HBM path (route_levels.cu) ----------------------------------
 // total = batch * N flat elements (<= 2^30), all blocks of one level per launch.
-// Level 0: S records from the caller's permutation, and Q[P[j]] = j.
-int launch_inverse(const uint32_t *perm, void *S, bool packed, uint32_t *Q, size_t total, int log2m,
+// The records of a level: packed, or wide (S = claim records, null without sampling; P = plain array,
+// null where it need not be written).
+struct LevelRecords {
+    void *S;
+    uint32_t *P;
+    bool packed;
+};
+// Level 0: records from the caller's permutation (rulers of salt 0), and Q[P[j]] = j.
+int launch_inverse(const uint32_t *perm, LevelRecords S, uint32_t *Q, size_t total, int log2m, int kappa,
                    cudaStream_t s);
 // The same for total >= 2^kInversePartitionMinLog2 in two streaming passes:
 // `pairs` = total x 8 bytes of scratch, `fill` = total >> 18 zero-initialised
 // counters (at most kInverseMaxBuckets).
 constexpr int kInversePartitionMinLog2 = 22;
 constexpr int kInverseMaxBuckets = 4096;
-int launch_inverse_partitioned(const uint32_t *perm, void *S, bool packed, uint32_t *Q, void *pairs,
-                               uint32_t *fill, size_t total, int log2m, cudaStream_t s);
+int launch_inverse_partitioned(const uint32_t *perm, LevelRecords S, uint32_t *Q, void *pairs,
+                               uint32_t *fill, size_t total, int log2m, int kappa, cudaStream_t s);
 int launch_inverse_clear(uint32_t *fill, size_t total, cudaStream_t s);
-int launch_inverse_partition_piece(const uint32_t *perm, void *S, bool packed, void *pairs, uint32_t *fill,
-                                   size_t total, size_t j_first, size_t count, int log2m,
+int launch_inverse_partition_piece(const uint32_t *perm, LevelRecords S, void *pairs, uint32_t *fill,
+                                   size_t total, size_t j_first, size_t count, int log2m, int kappa,
                                    cudaStream_t s);
 int launch_inverse_scatter(const void *pairs, uint32_t *Q, size_t total, int log2m, cudaStream_t s);
 // Pointer jumping over all outputs (successor build, log2m-2 in-place passes,
 // last pass + output-side bits) in ONE cooperative launch; `gate` (may be
 // null) is a device word: the kernel returns at once while it is 0.
-int launch_full_label(const void *S, bool packed, const uint32_t *Q, unsigned long long *Wd, size_t total,
+int launch_full_label(LevelRecords S, const uint32_t *Q, unsigned long long *Wd, size_t total,
                       int log2m, BitsLayout L, int out_stage, const uint32_t *gate, cudaStream_t s);
 // Input-side bits + next level's inverses; also the next level's records
-// (owner reset) if `gate` is null or *gate != 0 (otherwise the colouring kernel
+// (unclaimed, rulers of salt in_stage + 1) if `gate` is null or *gate != 0 (otherwise the colouring kernel
 // of the sampled labelling has written them already).
-int launch_split(const void *S, bool packed, const uint32_t *Q, void *Sn, bool next_packed, uint32_t *Qn,
-                 size_t total, int log2m, BitsLayout L, int in_stage, int out_stage, const uint32_t *gate,
+int launch_split(LevelRecords S, const uint32_t *Q, LevelRecords Sn, uint32_t *Qn,
+                 size_t total, int log2m, int kappa, BitsLayout L, int in_stage, int out_stage, const uint32_t *gate,
                  cudaStream_t s);
 
 // ---- ruler-sampled loop labelling (route_sampled.cu) --------------------------
@@ -277,9 +317,8 @@ void sampled_scratch_carve(char *base, size_t total, int kappa, SampledScratch *
 // Labels every loop of the level, writes the output-side stage and the next
 // level's records Sn; raises *gate if some walk exceeded `cap` hops (the level
 // must then be relabelled and Sn rewritten).
-int sampled_label(void *S, bool packed, const uint32_t *Q, void *Sn, bool next_packed,
-                  const SampledScratch &sc, size_t total, int log2m, int kappa, uint32_t salt, uint32_t cap,
-                  int walk_pairs, BitsLayout L, int out_stage, uint32_t *gate, cudaStream_t s);
+int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const SampledScratch &sc, size_t total,
+                  int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage, uint32_t *gate, cudaStream_t s);
 // owner[0] and owner[1] must be all kUnowned before the first sampled_label.
 int sampled_scratch_reset(const SampledScratch &sc, size_t total, int kappa, cudaStream_t s);
 
@@ -287,7 +326,7 @@ int sampled_scratch_reset(const SampledScratch &sc, size_t total, int kappa, cud
 // Finishes levels (n - log2m) .. n-1 of every block of size 2^log2m of the flat
 // level array (total elements), one CTA per block for log2m <= kFusedLog2M, one
 // cluster of two CTAs per block for log2m = kFusedLog2M + 1.
-// P is a plain uint32 array if records == 0, wide records if 1, packed records if 2.
+// P is a plain uint32 array if records == 0, packed records if 1.
 // `blocks` blocks from `first_block` on (blocks = 0: all from first_block).
 int launch_fused(const void *P, int records, size_t total, int log2m, uint32_t *bits, int log2n,
                  cudaStream_t s, size_t first_block = 0, size_t blocks = 0);

@@ -712,15 +712,10 @@ k_route_fused(const uint32_t *__restrict__ P, int records, uint32_t *__restrict_
         const size_t f = out.flat0 + 4u * i4;
         uint32_t v[4];
         if (4u * i4 + 4u <= out.valid && (records != 0 || aligned)) {
-            // plain array (0), wide switch records {P[2t], P[2t+1], -, -} (1), or packed records
-            // P[2t] | P[2t+1] << logs | ... (2)
+            // plain array (0) or packed records P[2t] | P[2t+1] << logs | ... (1)
             if (records == 0) {
                 const uint4 p = __ldcs(reinterpret_cast<const uint4 *>(P + f));
                 v[0] = p.x; v[1] = p.y; v[2] = p.z; v[3] = p.w;
-            } else if (records == 1) {
-                const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(P) + (f >> 1));
-                const uint4 b = __ldcs(reinterpret_cast<const uint4 *>(P) + (f >> 1) + 1);
-                v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
             } else {
                 const ulonglong2 p = __ldcs(reinterpret_cast<const ulonglong2 *>(P) + (f >> 2));
                 v[0] = uint32_t(p.x) & smask; v[1] = uint32_t(p.x >> logs) & smask;
@@ -818,13 +813,13 @@ k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restri
     for (int j = tid; j < M; j += T) {
         const size_t f = flat0 + rank * uint32_t(M) + j;
         uint32_t v;
-        if (records == 2) {
+        if (records) {
             const unsigned long long w = reinterpret_cast<const unsigned long long *>(P)[f >> 1];
-            v = uint32_t(w >> ((f & 1) ? kClusterLog2M : 0));
+            v = uint32_t(w >> ((f & 1) ? kClusterLog2M : 0)) & kBoth;
         } else {
-            v = records ? P[((f >> 1) << 2) | (f & 1)] : P[f];
+            v = P[f];
         }
-        Pa[j] = uint16_t(records == 2 ? (v & kBoth) : BENES_GUARD(v, kBoth));
+        Pa[j] = uint16_t(BENES_GUARD(v, kBoth));
     }
     for (int t = tid; t < M / 2; t += T) own[t] = uint16_t(kNone16);
     cluster.sync();           // both CTAs are running (and loaded) before either touches the other's memory

@@ -2,7 +2,7 @@
 // fit one CTA's shared memory.  One launch covers all 2^l blocks of a level
 // (and all permutations of a batch): arrays are flat, a block of size
 // M = 2^log2m owns flat indices [bM, (b+1)M), and P / Q hold block-local
-// values.  P lives in 16-byte switch records (see common.cuh).
+// values (record formats: see common.cuh).
 //
 // This file: the level-0 inverse scatter, the compaction that forms the next
 // level, and pointer jumping over ALL outputs (one cooperative kernel), which
@@ -59,7 +59,7 @@ inline int grid_for(size_t work_items, int per_sm = 8) {
 template <bool PACKED>
 __global__ void __launch_bounds__(kThreads)
 k_inverse(const uint4 *__restrict__ P4, void *__restrict__ S, uint32_t *__restrict__ Q,
-          size_t quads, int m) {
+          size_t quads, int m, int kappa) {
     const uint32_t mmask = (1u << m) - 1u;
     size_t stride = size_t(gridDim.x) * blockDim.x;
     for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < quads; i += stride) {
@@ -68,8 +68,7 @@ k_inverse(const uint4 *__restrict__ P4, void *__restrict__ S, uint32_t *__restri
         size_t j = i * 4;
         size_t base = j & ~size_t(mmask);
         uint32_t jl = uint32_t(j) & mmask;
-        rec_write<PACKED>(S, 2 * i, m, p.x, p.y);
-        rec_write<PACKED>(S, 2 * i + 1, m, p.z, p.w);
+        rec_write2<PACKED>(S, nullptr, 2 * i, m, p, kappa, 0u);
         Q[base + p.x] = jl;
         Q[base + p.y] = jl + 1;
         Q[base + p.z] = jl + 2;
@@ -106,7 +105,7 @@ inline size_t partition_smem(uint32_t buckets) { return size_t(kPartChunk) * 8 +
 template <bool PACKED>
 __global__ void __launch_bounds__(kPartThreads, 2)
 k_inverse_partition(const uint32_t *__restrict__ P, void *__restrict__ S, uint2 *__restrict__ pairs,
-                    uint32_t *__restrict__ fill, uint32_t buckets, int blog, int m, size_t j_first) {
+                    uint32_t *__restrict__ fill, uint32_t buckets, int blog, int m, size_t j_first, int kappa) {
     const uint32_t mmask = (1u << m) - 1u;
     extern __shared__ __align__(8) unsigned char part_smem[];
     uint2 *stage = reinterpret_cast<uint2 *>(part_smem);                  // the CTA's pairs, sorted by bucket
@@ -126,7 +125,7 @@ k_inverse_partition(const uint32_t *__restrict__ P, void *__restrict__ S, uint2 
         const size_t j = j0 + 2 * (size_t(i / 2) * kPartThreads + tid);
         const uint2 p = __ldcs(reinterpret_cast<const uint2 *>(P + j));
         const uint32_t px = BENES_GUARD(p.x, mmask), py = BENES_GUARD(p.y, mmask);
-        rec_write<PACKED>(S, j >> 1, m, px, py);
+        rec_write<PACKED>(S, nullptr, j >> 1, m, px, py, kappa, 0u);
         const uint32_t base = uint32_t(j) & ~mmask;
         dest[i] = base + px;
         dest[i + 1] = base + py;
@@ -244,7 +243,7 @@ __device__ __forceinline__ unsigned long long jump(unsigned long long w, unsigne
 //   last  : even outputs only; colour = leader & 1 -> output-side stage word
 template <bool PACKED>
 __global__ void __launch_bounds__(kThreads)
-k_full_label(const void *__restrict__ S, const uint32_t *__restrict__ Q,
+k_full_label(const void *__restrict__ S, const uint32_t *__restrict__ P, const uint32_t *__restrict__ Q,
              unsigned long long *__restrict__ Wd, size_t total, int m, int passes,
              BitsLayout L, int out_stage, const uint32_t *__restrict__ gate) {
     if (gate && *gate == 0u) return;        // same value for every thread of the grid
@@ -257,7 +256,7 @@ k_full_label(const void *__restrict__ S, const uint32_t *__restrict__ Q,
     const size_t switches = total / 2;
     for (size_t t = first; t < switches; t += stride) {
         uint32_t p0, p1;
-        rec_read<PACKED>(S, t, m, p0, p1);
+        rec_read<PACKED>(S, P, t, m, p0, p1);
         size_t j = 2 * t;
         size_t base = j & ~size_t(mmask);
         uint32_t b32 = uint32_t(base);
@@ -305,9 +304,9 @@ k_full_label(const void *__restrict__ S, const uint32_t *__restrict__ Q,
 // of each half-block and stores whole records.
 template <bool PACKED, bool NEXT_PACKED>
 __global__ void __launch_bounds__(kThreads, 8)
-k_split(const void *__restrict__ S, const uint4 *__restrict__ Q4, void *__restrict__ Sn,
-        uint32_t *__restrict__ Qn, uint32_t pairs, int m, BitsLayout L, int in_stage,
-        int out_stage, const uint32_t *__restrict__ gate, uint32_t rounds) {
+k_split(const void *__restrict__ S, const uint32_t *__restrict__ P, const uint4 *__restrict__ Q4,
+        void *__restrict__ Sn, uint32_t *__restrict__ Pn, uint32_t *__restrict__ Qn, uint32_t pairs, int m, int kappa,
+        BitsLayout L, int in_stage, int out_stage, const uint32_t *__restrict__ gate, uint32_t rounds) {
     const bool with_records = !gate || *gate != 0u;
     const uint32_t mmask = (1u << m) - 1u;
     // a CTA takes `rounds` consecutive groups of blockDim.x pairs: the colour
@@ -331,14 +330,15 @@ k_split(const void *__restrict__ S, const uint4 *__restrict__ Q4, void *__restri
         const uint32_t *colours = L.bits + L.word32(out_stage, (base >> 1) >> 5);   // the block's words of that stage
         if (with_records) {
             uint32_t px0, py0, px1, py1;
-            rec_read<PACKED>(S, t, m, px0, py0);
-            rec_read<PACKED>(S, t + 1, m, px1, py1);
+            rec_read<PACKED>(S, P, t, m, px0, py0);
+            rec_read<PACKED>(S, P, t + 1, m, px1, py1);
             // colours of outputs 2t and 2t+2
             const uint32_t cwd = colours[tl >> 5];
             const uint32_t c0 = (cwd >> (tl & 31u)) & 1u, c1 = (cwd >> ((tl + 1u) & 31u)) & 1u;
             const uint32_t r = (base >> 1) + (tl >> 1);
-            rec_write<NEXT_PACKED>(Sn, r, m - 1, (c0 ? py0 : px0) >> 1, (c1 ? py1 : px1) >> 1);
-            rec_write<NEXT_PACKED>(Sn, r + (H >> 1), m - 1, (c0 ? px0 : py0) >> 1, (c1 ? px1 : py1) >> 1);
+            const uint32_t salt = uint32_t(in_stage) + 1u;
+            rec_write<NEXT_PACKED>(Sn, Pn, r, m - 1, (c0 ? py0 : px0) >> 1, (c1 ? py1 : px1) >> 1, kappa, salt);
+            rec_write<NEXT_PACKED>(Sn, Pn, r + (H >> 1), m - 1, (c0 ? px0 : py0) >> 1, (c1 ? px1 : py1) >> 1, kappa, salt);
         }
         q.x = BENES_GUARD(q.x, mmask); q.y = BENES_GUARD(q.y, mmask); q.z = BENES_GUARD(q.z, mmask); q.w = BENES_GUARD(q.w, mmask);
         // colour of the output fed by input 2t (2t+2): that output's switch bit, flipped for an odd output
@@ -401,8 +401,8 @@ int launch_inverse_clear(uint32_t *fill, size_t total, cudaStream_t s) {
     return BENES_OK;
 }
 
-int launch_inverse_partition_piece(const uint32_t *perm, void *S, bool packed, void *pairs, uint32_t *fill,
-                                   size_t total, size_t j_first, size_t count, int log2m,
+int launch_inverse_partition_piece(const uint32_t *perm, LevelRecords S, void *pairs, uint32_t *fill,
+                                   size_t total, size_t j_first, size_t count, int log2m, int kappa,
                                    cudaStream_t s) {
     const int blog = bucket_log2(total);
     const uint32_t buckets = uint32_t(total >> blog);
@@ -420,12 +420,12 @@ int launch_inverse_partition_piece(const uint32_t *perm, void *S, bool packed, v
         });
         if (rc) return rc;
     }
-    if (packed)
+    if (S.packed)
         k_inverse_partition<true><<<grid, kPartThreads, smem, s>>>(
-            perm, S, static_cast<uint2 *>(pairs), fill, buckets, blog, log2m, j_first);
+            perm, S.S, static_cast<uint2 *>(pairs), fill, buckets, blog, log2m, j_first, kappa);
     else
         k_inverse_partition<false><<<grid, kPartThreads, smem, s>>>(
-            perm, S, static_cast<uint2 *>(pairs), fill, buckets, blog, log2m, j_first);
+            perm, S.S, static_cast<uint2 *>(pairs), fill, buckets, blog, log2m, j_first, kappa);
     return launch_status();
 }
 
@@ -439,25 +439,25 @@ int launch_inverse_scatter(const void *pairs, uint32_t *Q, size_t total, int log
     return launch_status();
 }
 
-int launch_inverse_partitioned(const uint32_t *perm, void *S, bool packed, uint32_t *Q, void *pairs,
-                               uint32_t *fill, size_t total, int log2m, cudaStream_t s) {
+int launch_inverse_partitioned(const uint32_t *perm, LevelRecords S, uint32_t *Q, void *pairs,
+                               uint32_t *fill, size_t total, int log2m, int kappa, cudaStream_t s) {
     int rc;
     if ((rc = launch_inverse_clear(fill, total, s))) return rc;
-    if ((rc = launch_inverse_partition_piece(perm, S, packed, pairs, fill, total, 0, total, log2m, s)))
+    if ((rc = launch_inverse_partition_piece(perm, S, pairs, fill, total, 0, total, log2m, kappa, s)))
         return rc;
     return launch_inverse_scatter(pairs, Q, total, log2m, s);
 }
 
-int launch_inverse(const uint32_t *perm, void *S, bool packed, uint32_t *Q, size_t total, int log2m,
+int launch_inverse(const uint32_t *perm, LevelRecords S, uint32_t *Q, size_t total, int log2m, int kappa,
                    cudaStream_t s) {
     size_t quads = total / 4;
     const uint4 *P4 = reinterpret_cast<const uint4 *>(perm);
-    if (packed) k_inverse<true><<<grid_for(quads), kThreads, 0, s>>>(P4, S, Q, quads, log2m);
-    else k_inverse<false><<<grid_for(quads), kThreads, 0, s>>>(P4, S, Q, quads, log2m);
+    if (S.packed) k_inverse<true><<<grid_for(quads), kThreads, 0, s>>>(P4, S.S, Q, quads, log2m, kappa);
+    else k_inverse<false><<<grid_for(quads), kThreads, 0, s>>>(P4, S.S, Q, quads, log2m, kappa);
     return launch_status();
 }
 
-int launch_full_label(const void *S, bool packed, const uint32_t *Q, unsigned long long *Wd, size_t total,
+int launch_full_label(LevelRecords S, const uint32_t *Q, unsigned long long *Wd, size_t total,
                       int log2m, BitsLayout L, int out_stage, const uint32_t *gate,
                       cudaStream_t s) {
     int grid = 0;
@@ -466,9 +466,9 @@ int launch_full_label(const void *S, bool packed, const uint32_t *Q, unsigned lo
     size_t need = (total / 2 + kThreads - 1) / kThreads;
     if (size_t(grid) > need) grid = int(need);
     int passes = log2m - 2;
-    void *args[] = {(void *)&S, (void *)&Q, (void *)&Wd, (void *)&total, (void *)&log2m,
+    void *args[] = {(void *)&S.S, (void *)&S.P, (void *)&Q, (void *)&Wd, (void *)&total, (void *)&log2m,
                     (void *)&passes, (void *)&L, (void *)&out_stage, (void *)&gate};
-    const void *kernel = packed ? (const void *)k_full_label<true> : (const void *)k_full_label<false>;
+    const void *kernel = S.packed ? (const void *)k_full_label<true> : (const void *)k_full_label<false>;
     if (cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(kThreads), args, 0, s) != cudaSuccess) {
         cudaGetLastError();
         return BENES_ERR_CUDA;
@@ -476,8 +476,8 @@ int launch_full_label(const void *S, bool packed, const uint32_t *Q, unsigned lo
     return launch_status();
 }
 
-int launch_split(const void *S, bool packed, const uint32_t *Q, void *Sn, bool next_packed, uint32_t *Qn,
-                 size_t total, int log2m, BitsLayout L, int in_stage, int out_stage, const uint32_t *gate,
+int launch_split(LevelRecords S, const uint32_t *Q, LevelRecords Sn, uint32_t *Qn,
+                 size_t total, int log2m, int kappa, BitsLayout L, int in_stage, int out_stage, const uint32_t *gate,
                  cudaStream_t s) {
     const uint32_t pairs = uint32_t(total / 4);                  // two switches per thread
     const uint4 *Q4 = reinterpret_cast<const uint4 *>(Q);
@@ -488,14 +488,14 @@ int launch_split(const void *S, bool packed, const uint32_t *Q, void *Sn, bool n
     uint32_t rounds = stream_rounds(pairs, kThreads);
     if (log2m >= 20 && log2m <= 22 && rounds > (1u << (log2m - 20))) rounds = 1u << (log2m - 20);
     const unsigned grid = unsigned((size_t(pairs) + size_t(kThreads) * rounds - 1) / (size_t(kThreads) * rounds));
-    if (packed)          // a packed level is followed by packed levels only
-        k_split<true, true><<<grid, kThreads, 0, s>>>(S, Q4, Sn, Qn, pairs, log2m, L, in_stage,
+    if (S.packed)          // a packed level is followed by packed levels only
+        k_split<true, true><<<grid, kThreads, 0, s>>>(S.S, S.P, Q4, Sn.S, Sn.P, Qn, pairs, log2m, kappa, L, in_stage,
                                                        out_stage, gate, rounds);
-    else if (next_packed)
-        k_split<false, true><<<grid, kThreads, 0, s>>>(S, Q4, Sn, Qn, pairs, log2m, L, in_stage,
+    else if (Sn.packed)
+        k_split<false, true><<<grid, kThreads, 0, s>>>(S.S, S.P, Q4, Sn.S, Sn.P, Qn, pairs, log2m, kappa, L, in_stage,
                                                         out_stage, gate, rounds);
     else
-        k_split<false, false><<<grid, kThreads, 0, s>>>(S, Q4, Sn, Qn, pairs, log2m, L, in_stage,
+        k_split<false, false><<<grid, kThreads, 0, s>>>(S.S, S.P, Q4, Sn.S, Sn.P, Qn, pairs, log2m, kappa, L, in_stage,
                                                          out_stage, gate, rounds);
     return launch_status();
 }

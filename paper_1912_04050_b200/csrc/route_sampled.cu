@@ -49,14 +49,6 @@ constexpr int kThreads = 256;
 constexpr int kWalkThreads = 128;             // a CTA's slots are free again when its longest walk ends
 constexpr int kListThreads = 1024;
 
-__device__ __forceinline__ uint32_t ruler_slot(uint32_t group, uint32_t salt, uint32_t kmask) {
-    uint32_t h = group * 0x9E3779B1u + salt;
-    h ^= h >> 15;
-    h *= 0x85EBCA6Bu;
-    h ^= h >> 13;
-    return h & kmask;
-}
-
 __device__ __forceinline__ bool gate_raised(const uint32_t *gate) {
     return *reinterpret_cast<const volatile uint32_t *>(gate) != 0u;
 }
@@ -64,15 +56,15 @@ __device__ __forceinline__ bool gate_raised(const uint32_t *gate) {
 // Step 2.  rulers = T / k threads, launched in index order so that the blocks
 // being walked at any moment are neighbours in memory.
 //
-// Wide records: the walker loads the record (16 B) and claims its owner word
-// with a compare-and-swap.  Packed records: one 64-bit atomic AND with
-// (my code << 2m | ones) returns the two P values and the previous owner and,
-// if the switch was free (owner all ones), leaves my code there; if it was
-// taken, the AND has mangled the other walker's code, and since nobody but the
-// two of us ever touches this switch, writing the old word back repairs it.
+// Wide records: one 64-bit exchange of the claim record for my code returns the
+// two P values, or the code of the walker that was here first.  Packed records: one
+// 64-bit atomic AND with (my code << 2m | ones) returns the two P values and the
+// previous owner and, if the switch was free (owner all ones), leaves my code
+// there.  If the switch was taken, the other walker's code is gone, and since nobody
+// but the two of us ever touches this switch, writing the old word back repairs it.
 template <bool PACKED>
 __global__ void __launch_bounds__(kWalkThreads)
-k_walk(void *__restrict__ Sv, const uint32_t *__restrict__ Q, uint4 *__restrict__ rec,
+k_walk(void *__restrict__ Sv, const uint32_t *__restrict__ P, const uint32_t *__restrict__ Q, uint4 *__restrict__ rec,
        uint32_t rulers, int m, int kappa, uint32_t salt, uint32_t cap,
        uint32_t *__restrict__ gate) {
     const uint32_t rho = blockIdx.x * kWalkThreads + threadIdx.x;
@@ -84,7 +76,6 @@ k_walk(void *__restrict__ Sv, const uint32_t *__restrict__ Q, uint4 *__restrict_
     uint32_t j = 2u * t0 + side0;
     const uint32_t base = j & ~mmask;
     uint32_t fwd = j, part = kUnowned, peer = rho ^ 1u, hops = 0;
-    uint4 *S16 = static_cast<uint4 *>(Sv);
     unsigned long long *S8 = static_cast<unsigned long long *>(Sv);
     // packed owners are local to the block: its first ruler output is base >> kappa
     const uint32_t rho_base = base >> kappa;
@@ -100,9 +91,8 @@ k_walk(void *__restrict__ Sv, const uint32_t *__restrict__ Q, uint4 *__restrict_
         else w = __ldcg(S8 + t0);
         p = uint32_t(w >> (side0 ? 0 : m)) & mmask;
     } else {
-        const uint4 r = __ldcg(S16 + t0);
-        if (!side0) reinterpret_cast<uint32_t *>(S16 + t0)[2] = rho << 1;
-        p = BENES_GUARD(side0 ? r.x : r.y, mmask);
+        // (the ruler switch carries its even-side walker's code from the start)
+        p = BENES_GUARD(__ldcs(P + (j ^ 1u)), mmask);
     }
     uint32_t q = BENES_GUARD(__ldcg(Q + base + (p ^ 1u)), mmask);
     for (;;) {
@@ -132,14 +122,15 @@ k_walk(void *__restrict__ Sv, const uint32_t *__restrict__ Q, uint4 *__restrict_
                 peer = rho_base + (prev >> 1);
             }
         } else {
-            const uint4 r = __ldcg(S16 + t);
-            p = BENES_GUARD(side ? r.x : r.y, mmask);
+            const unsigned long long w = atomicExch(S8 + t, kClaimed | (unsigned long long)((rho << 1) | side));
+            met = (w & kClaimed) != 0ull;
+            // (of a claimed record the lower word is a code: masked, the gather is harmless)
+            p = uint32_t(side ? w : (w >> 32)) & mmask;
             qn = BENES_GUARD(__ldcg(Q + base + (p ^ 1u)), mmask);
-            uint32_t prev = r.z;
-            if (prev == kUnowned)
-                prev = atomicCAS(reinterpret_cast<uint32_t *>(S16 + t) + 2, kUnowned, (rho << 1) | side);
-            met = prev != kUnowned;
-            if (met) peer = prev >> 1;
+            if (met) {
+                __stcg(S8 + t, w);
+                peer = uint32_t(w) >> 1;
+            }
         }
         if (met) break;                                           // met the walker from the other end
         fwd = min(fwd, j);
@@ -487,7 +478,7 @@ int launch_list_label_rec(const uint4 *rec, uint32_t *cb, uint32_t count, int be
 // they stop where they meet.  p_even / p_odd = P[2t] / P[2t+1], which the
 // caller holds already, start the two chains.
 template <bool PACKED>
-__device__ __forceinline__ uint32_t loop_colour(const void *S, const uint32_t *Q, uint32_t t, uint32_t base,
+__device__ __forceinline__ uint32_t loop_colour(const void *S, const uint32_t *P, const uint32_t *Q, uint32_t t, uint32_t base,
                                                 uint32_t p_even, uint32_t p_odd, int m, uint32_t mmask,
                                                 uint32_t cap, uint32_t *gate) {
     const uint32_t j0 = 2u * t;
@@ -508,8 +499,8 @@ __device__ __forceinline__ uint32_t loop_colour(const void *S, const uint32_t *Q
             break;
         }
         if ((hops & 63u) == 0u && gate_raised(gate)) break;
-        pf = rec_p<PACKED>(S, f ^ 1u, m);
-        pb = rec_p<PACKED>(S, bk, m);
+        pf = rec_p<PACKED>(S, P, f ^ 1u, m);
+        pb = rec_p<PACKED>(S, P, bk, m);
     }
     return mn & 1u;
 }
@@ -528,8 +519,8 @@ __device__ __forceinline__ uint32_t owner_colour(const uint32_t *cb, uint32_t co
 // the records from the relabelled stage.
 template <bool PACKED, bool NEXT_PACKED>
 __global__ void __launch_bounds__(kThreads)
-k_colour(const void *__restrict__ S, const uint32_t *__restrict__ Q,
-         const uint32_t *__restrict__ cb, void *__restrict__ Sn, uint32_t pairs,
+k_colour(const void *__restrict__ S, const uint32_t *__restrict__ P, const uint32_t *__restrict__ Q,
+         const uint32_t *__restrict__ cb, void *__restrict__ Sn, uint32_t *__restrict__ Pn, uint32_t salt_next, uint32_t pairs,
          uint32_t rulers, int m, int kappa, BitsLayout L, int out_stage, uint32_t cap,
          uint32_t *__restrict__ gate, uint32_t rounds) {
     // a CTA takes `rounds` consecutive groups of blockDim.x pairs: the ruler bits
@@ -538,7 +529,7 @@ k_colour(const void *__restrict__ S, const uint32_t *__restrict__ Q,
     const uint32_t last = min(pairs, (blockIdx.x + 1u) * rounds * stride);
     const uint32_t mmask = (1u << m) - 1u;
     const uint32_t H = (mmask + 1) >> 1;
-    const uint32_t none = PACKED ? uint32_t(~0ull >> (2 * m)) : kUnowned;
+    const uint32_t none = PACKED ? uint32_t(~0ull >> (2 * m)) : 0u;
     // packed fields with 32-bit operations (m < 32): the owner starts at bit 2m of
     // the word, the next level's owner (all ones) at bit 2(m-1)
     const int s_own = 2 * m, s_next = 2 * (m - 1);
@@ -547,19 +538,19 @@ k_colour(const void *__restrict__ S, const uint32_t *__restrict__ Q,
     // the records of the next round are on their way while this one is coloured
     // (pairs is a multiple of 32: a warp stays together)
     uint32_t i = blockIdx.x * rounds * stride + threadIdx.x;
-    ulonglong2 w = make_ulonglong2(0, 0);
-    uint4 r0 = make_uint4(0, 0, 0, 0), r1 = r0;
+    ulonglong2 w = make_ulonglong2(0, 0);                       // packed records, or claim records
+    uint4 p4 = make_uint4(0, 0, 0, 0);                          // wide: the P values beside them
     if (i < last) {
-        if (PACKED) w = __ldcs(static_cast<const ulonglong2 *>(S) + i);
-        else { r0 = __ldcs(static_cast<const uint4 *>(S) + 2 * size_t(i)); r1 = __ldcs(static_cast<const uint4 *>(S) + 2 * size_t(i) + 1); }
+        w = __ldcs(static_cast<const ulonglong2 *>(S) + i);
+        if (!PACKED) p4 = __ldcs(reinterpret_cast<const uint4 *>(P) + i);
     }
     while (i < last) {
         const uint32_t inext = i + stride;
         ulonglong2 wn = make_ulonglong2(0, 0);
-        uint4 r0n = make_uint4(0, 0, 0, 0), r1n = r0n;
+        uint4 p4n = make_uint4(0, 0, 0, 0);
         if (inext < last) {
-            if (PACKED) wn = __ldcs(static_cast<const ulonglong2 *>(S) + inext);
-            else { r0n = __ldcs(static_cast<const uint4 *>(S) + 2 * size_t(inext)); r1n = __ldcs(static_cast<const uint4 *>(S) + 2 * size_t(inext) + 1); }
+            wn = __ldcs(static_cast<const ulonglong2 *>(S) + inext);
+            if (!PACKED) p4n = __ldcs(reinterpret_cast<const uint4 *>(P) + inext);
         }
         const uint32_t t = 2u * i;                              // first switch of the pair
         const uint32_t base = (2u * t) & ~mmask;
@@ -576,14 +567,14 @@ k_colour(const void *__restrict__ S, const uint32_t *__restrict__ Q,
             own0 = l0 != none; own1 = l1 != none;
             code0 = rb + l0; code1 = rb + l1;                    // owner local to the block -> global
         } else {
-            px0 = BENES_GUARD(r0.x, mmask); py0 = BENES_GUARD(r0.y, mmask); code0 = r0.z; own0 = code0 != none;
-            px1 = BENES_GUARD(r1.x, mmask); py1 = BENES_GUARD(r1.y, mmask); code1 = r1.z; own1 = code1 != none;
+            px0 = BENES_GUARD(p4.x, mmask); py0 = BENES_GUARD(p4.y, mmask); code0 = uint32_t(w.x); own0 = (w.x & kClaimed) != 0ull;
+            px1 = BENES_GUARD(p4.z, mmask); py1 = BENES_GUARD(p4.w, mmask); code1 = uint32_t(w.y); own1 = (w.y & kClaimed) != 0ull;
         }
         // all but the switches of loops without ruler are owned
         const uint32_t c0 = own0 ? owner_colour(cb, code0, rulers)
-                                 : loop_colour<PACKED>(S, Q, t, base, px0, py0, m, mmask, cap, gate);
+                                 : loop_colour<PACKED>(S, P, Q, t, base, px0, py0, m, mmask, cap, gate);
         const uint32_t c1 = own1 ? owner_colour(cb, code1, rulers)
-                                 : loop_colour<PACKED>(S, Q, t + 1u, base, px1, py1, m, mmask, cap, gate);
+                                 : loop_colour<PACKED>(S, P, Q, t + 1u, base, px1, py1, m, mmask, cap, gate);
         // a warp covers 64 switches: two words of the output-side stage
         store_stage_bits64(L.bits + L.word32(out_stage, (t - 2u * (threadIdx.x & 31u)) >> 5), c0, c1);
         const uint32_t r = (base >> 1) + (((t - (base >> 1)) >> 1));   // record of the upper half
@@ -594,10 +585,10 @@ k_colour(const void *__restrict__ S, const uint32_t *__restrict__ Q,
             Sn8[r] = make_uint2(u0 | (u1 << (m - 1)) | ones_lo, (u1 >> (33 - m)) | ones_hi);
             Sn8[r + (H >> 1)] = make_uint2(d0 | (d1 << (m - 1)) | ones_lo, (d1 >> (33 - m)) | ones_hi);
         } else {
-            rec_write<false>(Sn, r, m - 1, u0, u1);
-            rec_write<false>(Sn, r + (H >> 1), m - 1, d0, d1);
+            rec_write<false>(Sn, Pn, r, m - 1, u0, u1, kappa, salt_next);
+            rec_write<false>(Sn, Pn, r + (H >> 1), m - 1, d0, d1, kappa, salt_next);
         }
-        w = wn; r0 = r0n; r1 = r1n;
+        w = wn; p4 = p4n;
         i = inext;
     }
 }
@@ -655,9 +646,9 @@ int sampled_scratch_reset(const SampledScratch &sc, size_t total, int kappa, cud
     return BENES_OK;
 }
 
-int sampled_label(void *S, bool packed, const uint32_t *Q, void *Sn, bool next_packed,
-                  const SampledScratch &sc, size_t total, int log2m, int kappa, uint32_t salt,
-                  uint32_t cap, int walk_pairs, BitsLayout L, int out_stage, uint32_t *gate, cudaStream_t s) {
+int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const SampledScratch &sc, size_t total,
+                  int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage,
+                  uint32_t *gate, cudaStream_t s) {
     const uint32_t R = uint32_t(total >> kappa);
     const unsigned rgrid = (R + kThreads - 1) / kThreads;
     {
@@ -668,11 +659,11 @@ int sampled_label(void *S, bool packed, const uint32_t *Q, void *Sn, bool next_p
         // lasts as long as its longest thread and one walker per thread is faster.  Four and
         // eight walkers per thread measured slower (0.60 and 0.90 ms).
         const bool pair = walk_pairs == 2 || (walk_pairs == 1 && size_t(R >> 1) >= size_t(sm_count()) * 2048);
-        if (packed && pair)
+        if (S.packed && pair)
             k_walk_multi<1><<<((R >> 1) + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s>>>(
-                static_cast<unsigned long long *>(S), Q, sc.rec, R >> 1, log2m, kappa, salt, cap, gate);
-        else if (packed) k_walk<true><<<wgrid, kWalkThreads, 0, s>>>(S, Q, sc.rec, R, log2m, kappa, salt, cap, gate);
-        else k_walk<false><<<wgrid, kWalkThreads, 0, s>>>(S, Q, sc.rec, R, log2m, kappa, salt, cap, gate);
+                static_cast<unsigned long long *>(S.S), Q, sc.rec, R >> 1, log2m, kappa, salt, cap, gate);
+        else if (S.packed) k_walk<true><<<wgrid, kWalkThreads, 0, s>>>(S.S, S.P, Q, sc.rec, R, log2m, kappa, salt, cap, gate);
+        else k_walk<false><<<wgrid, kWalkThreads, 0, s>>>(S.S, S.P, Q, sc.rec, R, log2m, kappa, salt, cap, gate);
         int rc = launch_status();
         if (rc) return rc;
     }
@@ -740,14 +731,14 @@ int sampled_label(void *S, bool packed, const uint32_t *Q, void *Sn, bool next_p
         const uint32_t switches = uint32_t(total / 4);           // pairs of switches, one per thread
         const uint32_t rounds = stream_rounds(switches, kThreads);
         const unsigned grid = unsigned((size_t(switches) + size_t(kThreads) * rounds - 1) / (size_t(kThreads) * rounds));
-        if (packed)          // a packed level is followed by packed levels only
-            k_colour<true, true><<<grid, kThreads, 0, s>>>(S, Q, cb, Sn, switches, R, log2m, kappa, L,
+        if (S.packed)        // a packed level is followed by packed levels only
+            k_colour<true, true><<<grid, kThreads, 0, s>>>(S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
                                                             out_stage, cap, gate, rounds);
-        else if (next_packed)
-            k_colour<false, true><<<grid, kThreads, 0, s>>>(S, Q, cb, Sn, switches, R, log2m, kappa, L,
+        else if (Sn.packed)
+            k_colour<false, true><<<grid, kThreads, 0, s>>>(S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
                                                              out_stage, cap, gate, rounds);
         else
-            k_colour<false, false><<<grid, kThreads, 0, s>>>(S, Q, cb, Sn, switches, R, log2m, kappa, L,
+            k_colour<false, false><<<grid, kThreads, 0, s>>>(S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
                                                               out_stage, cap, gate, rounds);
         return launch_status();
     }
