@@ -11,16 +11,14 @@
 //      and the g-cycle through j^1 are mirror images (g(g(j)^1) = j^1), so the
 //      walker that leaves ruler switch T forwards and the walker that leaves
 //      the next ruler switch T' backwards run over the same switches from the
-//      two ends.  Each claims the switches it reaches with a compare-and-swap
-//      on the record's owner field and stops at the first switch the other one
+//      two ends.  Each claims the switches it reaches with one atomic operation
+//      on the switch's record and stops at the first switch the other one
 //      owns: together they touch every switch of the segment once.  A walker
 //      keeps the smallest output index on its own side of the switches it
-//      claimed (fwd), the smallest on the far side (part), and its partner
-//      (peer).  The claim stores (walker, side of arrival).  At the levels with
-//      packed records and enough rulers to fill the GPU a thread advances the
-//      two walkers of one ruler switch together (k_walk_multi).
+//      claimed (on the far side it is the same with the last bit flipped) and its partner
+//      (peer).  The claim stores (walker, side of arrival).
 //   3. k_combine: the segment of walker rho ends at ruler output peer^1 and
-//      its minimum is min(fwd[rho], part[peer]): one 64-bit (next, min) word
+//      its minimum is min(least[rho], least[peer] ^ 1): one 64-bit (next, min) word
 //      per ruler output -- the contracted list.
 //   4. The contracted list is labelled with the minimum of every cycle:
 //      lists of up to 2^14 words per block in one CTA's shared memory, longer
@@ -53,8 +51,8 @@ __device__ __forceinline__ bool gate_raised(const uint32_t *gate) {
     return *reinterpret_cast<const volatile uint32_t *>(gate) != 0u;
 }
 
-// Step 2.  rulers = T / k threads, launched in index order so that the blocks
-// being walked at any moment are neighbours in memory.
+// Step 2.  W walks per thread, one after another, launched in index order so that the blocks being
+// walked at any moment are neighbours in memory.
 //
 // Wide records: one 64-bit exchange of the claim record for my code returns the
 // two P values, or the code of the walker that was here first.  Packed records: one
@@ -62,171 +60,125 @@ __device__ __forceinline__ bool gate_raised(const uint32_t *gate) {
 // previous owner and, if the switch was free (owner all ones), leaves my code
 // there.  If the switch was taken, the other walker's code is gone, and since nobody
 // but the two of us ever touches this switch, writing the old word back repairs it.
-template <bool PACKED>
+//
+// What bounds a launch is the latency of a hop, a chain of two dependent accesses (0.7 us with the
+// GPU full of them), times the longest walk of a warp: walks have all lengths, with one walk per
+// thread 9 of 32 lanes are active on average.  With W = 2 a thread has both walks of a ruler
+// switch, fetches the first hop of the two at once, and a lane whose walk ends goes on with its
+// second one in the same round.
+template <bool PACKED, int W>
 __global__ void __launch_bounds__(kWalkThreads)
-k_walk(void *__restrict__ Sv, const uint32_t *__restrict__ P, const uint32_t *__restrict__ Q, uint4 *__restrict__ rec,
-       uint32_t rulers, int m, int kappa, uint32_t salt, uint32_t cap,
+k_walk(unsigned long long *__restrict__ S8, const uint32_t *__restrict__ P, const uint32_t *__restrict__ Q,
+       uint2 *__restrict__ rec, uint32_t rulers, int m, int kappa, uint32_t salt, uint32_t cap,
        uint32_t *__restrict__ gate) {
-    const uint32_t rho = blockIdx.x * kWalkThreads + threadIdx.x;
-    if (rho >= rulers) return;
+    uint32_t rho = (blockIdx.x * kWalkThreads + threadIdx.x) * W;
+    if (rho >= rulers) return;                                       // rulers is a multiple of W
     const uint32_t mmask = (1u << m) - 1u;
     const uint32_t kmask = (1u << kappa) - 1u;
-    const uint32_t group = rho >> 1, side0 = rho & 1u;
-    const uint32_t t0 = (group << kappa) | ruler_slot(group, salt, kmask);
-    uint32_t j = 2u * t0 + side0;
-    const uint32_t base = j & ~mmask;
-    uint32_t fwd = j, part = kUnowned, peer = rho ^ 1u, hops = 0;
-    unsigned long long *S8 = static_cast<unsigned long long *>(Sv);
+    // the rulers of a thread lie in one block (a block has at least 2^7 ruler outputs)
+    const uint32_t base = ((rho >> 1) << (kappa + 1)) & ~mmask;
     // packed owners are local to the block: its first ruler output is base >> kappa
     const uint32_t rho_base = base >> kappa;
     const int cshift = 2 * m;
     const unsigned long long low_ones = PACKED ? ((1ull << cshift) - 1ull) : 0ull;
     const uint32_t none8 = PACKED ? uint32_t(~0ull >> cshift) : 0u;
 
-    uint32_t p;                                                   // P[j^1]
-    if (PACKED) {
-        unsigned long long w;
-        // the ruler switch belongs to its even-side walker (nobody else claims it)
-        if (!side0) w = atomicAnd(S8 + t0, ((unsigned long long)((rho - rho_base) << 1) << cshift) | low_ones);
-        else w = __ldcg(S8 + t0);
-        p = uint32_t(w >> (side0 ? 0 : m)) & mmask;
-    } else {
-        // (the ruler switch carries its even-side walker's code from the start)
-        p = BENES_GUARD(__ldcs(P + (j ^ 1u)), mmask);
-    }
-    uint32_t q = BENES_GUARD(__ldcg(Q + base + (p ^ 1u)), mmask);
-    for (;;) {
-        j = base + q;
-        const uint32_t t = j >> 1, side = j & 1u, g = t >> kappa;
-        if ((t & kmask) == ruler_slot(g, salt, kmask)) {          // reached the next ruler
-            peer = (2u * g + side) ^ 1u;
-            break;
-        }
-        if (++hops > cap) {
-            *gate = 1u;
-            break;
-        }
-        if ((hops & 63u) == 0u && gate_raised(gate)) break;       // the level is relabelled anyway
-        uint32_t qn;
-        bool met;
-        if (PACKED) {
-            const unsigned long long mine = (unsigned long long)(((rho - rho_base) << 1) | side) << cshift;
-            const unsigned long long w = atomicAnd(S8 + t, mine | low_ones);
-            p = uint32_t(w >> (side ? 0 : m)) & mmask;
-            // next hop's gather, issued before the claim is looked at (harmless if we stop)
-            qn = BENES_GUARD(__ldcg(Q + base + (p ^ 1u)), mmask);
-            const uint32_t prev = uint32_t(w >> cshift);
-            met = prev != none8;
-            if (met) {
-                __stcg(S8 + t, w);                                // put the other walker's code back
-                peer = rho_base + (prev >> 1);
-            }
-        } else {
-            const unsigned long long w = atomicExch(S8 + t, kClaimed | (unsigned long long)((rho << 1) | side));
-            met = (w & kClaimed) != 0ull;
-            // (of a claimed record the lower word is a code: masked, the gather is harmless)
-            p = uint32_t(side ? w : (w >> 32)) & mmask;
-            qn = BENES_GUARD(__ldcg(Q + base + (p ^ 1u)), mmask);
-            if (met) {
-                __stcg(S8 + t, w);
-                peer = uint32_t(w) >> 1;
-            }
-        }
-        if (met) break;                                           // met the walker from the other end
-        fwd = min(fwd, j);
-        part = min(part, j ^ 1u);
-        q = qn;
-    }
-    rec[rho] = make_uint4(fwd, part, peer, 0u);
-}
-
-// Step 2, packed records, 2 G walkers per thread: the two ruler outputs of each of G
-// neighbouring ruler switches (the two walks of a switch leave it in opposite
-// directions).  A hop is a chain of two dependent L2 accesses and most lanes of a
-// warp are idle while its longest walk lasts; advancing a thread's walks together,
-// one hop each per round, overlaps their chains.  Same claims and records as
-// k_walk<true>.  The hop limit counts rounds.
-template <int G>
-__global__ void __launch_bounds__(kWalkThreads)
-k_walk_multi(unsigned long long *__restrict__ S8, const uint32_t *__restrict__ Q, uint4 *__restrict__ rec,
-             uint32_t groups, int m, int kappa, uint32_t salt, uint32_t cap, uint32_t *__restrict__ gate) {
-    constexpr int W = 2 * G;
-    const uint32_t group0 = (blockIdx.x * kWalkThreads + threadIdx.x) * G;     // groups is a multiple of G
-    if (group0 >= groups) return;
-    const uint32_t mmask = (1u << m) - 1u;
-    const uint32_t kmask = (1u << kappa) - 1u;
-    const int cshift = 2 * m;
-    const unsigned long long low_ones = (1ull << cshift) - 1ull;
-    const uint32_t none8 = uint32_t(~0ull >> cshift);
-    const uint32_t rho0 = 2u * group0;                               // walker i is ruler output rho0 + i
-    // G neighbouring groups lie in one block (a block has at least 2^7 ruler outputs)
-    const uint32_t base = (2u * (group0 << kappa)) & ~mmask;
-    const uint32_t rho_base = base >> kappa;
-    uint32_t q[W], fwd[W], part[W], peer[W];
+    // where each walk goes first: g(j) of its ruler output j needs P[j^1]
+    uint32_t q[W];
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-        const uint32_t group = group0 + g;
+    for (int i = 0; i < (W > 1 ? W / 2 : 1); ++i) {
+        const uint32_t group = (rho >> 1) + uint32_t(i);
         const uint32_t t0 = (group << kappa) | ruler_slot(group, salt, kmask);
-        // the ruler switch belongs to its even-side walker; the claim returns both P values
-        const unsigned long long w0 = atomicAnd(S8 + t0, ((unsigned long long)((2u * group - rho_base) << 1) << cshift) | low_ones);
-        q[2 * g] = BENES_GUARD(__ldcg(Q + base + ((uint32_t(w0 >> m) & mmask) ^ 1u)), mmask);     // needs P[2 t0 + 1]
-        q[2 * g + 1] = BENES_GUARD(__ldcg(Q + base + ((uint32_t(w0) & mmask) ^ 1u)), mmask);      // needs P[2 t0]
-        fwd[2 * g] = 2u * t0; fwd[2 * g + 1] = 2u * t0 + 1u;
-        part[2 * g] = part[2 * g + 1] = kUnowned;
-        peer[2 * g] = (2u * group) ^ 1u; peer[2 * g + 1] = 2u * group;
+        uint32_t pe, po;
+        if (PACKED) {
+            // the ruler switch belongs to its even-side walker (nobody else claims it)
+            const unsigned long long w = (W > 1 || !(rho & 1u))
+                ? atomicAnd(S8 + t0, ((unsigned long long)((2u * group - rho_base) << 1) << cshift) | low_ones)
+                : __ldcg(S8 + t0);
+            pe = uint32_t(w) & mmask;
+            po = uint32_t(w >> m) & mmask;
+        } else {
+            // (the ruler switch carries its even-side walker's code from the start)
+            const uint2 p = __ldcs(reinterpret_cast<const uint2 *>(P) + t0);
+            pe = BENES_GUARD(p.x, mmask);
+            po = BENES_GUARD(p.y, mmask);
+        }
+        if (W > 1) {
+            q[2 * i] = BENES_GUARD(__ldcg(Q + base + (po ^ 1u)), mmask);
+            q[(2 * i + 1) % W] = BENES_GUARD(__ldcg(Q + base + (pe ^ 1u)), mmask);
+        } else {
+            q[0] = BENES_GUARD(__ldcg(Q + base + (((rho & 1u) ? pe : po) ^ 1u)), mmask);
+        }
     }
-    uint32_t active = (1u << W) - 1u, hops = 0;
-    while (active) {
-        if (++hops > cap) {
+    uint32_t walk = 0, hops = 0, rounds = 0;
+    uint32_t j = base + q[0];
+    uint32_t least = 2u * (((rho >> 1) << kappa) | ruler_slot(rho >> 1, salt, kmask)) + (rho & 1u);
+    for (;;) {
+        const uint32_t t = j >> 1, side = j & 1u, g = t >> kappa;
+        uint32_t peer = rho ^ 1u;
+        bool ends = true;
+        if ((t & kmask) == ruler_slot(g, salt, kmask)) {             // reached the next ruler
+            peer = (2u * g + side) ^ 1u;
+        } else if (++hops > cap) {
             *gate = 1u;
-            break;
-        }
-        if ((hops & 63u) == 0u && gate_raised(gate)) break;         // the level is relabelled anyway
-        unsigned long long w[W];
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-            w[i] = 0ull;
-            if (!((active >> i) & 1u)) continue;
-            const uint32_t j = base + q[i], t = j >> 1, side = j & 1u, g = t >> kappa;
-            if ((t & kmask) == ruler_slot(g, salt, kmask)) {        // reached the next ruler
-                peer[i] = (2u * g + side) ^ 1u;
-                active &= ~(1u << i);
+        } else {
+            uint32_t p, prev;
+            unsigned long long w;
+            bool met;
+            if (PACKED) {
+                w = atomicAnd(S8 + t, ((unsigned long long)(((rho - rho_base) << 1) | side) << cshift) | low_ones);
+                p = uint32_t(w >> (side ? 0 : m)) & mmask;
+                prev = rho_base + (uint32_t(w >> cshift) >> 1);
+                met = uint32_t(w >> cshift) != none8;
             } else {
-                w[i] = atomicAnd(S8 + t, ((unsigned long long)((((rho0 + i) - rho_base) << 1) | side) << cshift) | low_ones);
+                w = atomicExch(S8 + t, kClaimed | (unsigned long long)((rho << 1) | side));
+                p = uint32_t(side ? w : (w >> 32)) & mmask;          // (of a claimed record: some code, harmless)
+                prev = uint32_t(w) >> 1;
+                met = (w & kClaimed) != 0ull;
+            }
+            // next hop's gather, issued before the claim is looked at (harmless if we stop)
+            const uint32_t qn = BENES_GUARD(__ldcg(Q + base + (p ^ 1u)), mmask);
+            if (met) {                                               // the walker from the other end was here
+                __stcg(S8 + t, w);                                   // put its code back
+                peer = prev;
+            } else {
+                least = min(least, j);
+                j = base + qn;
+                ends = false;
             }
         }
-        uint32_t qn[W];
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-            qn[i] = 0u;
-            if (!((active >> i) & 1u)) continue;
-            const uint32_t side = q[i] & 1u;                        // base is even
-            const uint32_t p = uint32_t(w[i] >> (side ? 0 : m)) & mmask;
-            qn[i] = BENES_GUARD(__ldcg(Q + base + (p ^ 1u)), mmask);
+        if (W == 1 || (++rounds & 63u) == 0u) {
+            if (((W == 1 ? hops : rounds) & 63u) == 0u && gate_raised(gate)) break;      // the level is relabelled anyway
         }
+        if (ends) {
+            rec[rho] = make_uint2(least, peer);
+            if (W == 1 || ++walk == uint32_t(W)) break;
+            ++rho;
+            hops = 0;
+            uint32_t qk = q[0];
 #pragma unroll
-        for (int i = 0; i < W; ++i) {
-            if (!((active >> i) & 1u)) continue;
-            const uint32_t j = base + q[i];
-            const uint32_t prev = uint32_t(w[i] >> cshift);
-            if (prev != none8) {                                    // met the walker from the other end
-                __stcg(S8 + (j >> 1), w[i]);                        // put its code back
-                peer[i] = rho_base + (prev >> 1);
-                active &= ~(1u << i);
-            } else {
-                fwd[i] = min(fwd[i], j);
-                part[i] = min(part[i], j ^ 1u);
-                q[i] = qn[i];
-            }
+            for (int i = 1; i < W; ++i) qk = walk == uint32_t(i) ? q[i] : qk;
+            j = base + qk;
+            least = 2u * (((rho >> 1) << kappa) | ruler_slot(rho >> 1, salt, kmask)) + (rho & 1u);
         }
     }
-#pragma unroll
-    for (int i = 0; i < W; ++i) rec[rho0 + i] = make_uint4(fwd[i], part[i], peer[i], 0u);
 }
 
-// Step 3.
+// Step 3.  A switch walker's record is (minimum, peer): the outputs on the far side of the switches it
+// claimed are the ones it stood on with the last bit flipped, and so is their minimum.  (That counts
+// the far side of its own ruler switch too, which is where the other walker's segment ends.)
 __global__ void __launch_bounds__(kThreads)
-k_combine(const uint4 *__restrict__ rec, unsigned long long *__restrict__ W, uint32_t rulers) {
+k_combine(const uint2 *__restrict__ rec, unsigned long long *__restrict__ W, uint32_t rulers) {
+    const uint32_t rho = blockIdx.x * kThreads + threadIdx.x;
+    if (rho >= rulers) return;
+    const uint2 a = rec[rho];
+    const uint32_t peer = BENES_GUARD_BELOW(a.y, rulers, rho);
+    W[rho] = make_word(peer ^ 1u, min(a.x, __ldg(&rec[peer].x) ^ 1u));
+}
+
+// The same for walks over a list, whose far sides have a minimum of their own.
+__global__ void __launch_bounds__(kThreads)
+k_combine_list(const uint4 *__restrict__ rec, unsigned long long *__restrict__ W, uint32_t rulers) {
     const uint32_t rho = blockIdx.x * kThreads + threadIdx.x;
     if (rho >= rulers) return;
     const uint4 a = rec[rho];
@@ -415,12 +367,12 @@ int launch_list_label(unsigned long long *W, uint32_t count, int beta, uint32_t 
 // Steps 3 and 4 in one kernel for a level whose blocks have at most 2^18 outputs
 // and lists that fit one CTA (no sampling of the list): the CTA forms its
 // block's list words from the walk records, (next, min) = (peer ^ 1,
-// min(fwd[rho], part[peer])), as 14 + 18 bit, both local to the block, labels
+// min(least[rho], least[peer] ^ 1)), as 14 + 18 bit, both local to the block, labels
 // them by synchronous pointer jumping and writes the parity bits.  Indices a
 // raised gate may have left undefined are masked into the block.
 template <int PER>
 __global__ void __launch_bounds__(kListThreads)
-k_list_label_rec(const uint4 *__restrict__ rec, uint32_t *__restrict__ cb, int log2b, int m) {
+k_list_label_rec(const uint2 *__restrict__ rec, uint32_t *__restrict__ cb, int log2b, int m) {
     extern __shared__ uint32_t sw[];
     constexpr uint32_t kNext = (1u << kListSmemLog2) - 1u;
     const uint32_t B = 1u << log2b, bmask = B - 1u, mmask = (1u << m) - 1u;
@@ -429,10 +381,9 @@ k_list_label_rec(const uint4 *__restrict__ rec, uint32_t *__restrict__ cb, int l
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
         const uint32_t e = tid + uint32_t(i) * T;
-        const uint4 a = __ldcs(rec + base + e);
-        const uint32_t peer = a.z & bmask;
-        const uint4 b = __ldg(rec + base + peer);
-        sw[e] = (peer ^ 1u) | ((min(a.x, b.y) & mmask) << kListSmemLog2);
+        const uint2 a = __ldcs(rec + base + e);
+        const uint32_t peer = a.y & bmask;
+        sw[e] = (peer ^ 1u) | ((min(a.x, __ldg(&rec[base + peer].x) ^ 1u) & mmask) << kListSmemLog2);
     }
     __syncthreads();
     uint32_t v[PER];
@@ -457,7 +408,7 @@ k_list_label_rec(const uint4 *__restrict__ rec, uint32_t *__restrict__ cb, int l
 }
 
 template <int PER>
-int launch_list_label_rec(const uint4 *rec, uint32_t *cb, uint32_t count, int beta, int m, cudaStream_t s) {
+int launch_list_label_rec(const uint2 *rec, uint32_t *cb, uint32_t count, int beta, int m, cudaStream_t s) {
     static OncePerDevice configured;
     {
         const int rc = configured.run([]() -> int {
@@ -650,20 +601,22 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
                   int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage,
                   uint32_t *gate, cudaStream_t s) {
     const uint32_t R = uint32_t(total >> kappa);
+    uint2 *walk_rec = reinterpret_cast<uint2 *>(sc.rec);
     const unsigned rgrid = (R + kThreads - 1) / kThreads;
     {
         ProfileScope ps(kWalk, s);
-        const unsigned wgrid = (R + kWalkThreads - 1) / kWalkThreads;
-        // Two walkers per thread pay once the halved number of threads still fills the GPU
-        // (C4, cache-resident levels: 0.52-0.57 instead of 0.55-0.63 ms); below that the launch
-        // lasts as long as its longest thread and one walker per thread is faster.  Four and
-        // eight walkers per thread measured slower (0.60 and 0.90 ms).
-        const bool pair = walk_pairs == 2 || (walk_pairs == 1 && size_t(R >> 1) >= size_t(sm_count()) * 2048);
-        if (S.packed && pair)
-            k_walk_multi<1><<<((R >> 1) + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s>>>(
-                static_cast<unsigned long long *>(S.S), Q, sc.rec, R >> 1, log2m, kappa, salt, cap, gate);
-        else if (S.packed) k_walk<true><<<wgrid, kWalkThreads, 0, s>>>(S.S, S.P, Q, sc.rec, R, log2m, kappa, salt, cap, gate);
-        else k_walk<false><<<wgrid, kWalkThreads, 0, s>>>(S.S, S.P, Q, sc.rec, R, log2m, kappa, salt, cap, gate);
+        // Two walks per thread pay once half of the threads still fills the GPU (2^26, levels 0-3:
+        // 2.05 / 1.70 / 1.20 / 0.70 -> 1.98 / 1.62 / 1.08 / 0.67 ms, cache-resident levels 0.62 -> 0.53);
+        // below that the launch lasts as long as its longest thread and one walk per thread is
+        // faster.  More are slower: the rulers that are being walked at any moment then
+        // spread over more blocks than the L2 holds (four: 0.95 ms per cache-resident level, eight: 1.6).
+        const bool two = walk_pairs == 2 || (walk_pairs == 1 && size_t(R >> 1) >= size_t(sm_count()) * 2048);
+#define BENES_WALK(PACKED, W)                                                                            \
+    k_walk<PACKED, W><<<(R / W + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s>>>(                 \
+        static_cast<unsigned long long *>(S.S), S.P, Q, walk_rec, R, log2m, kappa, salt, cap, gate)
+        if (S.packed) { if (two) BENES_WALK(true, 2); else BENES_WALK(true, 1); }
+        else { if (two) BENES_WALK(false, 2); else BENES_WALK(false, 1); }
+#undef BENES_WALK
         int rc = launch_status();
         if (rc) return rc;
     }
@@ -677,13 +630,13 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
     const bool from_records = depth == 0 && log2m <= 32 - kListSmemLog2;
     if (from_records) {
         ProfileScope ps(kListLabel, s);
-        int rc = beta <= 12 ? launch_list_label_rec<4>(sc.rec, cb, count, beta, log2m, s)
-               : beta == 13 ? launch_list_label_rec<8>(sc.rec, cb, count, beta, log2m, s)
-                            : launch_list_label_rec<16>(sc.rec, cb, count, beta, log2m, s);
+        int rc = beta <= 12 ? launch_list_label_rec<4>(walk_rec, cb, count, beta, log2m, s)
+               : beta == 13 ? launch_list_label_rec<8>(walk_rec, cb, count, beta, log2m, s)
+                            : launch_list_label_rec<16>(walk_rec, cb, count, beta, log2m, s);
         if (rc) return rc;
     } else {
         ProfileScope ps(kCombine, s);
-        k_combine<<<rgrid, kThreads, 0, s>>>(sc.rec, sc.list[0], R);
+        k_combine<<<rgrid, kThreads, 0, s>>>(walk_rec, sc.list[0], R);
         int rc = launch_status();
         if (rc) return rc;
     }
@@ -701,7 +654,7 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
         }
         {
             ProfileScope ps(kCombine, s);
-            k_combine<<<(next + kThreads - 1) / kThreads, kThreads, 0, s>>>(sc.rec, sc.list[d + 1], next);
+            k_combine_list<<<(next + kThreads - 1) / kThreads, kThreads, 0, s>>>(sc.rec, sc.list[d + 1], next);
             int rc = launch_status();
             if (rc) return rc;
         }
