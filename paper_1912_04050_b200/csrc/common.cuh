@@ -336,8 +336,7 @@ int launch_apply_stage(const uint32_t *bits, const void *x, void *y, int elem_by
                        int log2n, size_t batch, cudaStream_t s);
 
 // ---- payload apply, several stages per pass (apply_fused.cu) -----------------
-// `scratch` (batch * N elements) is needed when apply_fused_passes(log2n) > 1.
-int apply_fused_passes(int log2n);
+// `scratch` (batch * N elements) is needed above 2^13 elements per permutation.
 // With a pipe the first pass runs part by part as the parts of `in` arrive
 // (in_ready[i], recorded on another stream), and the parts of `out` the last
 // pass has finished are copied to out_host on the side stream.

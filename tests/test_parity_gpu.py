@@ -252,6 +252,26 @@ def test_apply_random_settings(n, dtype, apply_mode):
     assert np.array_equal(gpu_apply(bits, x, n), oracle.apply(bits, x, n))
 
 
+@pytest.mark.parametrize("n,batch", [(1, 5000), (4, 77), (6, 33), (9, 2401), (10, 1), (10, 1301), (11, 3), (12, 301), (13, 149),
+                                     (14, 5), (22, 1), (23, 1), (24, 1)])
+@pytest.mark.parametrize("dtype", [np.uint32, np.uint64])
+def test_apply_chunks_and_passes(n, batch, dtype):
+    """Chunks of 2^10 and 2^13 that hold several networks and end in a partial one, the largest block of
+    a chunk, one outer pass per side with its shortest runs and two; payload off a 16-byte boundary too."""
+    rng = np.random.default_rng(100 * n + batch)
+    bits = rng.integers(0, 2 ** 32, size=(batch, 2 * n - 1, max(1, (1 << n) // 64)), dtype=np.uint64).astype(np.uint32)
+    if n < 6:
+        bits &= np.uint32((1 << (1 << (n - 1))) - 1)
+    x = rng.integers(0, 2 ** 63, size=(batch, 1 << n), dtype=np.uint64).astype(dtype)
+    want = oracle.apply(bits, x, n)
+    assert np.array_equal(gpu_apply(bits, x, n), want)
+    moved = dev(np.concatenate([x.ravel()[:1], x.ravel()]))[1:]
+    out = torch.empty_like(moved)
+    binding.benes_apply_ex(dev(bits), moved, out, x.dtype.itemsize, n, batch)
+    torch.cuda.synchronize()
+    assert np.array_equal(host(out, dtype).reshape(x.shape), want)
+
+
 def test_apply_does_not_touch_input():
     n = 12
     perm = inputs.random_perm(n, 1)
