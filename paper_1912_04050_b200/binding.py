@@ -124,8 +124,15 @@ def _host_ptr(t, what: str) -> int:
     return t.ctypes.data        # numpy array
 
 
+# handle of the current device's current stream, without building a torch.cuda.Stream for every call (3 us)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device_index = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and _device_index is not None and torch.cuda.is_initialized():
+            return _raw_stream(_device_index())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -353,14 +360,16 @@ def benes_fused_log2m() -> int:
 def route(perm: torch.Tensor, stream=None) -> torch.Tensor:
     """perm: (N,) or (batch, N) CUDA tensor holding uint32 values (dtype int32 or uint32).
     Returns the switch bits as an int32 tensor of shape ([batch,] 2n-1, W)."""
-    N = perm.shape[-1]
+    shape = tuple(perm.shape)
+    N = shape[-1]
     log2n = N.bit_length() - 1
     if N < 2 or (1 << log2n) != N:
         raise ValueError("N must be a power of two >= 2")
-    batch = perm.numel() // N
-    W = max(1, N // 64)
-    bits = torch.empty(perm.shape[:-1] + (2 * log2n - 1, W), dtype=torch.int32, device=perm.device)
-    benes_route(perm, log2n, batch, bits, stream)
+    if perm.dtype is torch.int32:           # (sizes one by one and no dtype: the cheapest way to a new tensor)
+        bits = perm.new_empty(*shape[:-1], 2 * log2n - 1, (N >> 6) or 1)
+    else:
+        bits = perm.new_empty(*shape[:-1], 2 * log2n - 1, (N >> 6) or 1, dtype=torch.int32)
+    benes_route(perm, log2n, perm.numel() >> log2n, bits, stream)
     return bits
 
 

@@ -735,6 +735,159 @@ k_route_fused(const uint32_t *__restrict__ P, int records, uint32_t *__restrict_
     fused_levels<Cfg>(sm, out, logs);
 }
 
+// ---- few outputs in all ---------------------------------------------------------------------
+// When every thread of the GPU could have a switch to itself, the time of a call is its chain of dependent
+// steps, and the labelling with the shortest one is pointer jumping over all outputs: one thread per
+// switch, one barrier per pass, and from sub-blocks of 64 down a warp in registers (a switch, then an output,
+// per lane; jumps by shuffle).  One permutation of 2^10: 22.8 -> 10.5 us; 32 of 2^6:
+// 8.7 -> 4 us; 290 of 2^10 (half of the GPU's threads): 43 -> 17 us.  From about twice the GPU's threads on the
+// kernels above are faster, which issue fewer instructions (5000 of 2^8: 37 us either way).
+
+// The levels of sub-blocks of 2^ls0 <= 32 outputs and less of 32 neighbouring outputs: p = the lane's entry, gathers
+// by shuffle, the inverse through the group's 32 entries of Q, which only this warp touches.  r = index of the
+// group in the CTA.
+__device__ __forceinline__ void few_tail32(uint32_t p, uint32_t r, uint16_t *Q, const FusedOut &out, int ls0) {
+    constexpr uint32_t kAll = 0xFFFFFFFFu;
+    const int n = out.n, lane = int(threadIdx.x & 31u);
+#pragma unroll
+    for (int ls = 5; ls >= 2; --ls) {
+        if (ls > ls0) continue;
+        const uint32_t smask = (1u << ls) - 1u, sb = uint32_t(lane) & ~smask;
+        const int level = n - ls;
+        Q[sb + p] = uint16_t(uint32_t(lane) & smask);
+        __syncwarp();
+        const uint32_t q = Q[lane];
+        __syncwarp();
+        const uint32_t p1 = __shfl_xor_sync(kAll, p, 1);
+        uint32_t next = sb + __shfl_sync(kAll, q, int(sb + (p1 ^ 1u))), least = uint32_t(lane);
+#pragma unroll
+        for (int pass = 0; pass < ls - 1; ++pass) {          // cycles of up to 2^(ls-1) outputs
+            const uint32_t m = __shfl_sync(kAll, least, int(next));
+            next = __shfl_sync(kAll, next, int(next));
+            least = min(least, m);
+        }
+        const uint32_t c = least & 1u;
+        // switch `lane` (< 16): colour of its even output; of the output its even input feeds
+        const uint32_t ce = __shfl_sync(kAll, c, (lane & 15) * 2);
+        const uint32_t out_half = __ballot_sync(kAll, int(ce)) & 0xFFFFu;
+        const uint32_t qe = __shfl_sync(kAll, q, (lane & 15) * 2);
+        const uint32_t ci = __shfl_sync(kAll, c, int((uint32_t((lane & 15) * 2) & ~smask) + qe));
+        const uint32_t in_half = __ballot_sync(kAll, int(ci)) & 0xFFFFu;
+        if (lane == 0) {
+            out.store16(2 * n - 2 - level, r, out_half);
+            out.store16(level, r, in_half);
+        }
+        // position dl of the upper (lower) half takes the colour-0 (1) output of switch tl
+        const uint32_t H = 1u << (ls - 1), dl = uint32_t(lane) & smask, tl = dl & (H - 1u), lower = dl >> (ls - 1);
+        const uint32_t c2 = __shfl_sync(kAll, c, int(sb + 2u * tl));
+        p = __shfl_sync(kAll, p, int(sb + 2u * tl + (c2 ^ lower))) >> 1;
+    }
+    const uint32_t mid = __ballot_sync(kAll, int(__shfl_sync(kAll, p, (lane & 15) * 2) & 1u)) & 0xFFFFu;
+    if (lane == 0) out.store16(n - 1, r, mid);
+}
+
+template <int LOGC>
+__global__ void __launch_bounds__((1 << LOGC) / 2)
+k_route_few(const uint32_t *__restrict__ P, uint32_t *__restrict__ bits, int n, size_t total) {
+    constexpr uint32_t C = 1u << LOGC, kAll = 0xFFFFFFFFu;
+    __shared__ uint32_t W[C];                  // (minimum << 16 | next) of every output
+    __shared__ uint32_t Q32[C / 2], Pn32[C / 2];
+    uint16_t *Q = reinterpret_cast<uint16_t *>(Q32), *Pn = reinterpret_cast<uint16_t *>(Pn32);
+    __shared__ uint32_t cw[C / 64];
+    FusedOut out;
+    out.bits = bits;
+    out.n = n;
+    out.flat0 = size_t(blockIdx.x) << LOGC;
+    out.valid = uint32_t(total - out.flat0 < size_t(C) ? total - out.flat0 : size_t(C));
+    const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5, j = 2u * t;
+    const uint32_t nmask = (1u << n) - 1u;
+    uint32_t p0 = j & nmask, p1 = (j + 1u) & nmask;            // padding: the identity
+    if (j < out.valid) {                                       // (valid is even)
+        p0 = BENES_GUARD(P[out.flat0 + j], nmask);
+        p1 = BENES_GUARD(P[out.flat0 + j + 1], nmask);
+    }
+    int logs = n;
+    for (; logs > 6; --logs) {
+        const int level = n - logs;
+        const uint32_t smask = (1u << logs) - 1u, sb = j & ~smask, H = (smask + 1u) >> 1;
+        Q[sb + p0] = uint16_t(j);
+        Q[sb + p1] = uint16_t(j + 1u);
+        __syncthreads();
+        const uint32_t q0 = BENES_GUARD(uint32_t(Q[j]), C - 1u);
+        uint32_t w0 = (j << 16) | BENES_GUARD(uint32_t(Q[sb + (p1 ^ 1u)]), C - 1u);
+        uint32_t w1 = ((j + 1u) << 16) | BENES_GUARD(uint32_t(Q[sb + (p0 ^ 1u)]), C - 1u);
+        *reinterpret_cast<uint2 *>(W + j) = make_uint2(w0, w1);
+        __syncthreads();
+        // in place: a word always holds the minimum of the path up to, but excluding, its next; a cycle has
+        // at most S/2 outputs
+        volatile uint32_t *Wv = W;
+        for (int pass = 1; pass < logs; ++pass) {
+            const uint32_t v0 = Wv[w0 & 0xFFFFu], v1 = Wv[w1 & 0xFFFFu];
+            w0 = (v0 & 0xFFFFu) | min(w0 & 0xFFFF0000u, v0 & 0xFFFF0000u);
+            w1 = (v1 & 0xFFFFu) | min(w1 & 0xFFFF0000u, v1 & 0xFFFF0000u);
+            Wv[j] = w0;
+            Wv[j + 1u] = w1;
+            __syncthreads();
+        }
+        const uint32_t c = (w0 >> 16) & 1u;
+        const uint32_t word = __ballot_sync(kAll, int(c));
+        if (lane == 0) cw[warp] = word;
+        const uint32_t at0 = sb + ((j - sb) >> 1);
+        Pn[at0] = uint16_t((c ? p1 : p0) >> 1);
+        Pn[at0 + H] = uint16_t((c ? p0 : p1) >> 1);
+        __syncthreads();
+        const uint32_t in = __ballot_sync(kAll, int(((cw[q0 >> 6] >> ((q0 >> 1) & 31u)) ^ q0) & 1u));
+        if (lane == 0 && 64u * warp < out.valid) {
+            *out.stage_word(2 * n - 2 - level, warp) = word;
+            *out.stage_word(level, warp) = in;
+        }
+        const uint32_t pp = Pn32[t];
+        p0 = pp & 0xFFFFu;
+        p1 = pp >> 16;
+    }
+    uint16_t *Qw = Q + 64u * warp;             // the warp's 64 outputs
+    __syncwarp();
+    if (logs == 6) {
+        // a lane has one of the sub-block's 32 switches; the (next, minimum) words of its two outputs share a register
+        const int level = n - 6;
+        Qw[p0] = uint16_t(2u * lane);
+        Qw[p1] = uint16_t(2u * lane + 1u);
+        __syncwarp();
+        const uint32_t q0 = BENES_GUARD(uint32_t(Qw[2u * lane]), 63u);
+        const uint32_t n0 = BENES_GUARD(uint32_t(Qw[p1 ^ 1u]), 63u), n1 = BENES_GUARD(uint32_t(Qw[p0 ^ 1u]), 63u);
+        __syncwarp();
+        uint32_t w = (n0 | ((2u * lane) << 8)) | ((n1 | ((2u * lane + 1u) << 8)) << 16);
+#pragma unroll
+        for (int pass = 0; pass < 5; ++pass) {
+            const uint32_t a0 = w & 0xFFu, a1 = (w >> 16) & 0xFFu;
+            const uint32_t v0 = (__shfl_sync(kAll, w, int(a0 >> 1)) >> ((a0 & 1u) * 16u)) & 0xFFFFu;
+            const uint32_t v1 = (__shfl_sync(kAll, w, int(a1 >> 1)) >> ((a1 & 1u) * 16u)) & 0xFFFFu;
+            w = ((v0 & 0xFFu) | min(w & 0xFF00u, v0 & 0xFF00u)) | (((v1 & 0xFFu) | min((w >> 16) & 0xFF00u, v1 & 0xFF00u)) << 16);
+        }
+        const uint32_t c = (w >> 8) & 1u;
+        const uint32_t word = __ballot_sync(kAll, int(c));
+        const uint32_t in = __ballot_sync(kAll, int((__shfl_sync(kAll, c, int(q0 >> 1)) ^ q0) & 1u));
+        if (lane == 0 && 64u * warp < out.valid) {
+            *out.stage_word(2 * n - 2 - level, warp) = word;
+            *out.stage_word(level, warp) = in;
+        }
+        few_tail32((c ? p1 : p0) >> 1, 2u * warp, Qw, out, 5);
+        few_tail32((c ? p0 : p1) >> 1, 2u * warp + 1u, Qw + 32, out, 5);
+    } else {
+        // several permutations of 2^n <= 32: from a switch to an output per lane
+        const uint32_t a0 = __shfl_sync(kAll, p0, int(lane >> 1)), a1 = __shfl_sync(kAll, p1, int(lane >> 1));
+        const uint32_t b0 = __shfl_sync(kAll, p0, int(16u + (lane >> 1))), b1 = __shfl_sync(kAll, p1, int(16u + (lane >> 1)));
+        few_tail32((lane & 1u) ? a1 : a0, 2u * warp, Qw, out, n);
+        few_tail32((lane & 1u) ? b1 : b0, 2u * warp + 1u, Qw + 32, out, n);
+    }
+}
+
+template <int LOGC>
+int launch_few(const uint32_t *P, size_t total, uint32_t *bits, int n, cudaStream_t s) {
+    k_route_few<LOGC><<<unsigned((total + (size_t(1) << LOGC) - 1) >> LOGC), (1 << LOGC) / 2, 0, s>>>(P, bits, n, total);
+    return launch_status();
+}
+
 // ---- a block of 2^16 outputs in a thread-block cluster of two CTAs ----------------
 // The level whose sub-block spans both CTAs runs on distributed shared memory:
 // CTA r keeps outputs / inputs [r 2^15, (r+1) 2^15) of P and Q, the owners of
@@ -995,6 +1148,12 @@ int launch_fused(const void *Pv, int records, size_t total, int log2m, uint32_t 
     if (first_block + blocks > (total >> log2m)) return BENES_ERR_BADARG;
     if (log2m == kClusterLog2M) return launch_cluster2(P, records, first_block, blocks, bits, log2n, s);
     const size_t first = first_block << log2m, end = first + (blocks << log2m);
+    // whole permutations of up to 2^11, and not more switches than the GPU has threads
+    if (records == 0 && log2m == log2n && log2m <= 11 && first == 0 && end / 2 <= size_t(sm_count()) * 2048) {
+        const int logc = log2m > 8 ? log2m : 8;
+        return logc == 8 ? launch_few<8>(P, end, bits, log2n, s) : logc == 9 ? launch_few<9>(P, end, bits, log2n, s)
+             : logc == 10 ? launch_few<10>(P, end, bits, log2n, s) : launch_few<11>(P, end, bits, log2n, s);
+    }
     // Small blocks share a CTA: a thread of the 8-bit levels takes a whole sub-block, so the more
     // sub-blocks a CTA holds, the fuller its warps.  Up to 2^13 outputs per CTA, as long as
     // every SM still gets a few CTAs.
