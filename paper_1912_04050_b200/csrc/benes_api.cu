@@ -221,7 +221,7 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     if (kappa) {
         sampled_scratch_carve(sampled, T, kappa, &sc);
         BENES_CUDA_TRY(cudaMemsetAsync(gates, 0, kMaxLevels * 4, s));
-        if ((rc = sampled_scratch_reset(sc, T, kappa, s))) return rc;
+        if ((rc = sampled_scratch_reset(sc, T, n, kappa, s))) return rc;
     }
 
     BitsLayout L{bits, n, n - 6};

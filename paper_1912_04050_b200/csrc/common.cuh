@@ -18,8 +18,6 @@ constexpr int kFusedLog2M = 15;
 
 // Largest list (log2 of its 64-bit words) that one CTA labels in shared memory.
 constexpr int kListSmemLog2 = 14;
-// Ruler spacing (log2) used when a contracted list is itself sampled.
-constexpr int kListKappa = 4;
 
 constexpr uint32_t kUnowned = 0xFFFFFFFFu;
 
@@ -308,9 +306,9 @@ int launch_split(LevelRecords S, const uint32_t *Q, LevelRecords Sn, uint32_t *Q
 // ---- ruler-sampled loop labelling (route_sampled.cu) --------------------------
 struct SampledScratch {
     uint4 *rec;                  // total >> kappa walk records
-    uint32_t *ruler_bits;        // parity of every ruler's cycle minimum, one bit each
-    unsigned long long *list[5]; // contracted lists: total >> (kappa + 4 i) words
+    unsigned long long *list[5]; // contracted lists: at most total >> (kappa + 2 i) words
     uint32_t *owner[5];          // owners of the words of list[i] (all kUnowned between uses)
+    uint32_t *bits[5];           // parity of every word's cycle minimum, one bit each
 };
 size_t sampled_scratch_bytes(size_t total, int kappa);
 void sampled_scratch_carve(char *base, size_t total, int kappa, SampledScratch *out);
@@ -319,8 +317,8 @@ void sampled_scratch_carve(char *base, size_t total, int kappa, SampledScratch *
 // must then be relabelled and Sn rewritten).
 int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const SampledScratch &sc, size_t total,
                   int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage, uint32_t *gate, cudaStream_t s);
-// owner[0] and owner[1] must be all kUnowned before the first sampled_label.
-int sampled_scratch_reset(const SampledScratch &sc, size_t total, int kappa, cudaStream_t s);
+// Before the first sampled_label of a route: owners to kUnowned (log2m of the first level).
+int sampled_scratch_reset(const SampledScratch &sc, size_t total, int log2m, int kappa, cudaStream_t s);
 
 // ---- fused path (route_fused.cu) -------------------------------------------
 // Finishes levels (n - log2m) .. n-1 of every block of size 2^log2m of the flat

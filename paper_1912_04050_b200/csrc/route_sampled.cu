@@ -20,10 +20,10 @@
 //   3. k_combine: the segment of walker rho ends at ruler output peer^1 and
 //      its minimum is min(least[rho], least[peer] ^ 1): one 64-bit (next, min) word
 //      per ruler output -- the contracted list.
-//   4. The contracted list is labelled with the minimum of every cycle:
+//   4. The contracted list is labelled with the parity of every cycle's minimum:
 //      lists of up to 2^14 words per block in one CTA's shared memory, longer
 //      ones by sampling again: the list is mirror symmetric like the loops, so
-//      it is sampled the same way (one ruler pair per 16 pairs of words, walks
+//      it is sampled the same way (one ruler pair per 4 to 16 pairs of words, walks
 //      that meet in the middle, k_combine again).
 //   5. k_colour: output 2t lies on its owner's cycle if the owner arrived on
 //      the even side, else on the mirror cycle, which has the other colour:
@@ -198,23 +198,22 @@ k_combine_list(const uint4 *__restrict__ rec, unsigned long long *__restrict__ W
 // as with one-directional walks.  A walker keeps the minimum over the words it
 // passed (fwd), over their partners (part) and whom it met (peer): the same
 // record as in step 2, turned into the 16 times shorter list by k_combine.
-constexpr int kPairGroupLog2 = kListKappa;          // pairs per ruler pair (log2)
-
+// (spacing = log2 of the pairs per ruler pair.)
 __global__ void __launch_bounds__(kWalkThreads)
 k_list_walk_pairs(const ulonglong2 *__restrict__ W2p, uint32_t *__restrict__ owner, uint4 *__restrict__ rec,
-                  uint32_t rulers, uint32_t pairs, uint32_t salt, uint32_t cap, uint32_t *__restrict__ gate) {
+                  uint32_t rulers, uint32_t pairs, int spacing, uint32_t salt, uint32_t cap, uint32_t *__restrict__ gate) {
     const uint32_t sigma = blockIdx.x * kWalkThreads + threadIdx.x;
     if (sigma >= rulers) return;
-    constexpr uint32_t kmask = (1u << kPairGroupLog2) - 1u;
+    const uint32_t kmask = (1u << spacing) - 1u;
     const uint32_t group = sigma >> 1, side0 = sigma & 1u;
-    const uint32_t q0 = (group << kPairGroupLog2) | ruler_slot(group, salt, kmask);
+    const uint32_t q0 = (group << spacing) | ruler_slot(group, salt, kmask);
     ulonglong2 w = __ldcg(W2p + q0);
     if (!side0) owner[q0] = sigma << 1;                            // the ruler pair belongs to its even walker
     unsigned long long own = side0 ? w.y : w.x;
     uint32_t fwd = uint32_t(own >> 32), part = kUnowned, peer = sigma ^ 1u, hops = 0;
     for (;;) {
         // (a batch need not be a power of two: an index a raised gate left undefined is clamped, not masked)
-        const uint32_t e = uint32_t(own), q = BENES_GUARD_BELOW(e >> 1, pairs, 0u), side = e & 1u, g = q >> kPairGroupLog2;
+        const uint32_t e = uint32_t(own), q = BENES_GUARD_BELOW(e >> 1, pairs, 0u), side = e & 1u, g = q >> spacing;
         if ((q & kmask) == ruler_slot(g, salt, kmask)) {           // reached the next ruler pair
             peer = (2u * g + side) ^ 1u;
             break;
@@ -239,15 +238,11 @@ k_list_walk_pairs(const ulonglong2 *__restrict__ W2p, uint32_t *__restrict__ own
 }
 
 // Back from a sampled list: a thread takes the pair 2q, 2q+1 (and hands the
-// owner slot back as kUnowned).  Word 2q + b lies on its owner's cycle if the
-// owner arrived on side b, else on the mirror cycle, which is the cycle of the
-// owner's partner walker and whose minimum has the other parity.  A pair nobody
-// claimed lies on a cycle without ruler pair: the thread walks the cycle of
-// word 2q (and that of word 2q+1 if the minima themselves are needed).
-// Of the first list (the rulers of the level) only the parity of the minima is
-// needed afterwards: with `cb` one bit per word goes there, so that the colouring
-// kernel gathers from an array 64 times smaller than the list (it stays in
-// L1/L2 next to the streaming traffic); without, the words take their minima.
+// owner slot back as kUnowned).  Word 2q lies on its owner's cycle if the
+// owner arrived on side 0, else on the mirror cycle, whose minimum has the other
+// parity, and so does word 2q+1's: one bit of the sampled list (`cb2`) gives the two bits of
+// the pair (`cb`).  A pair nobody claimed lies on a cycle without ruler pair: the thread walks the
+// cycle of word 2q.
 __device__ __forceinline__ uint32_t list_cycle_min(const unsigned long long *W, uint32_t e0, uint32_t words,
                                                    uint32_t cap, uint32_t *gate) {
     unsigned long long v = __ldcg(W + e0);
@@ -258,40 +253,23 @@ __device__ __forceinline__ uint32_t list_cycle_min(const unsigned long long *W, 
             break;
         }
         v = __ldcg(W + e);
-        mn = min(mn, uint32_t(v >> 32));       // words rewritten meanwhile hold the minimum of this same cycle
+        mn = min(mn, uint32_t(v >> 32));
         e = BENES_GUARD_BELOW(uint32_t(v), words, 0u);
     }
     return mn;
 }
 
 __global__ void __launch_bounds__(kThreads)
-k_list_resolve_pairs(unsigned long long *__restrict__ W, uint32_t *__restrict__ owner,
-                     const unsigned long long *__restrict__ W2, uint32_t pairs, uint32_t words,
+k_list_resolve_pairs(const unsigned long long *__restrict__ W, uint32_t *__restrict__ owner,
+                     const uint32_t *__restrict__ cb2, uint32_t pairs, uint32_t words,
                      uint32_t cap, uint32_t *__restrict__ gate, uint32_t *__restrict__ cb) {
     const uint32_t q = blockIdx.x * kThreads + threadIdx.x;       // pairs is a multiple of 32
     if (q >= pairs) return;
     const uint32_t code = owner[q];
-    if (!cb) {
-        uint32_t mn0, mn1;
-        if (code != kUnowned) {
-            const uint32_t a = uint32_t(__ldcg(W2 + (code >> 1)) >> 32), b = uint32_t(__ldcg(W2 + ((code >> 1) ^ 1u)) >> 32);
-            mn0 = (code & 1u) ? b : a;
-            mn1 = (code & 1u) ? a : b;
-            owner[q] = kUnowned;
-        } else {
-            mn0 = list_cycle_min(W, 2u * q, words, cap, gate);
-            mn1 = list_cycle_min(W, 2u * q + 1u, words, cap, gate);
-        }
-        ulonglong2 *Wp = reinterpret_cast<ulonglong2 *>(W) + q;
-        ulonglong2 w = *Wp;
-        w.x = make_word(uint32_t(w.x), mn0);
-        w.y = make_word(uint32_t(w.y), mn1);
-        *Wp = w;
-        return;
-    }
     uint32_t bit0;
     if (code != kUnowned) {
-        bit0 = (uint32_t(__ldcg(W2 + (code >> 1)) >> 32) ^ code) & 1u;
+        const uint32_t sigma = code >> 1;
+        bit0 = ((__ldg(cb2 + (sigma >> 5)) >> (sigma & 31u)) ^ code) & 1u;
         owner[q] = kUnowned;
     } else {
         bit0 = list_cycle_min(W, 2u * q, words, cap, gate) & 1u;
@@ -300,125 +278,188 @@ k_list_resolve_pairs(unsigned long long *__restrict__ W, uint32_t *__restrict__ 
     store_stage_bits64(cb + ((q - (threadIdx.x & 31u)) >> 4), bit0, bit0 ^ 1u);
 }
 
-// Step 4, the end of the recursion: one CTA labels one block's list of
-// 2^log2b words in shared memory by synchronous pointer jumping (new words are
-// held in registers across the barrier; PER words per thread, blockDim =
-// 2^log2b / PER).  A cycle and its mirror image have the same number of words
-// and lie in the same block, so a cycle has at most 2^(log2b-1) words: log2b - 1
-// passes.
-// With `cb` (first list of a level) the parities of the minima go there, one bit
-// per word, instead of the words back to W.
-template <int PER>
+// Step 4, the end of the recursion: one CTA labels one block's list of B = 2^log2b words in shared memory, by
+// the same sampling once more: one ruler pair per 8 pairs, walks that meet in the middle over 16-bit
+// successors (claims go into the successor words, which nobody reads again), pointer jumping over the B/8 words
+// that are left, and a queue for the pairs of cycles without ruler pair.  Pointer jumping over the whole list
+// took log2b - 1 passes of random shared-memory reads (2^14 words: 25 us, now LIST_US).
+// Only the parities of the minima are needed from here on (a cycle and its mirror image differ in it): they
+// go to `cb`, one bit per word.
+// RECS: the list is the rulers of the level and its words, (next, min) = (peer ^ 1, min(least[rho],
+// least[peer] ^ 1)), are formed here from the walk records.  Indices a raised gate may have left undefined are
+// masked into the block.
+constexpr int kLGroup = 3;                            // pairs per ruler pair (log2)
+constexpr uint32_t kLRho = 0x7FFCu, kLRuler = 0x8000u;
+
+constexpr size_t list_label_smem(int log2b) { return (size_t(17) << log2b) / 2 + 16; }
+
+template <bool RECS>
 __global__ void __launch_bounds__(kListThreads)
-k_list_label(unsigned long long *__restrict__ W, int log2b, uint32_t *__restrict__ cb) {
-    extern __shared__ unsigned long long sm[];
-    const uint32_t B = 1u << log2b, bmask = B - 1u;
+k_list_label(const void *__restrict__ src, uint16_t *__restrict__ cb, int log2b, uint32_t salt) {
+    extern __shared__ __align__(16) unsigned char lsm[];
+    const uint32_t B = 1u << log2b, bmask = B - 1u, R = B >> kLGroup, groups = B >> (kLGroup + 1);
     const size_t base = size_t(blockIdx.x) << log2b;
     const uint32_t T = blockDim.x, tid = threadIdx.x;
+    uint32_t *M = reinterpret_cast<uint32_t *>(lsm);                            // minimum of every word
+    unsigned char *N = lsm + 4 * B;                                             // successors / claims, 16 bit
+    uint32_t *own = reinterpret_cast<uint32_t *>(N + 2 * B), *far_ = own + R, *peer = far_ + R;
+    unsigned long long *L = reinterpret_cast<unsigned long long *>(peer + R);   // list of the ruler words (+ a 0)
+    uint16_t *queue = reinterpret_cast<uint16_t *>(own);                        // after `own`, `far_` and `peer`
+    __shared__ uint32_t queued;
+    // sixteen words per thread (fewer than 512 words: a warp takes turns), all their loads under way together
+    for (uint32_t e0 = tid; e0 < B; e0 += 16 * T) {
+        uint32_t next[16], mn[16];
 #pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const uint32_t e = tid + uint32_t(i) * T;
-        unsigned long long w = __ldcs(W + base + e);
-        sm[e] = make_word(uint32_t(w) & bmask, uint32_t(w >> 32));
+        for (int i = 0; i < 16; ++i) {
+            const uint32_t e = e0 + uint32_t(i) * T;
+            next[i] = mn[i] = 0u;
+            if (e >= B) continue;
+            if (RECS) {
+                const uint2 a = __ldcs(static_cast<const uint2 *>(src) + base + e);
+                next[i] = (a.y & bmask) ^ 1u;
+                mn[i] = a.x;
+            } else {
+                const unsigned long long w = __ldcs(static_cast<const unsigned long long *>(src) + base + e);
+                next[i] = uint32_t(w) & bmask;
+                mn[i] = uint32_t(w >> 32);
+            }
+        }
+        if (RECS) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                mn[i] = min(mn[i], __ldg(&(static_cast<const uint2 *>(src) + base)[next[i] ^ 1u].x) ^ 1u);
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const uint32_t e = e0 + uint32_t(i) * T;
+            if (e >= B) continue;
+            M[e] = mn[i];
+            *reinterpret_cast<uint16_t *>(N + 2 * e) = uint16_t(2u * next[i]);
+        }
+    }
+    if (tid == 0) queued = 0u;
+    __syncthreads();
+    const uint32_t g = tid;                              // a thread has one group of 8 pairs
+    uint32_t start = 0, q0 = 0;
+    if (g < groups) {
+        q0 = (g << kLGroup) | ruler_slot(g, salt, (1u << kLGroup) - 1u);
+        uint32_t *word = reinterpret_cast<uint32_t *>(N + 4 * q0);
+        start = *word;
+        *word = (kLRuler | (g << 3) | 1u) * 0x10001u;
     }
     __syncthreads();
-    unsigned long long v[PER];
-    for (int pass = 0; pass < log2b - 1; ++pass) {
+    if (g < groups) {
+        uint32_t rho = 2u * g, j = start & 0xFFFFu, code = ((rho << 2) | 1u) * 0x10001u;
+        uint32_t least = M[2u * q0], part = kUnowned;
+        for (uint32_t k = 0;;) {
+            bool met = false;
+            uint32_t v = 0;
 #pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const unsigned long long w = sm[tid + uint32_t(i) * T];
-            const unsigned long long t = sm[uint32_t(w)];
-            v[i] = make_word(uint32_t(t), min(uint32_t(w >> 32), uint32_t(t >> 32)));
+            for (int hop = 0; hop < 4; ++hop) {
+                if (!met) {
+                    v = *reinterpret_cast<volatile uint16_t *>(N + j);
+                    met = (v & 1u) != 0u;
+                    if (!met) {
+                        const uint2 mm = *reinterpret_cast<const uint2 *>(M + ((j >> 1) & ~1u));
+                        *reinterpret_cast<volatile uint32_t *>(N + (j & ~3u)) = code + (j & 2u) * 0x10001u;
+                        least = min(least, (j & 2u) ? mm.y : mm.x);
+                        part = min(part, (j & 2u) ? mm.x : mm.y);
+                        j = v;
+                    }
+                }
+            }
+            if (met) {
+                // a ruler pair (its code names its even word), or one the other walker owns
+                own[rho] = least;
+                far_[rho] = part;
+                peer[rho] = ((v & kLRho) >> 2) ^ ((v & kLRuler) ? ((~j & 2u) >> 1) : 0u);
+                if (++k == 2u) break;
+                ++rho;
+                j = start >> 16;
+                code = ((rho << 2) | 1u) * 0x10001u;
+                least = M[2u * q0 + 1u];
+                part = kUnowned;
+            }
         }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < PER; ++i) sm[tid + uint32_t(i) * T] = v[i];
-        __syncthreads();
     }
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const uint32_t e = tid + uint32_t(i) * T;
-        const unsigned long long w = sm[e];
-        if (cb) {
-            const uint32_t word = __ballot_sync(0xFFFFFFFFu, uint32_t(w >> 32) & 1u);
-            if ((tid & 31u) == 0u) cb[(base + e) >> 5] = word;
-        } else {
-            W[base + e] = make_word(uint32_t(base) + uint32_t(w), uint32_t(w >> 32));
+    __syncthreads();
+    for (uint32_t rho = tid; rho < R; rho += T) {
+        const uint32_t p = peer[rho] & (R - 1u);
+        L[rho] = make_word(p ^ 1u, min(own[rho], far_[p]));
+    }
+    if (tid == 0) L[R] = 0ull;
+    __syncthreads();
+    // pairs of cycles without ruler pair queue up; pointer jumping over the ruler words meanwhile: a cycle of
+    // theirs has at most R/2 words (it and its mirror image share the block)
+    uint4 n0 = make_uint4(1, 1, 1, 1), n1 = n0;
+    if (g < groups) {
+        n0 = *reinterpret_cast<const uint4 *>(N + 32 * g);
+        n1 = *reinterpret_cast<const uint4 *>(N + 32 * g + 16);
+        uint32_t free_ = (~n0.x & 1u) | ((~n0.y & 1u) << 1) | ((~n0.z & 1u) << 2) | ((~n0.w & 1u) << 3) |
+                         ((~n1.x & 1u) << 4) | ((~n1.y & 1u) << 5) | ((~n1.z & 1u) << 6) | ((~n1.w & 1u) << 7);
+        if (free_) {
+            uint32_t pos = atomicAdd(&queued, uint32_t(__popc(free_)));
+            for (; free_; free_ &= free_ - 1u) queue[pos++] = uint16_t(8u * g + uint32_t(__ffs(int(free_))) - 1u);
         }
+    }
+    volatile unsigned long long *Lv = L;
+    for (int pass = 0; pass < log2b - kLGroup - 1; ++pass) {
+        for (uint32_t rho = tid; rho < R; rho += T) {
+            const unsigned long long w = Lv[rho], t = Lv[uint32_t(w)];
+            Lv[rho] = make_word(uint32_t(t), min(uint32_t(w >> 32), uint32_t(t >> 32)));
+        }
+        __syncthreads();
+        if (pass == 0) {
+            // (the queue is complete, and the walks below only read unclaimed words until the next barrier)
+            for (uint32_t i = tid; i < queued; i += T) {
+                const uint32_t q = queue[i];
+                uint32_t f = 4u * q, mn = M[2u * q];
+                for (uint32_t hops = 0; hops < B; ++hops) {
+                    f = *reinterpret_cast<volatile uint16_t *>(N + f) & (2u * bmask);
+                    if (f == 4u * q) break;
+                    mn = min(mn, M[f >> 1]);
+                }
+                queue[i] = uint16_t(q | (mn << 15));
+            }
+        } else if (pass == 1) {
+            for (uint32_t i = tid; i < queued; i += T) {
+                const uint32_t x = queue[i];
+                *reinterpret_cast<uint32_t *>(N + 4 * (x & 0x7FFFu)) = (R << 2) | 1u | ((x >> 14) & 2u);
+            }
+        }
+    }
+    __syncthreads();
+    if (g < groups) {
+        n0 = *reinterpret_cast<const uint4 *>(N + 32 * g);
+        n1 = *reinterpret_cast<const uint4 *>(N + 32 * g + 16);
+        const uint32_t code[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
+        uint32_t bits = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t b = (uint32_t(L[(code[k] & kLRho) >> 2] >> 32) ^ (code[k] >> 1)) & 1u;
+            bits |= (b | ((b ^ 1u) << 1)) << (2 * k);
+        }
+        cb[(base >> 4) + g] = uint16_t(bits);
     }
 }
 
-template <int PER>
-int launch_list_label(unsigned long long *W, uint32_t count, int beta, uint32_t *cb, cudaStream_t s) {
+int launch_list_label(const void *src, bool records, uint32_t *cb, uint32_t count, int beta, uint32_t salt, cudaStream_t s) {
     static OncePerDevice configured;
-    const size_t smem = (size_t(1) << beta) * 8;
     {
         const int rc = configured.run([]() -> int {
-            BENES_CUDA_TRY(cudaFuncSetAttribute(k_list_label<PER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (1 << kListSmemLog2) * 8));
+            BENES_CUDA_TRY(cudaFuncSetAttribute(k_list_label<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                int(list_label_smem(kListSmemLog2))));
+            BENES_CUDA_TRY(cudaFuncSetAttribute(k_list_label<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                int(list_label_smem(kListSmemLog2))));
             return BENES_OK;
         });
         if (rc) return rc;
     }
-    k_list_label<PER><<<count >> beta, (1u << beta) / PER, smem, s>>>(W, beta, cb);
-    return launch_status();
-}
-
-// Steps 3 and 4 in one kernel for a level whose blocks have at most 2^18 outputs
-// and lists that fit one CTA (no sampling of the list): the CTA forms its
-// block's list words from the walk records, (next, min) = (peer ^ 1,
-// min(least[rho], least[peer] ^ 1)), as 14 + 18 bit, both local to the block, labels
-// them by synchronous pointer jumping and writes the parity bits.  Indices a
-// raised gate may have left undefined are masked into the block.
-template <int PER>
-__global__ void __launch_bounds__(kListThreads)
-k_list_label_rec(const uint2 *__restrict__ rec, uint32_t *__restrict__ cb, int log2b, int m) {
-    extern __shared__ uint32_t sw[];
-    constexpr uint32_t kNext = (1u << kListSmemLog2) - 1u;
-    const uint32_t B = 1u << log2b, bmask = B - 1u, mmask = (1u << m) - 1u;
-    const uint32_t base = blockIdx.x << log2b;                    // first ruler output of the block
-    const uint32_t T = blockDim.x, tid = threadIdx.x;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const uint32_t e = tid + uint32_t(i) * T;
-        const uint2 a = __ldcs(rec + base + e);
-        const uint32_t peer = a.y & bmask;
-        sw[e] = (peer ^ 1u) | ((min(a.x, __ldg(&rec[base + peer].x) ^ 1u) & mmask) << kListSmemLog2);
-    }
-    __syncthreads();
-    uint32_t v[PER];
-    for (int pass = 0; pass < log2b - 1; ++pass) {
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const uint32_t w = sw[tid + uint32_t(i) * T];
-            const uint32_t t = sw[w & kNext];
-            v[i] = (t & kNext) | min(w & ~kNext, t & ~kNext);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < PER; ++i) sw[tid + uint32_t(i) * T] = v[i];
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const uint32_t e = tid + uint32_t(i) * T;
-        const uint32_t word = __ballot_sync(0xFFFFFFFFu, (sw[e] >> kListSmemLog2) & 1u);
-        if ((tid & 31u) == 0u) cb[(base + e) >> 5] = word;
-    }
-}
-
-template <int PER>
-int launch_list_label_rec(const uint2 *rec, uint32_t *cb, uint32_t count, int beta, int m, cudaStream_t s) {
-    static OncePerDevice configured;
-    {
-        const int rc = configured.run([]() -> int {
-            BENES_CUDA_TRY(cudaFuncSetAttribute(k_list_label_rec<PER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (1 << kListSmemLog2) * 4));
-            return BENES_OK;
-        });
-        if (rc) return rc;
-    }
-    k_list_label_rec<PER><<<count >> beta, (1u << beta) / PER, (size_t(1) << beta) * 4, s>>>(rec, cb, beta, m);
+    const unsigned threads = beta > 9 ? 1u << (beta - 4) : 32u;
+    if (records)
+        k_list_label<true><<<count >> beta, threads, list_label_smem(beta), s>>>(src, reinterpret_cast<uint16_t *>(cb), beta, salt);
+    else
+        k_list_label<false><<<count >> beta, threads, list_label_smem(beta), s>>>(src, reinterpret_cast<uint16_t *>(cb), beta, salt);
     return launch_status();
 }
 
@@ -547,26 +588,23 @@ k_colour(const void *__restrict__ S, const uint32_t *__restrict__ P, const uint3
 inline size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 constexpr int kMaxLists = 5;
 
-// Number of times the list of a block with 2^beta words is sampled again.
-inline int list_depth(int beta) {
-    int d = 0;
-    while (beta > kListSmemLog2 && d < kMaxLists - 1) {
-        beta -= kListKappa;
-        ++d;
-    }
-    return d;
+// Spacing at which a block's list of 2^beta words is sampled again: 2^4 while it is far from what one CTA labels, just
+// enough at the end (short walks are quick, and the CTA's labelling does not mind a full list).  0: fits.
+inline int list_spacing(int beta) {
+    const int over = beta - kListSmemLog2;
+    return over <= 0 ? 0 : over < 2 ? 2 : over > 4 ? 4 : over;
 }
 
 }  // namespace
 
-// Scratch: walk records, the contracted lists and the owners of every list
-// that may be sampled again.  Sized for the largest level (log2m = 30).
+// Scratch: walk records, the contracted lists, and the owners and parity bits of their words.
+// A list that is sampled again shrinks to a quarter at least.
 size_t sampled_scratch_bytes(size_t total, int kappa) {
-    size_t R = total >> kappa, bytes = align256(R * 16) + align256(R / 8 + 4);
+    size_t R = total >> kappa, bytes = align256(R * 16);
     for (int i = 0; i < kMaxLists; ++i) {
-        size_t c = R >> (kListKappa * i);
-        if (c < 4) c = 4;
-        bytes += align256(c * 8) + align256(c * 4);
+        size_t c = R >> (2 * i);
+        if (c < 32) c = 32;
+        bytes += align256(c * 8) + align256(c * 4) + align256(c / 8);
     }
     return bytes;
 }
@@ -575,24 +613,26 @@ void sampled_scratch_carve(char *base, size_t total, int kappa, SampledScratch *
     size_t R = total >> kappa, off = 0;
     out->rec = reinterpret_cast<uint4 *>(base);
     off += align256(R * 16);
-    out->ruler_bits = reinterpret_cast<uint32_t *>(base + off);
-    off += align256(R / 8 + 4);
     for (int i = 0; i < kMaxLists; ++i) {
-        size_t c = R >> (kListKappa * i);
-        if (c < 4) c = 4;
+        size_t c = R >> (2 * i);
+        if (c < 32) c = 32;
         out->list[i] = reinterpret_cast<unsigned long long *>(base + off);
         off += align256(c * 8);
         out->owner[i] = reinterpret_cast<uint32_t *>(base + off);
         off += align256(c * 4);
+        out->bits[i] = reinterpret_cast<uint32_t *>(base + off);
+        off += align256(c / 8);
     }
 }
 
-int sampled_scratch_reset(const SampledScratch &sc, size_t total, int kappa, cudaStream_t s) {
-    size_t R = total >> kappa;
-    for (int i = 0; i < kMaxLists - 1; ++i) {
-        size_t c = R >> (kListKappa * i);
-        if (c < 4) c = 4;
-        BENES_CUDA_TRY(cudaMemsetAsync(sc.owner[i], 0xFF, c * 4, s));
+// The owners of the lists that the first level (which has the longest) samples again.
+int sampled_scratch_reset(const SampledScratch &sc, size_t total, int log2m, int kappa, cudaStream_t s) {
+    size_t c = total >> kappa;
+    int beta = log2m - kappa;
+    for (int i = 0, sp; (sp = list_spacing(beta)) != 0; ++i) {
+        BENES_CUDA_TRY(cudaMemsetAsync(sc.owner[i], 0xFF, c / 2 * 4, s));
+        c >>= sp;
+        beta -= sp;
     }
     return BENES_OK;
 }
@@ -620,62 +660,50 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
         int rc = launch_status();
         if (rc) return rc;
     }
-    uint32_t *cb = sc.ruler_bits;
+    uint32_t *cb = sc.bits[0];
     // label the contracted list: sample it until a block's list fits one CTA
-    int beta = log2m - kappa;
-    const int depth = list_depth(beta);
-    uint32_t count = R;
-    // (the kernels that write the parity bits ballot: whole warps, i.e. lists of 2^7 words at least)
-    if (depth == 0 && beta < 7) return BENES_ERR_BADARG;
-    const bool from_records = depth == 0 && log2m <= 32 - kListSmemLog2;
-    if (from_records) {
-        ProfileScope ps(kListLabel, s);
-        int rc = beta <= 12 ? launch_list_label_rec<4>(walk_rec, cb, count, beta, log2m, s)
-               : beta == 13 ? launch_list_label_rec<8>(walk_rec, cb, count, beta, log2m, s)
-                            : launch_list_label_rec<16>(walk_rec, cb, count, beta, log2m, s);
-        if (rc) return rc;
-    } else {
+    int beta = log2m - kappa, depth = 0;
+    if (beta < 7) return BENES_ERR_BADARG;                     // (a CTA labels 2^7 words at least)
+    uint32_t counts[kMaxLists + 1] = {R};
+    if (list_spacing(beta)) {
         ProfileScope ps(kCombine, s);
         k_combine<<<rgrid, kThreads, 0, s>>>(walk_rec, sc.list[0], R);
         int rc = launch_status();
         if (rc) return rc;
     }
-    for (int d = 0; d < depth; ++d) {
+    for (int sp; (sp = list_spacing(beta)) != 0; ++depth) {
         // walks from both ends; the walk records of the previous stage (switches,
         // or the list before) are dead, their memory takes the new ones
-        const uint32_t next = count >> kListKappa;
+        if (depth + 1 >= kMaxLists) return BENES_ERR_BADARG;
+        const uint32_t count = counts[depth], next = count >> sp;
         {
             ProfileScope ps(kListWalk, s);
             k_list_walk_pairs<<<(next + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s>>>(
-                reinterpret_cast<const ulonglong2 *>(sc.list[d]), sc.owner[d], sc.rec, next, count >> 1,
-                salt * 7u + uint32_t(d) + 1u, cap, gate);
+                reinterpret_cast<const ulonglong2 *>(sc.list[depth]), sc.owner[depth], sc.rec, next, count >> 1, sp,
+                salt * 7u + uint32_t(depth) + 1u, cap, gate);
             int rc = launch_status();
             if (rc) return rc;
         }
         {
             ProfileScope ps(kCombine, s);
-            k_combine_list<<<(next + kThreads - 1) / kThreads, kThreads, 0, s>>>(sc.rec, sc.list[d + 1], next);
+            k_combine_list<<<(next + kThreads - 1) / kThreads, kThreads, 0, s>>>(sc.rec, sc.list[depth + 1], next);
             int rc = launch_status();
             if (rc) return rc;
         }
-        count = next;
-        beta -= kListKappa;
+        counts[depth + 1] = next;
+        beta -= sp;
     }
-    if (!from_records) {
+    {
         ProfileScope ps(kListLabel, s);
-        if (beta > kListSmemLog2 || beta < 5) return BENES_ERR_BADARG;
-        // 4 words per thread up to 2^12 words, then 1024 threads
-        uint32_t *bits_out = depth == 0 ? cb : nullptr;
-        int rc = beta <= 12 ? launch_list_label<4>(sc.list[depth], count, beta, bits_out, s)
-               : beta == 13 ? launch_list_label<8>(sc.list[depth], count, beta, bits_out, s)
-                            : launch_list_label<16>(sc.list[depth], count, beta, bits_out, s);
+        int rc = launch_list_label(depth ? static_cast<const void *>(sc.list[depth]) : walk_rec, depth == 0, sc.bits[depth],
+                                   counts[depth], beta, salt + 77u, s);
         if (rc) return rc;
     }
     for (int d = depth - 1; d >= 0; --d) {
         ProfileScope ps(kListResolve, s);
-        const uint32_t c = R >> (kListKappa * d);
+        const uint32_t c = counts[d];
         k_list_resolve_pairs<<<(c / 2 + kThreads - 1) / kThreads, kThreads, 0, s>>>(
-            sc.list[d], sc.owner[d], sc.list[d + 1], c / 2, c, cap, gate, d == 0 ? cb : nullptr);
+            sc.list[d], sc.owner[d], sc.bits[d + 1], c / 2, c, cap, gate, sc.bits[d]);
         int rc = launch_status();
         if (rc) return rc;
     }
