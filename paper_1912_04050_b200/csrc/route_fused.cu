@@ -290,19 +290,16 @@ __device__ __forceinline__ void level16(unsigned char *sm, const FusedOut &out, 
         uint32_t least = 4u * ((g << kFKappa) | fused_slot(g, uint32_t(level))), j = start[0] & 0xFFFFu;
         uint32_t code = ((rho << 2) | 1u) * 0x10001u;
         for (;;) {
+            // (no branches: a lane that has met somebody reads the same code again)
             bool met = false;
             uint32_t v = 0;
 #pragma unroll
             for (int hop = 0; hop < 4; ++hop) {
-                if (!met) {
-                    v = at<volatile uint16_t>(sm, Cfg::kN + j);
-                    met = (v & 1u) != 0u;
-                    if (!met) {
-                        at<volatile uint32_t>(sm, Cfg::kN + (j & ~3u)) = code + (j & 2u) * 0x10001u;
-                        least = min(least, j);
-                        j = v;
-                    }
-                }
+                v = at<volatile uint16_t>(sm, Cfg::kN + j);
+                met = (v & 1u) != 0u;
+                if (!met) at<volatile uint32_t>(sm, Cfg::kN + (j & ~3u)) = code + (j & 2u) * 0x10001u;
+                least = met ? least : min(least, j);
+                j = met ? j : v;
             }
             if (met) {
                 // a ruler switch (its code names its even output), or one the other walker owns

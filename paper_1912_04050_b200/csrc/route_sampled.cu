@@ -352,21 +352,18 @@ k_list_label(const void *__restrict__ src, uint16_t *__restrict__ cb, int log2b,
         uint32_t rho = 2u * g, j = start & 0xFFFFu, code = ((rho << 2) | 1u) * 0x10001u;
         uint32_t least = M[2u * q0], part = kUnowned;
         for (uint32_t k = 0;;) {
+            // (no branches: a lane that has met somebody reads the same code again)
             bool met = false;
             uint32_t v = 0;
 #pragma unroll
             for (int hop = 0; hop < 4; ++hop) {
-                if (!met) {
-                    v = *reinterpret_cast<volatile uint16_t *>(N + j);
-                    met = (v & 1u) != 0u;
-                    if (!met) {
-                        const uint2 mm = *reinterpret_cast<const uint2 *>(M + ((j >> 1) & ~1u));
-                        *reinterpret_cast<volatile uint32_t *>(N + (j & ~3u)) = code + (j & 2u) * 0x10001u;
-                        least = min(least, (j & 2u) ? mm.y : mm.x);
-                        part = min(part, (j & 2u) ? mm.x : mm.y);
-                        j = v;
-                    }
-                }
+                v = *reinterpret_cast<volatile uint16_t *>(N + j);
+                met = (v & 1u) != 0u;
+                const uint2 mm = *reinterpret_cast<const uint2 *>(M + ((j >> 1) & ~1u));
+                if (!met) *reinterpret_cast<volatile uint32_t *>(N + (j & ~3u)) = code + (j & 2u) * 0x10001u;
+                least = met ? least : min(least, (j & 2u) ? mm.y : mm.x);
+                part = met ? part : min(part, (j & 2u) ? mm.x : mm.y);
+                j = met ? j : v;
             }
             if (met) {
                 // a ruler pair (its code names its even word), or one the other walker owns
