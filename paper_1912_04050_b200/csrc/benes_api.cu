@@ -141,13 +141,13 @@ inline size_t level_chunk(int log2n, size_t batch, int chunk_log2) {
 
 // Scratch of the per-level path for T flat elements: two generations of switch
 // records (16 B per switch) and of inverses, the 64-bit words of the full
-// pointer jumping, the scratch of the sampled labelling, per-level gate flags.
+// pointer jumping, the scratch of the sampled labelling, the gate.
 constexpr int kMaxKappa = 8, kMinKappa = 2;
 size_t route_ws_bytes(int log2n, size_t batch) {
     if (log2n <= kFusedLog2M) return 0;
     size_t T = level_chunk(log2n, batch, options().chunk_log2) << log2n;
     return 2 * align_up(T * 8) + 2 * align_up(T * 4) + align_up(T * 8) +
-           align_up(sampled_scratch_bytes(T, kMinKappa)) + align_up(kMaxLevels * 4) +
+           align_up(sampled_scratch_bytes(T, kMinKappa)) + kAlign +
            align_up(kInverseMaxBuckets * 4);
 }
 
@@ -168,6 +168,7 @@ struct HostPipe {
     cudaStream_t back = nullptr;       // a second stream for device -> host copies (benes_route_apply_host)
     cudaStream_t d2h = nullptr;        // where this call's finished stages leave: `side` or `back`
     cudaEvent_t part_ready[kApplyMaxParts] = {};   // parts of a payload that have arrived
+    uint32_t *gate_host = nullptr;     // pinned: the route's gate, valid once the stream has been waited for
     int pieces = 0;                    // the permutation arrives in this many equal pieces
     cudaEvent_t piece_ready[kMaxPieces] = {};
     cudaEvent_t stage_ready[kMaxLevels] = {};
@@ -200,8 +201,8 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     Qbuf[1] = reinterpret_cast<uint32_t *>(ws + off); off += align_up(T * 4);
     unsigned long long *Wd = reinterpret_cast<unsigned long long *>(ws + off); off += align_up(T * 8);
     char *sampled = ws + off; off += align_up(sampled_scratch_bytes(T, kMinKappa));
-    // per level: a gate, raised by a walk that gave up
-    uint32_t *gates = reinterpret_cast<uint32_t *>(ws + off); off += align_up(kMaxLevels * 4);
+    // raised by a walk that gave up
+    uint32_t *gate = reinterpret_cast<uint32_t *>(ws + off); off += kAlign;
     uint32_t *fill = reinterpret_cast<uint32_t *>(ws + off);
     // Small inputs are bound by the longest walk of a level, not by throughput:
     // closer rulers (shorter walks) pay there although the lists get longer.
@@ -220,12 +221,14 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     int rc;
     if (kappa) {
         sampled_scratch_carve(sampled, T, kappa, &sc);
-        BENES_CUDA_TRY(cudaMemsetAsync(gates, 0, kMaxLevels * 4, s));
+        BENES_CUDA_TRY(cudaMemsetAsync(gate, 0, 4, s));
         if ((rc = sampled_scratch_reset(sc, T, n, kappa, s))) return rc;
     }
 
     BitsLayout L{bits, n, n - 6};
-    {
+    if (!kappa)
+        for (int i = 0; i < (hp ? hp->pieces : 0); ++i) BENES_CUDA_TRY(cudaStreamWaitEvent(s, hp->piece_ready[i], 0));
+    if (kappa) {
         ProfileScope ps(kInverse, s);
         // the 64-bit word array is free until the first level is labelled
         // (the bucketed form needs whole buckets, of 2^18 entries at most)
@@ -254,41 +257,46 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     // one more level runs in HBM and twice as many CTAs finish blocks of 2^14.
     const int fused_m = opt.cluster ? kFusedLog2M + 1 : (T >> kFusedLog2M) <= 64 ? kFusedLog2M - 1 : kFusedLog2M;
     int cur = 0;
-    for (int level = 0; n - level > fused_m; ++level) {
+    for (int level = 0; kappa && n - level > fused_m; ++level) {
         const int m = n - level;
         const int out_stage = 2 * n - 2 - level;
         const LevelRecords S = records(level, cur), Sn = records(level + 1, cur ^ 1);
         uint32_t *Q = Qbuf[cur];
-        uint32_t *gate = nullptr;
-        if (kappa) {
-            // ruler-sampled labelling; raises `gate` if a walk had to give up
-            gate = gates + level;
-            if ((rc = sampled_label(S, Q, Sn, sc, T, m, kappa, uint32_t(level), cap, opt.walk_pairs, L, out_stage, gate, s)))
-                return rc;
-        }
-        // pointer jumping over all outputs: the whole labelling when sampling is
-        // off, otherwise gated (returns at once unless this level's walks gave up)
-        {
-            ProfileScope ps(kFullLabel, s);
-            if ((rc = launch_full_label(S, Q, Wd, T, m, L, out_stage, gate, s))) return rc;
-        }
+        // ruler-sampled labelling; raises the gate if a walk had to give up
+        if ((rc = sampled_label(S, Q, Sn, sc, T, m, kappa, uint32_t(level), cap, opt.walk_pairs, L, out_stage, gate, s)))
+            return rc;
         {
             ProfileScope ps(kSplit, s);
-            if ((rc = launch_split(S, Q, Sn, Qbuf[cur ^ 1], T, m, kappa, L, level, out_stage, gate, s)))
-                return rc;
+            if ((rc = launch_split(Q, Qbuf[cur ^ 1], T, m, L, level, out_stage, s))) return rc;
         }
         cur ^= 1;
         if (hp && hp->bits_host) {
-            // stages `level` and `out_stage` are final: send them home behind the computation
+            // stages `level` and `out_stage` are final (unless the gate is raised): send them home behind the computation
             BENES_CUDA_TRY(cudaEventRecord(hp->stage_ready[level], s));
             BENES_CUDA_TRY(cudaStreamWaitEvent(hp->d2h, hp->stage_ready[level], 0));
             if ((rc = copy_stage_rows(*hp, bits, n, batch, level, 1, hp->d2h))) return rc;
             if ((rc = copy_stage_rows(*hp, bits, n, batch, out_stage, 1, hp->d2h))) return rc;
         }
     }
+    // Pointer jumping over all outputs, all levels: the whole labelling when sampling is off, otherwise gated
+    // (returns at once unless some walk gave up).  Its sub-permutations go where the records were.
+    uint32_t *const jump_p[2] = {static_cast<uint32_t *>(Sbuf[0]), static_cast<uint32_t *>(Sbuf[1])};
+    const uint32_t *redone = jump_p[(n - fused_m) & 1];
+    {
+        ProfileScope ps(kFullLabel, s);
+        if ((rc = launch_route_jump(perm, jump_p, Qbuf, Wd, T, n, fused_m, L, kappa ? gate : nullptr, s))) return rc;
+    }
+    if (kappa && hp) BENES_CUDA_TRY(cudaMemcpyAsync(hp->gate_host, gate, 4, cudaMemcpyDeviceToHost, s));
+    if (!kappa && hp && hp->bits_host) {
+        for (int level = 0; n - level > fused_m; ++level) {
+            if ((rc = copy_stage_rows(*hp, bits, n, batch, level, 1, s))) return rc;
+            if ((rc = copy_stage_rows(*hp, bits, n, batch, 2 * n - 2 - level, 1, s))) return rc;
+        }
+    }
     const LevelRecords tail = records(n - fused_m, cur);
-    const void *tail_p = tail.packed ? tail.S : tail.P;
-    const int tail_format = tail.packed ? 1 : 0;
+    const void *tail_p = kappa == 0 ? redone : tail.packed ? tail.S : tail.P;
+    const int tail_format = kappa && tail.packed ? 1 : 0;
+    const uint32_t *tail_gate = kappa ? gate : nullptr;
     const size_t blocks = T >> fused_m;
     // the stages of the in-CTA levels are one run of rows in the middle
     const int first = n - fused_m, rows = 2 * fused_m - 1;
@@ -299,12 +307,12 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
         const size_t b1 = ((waves + 1) / 2) * kFusedSplitWave;
         {
             ProfileScope ps(kFused, s);
-            if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, 0, b1))) return rc;
+            if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, 0, b1, tail_gate, redone))) return rc;
         }
         BENES_CUDA_TRY(cudaEventRecord(hp->stage_ready[kMaxLevels - 2], s));
         {
             ProfileScope ps(kFused, s);
-            if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, b1, blocks - b1))) return rc;
+            if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, b1, blocks - b1, tail_gate, redone))) return rc;
         }
         // a block of 2^m outputs owns 2^(m-6) words of every stage
         const size_t w = stage_words(n) * 4, col1 = (b1 << (fused_m - 6)) * 4;
@@ -320,11 +328,20 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     }
     {
         ProfileScope ps(kFused, s);
-        if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s))) return rc;
+        if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, 0, 0, tail_gate, redone))) return rc;
     }
     if (hp && hp->bits_host) {
         if ((rc = copy_stage_rows(*hp, bits, n, batch, first, rows, s))) return rc;
     }
+    return BENES_OK;
+}
+
+// After a host-buffer route has been waited for: if a walk gave up, the stages that went home early have been
+// redone since.
+int fetch_redone_bits(const HostPipe &hp, const uint32_t *bits, size_t bytes, cudaStream_t s) {
+    if (!*hp.gate_host || !hp.bits_host) return BENES_OK;
+    BENES_CUDA_TRY(cudaMemcpyAsync(hp.bits_host, bits, bytes, cudaMemcpyDeviceToHost, s));
+    BENES_CUDA_TRY(cudaStreamSynchronize(s));
     return BENES_OK;
 }
 
@@ -340,6 +357,7 @@ int host_pipe_for_current_device(HostPipe **out) {
     if (!ready[dev]) {
         BENES_CUDA_TRY(cudaStreamCreateWithFlags(&hp.side, cudaStreamNonBlocking));
         BENES_CUDA_TRY(cudaStreamCreateWithFlags(&hp.back, cudaStreamNonBlocking));
+        BENES_CUDA_TRY(cudaMallocHost(&hp.gate_host, 4));
         for (cudaEvent_t &e : hp.part_ready) BENES_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         for (cudaEvent_t &e : hp.piece_ready) BENES_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         for (cudaEvent_t &e : hp.stage_ready) BENES_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -558,10 +576,12 @@ int benes_route_host(const uint32_t *perm_host, int log2n, int batch, uint32_t *
                                            cudaMemcpyHostToDevice, hp->side));
             BENES_CUDA_TRY(cudaEventRecord(hp->piece_ready[i], hp->side));
         }
+        *hp->gate_host = 0u;
         rc = route_levels(d_perm, n, size_t(batch), d_bits, base, s, opt, hp);
         cudaError_t e1 = cudaStreamSynchronize(hp->side), e2 = cudaStreamSynchronize(s);
         if (rc) return rc;
-        return (e1 == cudaSuccess && e2 == cudaSuccess) ? BENES_OK : BENES_ERR_CUDA;
+        if (e1 != cudaSuccess || e2 != cudaSuccess) return BENES_ERR_CUDA;
+        return fetch_redone_bits(*hp, d_bits, bits_bytes, s);
     }
     BENES_CUDA_TRY(cudaMemcpyAsync(d_perm, perm_host, perm_bytes, cudaMemcpyHostToDevice, s));
     rc = benes_route(d_perm, log2n, batch, d_bits, stream);
@@ -691,6 +711,7 @@ int benes_route_apply_host(const uint32_t *perm_host, const void *in_host, void 
         BENES_CUDA_TRY(cudaEventRecord(hp->part_ready[i], hp->side));
         pipe.in_ready[i] = hp->part_ready[i];
     }
+    *hp->gate_host = 0u;
     rc = route_levels(d_perm, n, size_t(batch), d_bits, base, s, opt, hp);
     if (!rc) {
         // the route no longer waits on these events; the apply's last pass reuses them
@@ -700,7 +721,8 @@ int benes_route_apply_host(const uint32_t *perm_host, const void *in_host, void 
     }
     cudaError_t e1 = cudaStreamSynchronize(s), e2 = cudaStreamSynchronize(hp->side), e3 = cudaStreamSynchronize(hp->back);
     if (rc) return rc;
-    return (e1 == cudaSuccess && e2 == cudaSuccess && e3 == cudaSuccess) ? BENES_OK : BENES_ERR_CUDA;
+    if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) return BENES_ERR_CUDA;
+    return fetch_redone_bits(*hp, d_bits, bits_bytes, s);
 }
 
 struct benes_plan {

@@ -185,20 +185,6 @@ __device__ __forceinline__ uint32_t ruler_slot(uint32_t group, uint32_t salt, ui
     return h & kmask;
 }
 
-template <bool PACKED>
-__device__ __forceinline__ void rec_read(const void *S, const uint32_t *P, size_t t, int m, uint32_t &p0, uint32_t &p1) {
-    const uint32_t mask = (1u << m) - 1u;
-    if (PACKED) {
-        const unsigned long long w = __ldcs(static_cast<const unsigned long long *>(S) + t);
-        p0 = uint32_t(w) & mask;
-        p1 = uint32_t(w >> m) & mask;
-    } else {
-        const uint2 r = __ldcs(reinterpret_cast<const uint2 *>(P) + t);
-        p0 = BENES_GUARD(r.x, mask);
-        p1 = BENES_GUARD(r.y, mask);
-    }
-}
-
 // one P value, P[j], read at random
 template <bool PACKED>
 __device__ __forceinline__ uint32_t rec_p(const void *S, const uint32_t *P, uint32_t j, int m) {
@@ -291,16 +277,13 @@ int launch_inverse_partition_piece(const uint32_t *perm, LevelRecords S, void *p
                                    size_t total, size_t j_first, size_t count, int log2m, int kappa,
                                    cudaStream_t s);
 int launch_inverse_scatter(const void *pairs, uint32_t *Q, size_t total, int log2m, cudaStream_t s);
-// Pointer jumping over all outputs (successor build, log2m-2 in-place passes,
-// last pass + output-side bits) in ONE cooperative launch; `gate` (may be
-// null) is a device word: the kernel returns at once while it is 0.
-int launch_full_label(LevelRecords S, const uint32_t *Q, unsigned long long *Wd, size_t total,
-                      int log2m, BitsLayout L, int out_stage, const uint32_t *gate, cudaStream_t s);
-// Input-side bits + next level's inverses; also the next level's records
-// (unclaimed, rulers of salt in_stage + 1) if `gate` is null or *gate != 0 (otherwise the colouring kernel
-// of the sampled labelling has written them already).
-int launch_split(LevelRecords S, const uint32_t *Q, LevelRecords Sn, uint32_t *Qn,
-                 size_t total, int log2m, int kappa, BitsLayout L, int in_stage, int out_stage, const uint32_t *gate,
+// Levels of blocks of 2^log2n .. 2^(last_m + 1) by pointer jumping over all outputs, in ONE cooperative launch;
+// `gate` (may be null) is a device word: the kernel returns at once while it is 0.  P[], Q[]: total words each; the
+// blocks of 2^last_m are left in P[(log2n - last_m) & 1].
+int launch_route_jump(const uint32_t *perm, uint32_t *const P[2], uint32_t *const Q[2], unsigned long long *Wd,
+                      size_t total, int log2n, int last_m, BitsLayout L, const uint32_t *gate, cudaStream_t s);
+// Input-side bits + next level's inverses.
+int launch_split(const uint32_t *Q, uint32_t *Qn, size_t total, int log2m, BitsLayout L, int in_stage, int out_stage,
                  cudaStream_t s);
 
 // ---- ruler-sampled loop labelling (route_sampled.cu) --------------------------
@@ -313,8 +296,8 @@ struct SampledScratch {
 size_t sampled_scratch_bytes(size_t total, int kappa);
 void sampled_scratch_carve(char *base, size_t total, int kappa, SampledScratch *out);
 // Labels every loop of the level, writes the output-side stage and the next
-// level's records Sn; raises *gate if some walk exceeded `cap` hops (the level
-// must then be relabelled and Sn rewritten).
+// level's records Sn; raises *gate if some walk exceeded `cap` hops (the route must then be
+// redone by launch_route_jump).
 int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const SampledScratch &sc, size_t total,
                   int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage, uint32_t *gate, cudaStream_t s);
 // Before the first sampled_label of a route: owners to kUnowned (log2m of the first level).
@@ -325,9 +308,11 @@ int sampled_scratch_reset(const SampledScratch &sc, size_t total, int log2m, int
 // level array (total elements), one CTA per block for log2m <= kFusedLog2M, one
 // cluster of two CTAs per block for log2m = kFusedLog2M + 1.
 // P is a plain uint32 array if records == 0, packed records if 1.
-// `blocks` blocks from `first_block` on (blocks = 0: all from first_block).
+// `blocks` blocks from `first_block` on (blocks = 0: all from first_block).  With a gate: if *gate is not 0, the
+// blocks are those of the plain array `redone`.
 int launch_fused(const void *P, int records, size_t total, int log2m, uint32_t *bits, int log2n,
-                 cudaStream_t s, size_t first_block = 0, size_t blocks = 0);
+                 cudaStream_t s, size_t first_block = 0, size_t blocks = 0, const uint32_t *gate = nullptr,
+                 const uint32_t *redone = nullptr);
 
 // ---- payload apply (apply.cu) ----------------------------------------------
 int launch_apply_stage(const uint32_t *bits, const void *x, void *y, int elem_bytes, int stage,

@@ -694,7 +694,7 @@ __device__ __forceinline__ void fused_enter4(unsigned char *sm, uint32_t i4, con
 template <int LOGC, int THREADS>
 __global__ void __launch_bounds__(THREADS, (FusedCfg<LOGC, THREADS>::kMinCtas))
 k_route_fused(const uint32_t *__restrict__ P, int records, uint32_t *__restrict__ bits, int log2n, int logs,
-              size_t first, size_t end) {
+              size_t first, size_t end, const uint32_t *__restrict__ gate, const uint32_t *__restrict__ redone) {
     using Cfg = FusedCfg<LOGC, THREADS>;
     constexpr uint32_t C = Cfg::C, T = Cfg::T;
     extern __shared__ __align__(16) unsigned char sm[];
@@ -704,6 +704,10 @@ k_route_fused(const uint32_t *__restrict__ P, int records, uint32_t *__restrict_
     out.flat0 = first + size_t(blockIdx.x) * C;
     out.valid = uint32_t(end - out.flat0 < size_t(C) ? end - out.flat0 : size_t(C));
     const uint32_t tid = threadIdx.x, smask = (1u << logs) - 1u;
+    if (gate && *gate != 0u) {
+        P = redone;
+        records = 0;
+    }
     const bool aligned = (reinterpret_cast<uintptr_t>(P) & 15u) == 0;
     for (uint32_t i4 = tid; i4 < C / 4; i4 += T) {
         const size_t f = out.flat0 + 4u * i4;
@@ -912,7 +916,11 @@ constexpr size_t kClusterSmemBytes = kClusterTopBytes > ClusterTailCfg::kSmemByt
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(ClusterTailCfg::T)
 k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restrict__ bits, int log2n,
-                 uint32_t block0) {
+                 uint32_t block0, const uint32_t *__restrict__ gate, const uint32_t *__restrict__ redone) {
+    if (gate && *gate != 0u) {
+        P = redone;
+        records = 0;
+    }
     constexpr int LOGM = kFusedLog2M;           // per CTA
     using Cfg = ClusterTailCfg;
     constexpr int M = Cfg::C;                      // outputs per CTA
@@ -1102,7 +1110,7 @@ k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restri
 
 template <int LOGC, int THREADS>
 int launch_one(const uint32_t *P, int records, size_t first, size_t end, uint32_t *bits, int log2n, int logs,
-               cudaStream_t s) {
+               cudaStream_t s, const uint32_t *gate, const uint32_t *redone) {
     using Cfg = FusedCfg<LOGC, THREADS>;
     static OncePerDevice configured;
     const int rc = configured.run([]() -> int {
@@ -1114,12 +1122,13 @@ int launch_one(const uint32_t *P, int records, size_t first, size_t end, uint32_
     });
     if (rc) return rc;
     const size_t ctas = (end - first + Cfg::C - 1) >> LOGC;
-    k_route_fused<LOGC, THREADS><<<unsigned(ctas), THREADS, Cfg::kSmemBytes, s>>>(P, records, bits, log2n, logs, first, end);
+    k_route_fused<LOGC, THREADS><<<unsigned(ctas), THREADS, Cfg::kSmemBytes, s>>>(P, records, bits, log2n, logs, first, end,
+                                                                                        gate, redone);
     return launch_status();
 }
 
 int launch_cluster2(const uint32_t *P, int records, size_t first_block, size_t blocks, uint32_t *bits,
-                    int log2n, cudaStream_t s) {
+                    int log2n, cudaStream_t s, const uint32_t *gate, const uint32_t *redone) {
     static OncePerDevice configured;
     const int rc = configured.run([]() -> int {
         BENES_CUDA_TRY(cudaFuncSetAttribute(k_route_cluster2, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1131,19 +1140,19 @@ int launch_cluster2(const uint32_t *P, int records, size_t first_block, size_t b
     if (rc) return rc;
     // two CTAs per block (the cluster size is part of the kernel)
     k_route_cluster2<<<unsigned(2 * blocks), ClusterTailCfg::T, kClusterSmemBytes, s>>>(P, records, bits, log2n,
-                                                                                        uint32_t(first_block));
+                                                                                        uint32_t(first_block), gate, redone);
     return launch_status();
 }
 
 }  // namespace
 
 int launch_fused(const void *Pv, int records, size_t total, int log2m, uint32_t *bits, int log2n,
-                 cudaStream_t s, size_t first_block, size_t blocks) {
+                 cudaStream_t s, size_t first_block, size_t blocks, const uint32_t *gate, const uint32_t *redone) {
     const uint32_t *P = static_cast<const uint32_t *>(Pv);
     if (log2m < 1 || log2m > kClusterLog2M) return BENES_ERR_BADARG;
     if (blocks == 0) blocks = (total >> log2m) - first_block;        // all the rest
     if (first_block + blocks > (total >> log2m)) return BENES_ERR_BADARG;
-    if (log2m == kClusterLog2M) return launch_cluster2(P, records, first_block, blocks, bits, log2n, s);
+    if (log2m == kClusterLog2M) return launch_cluster2(P, records, first_block, blocks, bits, log2n, s, gate, redone);
     const size_t first = first_block << log2m, end = first + (blocks << log2m);
     // whole permutations of up to 2^11, and not more switches than the GPU has threads
     if (records == 0 && log2m == log2n && log2m <= 11 && first == 0 && end / 2 <= size_t(sm_count()) * 2048) {
@@ -1159,7 +1168,7 @@ int launch_fused(const void *Pv, int records, size_t total, int log2m, uint32_t 
     // CTAs that have an SM to themselves get more threads: their time is a chain of short
     // phases, not the instructions they issue.
     const bool alone = ((end - first + (size_t(1) << logc) - 1) >> logc) <= size_t(sm_count());
-#define BENES_FUSED(LC, T) return launch_one<LC, T>(P, records, first, end, bits, log2n, log2m, s)
+#define BENES_FUSED(LC, T) return launch_one<LC, T>(P, records, first, end, bits, log2n, log2m, s, gate, redone)
     switch (logc) {
         case 10: if (alone) BENES_FUSED(10, 256); BENES_FUSED(10, 32);
         case 11: if (alone) BENES_FUSED(11, 512); BENES_FUSED(11, 64);

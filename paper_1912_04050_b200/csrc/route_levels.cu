@@ -4,10 +4,9 @@
 // M = 2^log2m owns flat indices [bM, (b+1)M), and P / Q hold block-local
 // values (record formats: see common.cuh).
 //
-// This file: the level-0 inverse scatter, the compaction that forms the next
-// level, and pointer jumping over ALL outputs (one cooperative kernel), which
-// is the labelling when sampling is switched off and the fallback when a walk
-// of the sampled labelling gives up.
+// This file: the level-0 inverse scatter, the input side of the compaction that forms the next
+// level, and the levels by pointer jumping over ALL outputs (one cooperative kernel for all of
+// them), used when sampling is switched off and when a walk of the sampled labelling gives up.
 //
 // Words of the pointer-jumping array: one 64-bit word per output,
 //   low 32 bits  = nxt (flat index of the current successor),
@@ -236,78 +235,90 @@ __device__ __forceinline__ unsigned long long jump(unsigned long long w, unsigne
     return (hi << 32) | (t & 0xFFFFFFFFull);
 }
 
-// a2 + a3 + a4 + output side of a5 over all outputs of the level, passes
-// separated by grid-wide barriers (cooperative launch).
-//   build : W[j] = (g(j), j), g(j) = base + Q[base + (P[j^1] ^ 1)]
-//   passes: W[j] <- (W[nxt].nxt, min(mn, W[nxt].mn)), in place
-//   last  : even outputs only; colour = leader & 1 -> output-side stage word
-template <bool PACKED>
-__global__ void __launch_bounds__(kThreads)
-k_full_label(const void *__restrict__ S, const uint32_t *__restrict__ P, const uint32_t *__restrict__ Q,
-             unsigned long long *__restrict__ Wd, size_t total, int m, int passes,
-             BitsLayout L, int out_stage, const uint32_t *__restrict__ gate) {
-    if (gate && *gate == 0u) return;        // same value for every thread of the grid
-    const uint32_t mmask = (1u << m) - 1u;
-    cg::grid_group grid = cg::this_grid();
-    const size_t stride = size_t(gridDim.x) * blockDim.x;
-    const size_t first = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    ulonglong2 *W2 = reinterpret_cast<ulonglong2 *>(Wd);
+// All levels from the caller's permutation down to blocks of 2^last_m outputs by pointer jumping over all
+// outputs, in one cooperative launch with grid-wide barriers (P and Q plain arrays).  Per level:
+//   build : W[j] = (g(j), j), g(j) = base + Q[base + (P[j^1] ^ 1)]                       (a2)
+//   passes: W[j] <- (W[nxt].nxt, min(mn, W[nxt].mn)), in place                            (a3)
+//   last  : even outputs only; colour = leader & 1 -> output-side stage word              (a4, a5)
+//   split : input-side stage word, the next level's P and Q                               (a5, a6)
+// It is the whole labelling when sampling is off, and the second attempt when a walk of the sampled
+// labelling gave up at some level and raised `gate` (it returns at once while the gate is 0).  One such launch
+// per route: one per level cost 6 us each, a twelfth of the route of 2^18.
+struct JumpArrays {
+    const uint32_t *perm;
+    uint32_t *P[2], *Q[2];
+    unsigned long long *W;
+};
 
-    const size_t switches = total / 2;
-    for (size_t t = first; t < switches; t += stride) {
-        uint32_t p0, p1;
-        rec_read<PACKED>(S, P, t, m, p0, p1);
-        size_t j = 2 * t;
-        size_t base = j & ~size_t(mmask);
-        uint32_t b32 = uint32_t(base);
-        uint32_t g0 = b32 + BENES_GUARD(__ldg(Q + base + (p1 ^ 1u)), mmask);
-        uint32_t g1 = b32 + BENES_GUARD(__ldg(Q + base + (p0 ^ 1u)), mmask);
-        ulonglong2 a;
-        a.x = make_word(g0, uint32_t(j));
-        a.y = make_word(g1, uint32_t(j) + 1u);
-        W2[t] = a;
+__global__ void __launch_bounds__(kThreads)
+k_route_jump(JumpArrays a, uint32_t total, int log2n, int last_m, BitsLayout L, const uint32_t *__restrict__ gate) {
+    if (gate && *gate == 0u) return;        // same value for every thread of the grid
+    cg::grid_group grid = cg::this_grid();
+    const uint32_t stride = gridDim.x * blockDim.x, first = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t switches = total / 2, quads = total / 4;     // multiples of 32: a warp stays together
+    ulonglong2 *W2 = reinterpret_cast<ulonglong2 *>(a.W);
+    {
+        const uint32_t mmask = (1u << log2n) - 1u;
+        for (uint32_t j = first; j < total; j += stride)
+            a.Q[0][(j & ~mmask) + BENES_GUARD(__ldcg(a.perm + j), mmask)] = j & mmask;
     }
     grid.sync();
-
-    const size_t quads = total / 4;
-    for (int r = 0; r < passes; ++r) {
-        for (size_t i = first; i < quads; i += stride) {
-            ulonglong2 a = __ldcg(W2 + 2 * i);
-            ulonglong2 b = __ldcg(W2 + 2 * i + 1);
-            unsigned long long t0 = __ldcg(Wd + uint32_t(a.x));
-            unsigned long long t1 = __ldcg(Wd + uint32_t(a.y));
-            unsigned long long t2 = __ldcg(Wd + uint32_t(b.x));
-            unsigned long long t3 = __ldcg(Wd + uint32_t(b.y));
-            a.x = jump(a.x, t0);
-            a.y = jump(a.y, t1);
-            b.x = jump(b.x, t2);
-            b.y = jump(b.y, t3);
-            __stcg(W2 + 2 * i, a);
-            __stcg(W2 + 2 * i + 1, b);
+    for (int m = log2n; m > last_m; --m) {
+        const int level = log2n - m, out_stage = 2 * log2n - 2 - level;
+        const uint32_t mmask = (1u << m) - 1u, H = (mmask + 1u) >> 1;
+        const uint32_t *P = level ? a.P[level & 1] : a.perm, *Q = a.Q[level & 1];
+        uint32_t *Pn = a.P[(level + 1) & 1], *Qn = a.Q[(level + 1) & 1];
+        for (uint32_t t = first; t < switches; t += stride) {
+            const uint32_t j = 2u * t, base = j & ~mmask;
+            const uint32_t p0 = BENES_GUARD(__ldcg(P + j), mmask), p1 = BENES_GUARD(__ldcg(P + j + 1), mmask);
+            ulonglong2 w;
+            w.x = make_word(base + BENES_GUARD(__ldcg(Q + base + (p1 ^ 1u)), mmask), j);
+            w.y = make_word(base + BENES_GUARD(__ldcg(Q + base + (p0 ^ 1u)), mmask), j + 1u);
+            __stcg(W2 + t, w);
+        }
+        grid.sync();
+        for (int r = 0; r < m - 2; ++r) {
+            for (uint32_t i = first; i < quads; i += stride) {
+                ulonglong2 x = __ldcg(W2 + 2 * size_t(i)), y = __ldcg(W2 + 2 * size_t(i) + 1);
+                const unsigned long long t0 = __ldcg(a.W + uint32_t(x.x)), t1 = __ldcg(a.W + uint32_t(x.y));
+                const unsigned long long t2 = __ldcg(a.W + uint32_t(y.x)), t3 = __ldcg(a.W + uint32_t(y.y));
+                x.x = jump(x.x, t0);
+                x.y = jump(x.y, t1);
+                y.x = jump(y.x, t2);
+                y.y = jump(y.y, t3);
+                __stcg(W2 + 2 * size_t(i), x);
+                __stcg(W2 + 2 * size_t(i) + 1, y);
+            }
+            grid.sync();
+        }
+        for (uint32_t t = first; t < switches; t += stride) {
+            const unsigned long long w = __ldcg(a.W + 2 * size_t(t)), v = __ldcg(a.W + uint32_t(w));
+            const uint32_t word = __ballot_sync(0xFFFFFFFFu, uint32_t(jump(w, v) >> 32) & 1u);
+            if ((threadIdx.x & 31) == 0) __stcg(L.bits + L.word32(out_stage, t >> 5), word);
+        }
+        grid.sync();
+        for (uint32_t t = first; t < switches; t += stride) {
+            const uint32_t j = 2u * t, base = j & ~mmask, tl = (j - base) >> 1;
+            const uint32_t *colours = L.bits + L.word32(out_stage, (base >> 1) >> 5);
+            const uint32_t c = (__ldcg(colours + (tl >> 5)) >> (tl & 31u)) & 1u;
+            const uint32_t p0 = BENES_GUARD(__ldcg(P + j), mmask), p1 = BENES_GUARD(__ldcg(P + j + 1), mmask);
+            __stcg(Pn + base + tl, (c ? p1 : p0) >> 1);
+            __stcg(Pn + base + H + tl, (c ? p0 : p1) >> 1);
+            const uint32_t q0 = BENES_GUARD(__ldcg(Q + j), mmask), q1 = BENES_GUARD(__ldcg(Q + j + 1), mmask);
+            const uint32_t cin = ((__ldcg(colours + (q0 >> 6)) >> ((q0 >> 1) & 31u)) ^ q0) & 1u;
+            __stcg(Qn + base + tl, (cin ? q1 : q0) >> 1);
+            __stcg(Qn + base + H + tl, (cin ? q0 : q1) >> 1);
+            const uint32_t word = __ballot_sync(0xFFFFFFFFu, cin);
+            if ((threadIdx.x & 31) == 0) L.bits[L.word32(level, t >> 5)] = word;
         }
         grid.sync();
     }
-
-    for (size_t t = first; t < switches; t += stride) {
-        unsigned long long w = __ldcg(Wd + 2 * t);
-        unsigned long long v = __ldcg(Wd + uint32_t(w));
-        uint32_t mn = uint32_t(jump(w, v) >> 32);
-        uint32_t word = __ballot_sync(0xFFFFFFFFu, mn & 1u);
-        if ((threadIdx.x & 31) == 0) L.bits[L.word(out_stage, t >> 5)] = word;
-    }
 }
 
-// in-side half of a5 + a6: input-side stage word and Q'.  With `with_records`
-// (no sampled labelling, or its gate raised) also the next level's records:
-// position tl of the upper half-block takes P[2t or 2t+1] >> 1 of switch tl,
-// so the thread that owns switches 2i and 2i+1 holds both values of one record
-// of each half-block and stores whole records.
-template <bool PACKED, bool NEXT_PACKED>
+// in-side half of a5 + a6: input-side stage word and Q' (the colouring kernel has written the next level's records).
 __global__ void __launch_bounds__(kThreads, 8)
-k_split(const void *__restrict__ S, const uint32_t *__restrict__ P, const uint4 *__restrict__ Q4,
-        void *__restrict__ Sn, uint32_t *__restrict__ Pn, uint32_t *__restrict__ Qn, uint32_t pairs, int m, int kappa,
-        BitsLayout L, int in_stage, int out_stage, const uint32_t *__restrict__ gate, uint32_t rounds) {
-    const bool with_records = !gate || *gate != 0u;
+k_split(const uint4 *__restrict__ Q4, uint32_t *__restrict__ Qn, uint32_t pairs, int m,
+        BitsLayout L, int in_stage, int out_stage, uint32_t rounds) {
     const uint32_t mmask = (1u << m) - 1u;
     // a CTA takes `rounds` consecutive groups of blockDim.x pairs: the colour
     // words it gathers belong to one block of the level for a long time (L1 hits)
@@ -328,18 +339,6 @@ k_split(const void *__restrict__ S, const uint32_t *__restrict__ P, const uint4 
         const uint32_t base = (2u * t) & ~mmask;
         const uint32_t tl = t - (base >> 1);
         const uint32_t *colours = L.bits + L.word32(out_stage, (base >> 1) >> 5);   // the block's words of that stage
-        if (with_records) {
-            uint32_t px0, py0, px1, py1;
-            rec_read<PACKED>(S, P, t, m, px0, py0);
-            rec_read<PACKED>(S, P, t + 1, m, px1, py1);
-            // colours of outputs 2t and 2t+2
-            const uint32_t cwd = colours[tl >> 5];
-            const uint32_t c0 = (cwd >> (tl & 31u)) & 1u, c1 = (cwd >> ((tl + 1u) & 31u)) & 1u;
-            const uint32_t r = (base >> 1) + (tl >> 1);
-            const uint32_t salt = uint32_t(in_stage) + 1u;
-            rec_write<NEXT_PACKED>(Sn, Pn, r, m - 1, (c0 ? py0 : px0) >> 1, (c1 ? py1 : px1) >> 1, kappa, salt);
-            rec_write<NEXT_PACKED>(Sn, Pn, r + (H >> 1), m - 1, (c0 ? px0 : py0) >> 1, (c1 ? px1 : py1) >> 1, kappa, salt);
-        }
         q.x = BENES_GUARD(q.x, mmask); q.y = BENES_GUARD(q.y, mmask); q.z = BENES_GUARD(q.z, mmask); q.w = BENES_GUARD(q.w, mmask);
         // colour of the output fed by input 2t (2t+2): that output's switch bit, flipped for an odd output
         const uint32_t cin0 = ((colours[q.x >> 6] >> ((q.x >> 1) & 31u)) ^ q.x) & 1u;
@@ -369,7 +368,7 @@ k_validate(const uint32_t *__restrict__ perm, size_t total, uint32_t nmask,
     }
 }
 
-// CTAs of k_full_label that are resident together on the current device.
+// CTAs of k_route_jump that are resident together on the current device.
 int cooperative_grid(int *out) {
     constexpr int kMaxDev = 64;
     static int cached[kMaxDev] = {};
@@ -381,10 +380,7 @@ int cooperative_grid(int *out) {
         BENES_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
         if (!coop) return BENES_ERR_CUDA;
         BENES_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        BENES_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_full_label<false>, kThreads, 0));
-        int per_sm_packed = 0;
-        BENES_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_packed, k_full_label<true>, kThreads, 0));
-        if (per_sm_packed < per_sm) per_sm = per_sm_packed;
+        BENES_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_route_jump, kThreads, 0));
         if (sms < 1 || per_sm < 1) return BENES_ERR_CUDA;
         cached[dev] = sms * per_sm;
     }
@@ -457,27 +453,24 @@ int launch_inverse(const uint32_t *perm, LevelRecords S, uint32_t *Q, size_t tot
     return launch_status();
 }
 
-int launch_full_label(LevelRecords S, const uint32_t *Q, unsigned long long *Wd, size_t total,
-                      int log2m, BitsLayout L, int out_stage, const uint32_t *gate,
-                      cudaStream_t s) {
+int launch_route_jump(const uint32_t *perm, uint32_t *const P[2], uint32_t *const Q[2], unsigned long long *Wd,
+                      size_t total, int log2n, int last_m, BitsLayout L, const uint32_t *gate, cudaStream_t s) {
     int grid = 0;
     int rc = cooperative_grid(&grid);
     if (rc) return rc;
     size_t need = (total / 2 + kThreads - 1) / kThreads;
     if (size_t(grid) > need) grid = int(need);
-    int passes = log2m - 2;
-    void *args[] = {(void *)&S.S, (void *)&S.P, (void *)&Q, (void *)&Wd, (void *)&total, (void *)&log2m,
-                    (void *)&passes, (void *)&L, (void *)&out_stage, (void *)&gate};
-    const void *kernel = S.packed ? (const void *)k_full_label<true> : (const void *)k_full_label<false>;
-    if (cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(kThreads), args, 0, s) != cudaSuccess) {
+    JumpArrays a{perm, {P[0], P[1]}, {Q[0], Q[1]}, Wd};
+    uint32_t total32 = uint32_t(total);
+    void *args[] = {(void *)&a, (void *)&total32, (void *)&log2n, (void *)&last_m, (void *)&L, (void *)&gate};
+    if (cudaLaunchCooperativeKernel((const void *)k_route_jump, dim3(grid), dim3(kThreads), args, 0, s) != cudaSuccess) {
         cudaGetLastError();
         return BENES_ERR_CUDA;
     }
     return launch_status();
 }
 
-int launch_split(LevelRecords S, const uint32_t *Q, LevelRecords Sn, uint32_t *Qn,
-                 size_t total, int log2m, int kappa, BitsLayout L, int in_stage, int out_stage, const uint32_t *gate,
+int launch_split(const uint32_t *Q, uint32_t *Qn, size_t total, int log2m, BitsLayout L, int in_stage, int out_stage,
                  cudaStream_t s) {
     const uint32_t pairs = uint32_t(total / 4);                  // two switches per thread
     const uint4 *Q4 = reinterpret_cast<const uint4 *>(Q);
@@ -488,15 +481,7 @@ int launch_split(LevelRecords S, const uint32_t *Q, LevelRecords Sn, uint32_t *Q
     uint32_t rounds = stream_rounds(pairs, kThreads);
     if (log2m >= 20 && log2m <= 22 && rounds > (1u << (log2m - 20))) rounds = 1u << (log2m - 20);
     const unsigned grid = unsigned((size_t(pairs) + size_t(kThreads) * rounds - 1) / (size_t(kThreads) * rounds));
-    if (S.packed)          // a packed level is followed by packed levels only
-        k_split<true, true><<<grid, kThreads, 0, s>>>(S.S, S.P, Q4, Sn.S, Sn.P, Qn, pairs, log2m, kappa, L, in_stage,
-                                                       out_stage, gate, rounds);
-    else if (Sn.packed)
-        k_split<false, true><<<grid, kThreads, 0, s>>>(S.S, S.P, Q4, Sn.S, Sn.P, Qn, pairs, log2m, kappa, L, in_stage,
-                                                        out_stage, gate, rounds);
-    else
-        k_split<false, false><<<grid, kThreads, 0, s>>>(S.S, S.P, Q4, Sn.S, Sn.P, Qn, pairs, log2m, kappa, L, in_stage,
-                                                         out_stage, gate, rounds);
+    k_split<<<grid, kThreads, 0, s>>>(Q4, Qn, pairs, log2m, L, in_stage, out_stage, rounds);
     return launch_status();
 }
 

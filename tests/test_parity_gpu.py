@@ -208,6 +208,23 @@ def test_route_walks_that_give_up_fall_back_to_full_pointer_jumping(cap, labelli
         assert np.array_equal(gpu_route(perm, n), oracle.route(perm, n))
 
 
+@pytest.mark.parametrize("kappa,cap", [(None, 2), (0, None), (5, 30)])
+@pytest.mark.parametrize("n,batch", [(16, 1), (16, 5), (17, 2), (19, 1), (21, 1)])
+def test_route_redone_as_a_whole(n, batch, kappa, cap, labelling_options):
+    """A walk that gives up (and sampling switched off) sends all levels above the in-CTA ones through one
+    pointer-jumping launch; the host entry point has sent stages home by then and fetches them again."""
+    if kappa is not None:
+        binding.benes_set_option(binding.OPT_SAMPLE_LOG2K, kappa)
+    if cap is not None:
+        binding.benes_set_option(binding.OPT_WALK_CAP, cap)
+    perm = inputs.random_perm_batch(n, batch, seed0=17 * n + batch)
+    want = oracle.route(perm, n)
+    assert np.array_equal(gpu_route(perm, n), want)
+    bits = np.zeros_like(want)
+    binding.benes_route_host(perm, n, batch, bits)
+    assert np.array_equal(bits, want)
+
+
 @pytest.mark.parametrize("kappa,cap", [(None, None), (2, None), (4, None), (None, 12)])
 @pytest.mark.parametrize("n,batch", [(18, 3), (19, 3), (20, 5), (19, 7)])
 def test_route_batch_not_a_power_of_two_with_resampled_lists(n, batch, kappa, cap, labelling_options):
