@@ -288,9 +288,9 @@ int launch_split(const uint32_t *Q, uint32_t *Qn, size_t total, int log2m, BitsL
 
 // ---- ruler-sampled loop labelling (route_sampled.cu) --------------------------
 struct SampledScratch {
-    uint4 *rec;                  // total >> kappa walk records
-    unsigned long long *list[5]; // contracted lists: at most total >> (kappa + 2 i) words
-    uint32_t *owner[5];          // owners of the words of list[i] (all kUnowned between uses)
+    uint2 *rec[5];               // walk records (minimum, peer), which are contracted lists: at most
+                                 // total >> (kappa + 2 i) words
+    uint32_t *owner[5];          // owners of the pairs of words of rec[i] (all kUnowned between uses)
     uint32_t *bits[5];           // parity of every word's cycle minimum, one bit each
 };
 size_t sampled_scratch_bytes(size_t total, int kappa);

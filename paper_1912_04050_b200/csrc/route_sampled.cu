@@ -17,14 +17,13 @@
 //      keeps the smallest output index on its own side of the switches it
 //      claimed (on the far side it is the same with the last bit flipped) and its partner
 //      (peer).  The claim stores (walker, side of arrival).
-//   3. k_combine: the segment of walker rho ends at ruler output peer^1 and
-//      its minimum is min(least[rho], least[peer] ^ 1): one 64-bit (next, min) word
-//      per ruler output -- the contracted list.
+//   3. The segment of walker rho ends at ruler output peer^1: the walk records are the
+//      contracted list as they are (see pair_least for the minima).
 //   4. The contracted list is labelled with the parity of every cycle's minimum:
 //      lists of up to 2^14 words per block in one CTA's shared memory, longer
 //      ones by sampling again: the list is mirror symmetric like the loops, so
 //      it is sampled the same way (one ruler pair per 4 to 16 pairs of words, walks
-//      that meet in the middle, k_combine again).
+//      that meet in the middle).
 //   5. k_colour: output 2t lies on its owner's cycle if the owner arrived on
 //      the even side, else on the mirror cycle, which has the other colour:
 //      colour = (cycle minimum of the owner & 1) ^ side.  A switch nobody
@@ -164,56 +163,36 @@ k_walk(unsigned long long *__restrict__ S8, const uint32_t *__restrict__ P, cons
     }
 }
 
-// Step 3.  A switch walker's record is (minimum, peer): the outputs on the far side of the switches it
-// claimed are the ones it stood on with the last bit flipped, and so is their minimum.  (That counts
-// the far side of its own ruler switch too, which is where the other walker's segment ends.)
-__global__ void __launch_bounds__(kThreads)
-k_combine(const uint2 *__restrict__ rec, unsigned long long *__restrict__ W, uint32_t rulers) {
-    const uint32_t rho = blockIdx.x * kThreads + threadIdx.x;
-    if (rho >= rulers) return;
-    const uint2 a = rec[rho];
-    const uint32_t peer = BENES_GUARD_BELOW(a.y, rulers, rho);
-    W[rho] = make_word(peer ^ 1u, min(a.x, __ldg(&rec[peer].x) ^ 1u));
-}
-
-// The same for walks over a list, whose far sides have a minimum of their own.
-__global__ void __launch_bounds__(kThreads)
-k_combine_list(const uint4 *__restrict__ rec, unsigned long long *__restrict__ W, uint32_t rulers) {
-    const uint32_t rho = blockIdx.x * kThreads + threadIdx.x;
-    if (rho >= rulers) return;
-    const uint4 a = rec[rho];
-    const uint32_t peer = BENES_GUARD_BELOW(a.z, rulers, rho);
-    const uint4 b = __ldg(rec + peer);
-    W[rho] = make_word(peer ^ 1u, min(a.x, b.y));
-}
+// Step 3, the contracted list.  It needs no pass of its own.  The segment of walker rho ends at ruler output
+// peer ^ 1, so that is the word after rho.  Words 2q and 2q + 1 (the two outputs of a ruler switch) form a pair; the
+// cycle through one and the cycle through the other are mirror images, so what walker 2q + 1 has seen, with
+// the last bit flipped, lies on the cycle of word 2q, and every segment of a cycle has both of its walkers in
+// pairs of the cycle: the minimum over a cycle is the minimum over its pairs of
+//     min(least[2q], least[2q + 1] ^ 1)          (on the side of word 2q; on the other side, that ^ 1).
+__device__ __forceinline__ uint32_t pair_least(uint32_t least0, uint32_t least1) { return min(least0, least1 ^ 1u); }
 
 // Step 4, sampling a list.  The contracted list inherits the mirror symmetry
 // of the loops (next[rho] = sigma implies next[sigma ^ 1] = rho ^ 1), and so does
-// every list sampled from it this way: a list is sampled the way the switches are.  Words 2q and 2q+1 form a pair; one pair per 16
+// every list sampled from it this way: a list is sampled the way the switches are.  One pair per 2^spacing
 // pairs is a ruler pair, both of its words start a walker; the walker from the
 // even word runs along its cycle, the walker from the odd word of the NEXT
 // ruler pair runs along the mirror cycle, i.e. over the same pairs from the
 // other end; each claims pairs (owner[q] = walker, side of arrival) and stops
-// where the other one has been.  The longest walk of a launch is half as long
-// as with one-directional walks.  A walker keeps the minimum over the words it
-// passed (fwd), over their partners (part) and whom it met (peer): the same
-// record as in step 2, turned into the 16 times shorter list by k_combine.
-// (spacing = log2 of the pairs per ruler pair.)
+// where the other one has been.  A walker's record is (minimum, peer) again.
 __global__ void __launch_bounds__(kWalkThreads)
-k_list_walk_pairs(const ulonglong2 *__restrict__ W2p, uint32_t *__restrict__ owner, uint4 *__restrict__ rec,
+k_list_walk_pairs(const uint4 *__restrict__ pair, uint32_t *__restrict__ owner, uint2 *__restrict__ rec,
                   uint32_t rulers, uint32_t pairs, int spacing, uint32_t salt, uint32_t cap, uint32_t *__restrict__ gate) {
     const uint32_t sigma = blockIdx.x * kWalkThreads + threadIdx.x;
     if (sigma >= rulers) return;
     const uint32_t kmask = (1u << spacing) - 1u;
     const uint32_t group = sigma >> 1, side0 = sigma & 1u;
     const uint32_t q0 = (group << spacing) | ruler_slot(group, salt, kmask);
-    ulonglong2 w = __ldcg(W2p + q0);
+    uint4 w = __ldcg(pair + q0);
     if (!side0) owner[q0] = sigma << 1;                            // the ruler pair belongs to its even walker
-    unsigned long long own = side0 ? w.y : w.x;
-    uint32_t fwd = uint32_t(own >> 32), part = kUnowned, peer = sigma ^ 1u, hops = 0;
+    uint32_t least = pair_least(w.x, w.z) ^ side0, next = (side0 ? w.w : w.y) ^ 1u, peer = sigma ^ 1u, hops = 0;
     for (;;) {
         // (a batch need not be a power of two: an index a raised gate left undefined is clamped, not masked)
-        const uint32_t e = uint32_t(own), q = BENES_GUARD_BELOW(e >> 1, pairs, 0u), side = e & 1u, g = q >> spacing;
+        const uint32_t q = BENES_GUARD_BELOW(next >> 1, pairs, 0u), side = next & 1u, g = q >> spacing;
         if ((q & kmask) == ruler_slot(g, salt, kmask)) {           // reached the next ruler pair
             peer = (2u * g + side) ^ 1u;
             break;
@@ -223,18 +202,16 @@ k_list_walk_pairs(const ulonglong2 *__restrict__ W2p, uint32_t *__restrict__ own
             break;
         }
         if ((hops & 63u) == 0u && gate_raised(gate)) break;
-        w = __ldcg(W2p + q);
+        w = __ldcg(pair + q);
         const uint32_t prev = atomicCAS(owner + q, kUnowned, (sigma << 1) | side);
         if (prev != kUnowned) {                                    // met the walker from the other end
             peer = prev >> 1;
             break;
         }
-        own = side ? w.y : w.x;
-        const unsigned long long far = side ? w.x : w.y;
-        fwd = min(fwd, uint32_t(own >> 32));
-        part = min(part, uint32_t(far >> 32));
+        least = min(least, pair_least(w.x, w.z) ^ side);
+        next = (side ? w.w : w.y) ^ 1u;
     }
-    rec[sigma] = make_uint4(fwd, part, peer, 0u);
+    rec[sigma] = make_uint2(least, peer);
 }
 
 // Back from a sampled list: a thread takes the pair 2q, 2q+1 (and hands the
@@ -243,25 +220,9 @@ k_list_walk_pairs(const ulonglong2 *__restrict__ W2p, uint32_t *__restrict__ own
 // parity, and so does word 2q+1's: one bit of the sampled list (`cb2`) gives the two bits of
 // the pair (`cb`).  A pair nobody claimed lies on a cycle without ruler pair: the thread walks the
 // cycle of word 2q.
-__device__ __forceinline__ uint32_t list_cycle_min(const unsigned long long *W, uint32_t e0, uint32_t words,
-                                                   uint32_t cap, uint32_t *gate) {
-    unsigned long long v = __ldcg(W + e0);
-    uint32_t mn = uint32_t(v >> 32), e = BENES_GUARD_BELOW(uint32_t(v), words, 0u), hops = 0;
-    while (e != e0) {
-        if (++hops > cap) {
-            *gate = 1u;
-            break;
-        }
-        v = __ldcg(W + e);
-        mn = min(mn, uint32_t(v >> 32));
-        e = BENES_GUARD_BELOW(uint32_t(v), words, 0u);
-    }
-    return mn;
-}
-
 __global__ void __launch_bounds__(kThreads)
-k_list_resolve_pairs(const unsigned long long *__restrict__ W, uint32_t *__restrict__ owner,
-                     const uint32_t *__restrict__ cb2, uint32_t pairs, uint32_t words,
+k_list_resolve_pairs(const uint4 *__restrict__ pair, uint32_t *__restrict__ owner,
+                     const uint32_t *__restrict__ cb2, uint32_t pairs,
                      uint32_t cap, uint32_t *__restrict__ gate, uint32_t *__restrict__ cb) {
     const uint32_t q = blockIdx.x * kThreads + threadIdx.x;       // pairs is a multiple of 32
     if (q >= pairs) return;
@@ -272,7 +233,19 @@ k_list_resolve_pairs(const unsigned long long *__restrict__ W, uint32_t *__restr
         bit0 = ((__ldg(cb2 + (sigma >> 5)) >> (sigma & 31u)) ^ code) & 1u;
         owner[q] = kUnowned;
     } else {
-        bit0 = list_cycle_min(W, 2u * q, words, cap, gate) & 1u;
+        uint4 w = __ldg(pair + q);
+        uint32_t least = pair_least(w.x, w.z), next = w.y ^ 1u, hops = 0;
+        while (next != 2u * q) {
+            if (++hops > cap) {
+                *gate = 1u;
+                break;
+            }
+            if ((hops & 63u) == 0u && gate_raised(gate)) break;
+            w = __ldg(pair + BENES_GUARD_BELOW(next >> 1, pairs, 0u));
+            least = min(least, pair_least(w.x, w.z) ^ (next & 1u));
+            next = ((next & 1u) ? w.w : w.y) ^ 1u;
+        }
+        bit0 = least & 1u;
     }
     // a warp covers 64 words: two words of cb
     store_stage_bits64(cb + ((q - (threadIdx.x & 31u)) >> 4), bit0, bit0 ^ 1u);
@@ -284,57 +257,38 @@ k_list_resolve_pairs(const unsigned long long *__restrict__ W, uint32_t *__restr
 // that are left, and a queue for the pairs of cycles without ruler pair.  Pointer jumping over the whole list
 // took log2b - 1 passes of random shared-memory reads (2^14 words: 25 us, now LIST_US).
 // Only the parities of the minima are needed from here on (a cycle and its mirror image differ in it): they
-// go to `cb`, one bit per word.
-// RECS: the list is the rulers of the level and its words, (next, min) = (peer ^ 1, min(least[rho],
-// least[peer] ^ 1)), are formed here from the walk records.  Indices a raised gate may have left undefined are
-// masked into the block.
+// go to `cb`, one bit per word.  Indices a raised gate may have left undefined are masked into the block.
 constexpr int kLGroup = 3;                            // pairs per ruler pair (log2)
 constexpr uint32_t kLRho = 0x7FFCu, kLRuler = 0x8000u;
 
-constexpr size_t list_label_smem(int log2b) { return (size_t(17) << log2b) / 2 + 16; }
+constexpr size_t list_label_smem(int log2b) { return (size_t(6) << log2b) + 16; }
 
-template <bool RECS>
 __global__ void __launch_bounds__(kListThreads)
-k_list_label(const void *__restrict__ src, uint16_t *__restrict__ cb, int log2b, uint32_t salt) {
+k_list_label(const uint4 *__restrict__ src, uint16_t *__restrict__ cb, int log2b, uint32_t salt) {
     extern __shared__ __align__(16) unsigned char lsm[];
     const uint32_t B = 1u << log2b, bmask = B - 1u, R = B >> kLGroup, groups = B >> (kLGroup + 1);
     const size_t base = size_t(blockIdx.x) << log2b;
     const uint32_t T = blockDim.x, tid = threadIdx.x;
-    uint32_t *M = reinterpret_cast<uint32_t *>(lsm);                            // minimum of every word
-    unsigned char *N = lsm + 4 * B;                                             // successors / claims, 16 bit
-    uint32_t *own = reinterpret_cast<uint32_t *>(N + 2 * B), *far_ = own + R, *peer = far_ + R;
+    uint32_t *M = reinterpret_cast<uint32_t *>(lsm);                            // minimum of every pair
+    unsigned char *N = lsm + 2 * B;                                             // successors / claims, 16 bit
+    uint32_t *own = reinterpret_cast<uint32_t *>(N + 2 * B), *peer = own + R;   // walk records
     unsigned long long *L = reinterpret_cast<unsigned long long *>(peer + R);   // list of the ruler words (+ a 0)
-    uint16_t *queue = reinterpret_cast<uint16_t *>(own);                        // after `own`, `far_` and `peer`
+    uint16_t *queue = reinterpret_cast<uint16_t *>(own);                        // after `own` and `peer`
     __shared__ uint32_t queued;
-    // sixteen words per thread (fewer than 512 words: a warp takes turns), all their loads under way together
-    for (uint32_t e0 = tid; e0 < B; e0 += 16 * T) {
-        uint32_t next[16], mn[16];
+    // eight pairs per thread (fewer than 512 words: a warp takes turns), all their loads under way together
+    for (uint32_t e0 = tid; e0 < B / 2; e0 += 8 * T) {
+        uint4 w[8];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const uint32_t e = e0 + uint32_t(i) * T;
-            next[i] = mn[i] = 0u;
-            if (e >= B) continue;
-            if (RECS) {
-                const uint2 a = __ldcs(static_cast<const uint2 *>(src) + base + e);
-                next[i] = (a.y & bmask) ^ 1u;
-                mn[i] = a.x;
-            } else {
-                const unsigned long long w = __ldcs(static_cast<const unsigned long long *>(src) + base + e);
-                next[i] = uint32_t(w) & bmask;
-                mn[i] = uint32_t(w >> 32);
-            }
-        }
-        if (RECS) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-                mn[i] = min(mn[i], __ldg(&(static_cast<const uint2 *>(src) + base)[next[i] ^ 1u].x) ^ 1u);
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t q = e0 + uint32_t(i) * T;
+            w[i] = q < B / 2 ? __ldcs(src + base / 2 + q) : make_uint4(0, 0, 0, 0);
         }
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const uint32_t e = e0 + uint32_t(i) * T;
-            if (e >= B) continue;
-            M[e] = mn[i];
-            *reinterpret_cast<uint16_t *>(N + 2 * e) = uint16_t(2u * next[i]);
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t q = e0 + uint32_t(i) * T;
+            if (q >= B / 2) continue;
+            M[q] = pair_least(w[i].x, w[i].z);
+            *reinterpret_cast<uint32_t *>(N + 4 * q) = 2u * ((w[i].y & bmask) ^ 1u) | (2u * ((w[i].w & bmask) ^ 1u)) << 16;
         }
     }
     if (tid == 0) queued = 0u;
@@ -350,7 +304,7 @@ k_list_label(const void *__restrict__ src, uint16_t *__restrict__ cb, int log2b,
     __syncthreads();
     if (g < groups) {
         uint32_t rho = 2u * g, j = start & 0xFFFFu, code = ((rho << 2) | 1u) * 0x10001u;
-        uint32_t least = M[2u * q0], part = kUnowned;
+        uint32_t least = M[q0];
         for (uint32_t k = 0;;) {
             // (no branches: a lane that has met somebody reads the same code again)
             bool met = false;
@@ -359,30 +313,26 @@ k_list_label(const void *__restrict__ src, uint16_t *__restrict__ cb, int log2b,
             for (int hop = 0; hop < 4; ++hop) {
                 v = *reinterpret_cast<volatile uint16_t *>(N + j);
                 met = (v & 1u) != 0u;
-                const uint2 mm = *reinterpret_cast<const uint2 *>(M + ((j >> 1) & ~1u));
+                const uint32_t mm = M[j >> 2] ^ ((j >> 1) & 1u);
                 if (!met) *reinterpret_cast<volatile uint32_t *>(N + (j & ~3u)) = code + (j & 2u) * 0x10001u;
-                least = met ? least : min(least, (j & 2u) ? mm.y : mm.x);
-                part = met ? part : min(part, (j & 2u) ? mm.x : mm.y);
+                least = met ? least : min(least, mm);
                 j = met ? j : v;
             }
             if (met) {
                 // a ruler pair (its code names its even word), or one the other walker owns
                 own[rho] = least;
-                far_[rho] = part;
                 peer[rho] = ((v & kLRho) >> 2) ^ ((v & kLRuler) ? ((~j & 2u) >> 1) : 0u);
                 if (++k == 2u) break;
                 ++rho;
                 j = start >> 16;
                 code = ((rho << 2) | 1u) * 0x10001u;
-                least = M[2u * q0 + 1u];
-                part = kUnowned;
+                least = M[q0] ^ 1u;
             }
         }
     }
     __syncthreads();
     for (uint32_t rho = tid; rho < R; rho += T) {
-        const uint32_t p = peer[rho] & (R - 1u);
-        L[rho] = make_word(p ^ 1u, min(own[rho], far_[p]));
+        L[rho] = make_word((peer[rho] & (R - 1u)) ^ 1u, min(own[rho], own[rho ^ 1u] ^ 1u));
     }
     if (tid == 0) L[R] = 0ull;
     __syncthreads();
@@ -410,11 +360,11 @@ k_list_label(const void *__restrict__ src, uint16_t *__restrict__ cb, int log2b,
             // (the queue is complete, and the walks below only read unclaimed words until the next barrier)
             for (uint32_t i = tid; i < queued; i += T) {
                 const uint32_t q = queue[i];
-                uint32_t f = 4u * q, mn = M[2u * q];
+                uint32_t f = 4u * q, mn = M[q];
                 for (uint32_t hops = 0; hops < B; ++hops) {
                     f = *reinterpret_cast<volatile uint16_t *>(N + f) & (2u * bmask);
                     if (f == 4u * q) break;
-                    mn = min(mn, M[f >> 1]);
+                    mn = min(mn, M[f >> 2] ^ ((f >> 1) & 1u));
                 }
                 queue[i] = uint16_t(q | (mn << 15));
             }
@@ -440,23 +390,19 @@ k_list_label(const void *__restrict__ src, uint16_t *__restrict__ cb, int log2b,
     }
 }
 
-int launch_list_label(const void *src, bool records, uint32_t *cb, uint32_t count, int beta, uint32_t salt, cudaStream_t s) {
+int launch_list_label(const uint2 *rec, uint32_t *cb, uint32_t count, int beta, uint32_t salt, cudaStream_t s) {
     static OncePerDevice configured;
     {
         const int rc = configured.run([]() -> int {
-            BENES_CUDA_TRY(cudaFuncSetAttribute(k_list_label<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                int(list_label_smem(kListSmemLog2))));
-            BENES_CUDA_TRY(cudaFuncSetAttribute(k_list_label<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            BENES_CUDA_TRY(cudaFuncSetAttribute(k_list_label, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 int(list_label_smem(kListSmemLog2))));
             return BENES_OK;
         });
         if (rc) return rc;
     }
     const unsigned threads = beta > 9 ? 1u << (beta - 4) : 32u;
-    if (records)
-        k_list_label<true><<<count >> beta, threads, list_label_smem(beta), s>>>(src, reinterpret_cast<uint16_t *>(cb), beta, salt);
-    else
-        k_list_label<false><<<count >> beta, threads, list_label_smem(beta), s>>>(src, reinterpret_cast<uint16_t *>(cb), beta, salt);
+    k_list_label<<<count >> beta, threads, list_label_smem(beta), s>>>(reinterpret_cast<const uint4 *>(rec),
+                                                                       reinterpret_cast<uint16_t *>(cb), beta, salt);
     return launch_status();
 }
 
@@ -594,29 +540,27 @@ inline int list_spacing(int beta) {
 
 }  // namespace
 
-// Scratch: walk records, the contracted lists, and the owners and parity bits of their words.
+// Scratch: walk records (each a list), and the owners and parity bits of their words.
 // A list that is sampled again shrinks to a quarter at least.
 size_t sampled_scratch_bytes(size_t total, int kappa) {
-    size_t R = total >> kappa, bytes = align256(R * 16);
+    size_t R = total >> kappa, bytes = 0;
     for (int i = 0; i < kMaxLists; ++i) {
         size_t c = R >> (2 * i);
         if (c < 32) c = 32;
-        bytes += align256(c * 8) + align256(c * 4) + align256(c / 8);
+        bytes += align256(c * 8) + align256(c * 2) + align256(c / 8);
     }
     return bytes;
 }
 
 void sampled_scratch_carve(char *base, size_t total, int kappa, SampledScratch *out) {
     size_t R = total >> kappa, off = 0;
-    out->rec = reinterpret_cast<uint4 *>(base);
-    off += align256(R * 16);
     for (int i = 0; i < kMaxLists; ++i) {
         size_t c = R >> (2 * i);
         if (c < 32) c = 32;
-        out->list[i] = reinterpret_cast<unsigned long long *>(base + off);
+        out->rec[i] = reinterpret_cast<uint2 *>(base + off);
         off += align256(c * 8);
         out->owner[i] = reinterpret_cast<uint32_t *>(base + off);
-        off += align256(c * 4);
+        off += align256(c * 2);
         out->bits[i] = reinterpret_cast<uint32_t *>(base + off);
         off += align256(c / 8);
     }
@@ -638,8 +582,6 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
                   int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage,
                   uint32_t *gate, cudaStream_t s) {
     const uint32_t R = uint32_t(total >> kappa);
-    uint2 *walk_rec = reinterpret_cast<uint2 *>(sc.rec);
-    const unsigned rgrid = (R + kThreads - 1) / kThreads;
     {
         ProfileScope ps(kWalk, s);
         // Two walks per thread pay once half of the threads still fills the GPU (2^26, levels 0-3:
@@ -650,7 +592,7 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
         const bool two = walk_pairs == 2 || (walk_pairs == 1 && size_t(R >> 1) >= size_t(sm_count()) * 2048);
 #define BENES_WALK(PACKED, W)                                                                            \
     k_walk<PACKED, W><<<(R / W + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s>>>(                 \
-        static_cast<unsigned long long *>(S.S), S.P, Q, walk_rec, R, log2m, kappa, salt, cap, gate)
+        static_cast<unsigned long long *>(S.S), S.P, Q, sc.rec[0], R, log2m, kappa, salt, cap, gate)
         if (S.packed) { if (two) BENES_WALK(true, 2); else BENES_WALK(true, 1); }
         else { if (two) BENES_WALK(false, 2); else BENES_WALK(false, 1); }
 #undef BENES_WALK
@@ -662,45 +604,29 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
     int beta = log2m - kappa, depth = 0;
     if (beta < 7) return BENES_ERR_BADARG;                     // (a CTA labels 2^7 words at least)
     uint32_t counts[kMaxLists + 1] = {R};
-    if (list_spacing(beta)) {
-        ProfileScope ps(kCombine, s);
-        k_combine<<<rgrid, kThreads, 0, s>>>(walk_rec, sc.list[0], R);
-        int rc = launch_status();
-        if (rc) return rc;
-    }
     for (int sp; (sp = list_spacing(beta)) != 0; ++depth) {
-        // walks from both ends; the walk records of the previous stage (switches,
-        // or the list before) are dead, their memory takes the new ones
+        // walks from both ends
         if (depth + 1 >= kMaxLists) return BENES_ERR_BADARG;
         const uint32_t count = counts[depth], next = count >> sp;
-        {
-            ProfileScope ps(kListWalk, s);
-            k_list_walk_pairs<<<(next + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s>>>(
-                reinterpret_cast<const ulonglong2 *>(sc.list[depth]), sc.owner[depth], sc.rec, next, count >> 1, sp,
-                salt * 7u + uint32_t(depth) + 1u, cap, gate);
-            int rc = launch_status();
-            if (rc) return rc;
-        }
-        {
-            ProfileScope ps(kCombine, s);
-            k_combine_list<<<(next + kThreads - 1) / kThreads, kThreads, 0, s>>>(sc.rec, sc.list[depth + 1], next);
-            int rc = launch_status();
-            if (rc) return rc;
-        }
+        ProfileScope ps(kListWalk, s);
+        k_list_walk_pairs<<<(next + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s>>>(
+            reinterpret_cast<const uint4 *>(sc.rec[depth]), sc.owner[depth], sc.rec[depth + 1], next, count >> 1, sp,
+            salt * 7u + uint32_t(depth) + 1u, cap, gate);
+        int rc = launch_status();
+        if (rc) return rc;
         counts[depth + 1] = next;
         beta -= sp;
     }
     {
         ProfileScope ps(kListLabel, s);
-        int rc = launch_list_label(depth ? static_cast<const void *>(sc.list[depth]) : walk_rec, depth == 0, sc.bits[depth],
-                                   counts[depth], beta, salt + 77u, s);
+        int rc = launch_list_label(sc.rec[depth], sc.bits[depth], counts[depth], beta, salt + 77u, s);
         if (rc) return rc;
     }
     for (int d = depth - 1; d >= 0; --d) {
         ProfileScope ps(kListResolve, s);
         const uint32_t c = counts[d];
         k_list_resolve_pairs<<<(c / 2 + kThreads - 1) / kThreads, kThreads, 0, s>>>(
-            sc.list[d], sc.owner[d], sc.bits[d + 1], c / 2, c, cap, gate, sc.bits[d]);
+            reinterpret_cast<const uint4 *>(sc.rec[d]), sc.owner[d], sc.bits[d + 1], c / 2, cap, gate, sc.bits[d]);
         int rc = launch_status();
         if (rc) return rc;
     }
