@@ -252,10 +252,7 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
         }
         if (rc) return rc;
     }
-    // Blocks of 2^15 are finished by one CTA each.  Up to 64 of them would leave
-    // more than half of the SMs idle during the longest kernel of the route: then
-    // one more level runs in HBM and twice as many CTAs finish blocks of 2^14.
-    const int fused_m = opt.cluster ? kFusedLog2M + 1 : (T >> kFusedLog2M) <= 64 ? kFusedLog2M - 1 : kFusedLog2M;
+    const int fused_m = opt.cluster ? kFusedLog2M + 1 : kFusedLog2M;
     int cur = 0;
     for (int level = 0; kappa && n - level > fused_m; ++level) {
         const int m = n - level;
@@ -328,7 +325,7 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     }
     {
         ProfileScope ps(kFused, s);
-        if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, 0, 0, tail_gate, redone))) return rc;
+        if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, 0, 0, tail_gate, redone, Qbuf))) return rc;
     }
     if (hp && hp->bits_host) {
         if ((rc = copy_stage_rows(*hp, bits, n, batch, first, rows, s))) return rc;
@@ -409,6 +406,23 @@ int benes_release_workspace(void) {
     return drop_own(g_ws[dev], dev, false, nullptr);
 }
 
+// What splitting the levels of a few permutations of 2^12 .. 2^15 over the SMs takes on top of route_ws_bytes (which
+// is 0 there): only ever from a buffer of the library's own, and a call does without where there is none.
+static size_t peel_bytes(int n, size_t batch) {
+    return n >= kPeelLog2 && n <= kFusedLog2M && 2 * batch <= size_t(sm_count()) ? 2 * align_up((batch << n) * 4) : 0;
+}
+static bool caller_workspace() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return true; }
+    std::lock_guard<std::mutex> lk(g_mu);
+    return g_ws[dev].user != nullptr;
+}
+// the part of the workspace that benes_route uses inside a call that keeps buffers of its own behind it
+static size_t route_inner_bytes(int n, size_t batch) {
+    const size_t need = route_ws_bytes(n, batch), more = need ? 0 : peel_bytes(n, batch);
+    return align_up(need + (more && !caller_workspace() ? more : 0));
+}
+
 // benes_route on a given scratch buffer (`ws` may be null when route_ws_bytes is 0)
 static int route_on(const uint32_t *perm, int n, int batch, uint32_t *switch_bits, char *ws, cudaStream_t s,
                     const Options &opt) {
@@ -418,8 +432,11 @@ static int route_on(const uint32_t *perm, int n, int batch, uint32_t *switch_bit
         ProfileScope ps(kFused, s);
         for (size_t b0 = 0; b0 < size_t(batch); b0 += max_ctas) {
             size_t nb = size_t(batch) - b0 < max_ctas ? size_t(batch) - b0 : max_ctas;
+            uint32_t *const spare[2] = {reinterpret_cast<uint32_t *>(ws),
+                                        reinterpret_cast<uint32_t *>(ws + align_up((nb << n) * 4))};
             int rc = launch_fused(perm + (b0 << n), 0, nb << n, n,
-                                  switch_bits + b0 * size_t(2 * n - 1) * stage_words(n), n, s);
+                                  switch_bits + b0 * size_t(2 * n - 1) * stage_words(n), n, s, 0, 0, nullptr, nullptr,
+                                  ws ? spare : nullptr);
             if (rc) return rc;
         }
         return BENES_OK;
@@ -473,6 +490,8 @@ int benes_route(const uint32_t *perm, int log2n, int batch, uint32_t *switch_bit
     if (route_needs_ws(log2n, opt)) {
         int rc = get_workspace(route_ws_bytes(log2n, size_t(batch)), &ws, s);
         if (rc) return rc;
+    } else if (const size_t more = peel_bytes(log2n, size_t(batch))) {
+        if (caller_workspace() || get_workspace(more, &ws, s)) ws = nullptr;
     }
     return route_on(perm, log2n, batch, switch_bits, static_cast<char *>(ws), s, opt);
 }
@@ -516,7 +535,7 @@ int benes_route_padded(const uint32_t *perm, size_t n_elems, int batch, uint32_t
     if (!perm || !switch_bits || n == 0 || batch < 1) return BENES_ERR_BADARG;
     if ((size_t(1) << n) == n_elems) return benes_route(perm, n, batch, switch_bits, stream);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    const size_t inner = align_up(route_ws_bytes(n, size_t(batch)));
+    const size_t inner = route_inner_bytes(n, size_t(batch));
     void *ws = nullptr;
     int rc = get_workspace(inner + align_up((size_t(batch) << n) * 4), &ws, s);
     if (rc) return rc;
@@ -549,7 +568,7 @@ int benes_route_host(const uint32_t *perm_host, int log2n, int batch, uint32_t *
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const size_t perm_bytes = (size_t(batch) << log2n) * 4;
     const size_t bits_bytes = benes_switch_words(log2n, batch) * 4;
-    const size_t inner = route_ws_bytes(log2n, size_t(batch));
+    const size_t inner = route_inner_bytes(log2n, size_t(batch));
     void *ws = nullptr;
     int rc = get_workspace(align_up(inner) + align_up(perm_bytes) + align_up(bits_bytes), &ws, s);
     if (rc) return rc;
@@ -763,7 +782,7 @@ int benes_plan_create(benes_plan_t **plan_out, const uint32_t *perm, int log2n, 
         return code;
     };
     if (cudaGetDevice(&p->dev) != cudaSuccess) return fail(BENES_ERR_CUDA);
-    const size_t route_ws = route_needs_ws(n, opt) ? align_up(route_ws_bytes(n, size_t(batch))) : 0;
+    const size_t route_ws = route_needs_ws(n, opt) ? align_up(route_ws_bytes(n, size_t(batch))) : peel_bytes(n, size_t(batch));
     const size_t apply_ws = with_apply ? align_up(apply_ws_bytes(elem_bytes, n, size_t(batch))) : 0;
     if (route_ws + apply_ws) {
         if (cudaMalloc(&p->ws, route_ws + apply_ws) != cudaSuccess) return fail(BENES_ERR_NOMEM);
@@ -771,7 +790,7 @@ int benes_plan_create(benes_plan_t **plan_out, const uint32_t *perm, int log2n, 
     char *ws = static_cast<char *>(p->ws);
     if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return fail(BENES_ERR_CUDA);
     auto enqueue = [&]() -> int {
-        int r = route_on(perm, n, batch, switch_bits, ws, cap, opt);
+        int r = route_on(perm, n, batch, switch_bits, route_ws ? ws : nullptr, cap, opt);
         if (!r && with_apply) r = apply_on(switch_bits, in, out, elem_bytes, n, batch, ws + route_ws, cap, opt);
         return r;
     };

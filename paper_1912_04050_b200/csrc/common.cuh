@@ -312,7 +312,10 @@ int sampled_scratch_reset(const SampledScratch &sc, size_t total, int log2m, int
 // blocks are those of the plain array `redone`.
 int launch_fused(const void *P, int records, size_t total, int log2m, uint32_t *bits, int log2n,
                  cudaStream_t s, size_t first_block = 0, size_t blocks = 0, const uint32_t *gate = nullptr,
-                 const uint32_t *redone = nullptr);
+                 const uint32_t *redone = nullptr, uint32_t *const spare[2] = nullptr);
+// With `spare` (two arrays of total words), blocks of 2^kPeelLog2 and more that leave at least half of the SMs without
+// one run a level at a time, on twice as many SMs each time.
+constexpr int kPeelLog2 = 12;
 
 // ---- payload apply (apply.cu) ----------------------------------------------
 int launch_apply_stage(const uint32_t *bits, const void *x, void *y, int elem_bytes, int stage,

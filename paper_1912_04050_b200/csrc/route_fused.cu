@@ -209,6 +209,19 @@ __device__ __forceinline__ uint32_t spread4(uint32_t c) {
 __device__ __forceinline__ uint32_t fields_of_bytes(uint32_t x) { return (x * 0x40100401u) >> 24; }
 
 // ---- a level with 16-bit entries -------------------------------------------------------
+// Input-side bits of the level above a level of sub-blocks of 2^logs: the parities in the upper half-blocks, in input order.
+template <class Cfg>
+__device__ __forceinline__ void input_bits16(unsigned char *sm, int logs) {
+    constexpr uint32_t C = Cfg::C, T = Cfg::T;
+    for (uint32_t c = threadIdx.x; c < C / 16; c += T) {
+        const uint32_t i = ((c >> (logs - 3)) << (logs + 1)) + ((c & ((1u << (logs - 3)) - 1u)) << 3);
+        const uint4 q = at<uint4>(sm, Cfg::kQ + 2 * i);
+        const uint32_t x = (q.x & 0x00010001u) | ((q.y & 0x00010001u) << 2) | ((q.z & 0x00010001u) << 4) |
+                           ((q.w & 0x00010001u) << 6);
+        at<uint8_t>(sm, Cfg::kInw + c) = uint8_t(x | (x >> 15));
+    }
+}
+
 // Colour of output 2t of a switch nobody claimed: its g-cycle (at most S/2 outputs) from both ends;
 // g(b ^ 1) ^ 1 is the predecessor of b on the cycle (the cycle of 2t+1 is its mirror image).
 template <class Cfg>
@@ -237,16 +250,7 @@ __device__ __forceinline__ void level16(unsigned char *sm, const FusedOut &out, 
     const uint32_t tid = threadIdx.x;
     const uint32_t S = 1u << logs;
 
-    // input-side bits of the level above: the parities in the upper half-blocks, in input order
-    if (!first) {
-        for (uint32_t c = tid; c < C / 16; c += T) {
-            const uint32_t i = ((c >> (logs - 3)) << (logs + 1)) + ((c & ((S >> 3) - 1u)) << 3);
-            const uint4 q = at<uint4>(sm, Cfg::kQ + 2 * i);
-            const uint32_t x = (q.x & 0x00010001u) | ((q.y & 0x00010001u) << 2) | ((q.z & 0x00010001u) << 4) |
-                               ((q.w & 0x00010001u) << 6);
-            at<uint8_t>(sm, Cfg::kInw + c) = uint8_t(x | (x >> 15));
-        }
-    }
+    if (!first) input_bits16<Cfg>(sm, logs);
     // Successors g(j) = Q[P[j^1] ^ 1], so that a hop of a walk is one load: the gathers here run
     // with all lanes, those of the walks with a quarter of them.  The word of a ruler switch is its
     // code from the start; its thread keeps the successors, with which it starts the two walks.
@@ -323,16 +327,17 @@ __device__ __forceinline__ void level16(unsigned char *sm, const FusedOut &out, 
     }
     __syncthreads();
 
-    // contracted list: next = peer ^ 1, minimum = own side of mine, far side of the peer's
+    // Contracted list: next = peer ^ 1.  What the other walker of my ruler switch has seen, with the last bit
+    // flipped, lies on my cycle too, and every segment of a cycle has both of its walkers in such pairs of the cycle:
+    // no need to fetch the minimum of the peer.
     constexpr int kPer = int(R / T) > 0 ? int(R / T) : 1;
     uint32_t w[kPer];
 #pragma unroll
     for (int r = 0; r < kPer; ++r) {
         const uint32_t rho = tid + uint32_t(r) * T;
         if (rho < R) {
-            const uint32_t a = at<uint32_t>(sm, Cfg::kRec + rho * 4), pr4 = a & (R * 4u - 4u);
-            const uint32_t b = at<uint32_t>(sm, Cfg::kRec + pr4);
-            w[r] = (pr4 ^ 4u) | min(a & 0xFFFF0000u, (b ^ 0x00020000u) & 0xFFFF0000u);
+            const uint32_t a = at<uint32_t>(sm, Cfg::kRec + rho * 4), b = at<uint32_t>(sm, Cfg::kRec + (rho ^ 1u) * 4);
+            w[r] = ((a & (R * 4u - 4u)) ^ 4u) | min(a & 0xFFFF0000u, (b ^ 0x00020000u) & 0xFFFF0000u);
             at<uint32_t>(sm, Cfg::kList + rho * 4) = w[r];
         }
     }
@@ -691,49 +696,92 @@ __device__ __forceinline__ void fused_enter4(unsigned char *sm, uint32_t i4, con
     }
 }
 
+// The CTA's blocks of 2^logs outputs from a plain array (records = 0) or from packed records
+// P[2t] | P[2t+1] << logs | ... (1), four entries per load, four loads of a thread under way together.
+template <class Cfg>
+__device__ __forceinline__ void fused_load(unsigned char *sm, const FusedOut &out, const uint32_t *P, int records, int logs) {
+    constexpr uint32_t T = Cfg::T, kItems = Cfg::C / 4, kBatch = kItems / T >= 4 ? 4 : 1;
+    const uint32_t smask = (1u << logs) - 1u;
+    const bool aligned = (reinterpret_cast<uintptr_t>(P) & 15u) == 0;
+    for (uint32_t i0 = threadIdx.x; i0 < kItems; i0 += kBatch * T) {
+        uint32_t v[kBatch][4];
+#pragma unroll
+        for (uint32_t r = 0; r < kBatch; ++r) {
+            const uint32_t i4 = i0 + r * T;
+            const size_t f = out.flat0 + 4u * i4;
+            if (4u * i4 + 4u <= out.valid && (records != 0 || aligned)) {
+                if (records == 0) {
+                    const uint4 p = __ldcs(reinterpret_cast<const uint4 *>(P + f));
+                    v[r][0] = p.x; v[r][1] = p.y; v[r][2] = p.z; v[r][3] = p.w;
+                } else {
+                    const ulonglong2 p = __ldcs(reinterpret_cast<const ulonglong2 *>(P) + (f >> 2));
+                    v[r][0] = uint32_t(p.x) & smask; v[r][1] = uint32_t(p.x >> logs) & smask;
+                    v[r][2] = uint32_t(p.y) & smask; v[r][3] = uint32_t(p.y >> logs) & smask;
+                }
+            } else {
+                // a permutation that does not start on 16 bytes, the end of a batch of permutations of 2,
+                // or padding: the identity
+#pragma unroll
+                for (uint32_t k = 0; k < 4; ++k)
+                    v[r][k] = (records == 0 && 4u * i4 + k < out.valid) ? P[f + k] : (4u * i4 + k) & smask;
+            }
+        }
+#pragma unroll
+        for (uint32_t r = 0; r < kBatch; ++r) {
+#pragma unroll
+            for (uint32_t k = 0; k < 4; ++k) v[r][k] = BENES_GUARD(v[r][k], smask);
+            fused_enter4<Cfg>(sm, i0 + r * T, v[r], logs);
+        }
+    }
+    __syncthreads();
+}
+
 template <int LOGC, int THREADS>
 __global__ void __launch_bounds__(THREADS, (FusedCfg<LOGC, THREADS>::kMinCtas))
 k_route_fused(const uint32_t *__restrict__ P, int records, uint32_t *__restrict__ bits, int log2n, int logs,
               size_t first, size_t end, const uint32_t *__restrict__ gate, const uint32_t *__restrict__ redone) {
     using Cfg = FusedCfg<LOGC, THREADS>;
-    constexpr uint32_t C = Cfg::C, T = Cfg::T;
+    constexpr uint32_t C = Cfg::C;
     extern __shared__ __align__(16) unsigned char sm[];
     FusedOut out;
     out.bits = bits;
     out.n = log2n;
     out.flat0 = first + size_t(blockIdx.x) * C;
     out.valid = uint32_t(end - out.flat0 < size_t(C) ? end - out.flat0 : size_t(C));
-    const uint32_t tid = threadIdx.x, smask = (1u << logs) - 1u;
-    if (gate && *gate != 0u) {
-        P = redone;
-        records = 0;
-    }
-    const bool aligned = (reinterpret_cast<uintptr_t>(P) & 15u) == 0;
-    for (uint32_t i4 = tid; i4 < C / 4; i4 += T) {
-        const size_t f = out.flat0 + 4u * i4;
-        uint32_t v[4];
-        if (4u * i4 + 4u <= out.valid && (records != 0 || aligned)) {
-            // plain array (0) or packed records P[2t] | P[2t+1] << logs | ... (1)
-            if (records == 0) {
-                const uint4 p = __ldcs(reinterpret_cast<const uint4 *>(P + f));
-                v[0] = p.x; v[1] = p.y; v[2] = p.z; v[3] = p.w;
-            } else {
-                const ulonglong2 p = __ldcs(reinterpret_cast<const ulonglong2 *>(P) + (f >> 2));
-                v[0] = uint32_t(p.x) & smask; v[1] = uint32_t(p.x >> logs) & smask;
-                v[2] = uint32_t(p.y) & smask; v[3] = uint32_t(p.y >> logs) & smask;
-            }
-        } else {
-            // a permutation that does not start on 16 bytes, the end of a batch of permutations of 2,
-            // or padding: the identity
-#pragma unroll
-            for (uint32_t k = 0; k < 4; ++k) v[k] = (records == 0 && 4u * i4 + k < out.valid) ? P[f + k] : (4u * i4 + k) & smask;
-        }
-#pragma unroll
-        for (uint32_t k = 0; k < 4; ++k) v[k] = BENES_GUARD(v[k], smask);
-        fused_enter4<Cfg>(sm, i4, v, logs);
-    }
-    __syncthreads();
+    const bool redo = gate && *gate != 0u;
+    fused_load<Cfg>(sm, out, redo ? redone : P, redo ? 0 : records, logs);
     fused_levels<Cfg>(sm, out, logs);
+}
+
+// One level of one block of 2^LOGC outputs per CTA; the two half-blocks go to `next` (a plain array), where the
+// next launch finds them with twice as many CTAs.  While more than half of the SMs would have no block, that is how the
+// in-CTA levels run: a level takes a time in proportion to the CTA's outputs, so halving the block with every level
+// costs about two levels of the first block instead of one for each (one block of 2^15: 172 -> 82 us,
+// 2^13: 51 -> 37; the route of 2^16: 206 -> 140, of 2^20: 545 -> 497).
+template <int LOGC, int THREADS>
+__global__ void __launch_bounds__(THREADS)
+k_route_peel(const uint32_t *__restrict__ P, int records, uint32_t *__restrict__ bits, int log2n,
+             uint32_t *__restrict__ next, const uint32_t *__restrict__ gate, const uint32_t *__restrict__ redone) {
+    using Cfg = FusedCfg<LOGC, THREADS>;
+    constexpr uint32_t C = Cfg::C, T = Cfg::T, H = C / 2;
+    extern __shared__ __align__(16) unsigned char sm[];
+    FusedOut out;
+    out.bits = bits;
+    out.n = log2n;
+    out.flat0 = size_t(blockIdx.x) * C;
+    out.valid = C;
+    const bool redo = gate && *gate != 0u;
+    fused_load<Cfg>(sm, out, redo ? redone : P, redo ? 0 : records, LOGC);
+    level16<Cfg>(sm, out, LOGC, log2n - LOGC, true);
+    // entries 2 (base of the half + value) | parity -> values; input-side bits from the inverse of the upper half
+    for (uint32_t i4 = threadIdx.x; i4 < C / 4; i4 += T) {
+        const uint2 e = at<uint2>(sm, 8 * i4);
+        const uint32_t x = (e.x >> 1) & ((H - 1u) * 0x10001u), y = (e.y >> 1) & ((H - 1u) * 0x10001u);
+        *reinterpret_cast<uint4 *>(next + out.flat0 + 4u * i4) = make_uint4(x & 0xFFFFu, x >> 16, y & 0xFFFFu, y >> 16);
+    }
+    input_bits16<Cfg>(sm, LOGC - 1);
+    __syncthreads();
+    out.store_row<Cfg>(sm, Cfg::kInw, log2n - LOGC);
 }
 
 // ---- few outputs in all ---------------------------------------------------------------------
@@ -789,7 +837,7 @@ __device__ __forceinline__ void few_tail32(uint32_t p, uint32_t r, uint16_t *Q, 
 
 template <int LOGC>
 __global__ void __launch_bounds__((1 << LOGC) / 2)
-k_route_few(const uint32_t *__restrict__ P, uint32_t *__restrict__ bits, int n, size_t total) {
+k_route_few(const uint32_t *__restrict__ P, uint32_t *__restrict__ bits, int n, int logs, size_t total) {
     constexpr uint32_t C = 1u << LOGC, kAll = 0xFFFFFFFFu;
     __shared__ uint32_t W[C];                  // (minimum << 16 | next) of every output
     __shared__ uint32_t Q32[C / 2], Pn32[C / 2];
@@ -801,13 +849,12 @@ k_route_few(const uint32_t *__restrict__ P, uint32_t *__restrict__ bits, int n, 
     out.flat0 = size_t(blockIdx.x) << LOGC;
     out.valid = uint32_t(total - out.flat0 < size_t(C) ? total - out.flat0 : size_t(C));
     const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5, j = 2u * t;
-    const uint32_t nmask = (1u << n) - 1u;
-    uint32_t p0 = j & nmask, p1 = (j + 1u) & nmask;            // padding: the identity
+    const uint32_t block = (1u << logs) - 1u;
+    uint32_t p0 = j & block, p1 = (j + 1u) & block;            // padding: the identity
     if (j < out.valid) {                                       // (valid is even)
-        p0 = BENES_GUARD(P[out.flat0 + j], nmask);
-        p1 = BENES_GUARD(P[out.flat0 + j + 1], nmask);
+        p0 = BENES_GUARD(P[out.flat0 + j], block);
+        p1 = BENES_GUARD(P[out.flat0 + j + 1], block);
     }
-    int logs = n;
     for (; logs > 6; --logs) {
         const int level = n - logs;
         const uint32_t smask = (1u << logs) - 1u, sb = j & ~smask, H = (smask + 1u) >> 1;
@@ -878,14 +925,14 @@ k_route_few(const uint32_t *__restrict__ P, uint32_t *__restrict__ bits, int n, 
         // several permutations of 2^n <= 32: from a switch to an output per lane
         const uint32_t a0 = __shfl_sync(kAll, p0, int(lane >> 1)), a1 = __shfl_sync(kAll, p1, int(lane >> 1));
         const uint32_t b0 = __shfl_sync(kAll, p0, int(16u + (lane >> 1))), b1 = __shfl_sync(kAll, p1, int(16u + (lane >> 1)));
-        few_tail32((lane & 1u) ? a1 : a0, 2u * warp, Qw, out, n);
-        few_tail32((lane & 1u) ? b1 : b0, 2u * warp + 1u, Qw + 32, out, n);
+        few_tail32((lane & 1u) ? a1 : a0, 2u * warp, Qw, out, logs);
+        few_tail32((lane & 1u) ? b1 : b0, 2u * warp + 1u, Qw + 32, out, logs);
     }
 }
 
 template <int LOGC>
-int launch_few(const uint32_t *P, size_t total, uint32_t *bits, int n, cudaStream_t s) {
-    k_route_few<LOGC><<<unsigned((total + (size_t(1) << LOGC) - 1) >> LOGC), (1 << LOGC) / 2, 0, s>>>(P, bits, n, total);
+int launch_few(const uint32_t *P, size_t total, uint32_t *bits, int n, int logs, cudaStream_t s) {
+    k_route_few<LOGC><<<unsigned((total + (size_t(1) << LOGC) - 1) >> LOGC), (1 << LOGC) / 2, 0, s>>>(P, bits, n, logs, total);
     return launch_status();
 }
 
@@ -1127,6 +1174,22 @@ int launch_one(const uint32_t *P, int records, size_t first, size_t end, uint32_
     return launch_status();
 }
 
+template <int LOGC>
+int launch_peel(const uint32_t *P, int records, size_t total, uint32_t *bits, int log2n, uint32_t *next, cudaStream_t s,
+                const uint32_t *gate, const uint32_t *redone) {
+    constexpr int T = 1024;
+    using Cfg = FusedCfg<LOGC, T>;
+    static OncePerDevice configured;
+    const int rc = configured.run([]() -> int {
+        BENES_CUDA_TRY(cudaFuncSetAttribute(k_route_peel<LOGC, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            int(Cfg::kSmemBytes)));
+        return BENES_OK;
+    });
+    if (rc) return rc;
+    k_route_peel<LOGC, T><<<unsigned(total >> LOGC), T, Cfg::kSmemBytes, s>>>(P, records, bits, log2n, next, gate, redone);
+    return launch_status();
+}
+
 int launch_cluster2(const uint32_t *P, int records, size_t first_block, size_t blocks, uint32_t *bits,
                     int log2n, cudaStream_t s, const uint32_t *gate, const uint32_t *redone) {
     static OncePerDevice configured;
@@ -1147,28 +1210,41 @@ int launch_cluster2(const uint32_t *P, int records, size_t first_block, size_t b
 }  // namespace
 
 int launch_fused(const void *Pv, int records, size_t total, int log2m, uint32_t *bits, int log2n,
-                 cudaStream_t s, size_t first_block, size_t blocks, const uint32_t *gate, const uint32_t *redone) {
+                 cudaStream_t s, size_t first_block, size_t blocks, const uint32_t *gate, const uint32_t *redone,
+                 uint32_t *const spare[2]) {
     const uint32_t *P = static_cast<const uint32_t *>(Pv);
     if (log2m < 1 || log2m > kClusterLog2M) return BENES_ERR_BADARG;
     if (blocks == 0) blocks = (total >> log2m) - first_block;        // all the rest
     if (first_block + blocks > (total >> log2m)) return BENES_ERR_BADARG;
     if (log2m == kClusterLog2M) return launch_cluster2(P, records, first_block, blocks, bits, log2n, s, gate, redone);
     const size_t first = first_block << log2m, end = first + (blocks << log2m);
-    // whole permutations of up to 2^11, and not more switches than the GPU has threads
-    if (records == 0 && log2m == log2n && log2m <= 11 && first == 0 && end / 2 <= size_t(sm_count()) * 2048) {
-        const int logc = log2m > 8 ? log2m : 8;
-        return logc == 8 ? launch_few<8>(P, end, bits, log2n, s) : logc == 9 ? launch_few<9>(P, end, bits, log2n, s)
-             : logc == 10 ? launch_few<10>(P, end, bits, log2n, s) : launch_few<11>(P, end, bits, log2n, s);
+    int m = log2m;
+    if (spare && first == 0 && end == total)
+        for (int i = 0; m >= kPeelLog2 && 2 * (total >> m) <= size_t(sm_count()); --m, i ^= 1) {
+            const int rc = m == 15 ? launch_peel<15>(P, records, total, bits, log2n, spare[i], s, gate, redone)
+                         : m == 14 ? launch_peel<14>(P, records, total, bits, log2n, spare[i], s, gate, redone)
+                         : m == 13 ? launch_peel<13>(P, records, total, bits, log2n, spare[i], s, gate, redone)
+                                   : launch_peel<12>(P, records, total, bits, log2n, spare[i], s, gate, redone);
+            if (rc) return rc;
+            P = spare[i];
+            records = 0;
+            gate = nullptr;
+        }
+    // blocks of up to 2^11 in a plain array, and not more switches than the GPU has threads
+    if (records == 0 && !gate && m <= 11 && first == 0 && end / 2 <= size_t(sm_count()) * 2048) {
+        const int logc = m > 8 ? m : 8;
+        return logc == 8 ? launch_few<8>(P, end, bits, log2n, m, s) : logc == 9 ? launch_few<9>(P, end, bits, log2n, m, s)
+             : logc == 10 ? launch_few<10>(P, end, bits, log2n, m, s) : launch_few<11>(P, end, bits, log2n, m, s);
     }
     // Small blocks share a CTA: a thread of the 8-bit levels takes a whole sub-block, so the more
     // sub-blocks a CTA holds, the fuller its warps.  Up to 2^13 outputs per CTA, as long as
     // every SM still gets a few CTAs.
-    int logc = log2m > 10 ? log2m : 10;
+    int logc = m > 10 ? m : 10;
     while (logc < 13 && ((end - first) >> logc) > 4 * size_t(sm_count())) ++logc;
     // CTAs that have an SM to themselves get more threads: their time is a chain of short
     // phases, not the instructions they issue.
     const bool alone = ((end - first + (size_t(1) << logc) - 1) >> logc) <= size_t(sm_count());
-#define BENES_FUSED(LC, T) return launch_one<LC, T>(P, records, first, end, bits, log2n, log2m, s, gate, redone)
+#define BENES_FUSED(LC, T) return launch_one<LC, T>(P, records, first, end, bits, log2n, m, s, gate, redone)
     switch (logc) {
         case 10: if (alone) BENES_FUSED(10, 256); BENES_FUSED(10, 32);
         case 11: if (alone) BENES_FUSED(11, 512); BENES_FUSED(11, 64);

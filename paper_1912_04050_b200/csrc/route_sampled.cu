@@ -255,7 +255,7 @@ k_list_resolve_pairs(const uint4 *__restrict__ pair, uint32_t *__restrict__ owne
 // the same sampling once more: one ruler pair per 8 pairs, walks that meet in the middle over 16-bit
 // successors (claims go into the successor words, which nobody reads again), pointer jumping over the B/8 words
 // that are left, and a queue for the pairs of cycles without ruler pair.  Pointer jumping over the whole list
-// took log2b - 1 passes of random shared-memory reads (2^14 words: 25 us, now LIST_US).
+// took log2b - 1 passes of random shared-memory reads (2^14 words: 25 us, now 16).
 // Only the parities of the minima are needed from here on (a cycle and its mirror image differ in it): they
 // go to `cb`, one bit per word.  Indices a raised gate may have left undefined are masked into the block.
 constexpr int kLGroup = 3;                            // pairs per ruler pair (log2)

@@ -61,6 +61,24 @@ def test_route_batched(n, batch):
     assert np.array_equal(gpu_route(perm, n), oracle.route(perm, n))
 
 
+@pytest.mark.parametrize("n,batch", [(12, 1), (12, 37), (12, 75), (13, 3), (14, 1), (14, 19), (15, 1), (15, 5), (16, 3), (18, 1)])
+def test_route_levels_split_over_the_sms(n, batch):
+    """Few blocks: a level at a time on twice as many SMs, which takes scratch of the library's own; with a
+    caller's workspace too small for it the blocks stay in their CTAs.  Same bits."""
+    perm = inputs.random_perm_batch(n, batch, seed0=23 * n)
+    want = oracle.route(perm, n)
+    assert np.array_equal(gpu_route(perm, n), want)
+    bits = np.zeros_like(want)
+    binding.benes_route_host(perm, n, batch, bits)
+    assert np.array_equal(bits, want)
+    if n <= 15:
+        binding.benes_set_workspace(torch.zeros(256, dtype=torch.uint8, device="cuda"))
+        try:
+            assert np.array_equal(gpu_route(perm, n), want)
+        finally:
+            binding.benes_set_workspace(None)
+
+
 @pytest.mark.parametrize("n,batch", [(1, 2049), (2, 1031), (3, 131), (4, 67), (5, 33), (6, 17), (6, 10007), (7, 2401), (8, 5),
                                      (8, 601), (9, 1201), (10, 149), (10, 593), (11, 297), (12, 149), (13, 149), (14, 149)])
 def test_route_blocks_that_share_a_cta(n, batch):
