@@ -165,7 +165,7 @@ int benes_apply_static(const uint32_t *switch_bits, const void *in, void *out, i
  * copies with the computation on a second stream the library owns (one per
  * device, created on the first call).  benes_route_host: the permutation
  * arrives in pieces, and the stages a level has finished go back while the next
- * levels run.  benes_apply_host (payloads of 64 MiB and more): the first pass
+ * levels run.  benes_apply_host (payloads of 8 MiB and more): the first pass
  * starts on each part of the payload as it arrives, and the parts the last
  * pass has finished go back while it still runs.
  */
@@ -176,9 +176,9 @@ int benes_apply_host(const uint32_t *switch_bits_host, const void *in_host, void
 
 /*
  * Both steps for host buffers in one call: out_host[b][j] = in_host[b][pi_b[j]].
- * switch_bits_host may be NULL if the settings themselves are not wanted.  For
- * batch * N >= 2^23 the payload travels to the device while the levels run, the
- * finished stages and the finished parts of the routed payload travel back on a
+ * switch_bits_host may be NULL if the settings themselves are not wanted.  The
+ * payload travels to the device while the levels run, the
+ * finished stages and (from 8 MiB on) the finished parts of the routed payload travel back on a
  * second copy stream, and the switch words never make the round trip through
  * host memory that calling benes_route_host and benes_apply_host one after the
  * other costs.  Synchronises `stream` before returning.

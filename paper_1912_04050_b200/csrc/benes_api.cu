@@ -161,6 +161,8 @@ size_t apply_ws_bytes(int elem_bytes, int log2n, size_t batch) {
 // piece as soon as it is there), and the two stages a level has finished are
 // copied to the host on the side stream while the next levels run.
 constexpr int kMaxPieces = 8;
+// A payload travels in parts from here on: a part is 1 MiB at least, 20 us over the bus, against some 5 us for a copy.
+constexpr size_t kPipeMinBytes = size_t(1) << 23;
 static_assert(kMaxPieces >= kApplyMaxParts, "the host pipe's events serve the apply parts too");
 struct HostPipe {
     uint32_t *bits_host = nullptr;     // finished stages go here (same layout as `bits`)
@@ -328,7 +330,9 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
         if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, 0, 0, tail_gate, redone, Qbuf))) return rc;
     }
     if (hp && hp->bits_host) {
-        if ((rc = copy_stage_rows(*hp, bits, n, batch, first, rows, s))) return rc;
+        BENES_CUDA_TRY(cudaEventRecord(hp->stage_ready[kMaxLevels - 2], s));
+        BENES_CUDA_TRY(cudaStreamWaitEvent(hp->d2h, hp->stage_ready[kMaxLevels - 2], 0));
+        if ((rc = copy_stage_rows(*hp, bits, n, batch, first, rows, hp->d2h))) return rc;
     }
     return BENES_OK;
 }
@@ -584,7 +588,7 @@ int benes_route_host(const uint32_t *perm_host, int log2n, int batch, uint32_t *
         const size_t T = size_t(batch) << n;
         hp->bits_host = switch_bits_host;
         hp->d2h = hp->side;
-        hp->pieces = (T >= (size_t(1) << 23)) ? kMaxPieces : 1;
+        hp->pieces = T >= (size_t(1) << kInversePartitionMinLog2) ? kMaxPieces : 1;
         // the side stream must not touch the workspace before earlier work on `s` is done
         BENES_CUDA_TRY(cudaEventRecord(hp->stage_ready[kMaxLevels - 1], s));
         BENES_CUDA_TRY(cudaStreamWaitEvent(hp->side, hp->stage_ready[kMaxLevels - 1], 0));
@@ -627,7 +631,7 @@ int benes_apply_host(const uint32_t *switch_bits_host, const void *in_host, void
     uint32_t *d_bits = reinterpret_cast<uint32_t *>(d_out + align_up(data_bytes));
     BENES_CUDA_TRY(cudaMemcpyAsync(d_bits, switch_bits_host, bits_bytes, cudaMemcpyHostToDevice, s));
     const size_t chunks = apply_fused_chunks(log2n, size_t(batch));
-    if (options().apply_fused && data_bytes >= (size_t(1) << 26) && chunks % kApplyMaxParts == 0 && chunks > 0) {
+    if (options().apply_fused && data_bytes >= kPipeMinBytes && chunks % kApplyMaxParts == 0 && chunks > 0) {
         // The payload arrives in parts on the side stream, behind the switch words:
         // the first pass starts on a part as soon as it is there, and the parts the
         // last pass has finished leave on the side stream while it still runs.
@@ -673,11 +677,9 @@ int benes_route_apply_host(const uint32_t *perm_host, const void *in_host, void 
     const Options opt = options();
     const size_t T = size_t(batch) << n;
     const size_t data_bytes = T * size_t(elem_bytes);
-    const size_t chunks = apply_fused_chunks(n, size_t(batch));
-    const bool piped = n > kFusedLog2M && level_chunk(n, size_t(batch), opt.chunk_log2) == size_t(batch) &&
-                       opt.apply_fused && T >= (size_t(1) << 23) && chunks > 0 && chunks % kApplyMaxParts == 0;
-    if (!piped) {
-        // small or chunked inputs: one call after the other (the switch words stay on the host side
+    const bool levels = route_needs_ws(n, opt);
+    if (!opt.apply_fused || (levels && level_chunk(n, size_t(batch), opt.chunk_log2) != size_t(batch))) {
+        // chunked inputs: one call after the other (the switch words stay on the host side
         // of the first call only if the caller wants them)
         const size_t words = benes_switch_words(n, batch);
         uint32_t *bits_tmp = switch_bits_host;
@@ -689,8 +691,10 @@ int benes_route_apply_host(const uint32_t *perm_host, const void *in_host, void 
         if (!switch_bits_host) cudaFreeHost(bits_tmp);
         return rc;
     }
+    const size_t chunks = apply_fused_chunks(n, size_t(batch));
+    const int parts = data_bytes >= kPipeMinBytes && chunks > 0 && chunks % kApplyMaxParts == 0 ? kApplyMaxParts : 1;
     const size_t perm_bytes = T * 4, bits_bytes = benes_switch_words(n, batch) * 4;
-    const size_t route_ws = align_up(route_ws_bytes(n, size_t(batch)));
+    const size_t route_ws = route_inner_bytes(n, size_t(batch));
     const size_t apply_ws = align_up(apply_ws_bytes(elem_bytes, n, size_t(batch)));
     void *ws = nullptr;
     int rc = get_workspace(route_ws + apply_ws + align_up(perm_bytes) + align_up(bits_bytes) + 2 * align_up(data_bytes), &ws, s);
@@ -705,7 +709,7 @@ int benes_route_apply_host(const uint32_t *perm_host, const void *in_host, void 
     if ((rc = host_pipe_for_current_device(&hp))) return rc;
     hp->bits_host = switch_bits_host;              // null: the switch words stay on the device
     hp->d2h = hp->back;
-    hp->pieces = kMaxPieces;
+    hp->pieces = levels && T >= (size_t(1) << kInversePartitionMinLog2) ? kMaxPieces : 1;
     // the copy streams must not touch the workspace before earlier work on `s` is done
     BENES_CUDA_TRY(cudaEventRecord(hp->stage_ready[kMaxLevels - 1], s));
     BENES_CUDA_TRY(cudaStreamWaitEvent(hp->side, hp->stage_ready[kMaxLevels - 1], 0));
@@ -720,23 +724,38 @@ int benes_route_apply_host(const uint32_t *perm_host, const void *in_host, void 
         BENES_CUDA_TRY(cudaEventRecord(hp->piece_ready[i], hp->side));
     }
     ApplyHostPipe pipe;
-    pipe.parts = kApplyMaxParts;
+    pipe.parts = parts;
     pipe.side = hp->back;
     pipe.out_host = out_host;
-    const size_t part = data_bytes / size_t(pipe.parts);
-    for (int i = 0; i < pipe.parts; ++i) {
+    const size_t part = data_bytes / size_t(parts);
+    for (int i = 0; i < parts; ++i) {
         BENES_CUDA_TRY(cudaMemcpyAsync(d_in + part * size_t(i), static_cast<const char *>(in_host) + part * size_t(i),
                                        part, cudaMemcpyHostToDevice, hp->side));
         BENES_CUDA_TRY(cudaEventRecord(hp->part_ready[i], hp->side));
         pipe.in_ready[i] = hp->part_ready[i];
     }
     *hp->gate_host = 0u;
-    rc = route_levels(d_perm, n, size_t(batch), d_bits, base, s, opt, hp);
-    if (!rc) {
+    if (levels) {
+        rc = route_levels(d_perm, n, size_t(batch), d_bits, base, s, opt, hp);
+    } else {
+        // whole permutations in their CTAs: the settings leave in one piece while the payload is routed
+        BENES_CUDA_TRY(cudaStreamWaitEvent(s, hp->piece_ready[0], 0));
+        rc = route_on(d_perm, n, batch, d_bits, route_ws ? base : nullptr, s, opt);
+        if (!rc && switch_bits_host) {
+            BENES_CUDA_TRY(cudaEventRecord(hp->stage_ready[0], s));
+            BENES_CUDA_TRY(cudaStreamWaitEvent(hp->back, hp->stage_ready[0], 0));
+            BENES_CUDA_TRY(cudaMemcpyAsync(switch_bits_host, d_bits, bits_bytes, cudaMemcpyDeviceToHost, hp->back));
+        }
+    }
+    if (!rc && parts > 1) {
         // the route no longer waits on these events; the apply's last pass reuses them
-        for (int i = 0; i < pipe.parts; ++i) pipe.out_done[i] = hp->stage_ready[i];
+        for (int i = 0; i < parts; ++i) pipe.out_done[i] = hp->stage_ready[i];
         ProfileScope ps(kApplyFused, s);
         rc = launch_apply_fused(d_bits, d_in, d_out, scratch, elem_bytes, n, size_t(batch), s, &pipe);
+    } else if (!rc) {
+        BENES_CUDA_TRY(cudaStreamWaitEvent(s, hp->part_ready[0], 0));
+        rc = apply_on(d_bits, d_in, d_out, elem_bytes, n, batch, scratch, s, opt);
+        if (!rc) BENES_CUDA_TRY(cudaMemcpyAsync(out_host, d_out, data_bytes, cudaMemcpyDeviceToHost, s));
     }
     cudaError_t e1 = cudaStreamSynchronize(s), e2 = cudaStreamSynchronize(hp->side), e3 = cudaStreamSynchronize(hp->back);
     if (rc) return rc;
