@@ -22,6 +22,7 @@ template <typename E, int SIDE>
 __global__ void __launch_bounds__(kThreads)
 k_apply_stage(const uint32_t *__restrict__ bits, const E *__restrict__ x, E *__restrict__ y,
               size_t switches, int log2m, int stage, int log2n) {
+    after_previous_kernel();
     using P2 = typename Pair<E>::type;
     const size_t stride = size_t(gridDim.x) * blockDim.x;
     const size_t half_n = size_t(1) << (log2n - 1);
@@ -64,11 +65,11 @@ int launch_typed(const uint32_t *bits, const void *x, void *y, int stage, int lo
     size_t cap = size_t(sm_count()) * 16;
     int grid = int(blocks < cap ? blocks : cap);
     if (stage <= log2n - 1)
-        k_apply_stage<E, 0><<<grid, kThreads, 0, s>>>(bits, static_cast<const E *>(x),
-                                                      static_cast<E *>(y), switches, log2m, stage, log2n);
+        launch_kernel(k_apply_stage<E, 0>, grid, kThreads, 0, s, bits, static_cast<const E *>(x),
+                      static_cast<E *>(y), switches, log2m, stage, log2n);
     else
-        k_apply_stage<E, 1><<<grid, kThreads, 0, s>>>(bits, static_cast<const E *>(x),
-                                                      static_cast<E *>(y), switches, log2m, stage, log2n);
+        launch_kernel(k_apply_stage<E, 1>, grid, kThreads, 0, s, bits, static_cast<const E *>(x),
+                      static_cast<E *>(y), switches, log2m, stage, log2n);
     return launch_status();
 }
 

@@ -312,6 +312,7 @@ template <typename E, int C>
 __global__ void __launch_bounds__(kApplyThreads<C>, (C == kChunkLog2 ? (sizeof(E) == 8 ? 2 : 3) : 8))
 k_apply_inner(const uint32_t *__restrict__ bits, const E *__restrict__ x, E *__restrict__ y, int n, int b,
               size_t total, uint32_t cta0) {
+    after_previous_kernel();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr uint32_t T = kApplyThreads<C>, kHalf = 1u << (C - 1);
     E *sm = reinterpret_cast<E *>(smem_raw);
@@ -387,6 +388,7 @@ template <typename E, int C, bool OUT>
 __global__ void __launch_bounds__(kApplyThreads<C>, (sizeof(E) == 8 ? (C == 13 ? 2 : 5) : 4))
 k_apply_outer(const uint32_t *__restrict__ bits, const E *__restrict__ x, E *__restrict__ y, int n,
               int l0, int k, uint32_t cta0) {
+    after_previous_kernel();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr uint32_t T = kApplyThreads<C>, kHalf = 1u << (C - 1);
     E *sm = reinterpret_cast<E *>(smem_raw);
@@ -482,6 +484,7 @@ constexpr int kTraceThreads = 1024;
 template <typename E>
 __global__ void __launch_bounds__(kTraceThreads)
 k_apply_trace(const uint32_t *__restrict__ bits, const E *__restrict__ x, E *__restrict__ y, int n, size_t total) {
+    after_previous_kernel();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t *sb = reinterpret_cast<uint32_t *>(smem_raw);
     const uint32_t N = 1u << n, W = n >= 6 ? N >> 6 : 1u, per = uint32_t(2 * n - 1) * W;     // words per permutation
@@ -536,7 +539,7 @@ int apply_fused_typed(const uint32_t *bits, const E *in, E *out, E *scratch, int
         const unsigned threads = n < 7 ? 128u : n < 10 ? 1u << n : unsigned(kTraceThreads);
         const size_t words = size_t(2 * n - 1) * (n >= 6 ? size_t(1) << (n - 6) : 1);
         const size_t perms = (threads >> n) > 1 ? threads >> n : 1;
-        k_apply_trace<E><<<unsigned((total + threads - 1) / threads), threads, words * perms * 4, s>>>(bits, in, out, n, total);
+        launch_kernel(k_apply_trace<E>, unsigned((total + threads - 1) / threads), threads, words * perms * 4, s, bits, in, out, n, total);
         return launch_status();
     }
     static OncePerDevice configured;
@@ -593,7 +596,7 @@ int apply_fused_typed(const uint32_t *bits, const E *in, E *out, E *scratch, int
         E *dst = next_dst();
         const int k = ks[i], lvl = l0;
         if ((rc = run_pass(index++, chunks, size_t(1) << kOuterLog2<E>, [&](unsigned ctas, unsigned cta0) {
-                 k_apply_outer<E, kOuterLog2<E>, false><<<ctas, kApplyThreads<kOuterLog2<E>>, apply_smem<E, kOuterLog2<E>>(k), s>>>(bits, src, dst, n, lvl, k, cta0);
+                 launch_kernel(k_apply_outer<E, kOuterLog2<E>, false>, ctas, kApplyThreads<kOuterLog2<E>>, apply_smem<E, kOuterLog2<E>>(k), s, bits, src, dst, n, lvl, k, cta0);
              })))
             return rc;
         src = dst;
@@ -607,10 +610,10 @@ int apply_fused_typed(const uint32_t *bits, const E *in, E *out, E *scratch, int
         const unsigned blocks = unsigned((total + (size_t(1) << c) - 1) >> c);
         if ((rc = run_pass(index++, blocks, size_t(1) << c, [&](unsigned ctas, unsigned cta0) {
                  if (small)
-                     k_apply_inner<E, kSmallLog2><<<ctas, kApplyThreads<kSmallLog2>, apply_smem<E, kSmallLog2>(2 * b - 1), s>>>(
+                     launch_kernel(k_apply_inner<E, kSmallLog2>, ctas, kApplyThreads<kSmallLog2>, apply_smem<E, kSmallLog2>(2 * b - 1), s,
                          bits, src, dst, n, b, total, cta0);
                  else
-                     k_apply_inner<E, kChunkLog2><<<ctas, kApplyThreads<kChunkLog2>, apply_smem<E, kChunkLog2>(2 * b - 1), s>>>(
+                     launch_kernel(k_apply_inner<E, kChunkLog2>, ctas, kApplyThreads<kChunkLog2>, apply_smem<E, kChunkLog2>(2 * b - 1), s,
                          bits, src, dst, n, b, total, cta0);
              })))
             return rc;
@@ -621,7 +624,7 @@ int apply_fused_typed(const uint32_t *bits, const E *in, E *out, E *scratch, int
         l0 -= ks[i];
         const int k = ks[i], lvl = l0;
         if ((rc = run_pass(index++, chunks, size_t(1) << kOuterLog2<E>, [&](unsigned ctas, unsigned cta0) {
-                 k_apply_outer<E, kOuterLog2<E>, true><<<ctas, kApplyThreads<kOuterLog2<E>>, apply_smem<E, kOuterLog2<E>>(k), s>>>(bits, src, dst, n, lvl, k, cta0);
+                 launch_kernel(k_apply_outer<E, kOuterLog2<E>, true>, ctas, kApplyThreads<kOuterLog2<E>>, apply_smem<E, kOuterLog2<E>>(k), s, bits, src, dst, n, lvl, k, cta0);
              })))
             return rc;
         src = dst;

@@ -202,10 +202,10 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     Qbuf[0] = reinterpret_cast<uint32_t *>(ws + off); off += align_up(T * 4);
     Qbuf[1] = reinterpret_cast<uint32_t *>(ws + off); off += align_up(T * 4);
     unsigned long long *Wd = reinterpret_cast<unsigned long long *>(ws + off); off += align_up(T * 8);
-    char *sampled = ws + off; off += align_up(sampled_scratch_bytes(T, kMinKappa));
     // raised by a walk that gave up
     uint32_t *gate = reinterpret_cast<uint32_t *>(ws + off); off += kAlign;
-    uint32_t *fill = reinterpret_cast<uint32_t *>(ws + off);
+    uint32_t *fill = reinterpret_cast<uint32_t *>(ws + off); off += align_up(kInverseMaxBuckets * 4);
+    char *sampled = ws + off;
     // Small inputs are bound by the longest walk of a level, not by throughput:
     // closer rulers (shorter walks) pay there although the lists get longer.
     const int kappa = (opt.kappa > 3 && T <= (size_t(1) << 22)) ? 3 : opt.kappa;
@@ -223,8 +223,9 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     int rc;
     if (kappa) {
         sampled_scratch_carve(sampled, T, kappa, &sc);
-        BENES_CUDA_TRY(cudaMemsetAsync(gate, 0, 4, s));
-        if ((rc = sampled_scratch_reset(sc, T, n, kappa, s))) return rc;
+        // the gate, the bucket counters and the owners lie one after the other
+        const char *end = sampled + sampled_owner_bytes(sc, T, n, kappa);
+        BENES_CUDA_TRY(cudaMemsetAsync(gate, 0, size_t(end - reinterpret_cast<char *>(gate)), s));
     }
 
     BitsLayout L{bits, n, n - 6};
@@ -239,7 +240,6 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
         const int pieces = hp ? hp->pieces : 0;
         const LevelRecords S0 = records(0, 0);
         if (bucketed && pieces > 1) {
-            if ((rc = launch_inverse_clear(fill, T, s))) return rc;
             const size_t per = T / size_t(pieces);
             for (int i = 0; i < pieces; ++i) {
                 BENES_CUDA_TRY(cudaStreamWaitEvent(s, hp->piece_ready[i], 0));

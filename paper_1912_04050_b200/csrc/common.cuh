@@ -19,7 +19,9 @@ constexpr int kFusedLog2M = 15;
 // Largest list (log2 of its 64-bit words) that one CTA labels in shared memory.
 constexpr int kListSmemLog2 = 14;
 
-constexpr uint32_t kUnowned = 0xFFFFFFFFu;
+// Owner of a pair of list words nobody has claimed; a claim is ~(walker << 1 | side of arrival).  Zero, so that one
+// memset clears it with the gate and the bucket counters.
+constexpr uint32_t kUnowned = 0u;
 
 // Every kernel launch of the library goes through this counter.
 extern unsigned long long g_launches;
@@ -38,6 +40,33 @@ extern unsigned long long g_launches;
 inline int launch_status() {
     ++g_launches;
     return cudaGetLastError() == cudaSuccess ? BENES_OK : BENES_ERR_CUDA;
+}
+
+// Launches `kernel` so that its CTAs may take their places while the last CTAs of the kernel before it in the stream
+// are ending (programmatic dependent launch).  Every kernel of the library begins with after_previous_kernel(), so none
+// of it runs before that kernel has finished and its memory operations are visible; what overlaps is the launch itself
+// and the start of the CTAs.  A route above 2^15 is a chain of 10 to 60 launches, most of them of 5 to 60 us: 2^18 272
+// -> 230 us, 2^20 499 -> 434, 2^24 3.71 -> 3.59 ms, 2^20 apply 24.8 -> 18.3 us.
+template <class... P, class... A>
+inline void launch_kernel(void (*kernel)(P...), size_t grid, size_t threads, size_t smem, cudaStream_t s, A &&...args) {
+    cudaLaunchAttribute overlap = {};
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(grid));
+    cfg.blockDim = dim3(unsigned(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &overlap;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);               // launch_status() has the result
+}
+// Waits for the previous grid.  The wait comes before any access, so that a kernel that has ended implies that all
+// kernels before it in the stream have.  (No explicit trigger, which would let the next grid's CTAs in as soon as all of this
+// grid have started: they fill the SMs that happen to have room, two and three on one SM, and are slower for it: 2^20
+// apply 39 us, route 442.)
+__device__ __forceinline__ void after_previous_kernel() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Kernel attributes (opt-in shared memory) belong to a device: a launcher sets
@@ -272,7 +301,6 @@ constexpr int kInversePartitionMinLog2 = 22;
 constexpr int kInverseMaxBuckets = 4096;
 int launch_inverse_partitioned(const uint32_t *perm, LevelRecords S, uint32_t *Q, void *pairs,
                                uint32_t *fill, size_t total, int log2m, int kappa, cudaStream_t s);
-int launch_inverse_clear(uint32_t *fill, size_t total, cudaStream_t s);
 int launch_inverse_partition_piece(const uint32_t *perm, LevelRecords S, void *pairs, uint32_t *fill,
                                    size_t total, size_t j_first, size_t count, int log2m, int kappa,
                                    cudaStream_t s);
@@ -300,8 +328,9 @@ void sampled_scratch_carve(char *base, size_t total, int kappa, SampledScratch *
 // redone by launch_route_jump).
 int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const SampledScratch &sc, size_t total,
                   int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage, uint32_t *gate, cudaStream_t s);
-// Before the first sampled_label of a route: owners to kUnowned (log2m of the first level).
-int sampled_scratch_reset(const SampledScratch &sc, size_t total, int log2m, int kappa, cudaStream_t s);
+// The bytes from the start of the scratch that have to be zero (owners kUnowned) before the first sampled_label of a
+// route (log2m of the first level).
+size_t sampled_owner_bytes(const SampledScratch &sc, size_t total, int log2m, int kappa);
 
 // ---- fused path (route_fused.cu) -------------------------------------------
 // Finishes levels (n - log2m) .. n-1 of every block of size 2^log2m of the flat

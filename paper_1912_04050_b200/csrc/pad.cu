@@ -19,6 +19,7 @@ inline unsigned grid_for(size_t items) {
 __global__ void __launch_bounds__(kThreads)
 k_pad_perm(const uint32_t *__restrict__ src, uint32_t *__restrict__ dst, size_t n_elems, int log2n,
            size_t total) {
+    after_previous_kernel();
     const size_t stride = size_t(gridDim.x) * blockDim.x;
     const size_t nmask = (size_t(1) << log2n) - 1;
     for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += stride) {
@@ -31,6 +32,7 @@ k_pad_perm(const uint32_t *__restrict__ src, uint32_t *__restrict__ dst, size_t 
 template <typename E, bool PAD>
 __global__ void __launch_bounds__(kThreads)
 k_pad_rows(const E *__restrict__ src, E *__restrict__ dst, size_t n_elems, int log2n, size_t total) {
+    after_previous_kernel();
     const size_t stride = size_t(gridDim.x) * blockDim.x;
     const size_t nmask = (size_t(1) << log2n) - 1;
     for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += stride) {
@@ -45,7 +47,7 @@ k_pad_rows(const E *__restrict__ src, E *__restrict__ dst, size_t n_elems, int l
 int launch_pad_perm(const uint32_t *src, uint32_t *dst, size_t n_elems, int log2n, size_t batch,
                     cudaStream_t s) {
     const size_t total = batch << log2n;
-    k_pad_perm<<<grid_for(total), kThreads, 0, s>>>(src, dst, n_elems, log2n, total);
+    launch_kernel(k_pad_perm, grid_for(total), kThreads, 0, s, src, dst, n_elems, log2n, total);
     return launch_status();
 }
 
@@ -54,15 +56,15 @@ int launch_pad_rows(const void *src, void *dst, int elem_bytes, bool pad, size_t
     const size_t total = batch << log2n;
     const unsigned grid = grid_for(total);
     if (elem_bytes == 4) {
-        if (pad) k_pad_rows<uint32_t, true><<<grid, kThreads, 0, s>>>(
+        if (pad) launch_kernel(k_pad_rows<uint32_t, true>, grid, kThreads, 0, s,
             static_cast<const uint32_t *>(src), static_cast<uint32_t *>(dst), n_elems, log2n, total);
-        else k_pad_rows<uint32_t, false><<<grid, kThreads, 0, s>>>(
+        else launch_kernel(k_pad_rows<uint32_t, false>, grid, kThreads, 0, s,
             static_cast<const uint32_t *>(src), static_cast<uint32_t *>(dst), n_elems, log2n, total);
     } else if (elem_bytes == 8) {
-        if (pad) k_pad_rows<unsigned long long, true><<<grid, kThreads, 0, s>>>(
+        if (pad) launch_kernel(k_pad_rows<unsigned long long, true>, grid, kThreads, 0, s,
             static_cast<const unsigned long long *>(src), static_cast<unsigned long long *>(dst), n_elems,
             log2n, total);
-        else k_pad_rows<unsigned long long, false><<<grid, kThreads, 0, s>>>(
+        else launch_kernel(k_pad_rows<unsigned long long, false>, grid, kThreads, 0, s,
             static_cast<const unsigned long long *>(src), static_cast<unsigned long long *>(dst), n_elems,
             log2n, total);
     } else {
@@ -88,6 +90,7 @@ namespace {
 __global__ void __launch_bounds__(256)
 k_export_butterfly(const uint32_t *__restrict__ bits, uint32_t *__restrict__ out, int n, size_t rows,
                    uint32_t words_per_row) {
+    after_previous_kernel();
     const uint32_t half = 1u << (n - 1);                       // switches per row
     const size_t lanes_per_row = size_t(words_per_row) * 32;
     const size_t total = rows * lanes_per_row;
@@ -118,7 +121,7 @@ int launch_export_butterfly(const uint32_t *bits, uint32_t *out, int log2n, size
     const size_t total = rows * words * 32;
     size_t blocks = (total + 255) / 256;
     if (blocks > size_t(sm_count()) * 16) blocks = size_t(sm_count()) * 16;
-    k_export_butterfly<<<unsigned(blocks), 256, 0, s>>>(bits, out, log2n, rows, words);
+    launch_kernel(k_export_butterfly, unsigned(blocks), 256, 0, s, bits, out, log2n, rows, words);
     return launch_status();
 }
 

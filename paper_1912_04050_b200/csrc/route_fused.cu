@@ -740,6 +740,7 @@ template <int LOGC, int THREADS>
 __global__ void __launch_bounds__(THREADS, (FusedCfg<LOGC, THREADS>::kMinCtas))
 k_route_fused(const uint32_t *__restrict__ P, int records, uint32_t *__restrict__ bits, int log2n, int logs,
               size_t first, size_t end, const uint32_t *__restrict__ gate, const uint32_t *__restrict__ redone) {
+    after_previous_kernel();
     using Cfg = FusedCfg<LOGC, THREADS>;
     constexpr uint32_t C = Cfg::C;
     extern __shared__ __align__(16) unsigned char sm[];
@@ -762,6 +763,7 @@ template <int LOGC, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 k_route_peel(const uint32_t *__restrict__ P, int records, uint32_t *__restrict__ bits, int log2n,
              uint32_t *__restrict__ next, const uint32_t *__restrict__ gate, const uint32_t *__restrict__ redone) {
+    after_previous_kernel();
     using Cfg = FusedCfg<LOGC, THREADS>;
     constexpr uint32_t C = Cfg::C, T = Cfg::T, H = C / 2;
     extern __shared__ __align__(16) unsigned char sm[];
@@ -838,6 +840,7 @@ __device__ __forceinline__ void few_tail32(uint32_t p, uint32_t r, uint16_t *Q, 
 template <int LOGC>
 __global__ void __launch_bounds__((1 << LOGC) / 2)
 k_route_few(const uint32_t *__restrict__ P, uint32_t *__restrict__ bits, int n, int logs, size_t total) {
+    after_previous_kernel();
     constexpr uint32_t C = 1u << LOGC, kAll = 0xFFFFFFFFu;
     __shared__ uint32_t W[C];                  // (minimum << 16 | next) of every output
     __shared__ uint32_t Q32[C / 2], Pn32[C / 2];
@@ -932,7 +935,7 @@ k_route_few(const uint32_t *__restrict__ P, uint32_t *__restrict__ bits, int n, 
 
 template <int LOGC>
 int launch_few(const uint32_t *P, size_t total, uint32_t *bits, int n, int logs, cudaStream_t s) {
-    k_route_few<LOGC><<<unsigned((total + (size_t(1) << LOGC) - 1) >> LOGC), (1 << LOGC) / 2, 0, s>>>(P, bits, n, logs, total);
+    launch_kernel(k_route_few<LOGC>, unsigned((total + (size_t(1) << LOGC) - 1) >> LOGC), (1 << LOGC) / 2, 0, s, P, bits, n, logs, total);
     return launch_status();
 }
 
@@ -964,6 +967,7 @@ constexpr size_t kClusterSmemBytes = kClusterTopBytes > ClusterTailCfg::kSmemByt
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(ClusterTailCfg::T)
 k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restrict__ bits, int log2n,
                  uint32_t block0, const uint32_t *__restrict__ gate, const uint32_t *__restrict__ redone) {
+    after_previous_kernel();
     if (gate && *gate != 0u) {
         P = redone;
         records = 0;
@@ -1169,8 +1173,8 @@ int launch_one(const uint32_t *P, int records, size_t first, size_t end, uint32_
     });
     if (rc) return rc;
     const size_t ctas = (end - first + Cfg::C - 1) >> LOGC;
-    k_route_fused<LOGC, THREADS><<<unsigned(ctas), THREADS, Cfg::kSmemBytes, s>>>(P, records, bits, log2n, logs, first, end,
-                                                                                        gate, redone);
+    launch_kernel(k_route_fused<LOGC, THREADS>, unsigned(ctas), THREADS, Cfg::kSmemBytes, s, P, records, bits, log2n, logs, first, end,
+                  gate, redone);
     return launch_status();
 }
 
@@ -1186,7 +1190,7 @@ int launch_peel(const uint32_t *P, int records, size_t total, uint32_t *bits, in
         return BENES_OK;
     });
     if (rc) return rc;
-    k_route_peel<LOGC, T><<<unsigned(total >> LOGC), T, Cfg::kSmemBytes, s>>>(P, records, bits, log2n, next, gate, redone);
+    launch_kernel(k_route_peel<LOGC, T>, unsigned(total >> LOGC), T, Cfg::kSmemBytes, s, P, records, bits, log2n, next, gate, redone);
     return launch_status();
 }
 
@@ -1202,8 +1206,8 @@ int launch_cluster2(const uint32_t *P, int records, size_t first_block, size_t b
     });
     if (rc) return rc;
     // two CTAs per block (the cluster size is part of the kernel)
-    k_route_cluster2<<<unsigned(2 * blocks), ClusterTailCfg::T, kClusterSmemBytes, s>>>(P, records, bits, log2n,
-                                                                                        uint32_t(first_block), gate, redone);
+    launch_kernel(k_route_cluster2, unsigned(2 * blocks), ClusterTailCfg::T, kClusterSmemBytes, s, P, records, bits, log2n,
+                  uint32_t(first_block), gate, redone);
     return launch_status();
 }
 

@@ -59,6 +59,7 @@ template <bool PACKED>
 __global__ void __launch_bounds__(kThreads)
 k_inverse(const uint4 *__restrict__ P4, void *__restrict__ S, uint32_t *__restrict__ Q,
           size_t quads, int m, int kappa) {
+    after_previous_kernel();
     const uint32_t mmask = (1u << m) - 1u;
     size_t stride = size_t(gridDim.x) * blockDim.x;
     for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < quads; i += stride) {
@@ -105,6 +106,7 @@ template <bool PACKED>
 __global__ void __launch_bounds__(kPartThreads, 2)
 k_inverse_partition(const uint32_t *__restrict__ P, void *__restrict__ S, uint2 *__restrict__ pairs,
                     uint32_t *__restrict__ fill, uint32_t buckets, int blog, int m, size_t j_first, int kappa) {
+    after_previous_kernel();
     const uint32_t mmask = (1u << m) - 1u;
     extern __shared__ __align__(8) unsigned char part_smem[];
     uint2 *stage = reinterpret_cast<uint2 *>(part_smem);                  // the CTA's pairs, sorted by bucket
@@ -182,6 +184,7 @@ k_inverse_partition(const uint32_t *__restrict__ P, void *__restrict__ S, uint2 
 // Pass 2, buckets of 2^kBucketSmemLog2 entries: one CTA per bucket.
 __global__ void __launch_bounds__(1024)
 k_inverse_scatter_smem(const uint2 *__restrict__ pairs, uint32_t *__restrict__ Q, uint32_t mmask) {
+    after_previous_kernel();
     extern __shared__ __align__(16) uint32_t piece[];
     constexpr uint32_t kEntries = 1u << kBucketSmemLog2, kInBucket = kEntries - 1u;
     const size_t b0 = size_t(blockIdx.x) << kBucketSmemLog2;
@@ -220,6 +223,7 @@ k_inverse_scatter_smem(const uint2 *__restrict__ pairs, uint32_t *__restrict__ Q
 // Pass 2, buckets of 2^kBucketL2Log2 entries.
 __global__ void __launch_bounds__(kThreads)
 k_inverse_scatter(const uint2 *__restrict__ pairs, uint32_t *__restrict__ Q, size_t total, uint32_t mmask) {
+    after_previous_kernel();
     const size_t i = size_t(blockIdx.x) * kThreads + threadIdx.x;
     if (i >= total) return;
     const uint2 pr = __ldcs(pairs + i);
@@ -252,6 +256,7 @@ struct JumpArrays {
 
 __global__ void __launch_bounds__(kThreads)
 k_route_jump(JumpArrays a, uint32_t total, int log2n, int last_m, BitsLayout L, const uint32_t *__restrict__ gate) {
+    after_previous_kernel();
     if (gate && *gate == 0u) return;        // same value for every thread of the grid
     cg::grid_group grid = cg::this_grid();
     const uint32_t stride = gridDim.x * blockDim.x, first = blockIdx.x * blockDim.x + threadIdx.x;
@@ -319,6 +324,7 @@ k_route_jump(JumpArrays a, uint32_t total, int log2n, int last_m, BitsLayout L, 
 __global__ void __launch_bounds__(kThreads, 8)
 k_split(const uint4 *__restrict__ Q4, uint32_t *__restrict__ Qn, uint32_t pairs, int m,
         BitsLayout L, int in_stage, int out_stage, uint32_t rounds) {
+    after_previous_kernel();
     const uint32_t mmask = (1u << m) - 1u;
     // a CTA takes `rounds` consecutive groups of blockDim.x pairs: the colour
     // words it gathers belong to one block of the level for a long time (L1 hits)
@@ -358,6 +364,7 @@ k_split(const uint4 *__restrict__ Q4, uint32_t *__restrict__ Qn, uint32_t pairs,
 __global__ void __launch_bounds__(kThreads)
 k_validate(const uint32_t *__restrict__ perm, size_t total, uint32_t nmask,
            uint32_t *__restrict__ seen, uint32_t *__restrict__ flag) {
+    after_previous_kernel();
     size_t stride = size_t(gridDim.x) * blockDim.x;
     for (size_t j = size_t(blockIdx.x) * blockDim.x + threadIdx.x; j < total; j += stride) {
         uint32_t v = perm[j];
@@ -390,13 +397,7 @@ int cooperative_grid(int *out) {
 
 }  // namespace
 
-// Pass 1 over elements [j_first, j_first + count) (a multiple of 8192); `fill`
-// must have been cleared before the first piece.  Pass 2 over everything.
-int launch_inverse_clear(uint32_t *fill, size_t total, cudaStream_t s) {
-    BENES_CUDA_TRY(cudaMemsetAsync(fill, 0, (total >> bucket_log2(total)) * 4, s));
-    return BENES_OK;
-}
-
+// Pass 1 over elements [j_first, j_first + count) (a multiple of 8192).  Pass 2 over everything.
 int launch_inverse_partition_piece(const uint32_t *perm, LevelRecords S, void *pairs, uint32_t *fill,
                                    size_t total, size_t j_first, size_t count, int log2m, int kappa,
                                    cudaStream_t s) {
@@ -417,30 +418,28 @@ int launch_inverse_partition_piece(const uint32_t *perm, LevelRecords S, void *p
         if (rc) return rc;
     }
     if (S.packed)
-        k_inverse_partition<true><<<grid, kPartThreads, smem, s>>>(
+        launch_kernel(k_inverse_partition<true>, grid, kPartThreads, smem, s,
             perm, S.S, static_cast<uint2 *>(pairs), fill, buckets, blog, log2m, j_first, kappa);
     else
-        k_inverse_partition<false><<<grid, kPartThreads, smem, s>>>(
+        launch_kernel(k_inverse_partition<false>, grid, kPartThreads, smem, s,
             perm, S.S, static_cast<uint2 *>(pairs), fill, buckets, blog, log2m, j_first, kappa);
     return launch_status();
 }
 
 int launch_inverse_scatter(const void *pairs, uint32_t *Q, size_t total, int log2m, cudaStream_t s) {
     if (bucket_log2(total) == kBucketSmemLog2)
-        k_inverse_scatter_smem<<<unsigned(total >> kBucketSmemLog2), 1024, 4 << kBucketSmemLog2, s>>>(
+        launch_kernel(k_inverse_scatter_smem, unsigned(total >> kBucketSmemLog2), 1024, 4 << kBucketSmemLog2, s,
             static_cast<const uint2 *>(pairs), Q, (1u << log2m) - 1u);
     else
-        k_inverse_scatter<<<unsigned((total + kThreads - 1) / kThreads), kThreads, 0, s>>>(
+        launch_kernel(k_inverse_scatter, unsigned((total + kThreads - 1) / kThreads), kThreads, 0, s,
             static_cast<const uint2 *>(pairs), Q, total, (1u << log2m) - 1u);
     return launch_status();
 }
 
 int launch_inverse_partitioned(const uint32_t *perm, LevelRecords S, uint32_t *Q, void *pairs,
                                uint32_t *fill, size_t total, int log2m, int kappa, cudaStream_t s) {
-    int rc;
-    if ((rc = launch_inverse_clear(fill, total, s))) return rc;
-    if ((rc = launch_inverse_partition_piece(perm, S, pairs, fill, total, 0, total, log2m, kappa, s)))
-        return rc;
+    const int rc = launch_inverse_partition_piece(perm, S, pairs, fill, total, 0, total, log2m, kappa, s);
+    if (rc) return rc;
     return launch_inverse_scatter(pairs, Q, total, log2m, s);
 }
 
@@ -448,8 +447,8 @@ int launch_inverse(const uint32_t *perm, LevelRecords S, uint32_t *Q, size_t tot
                    cudaStream_t s) {
     size_t quads = total / 4;
     const uint4 *P4 = reinterpret_cast<const uint4 *>(perm);
-    if (S.packed) k_inverse<true><<<grid_for(quads), kThreads, 0, s>>>(P4, S.S, Q, quads, log2m, kappa);
-    else k_inverse<false><<<grid_for(quads), kThreads, 0, s>>>(P4, S.S, Q, quads, log2m, kappa);
+    if (S.packed) launch_kernel(k_inverse<true>, grid_for(quads), kThreads, 0, s, P4, S.S, Q, quads, log2m, kappa);
+    else launch_kernel(k_inverse<false>, grid_for(quads), kThreads, 0, s, P4, S.S, Q, quads, log2m, kappa);
     return launch_status();
 }
 
@@ -481,13 +480,13 @@ int launch_split(const uint32_t *Q, uint32_t *Qn, size_t total, int log2m, BitsL
     uint32_t rounds = stream_rounds(pairs, kThreads);
     if (log2m >= 20 && log2m <= 22 && rounds > (1u << (log2m - 20))) rounds = 1u << (log2m - 20);
     const unsigned grid = unsigned((size_t(pairs) + size_t(kThreads) * rounds - 1) / (size_t(kThreads) * rounds));
-    k_split<<<grid, kThreads, 0, s>>>(Q4, Qn, pairs, log2m, L, in_stage, out_stage, rounds);
+    launch_kernel(k_split, grid, kThreads, 0, s, Q4, Qn, pairs, log2m, L, in_stage, out_stage, rounds);
     return launch_status();
 }
 
 int launch_validate(const uint32_t *perm, size_t total, int log2n, uint32_t *seen_words,
                     uint32_t *flag, cudaStream_t s) {
-    k_validate<<<grid_for(total), kThreads, 0, s>>>(perm, total, (1u << log2n) - 1u, seen_words, flag);
+    launch_kernel(k_validate, grid_for(total), kThreads, 0, s, perm, total, (1u << log2n) - 1u, seen_words, flag);
     return launch_status();
 }
 

@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(kWalkThreads)
 k_walk(unsigned long long *__restrict__ S8, const uint32_t *__restrict__ P, const uint32_t *__restrict__ Q,
        uint2 *__restrict__ rec, uint32_t rulers, int m, int kappa, uint32_t salt, uint32_t cap,
        uint32_t *__restrict__ gate) {
+    after_previous_kernel();
     uint32_t rho = (blockIdx.x * kWalkThreads + threadIdx.x) * W;
     if (rho >= rulers) return;                                       // rulers is a multiple of W
     const uint32_t mmask = (1u << m) - 1u;
@@ -182,13 +183,14 @@ __device__ __forceinline__ uint32_t pair_least(uint32_t least0, uint32_t least1)
 __global__ void __launch_bounds__(kWalkThreads)
 k_list_walk_pairs(const uint4 *__restrict__ pair, uint32_t *__restrict__ owner, uint2 *__restrict__ rec,
                   uint32_t rulers, uint32_t pairs, int spacing, uint32_t salt, uint32_t cap, uint32_t *__restrict__ gate) {
+    after_previous_kernel();
     const uint32_t sigma = blockIdx.x * kWalkThreads + threadIdx.x;
     if (sigma >= rulers) return;
     const uint32_t kmask = (1u << spacing) - 1u;
     const uint32_t group = sigma >> 1, side0 = sigma & 1u;
     const uint32_t q0 = (group << spacing) | ruler_slot(group, salt, kmask);
     uint4 w = __ldcg(pair + q0);
-    if (!side0) owner[q0] = sigma << 1;                            // the ruler pair belongs to its even walker
+    if (!side0) owner[q0] = ~(sigma << 1);                          // the ruler pair belongs to its even walker
     uint32_t least = pair_least(w.x, w.z) ^ side0, next = (side0 ? w.w : w.y) ^ 1u, peer = sigma ^ 1u, hops = 0;
     for (;;) {
         // (a batch need not be a power of two: an index a raised gate left undefined is clamped, not masked)
@@ -203,9 +205,9 @@ k_list_walk_pairs(const uint4 *__restrict__ pair, uint32_t *__restrict__ owner, 
         }
         if ((hops & 63u) == 0u && gate_raised(gate)) break;
         w = __ldcg(pair + q);
-        const uint32_t prev = atomicCAS(owner + q, kUnowned, (sigma << 1) | side);
+        const uint32_t prev = atomicCAS(owner + q, kUnowned, ~((sigma << 1) | side));
         if (prev != kUnowned) {                                    // met the walker from the other end
-            peer = prev >> 1;
+            peer = ~prev >> 1;
             break;
         }
         least = min(least, pair_least(w.x, w.z) ^ side);
@@ -224,13 +226,14 @@ __global__ void __launch_bounds__(kThreads)
 k_list_resolve_pairs(const uint4 *__restrict__ pair, uint32_t *__restrict__ owner,
                      const uint32_t *__restrict__ cb2, uint32_t pairs,
                      uint32_t cap, uint32_t *__restrict__ gate, uint32_t *__restrict__ cb) {
+    after_previous_kernel();
     const uint32_t q = blockIdx.x * kThreads + threadIdx.x;       // pairs is a multiple of 32
     if (q >= pairs) return;
     const uint32_t code = owner[q];
     uint32_t bit0;
     if (code != kUnowned) {
-        const uint32_t sigma = code >> 1;
-        bit0 = ((__ldg(cb2 + (sigma >> 5)) >> (sigma & 31u)) ^ code) & 1u;
+        const uint32_t sigma = ~code >> 1;
+        bit0 = ((__ldg(cb2 + (sigma >> 5)) >> (sigma & 31u)) ^ ~code) & 1u;
         owner[q] = kUnowned;
     } else {
         uint4 w = __ldg(pair + q);
@@ -265,6 +268,7 @@ constexpr size_t list_label_smem(int log2b) { return (size_t(6) << log2b) + 16; 
 
 __global__ void __launch_bounds__(kListThreads)
 k_list_label(const uint4 *__restrict__ src, uint16_t *__restrict__ cb, int log2b, uint32_t salt) {
+    after_previous_kernel();
     extern __shared__ __align__(16) unsigned char lsm[];
     const uint32_t B = 1u << log2b, bmask = B - 1u, R = B >> kLGroup, groups = B >> (kLGroup + 1);
     const size_t base = size_t(blockIdx.x) << log2b;
@@ -401,8 +405,8 @@ int launch_list_label(const uint2 *rec, uint32_t *cb, uint32_t count, int beta, 
         if (rc) return rc;
     }
     const unsigned threads = beta > 9 ? 1u << (beta - 4) : 32u;
-    k_list_label<<<count >> beta, threads, list_label_smem(beta), s>>>(reinterpret_cast<const uint4 *>(rec),
-                                                                       reinterpret_cast<uint16_t *>(cb), beta, salt);
+    launch_kernel(k_list_label, count >> beta, threads, list_label_smem(beta), s, reinterpret_cast<const uint4 *>(rec),
+                  reinterpret_cast<uint16_t *>(cb), beta, salt);
     return launch_status();
 }
 
@@ -458,6 +462,7 @@ k_colour(const void *__restrict__ S, const uint32_t *__restrict__ P, const uint3
          const uint32_t *__restrict__ cb, void *__restrict__ Sn, uint32_t *__restrict__ Pn, uint32_t salt_next, uint32_t pairs,
          uint32_t rulers, int m, int kappa, BitsLayout L, int out_stage, uint32_t cap,
          uint32_t *__restrict__ gate, uint32_t rounds) {
+    after_previous_kernel();
     // a CTA takes `rounds` consecutive groups of blockDim.x pairs: the ruler bits
     // it gathers belong to one block of the level for a long time (L1 hits)
     const uint32_t stride = blockDim.x;
@@ -547,35 +552,40 @@ size_t sampled_scratch_bytes(size_t total, int kappa) {
     for (int i = 0; i < kMaxLists; ++i) {
         size_t c = R >> (2 * i);
         if (c < 32) c = 32;
-        bytes += align256(c * 8) + align256(c * 2) + align256(c / 8);
+        bytes += align256(c * 2) + align256(c * 8) + align256(c / 8);
     }
     return bytes;
 }
 
 void sampled_scratch_carve(char *base, size_t total, int kappa, SampledScratch *out) {
     size_t R = total >> kappa, off = 0;
+    for (int i = 0; i < kMaxLists; ++i) {                      // the owners of all lists lie together
+        size_t c = R >> (2 * i);
+        if (c < 32) c = 32;
+        out->owner[i] = reinterpret_cast<uint32_t *>(base + off);
+        off += align256(c * 2);
+    }
     for (int i = 0; i < kMaxLists; ++i) {
         size_t c = R >> (2 * i);
         if (c < 32) c = 32;
         out->rec[i] = reinterpret_cast<uint2 *>(base + off);
         off += align256(c * 8);
-        out->owner[i] = reinterpret_cast<uint32_t *>(base + off);
-        off += align256(c * 2);
         out->bits[i] = reinterpret_cast<uint32_t *>(base + off);
         off += align256(c / 8);
     }
 }
 
-// The owners of the lists that the first level (which has the longest) samples again.
-int sampled_scratch_reset(const SampledScratch &sc, size_t total, int log2m, int kappa, cudaStream_t s) {
-    size_t c = total >> kappa;
+// From the start of the scratch to the end of the owners of the lists that the first level (which has the longest)
+// samples again.
+size_t sampled_owner_bytes(const SampledScratch &sc, size_t total, int log2m, int kappa) {
+    size_t c = total >> kappa, bytes = 0;
     int beta = log2m - kappa;
     for (int i = 0, sp; (sp = list_spacing(beta)) != 0; ++i) {
-        BENES_CUDA_TRY(cudaMemsetAsync(sc.owner[i], 0xFF, c / 2 * 4, s));
+        bytes = size_t(reinterpret_cast<char *>(sc.owner[i]) - reinterpret_cast<char *>(sc.owner[0])) + c * 2;
         c >>= sp;
         beta -= sp;
     }
-    return BENES_OK;
+    return bytes;
 }
 
 int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const SampledScratch &sc, size_t total,
@@ -591,7 +601,7 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
         // spread over more blocks than the L2 holds (four: 0.95 ms per cache-resident level, eight: 1.6).
         const bool two = walk_pairs == 2 || (walk_pairs == 1 && size_t(R >> 1) >= size_t(sm_count()) * 2048);
 #define BENES_WALK(PACKED, W)                                                                            \
-    k_walk<PACKED, W><<<(R / W + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s>>>(                 \
+    launch_kernel(k_walk<PACKED, W>, (R / W + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s, \
         static_cast<unsigned long long *>(S.S), S.P, Q, sc.rec[0], R, log2m, kappa, salt, cap, gate)
         if (S.packed) { if (two) BENES_WALK(true, 2); else BENES_WALK(true, 1); }
         else { if (two) BENES_WALK(false, 2); else BENES_WALK(false, 1); }
@@ -609,7 +619,7 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
         if (depth + 1 >= kMaxLists) return BENES_ERR_BADARG;
         const uint32_t count = counts[depth], next = count >> sp;
         ProfileScope ps(kListWalk, s);
-        k_list_walk_pairs<<<(next + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s>>>(
+        launch_kernel(k_list_walk_pairs, (next + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s,
             reinterpret_cast<const uint4 *>(sc.rec[depth]), sc.owner[depth], sc.rec[depth + 1], next, count >> 1, sp,
             salt * 7u + uint32_t(depth) + 1u, cap, gate);
         int rc = launch_status();
@@ -625,7 +635,7 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
     for (int d = depth - 1; d >= 0; --d) {
         ProfileScope ps(kListResolve, s);
         const uint32_t c = counts[d];
-        k_list_resolve_pairs<<<(c / 2 + kThreads - 1) / kThreads, kThreads, 0, s>>>(
+        launch_kernel(k_list_resolve_pairs, (c / 2 + kThreads - 1) / kThreads, kThreads, 0, s,
             reinterpret_cast<const uint4 *>(sc.rec[d]), sc.owner[d], sc.bits[d + 1], c / 2, cap, gate, sc.bits[d]);
         int rc = launch_status();
         if (rc) return rc;
@@ -636,14 +646,14 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
         const uint32_t rounds = stream_rounds(switches, kThreads);
         const unsigned grid = unsigned((size_t(switches) + size_t(kThreads) * rounds - 1) / (size_t(kThreads) * rounds));
         if (S.packed)        // a packed level is followed by packed levels only
-            k_colour<true, true><<<grid, kThreads, 0, s>>>(S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
-                                                            out_stage, cap, gate, rounds);
+            launch_kernel(k_colour<true, true>, grid, kThreads, 0, s, S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
+                          out_stage, cap, gate, rounds);
         else if (Sn.packed)
-            k_colour<false, true><<<grid, kThreads, 0, s>>>(S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
-                                                             out_stage, cap, gate, rounds);
+            launch_kernel(k_colour<false, true>, grid, kThreads, 0, s, S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
+                          out_stage, cap, gate, rounds);
         else
-            k_colour<false, false><<<grid, kThreads, 0, s>>>(S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
-                                                              out_stage, cap, gate, rounds);
+            launch_kernel(k_colour<false, false>, grid, kThreads, 0, s, S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
+                          out_stage, cap, gate, rounds);
         return launch_status();
     }
 }
