@@ -62,22 +62,23 @@ def algorithmic_bytes_per_element(kind: str, ebytes: int, kappa: int) -> float:
     """Useful bytes one launch of a kernel kind moves per permutation element."""
     k = float(1 << max(kappa, 1))
     return {
-        # per switch, visited once: P[j^1] read (4 B), owner word read and written (8 B),
-        # Q[.] read (4 B) -> 8 B per element; one 16-byte walk record per ruler output
-        "walk": 8.0 + 16.0 / k,
-        # build 16 B + (m-2) passes of 24 B + last 8 B per element, m ~ 20 on average
-        "full_label": 16.0 + 18 * 24.0 + 8.0,
+        # per switch, visited once: P[j^1] read (4 B), owner read and written (8 B),
+        # Q[.] read (4 B) -> 8 B per element; one 8-byte walk record per ruler output
+        "walk": 8.0 + 8.0 / k,
+        # one level of blocks of 2^20: build 16 B + 18 passes of 24 B + last 8 B, then compaction 16 B
+        # (a launch does all levels when sampling is off, and returns at once otherwise)
+        "full_label": 16.0 + 18 * 24.0 + 8.0 + 16.0,
         # payload pair in, pair out, one switch bit per pair
         "apply": 2.0 * ebytes + 1.0 / 16.0,
         "apply_fused": 2.0 * ebytes + 1.0 / 16.0,
-        # P read (4 B), record written (8 B), Q scattered (4 B)
-        "inverse": 16.0,
-        # record (8 B) and Q (4 B) read, record (8 B) and Q' (4 B) written, two stage bits
-        "split": 24.0 + 1.0 / 8.0,
-        # owner word per switch, contracted word per switch, one stage bit
-        "colour": 2.0 + 4.0 + 1.0 / 16.0,
-        "combine": (16.0 + 16.0 + 8.0) / k, "list_walk": 20.0 / k, "list_label": 16.0 / k / 16.0,
-        "list_resolve": 24.0 / k,
+        # P read (4 B), claim record written (4 B), Q scattered (4 B)
+        "inverse": 12.0,
+        # Q (4 B) read, Q' (4 B) written, a stage bit per switch read and one written
+        "split": 8.0 + 1.0 / 8.0,
+        # P (4 B) and an 8-byte claim per switch read, P' (4 B) written, a stage bit per switch written
+        "colour": 12.0 + 1.0 / 16.0,
+        # records of 8 B per ruler output, an owner per pair of them, a bit each
+        "list_walk": (8.0 + 4.0) / k, "list_label": 8.0 / k, "list_resolve": (2.0 + 1.0 / 4.0) / k,
         "fused": 4.0 + (2 * 15 - 1) / 16.0,
     }[kind]
 
@@ -86,11 +87,6 @@ FALLBACK_HBM_GBS = 6650.0
 # which source file holds the kernels of a profile kind (its hash guards the stored ncu counters)
 KIND_SOURCE = {"walk": "route_sampled.cu", "colour": "route_sampled.cu", "fused": "route_fused.cu",
                "split": "route_levels.cu", "inverse": "route_levels.cu", "apply_fused": "apply_fused.cu"}
-
-
-def binding_packed_level0(n: int, kappa: int) -> bool:
-    """Whether level 0 of a permutation of 2^n uses packed 8-byte records (the library's rule)."""
-    return kappa != 0 and 3 * n - kappa + 1 < 64
 
 
 def measured_peaks():
@@ -464,9 +460,9 @@ def time_steps(case: GpuCase, steps: int, flush):
 PROBE_MODES = {
     # name: (mode, record bytes, records = elements >> shift, what it stands for)
     "load4": (0, 4, 0, "4-byte load from an array of one word per element (the inverse entry of a hop)"),
-    "load16": (1, 16, 1, "16-byte load of a wide switch record"),
-    "load16_cas": (2, 16, 1, "16-byte load + compare-and-swap on its owner word (a visit of a wide record)"),
-    "and64": (3, 8, 1, "64-bit atomic AND on an 8-byte record (a visit of a packed record)"),
+    "load16": (1, 16, 1, "16-byte load of a 16-byte record"),
+    "load16_cas": (2, 16, 1, "16-byte load + compare-and-swap on a word of it"),
+    "and64": (3, 8, 1, "64-bit atomic on an 8-byte record (a visit of a switch record)"),
     "store4": (4, 16, 1, "4-byte store into a 16-byte record"),
 }
 
@@ -693,11 +689,11 @@ def run_gpu(args):
                 roofline["dram_frac"] = traffic / per_launch_s / 1e9 / peak
                 roofline["dram_frac_of_nominal_8tbs"] = traffic / per_launch_s / 1e9 / 8000.0
             if top == "walk" and per_level.get("walk") and probe:
-                # The walk is a chain of dependent random accesses: per switch one record visit
-                # (load + claim) and one 4-byte inverse entry.  Level 0 is the launch whose block
+                # The walk is a chain of dependent random accesses: per switch one 64-bit atomic on its
+                # 8-byte record and one 4-byte inverse entry.  Level 0 is the launch whose block
                 # is furthest above the L2.  The time the same accesses take when they are
                 # independent (measured in this run on arrays of the same sizes) is the floor.
-                visit = "load16_cas" if per_level["walk"][0] and not binding_packed_level0(n, kappa) else "and64"
+                visit = "and64"
                 floor_ms = probe[visit]["ms"] + probe["load4"]["ms"]
                 roofline["random_access"] = {
                     "launch": "level 0", "ms": per_level["walk"][0],

@@ -65,7 +65,7 @@ enum {
 };
 /* There is no time-out status: no kernel of the library waits on a flag, a peer
  * or another launch.  The only loops whose length depends on the data are the
- * walks, and those stop after BENES_OPT_WALK_CAP hops and hand the level to the
+ * walks, and those stop after BENES_OPT_WALK_CAP hops and hand the route to the
  * pointer-jumping kernel, whose pass count is fixed by the block size. */
 
 #define BENES_MAX_LOG2N 30
@@ -239,7 +239,7 @@ int benes_validate_perm(const uint32_t *perm, int log2n, int batch, benes_stream
  *       walks matter more than short lists there).  The result is identical
  *       either way.
  *   BENES_OPT_WALK_CAP : hops (1 .. 2^24, default 2^14) after which a walk gives
- *       up; a level in which that happens is relabelled by full pointer jumping.
+ *       up; a route in which that happens is redone by full pointer jumping.
  *   BENES_OPT_APPLY_FUSED : 1 (default) = benes_apply / benes_apply_ex run up to
  *       25 stages per pass over the payload in shared memory; 0 = one stage per
  *       pass.  Same result.
@@ -277,9 +277,9 @@ unsigned long long benes_launch_count(void);
  * of consecutive launches of one kernel kind with a pair of CUDA events on the
  * caller's stream.  benes_profile_read synchronises those events and returns,
  * for one kind, the launches and the summed device time since the last reset.
- * Kinds: 0 inverse scatter, 1 pointer jumping over all outputs (one launch per
- * level), 2 input-side bits + compaction, 3 fused in-CTA levels, 4 payload-apply
- * stage, 5 ruler walk, 6 contracted-list assembly, 7 walk over a contracted
+ * Kinds: 0 inverse scatter, 1 pointer jumping over all outputs (one launch for all
+ * levels), 2 input-side bits + compaction, 3 fused in-CTA levels, 4 payload-apply
+ * stage, 5 ruler walk, 6 unused (always 0), 7 walk over a contracted
  * list, 8 in-CTA labelling of a contracted list, 9 labels back to a sampled
  * list, 10 colouring + output-side bits, 11 payload-apply over several stages.
  * BENES_PROFILE_KINDS = number of kinds.
