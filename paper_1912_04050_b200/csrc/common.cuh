@@ -276,10 +276,14 @@ __device__ __forceinline__ unsigned long long make_word(uint32_t nxt, uint32_t m
 }
 
 // The streaming kernels of a level give every CTA `rounds` consecutive groups of
-// `threads` items: as many as keep 8 CTAs per SM busy, at most 16.
+// `threads` items: as many as keep 8 CTAs per SM busy, at most 4.  More than one, because the next group's loads
+// are under way while one is worked on and the words a CTA gathers stay in the L1; few, because with 16 the last wave of
+// the 1184 CTAs that run together was nearly as long as the others (2^24: 1.7 waves) and the CTAs whose loops have no
+// ruler ended late.  Colouring + split, 16 -> 4 (2: the same, 1: slower at 2^26): 2^24 0.82 -> 0.70 ms, transposed 1.33
+// -> 1.09, 2^26 3.16 -> 2.97, 256 x 2^16 0.101 -> 0.079.
 inline uint32_t stream_rounds(size_t items, int threads) {
     const size_t r = items / (size_t(threads) * size_t(sm_count()) * 8);
-    return uint32_t(r < 1 ? 1 : (r > 16 ? 16 : r));
+    return uint32_t(r < 1 ? 1 : (r > 4 ? 4 : r));
 }
 
 // ---- per-level HBM path (route_levels.cu) ----------------------------------

@@ -475,10 +475,10 @@ int launch_split(const uint32_t *Q, uint32_t *Qn, size_t total, int log2m, BitsL
     const uint4 *Q4 = reinterpret_cast<const uint4 *>(Q);
     // Colour words are gathered at random from the block's row of the output-side
     // stage (2^(m-1) bits).  Rows of 32 KiB and less stay in L1 whatever the CTAs
-    // of an SM work on; for rows of 64 to 256 KiB the CTAs that are resident
+    // of an SM work on; for rows of 64 and 128 KiB the CTAs that are resident
     // together (8 per SM) should cover about one block, so that an SM sees one row.
     uint32_t rounds = stream_rounds(pairs, kThreads);
-    if (log2m >= 20 && log2m <= 22 && rounds > (1u << (log2m - 20))) rounds = 1u << (log2m - 20);
+    if (log2m >= 20 && log2m <= 21 && rounds > (1u << (log2m - 20))) rounds = 1u << (log2m - 20);
     const unsigned grid = unsigned((size_t(pairs) + size_t(kThreads) * rounds - 1) / (size_t(kThreads) * rounds));
     launch_kernel(k_split, grid, kThreads, 0, s, Q4, Qn, pairs, log2m, L, in_stage, out_stage, rounds);
     return launch_status();
