@@ -210,8 +210,11 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     // closer rulers (shorter walks) pay there although the lists get longer.
     const int kappa = (opt.kappa > 3 && T <= (size_t(1) << 22)) ? 3 : opt.kappa;
     const uint32_t cap = uint32_t(opt.walk_cap);
-    // (level 0: P is the caller's permutation, which nobody writes; the kernels load 16 bytes at a time)
-    if (reinterpret_cast<uintptr_t>(perm) % 16) {
+    // Level 0: P is the caller's permutation, which nobody writes.  The kernels of the sampled levels load it 16 bytes at
+    // a time, from a copy where it does not start on 16 bytes.  The copy lasts as long as level 0 only (level 2
+    // writes its plain P there), so pointer jumping, which begins again from level 0, reads the caller's (4 bytes at a time).
+    const uint32_t *const given = perm;
+    if (kappa && reinterpret_cast<uintptr_t>(perm) % 16) {
         BENES_CUDA_TRY(cudaMemcpyAsync(Pbuf[0], perm, T * 4, cudaMemcpyDeviceToDevice, s));
         perm = Pbuf[0];
     }
@@ -283,7 +286,7 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     const uint32_t *redone = jump_p[(n - fused_m) & 1];
     {
         ProfileScope ps(kFullLabel, s);
-        if ((rc = launch_route_jump(perm, jump_p, Qbuf, Wd, T, n, fused_m, L, kappa ? gate : nullptr, s))) return rc;
+        if ((rc = launch_route_jump(given, jump_p, Qbuf, Wd, T, n, fused_m, L, kappa ? gate : nullptr, s))) return rc;
     }
     if (kappa && hp) BENES_CUDA_TRY(cudaMemcpyAsync(hp->gate_host, gate, 4, cudaMemcpyDeviceToHost, s));
     if (!kappa && hp && hp->bits_host) {

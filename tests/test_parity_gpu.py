@@ -243,6 +243,27 @@ def test_route_redone_as_a_whole(n, batch, kappa, cap, labelling_options):
     assert np.array_equal(bits, want)
 
 
+@pytest.mark.parametrize("n,batch,kappa,cap", [(16, 1, None, None), (16, 3, None, None), (20, 1, None, None), (22, 1, None, None),
+                                               (17, 2, 0, None), (18, 1, None, 2), (24, 1, 2, 2)])
+def test_route_of_a_permutation_off_a_16_byte_boundary(n, batch, kappa, cap, labelling_options):
+    """Above the in-CTA sizes: the levels as usual, without sampling, and redone after a walk that gave up.  At 2^24 with
+    rulers 2^2 apart level 2 has wide records, whose plain array lies where an aligned copy of the permutation
+    was made; the second attempt has to start from the caller's own."""
+    if kappa is not None:
+        binding.benes_set_option(binding.OPT_SAMPLE_LOG2K, kappa)
+    if cap is not None:
+        binding.benes_set_option(binding.OPT_WALK_CAP, cap)
+    perm = inputs.random_perm_batch(n, batch, seed0=41 * n + batch)
+    want = oracle.route(perm, n)
+    for off in (1, 2, 3):                                       # words off the boundary
+        moved = dev(np.concatenate([np.zeros(off, dtype=np.uint32), perm.ravel()]))[off:]
+        bits = torch.full((binding.benes_switch_words(n, batch),), -1, dtype=torch.int32, device="cuda")
+        binding.benes_route(moved, n, batch, bits)
+        torch.cuda.synchronize()
+        assert np.array_equal(host(bits, np.uint32).reshape(want.shape), want), off
+        assert np.array_equal(host(moved, np.uint32).reshape(perm.shape), perm)
+
+
 @pytest.mark.parametrize("kappa,cap", [(None, None), (2, None), (4, None), (None, 12)])
 @pytest.mark.parametrize("n,batch", [(18, 3), (19, 3), (20, 5), (19, 7)])
 def test_route_batch_not_a_power_of_two_with_resampled_lists(n, batch, kappa, cap, labelling_options):
