@@ -39,9 +39,16 @@
  * they can be captured into a CUDA graph and replayed on new contents of the
  * same buffers; with the 2-50 small dependent launches of inputs up to about
  * 2^22 elements a replay is 10-40 % faster than the launches.
- * Nothing throws, aborts or traps.  The library is not re-entrant: calls that
- * share the workspace must be ordered (same stream, or externally
- * synchronised).
+ * Nothing throws, aborts or traps.  Calls that share the workspace must be
+ * ordered (same stream, or externally synchronised).  benes_route of sizes for
+ * which benes_route_workspace_bytes is 0 does not use it: such calls may run at
+ * once, on several streams and from several threads.  Where splitting the levels
+ * of a few permutations of 2^12 .. 2^15 over more SMs is faster, such a call takes
+ * scratch of its own in stream order (at most 19 MiB, from a memory pool of the
+ * library's own that keeps up to 32 MiB per device and gives them back in
+ * benes_release_workspace); with a caller's workspace installed and inside a
+ * capture it takes none and those levels stay in their CTAs (same result, up to
+ * about twice the time; a plan has scratch of its own and splits them).
  */
 #ifndef BENES_H_
 #define BENES_H_
@@ -209,7 +216,7 @@ int benes_plan_destroy(benes_plan_t *plan);
 /* Number of 32-bit words of switch_bits for (log2n, batch); 0 on bad arguments. */
 size_t benes_switch_words(int log2n, int batch);
 
-/* Scratch bytes benes_route / benes_apply_ex need for these arguments. */
+/* Workspace bytes benes_route / benes_apply_ex need for these arguments. */
 size_t benes_route_workspace_bytes(int log2n, int batch);
 size_t benes_apply_workspace_bytes(int elem_bytes, int log2n, int batch);
 
@@ -221,7 +228,8 @@ size_t benes_apply_workspace_bytes(int elem_bytes, int log2n, int batch);
  */
 int benes_set_workspace(void *dev_ptr, size_t bytes);
 
-/* Free the internal workspace of the current device (synchronises the device). */
+/* Free the internal workspace of the current device and what the pool behind the calls without one has kept
+ * (synchronises the device). */
 int benes_release_workspace(void);
 
 /*

@@ -126,6 +126,66 @@ int get_workspace(size_t bytes, void **out, cudaStream_t s) {
     return BENES_OK;
 }
 
+// Scratch that belongs to one call.  A route of at most 2^15 needs no workspace, so such calls may run at once, on
+// several streams and from several threads; what one of them passes from launch to launch must not lie in the
+// workspace, which they would share.  It comes and goes in stream order from a memory pool of the library's own,
+// one per device, that keeps up to kCallPoolKeep bytes when it is idle (a call takes 19 MiB at most) and returns
+// them in benes_release_workspace.  (The device's default pool keeps nothing across a synchronisation unless the
+// program has changed that, and then an allocation takes longer than the route.)
+constexpr uint64_t kCallPoolKeep = uint64_t(32) << 20;
+cudaMemPool_t g_call_pool[kMaxDevices] = {};
+
+class CallScratch {
+public:
+    CallScratch() = default;
+    CallScratch(const CallScratch &) = delete;
+    CallScratch &operator=(const CallScratch &) = delete;
+    ~CallScratch() {
+        if (p_ && cudaFreeAsync(p_, s_) != cudaSuccess) cudaGetLastError();
+    }
+    // Null where there is none to be had: with a caller's workspace no call allocates, and a graph must not hold
+    // memory of a call (an allocation in a capture would become part of the caller's graph).
+    void *take(size_t bytes, cudaStream_t s) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        int dev = 0;
+        if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
+            cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        cudaMemPool_t pool = nullptr;
+        {
+            std::lock_guard<std::mutex> lk(g_mu);
+            if (g_ws[dev].user || !pool_supported(dev)) return nullptr;
+            if (!g_call_pool[dev]) {
+                cudaMemPoolProps props = {};
+                props.allocType = cudaMemAllocationTypePinned;
+                props.location.type = cudaMemLocationTypeDevice;
+                props.location.id = dev;
+                uint64_t keep = kCallPoolKeep;
+                if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+                    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+                    if (pool) cudaMemPoolDestroy(pool);
+                    cudaGetLastError();
+                    return nullptr;
+                }
+                g_call_pool[dev] = pool;
+            }
+            pool = g_call_pool[dev];
+        }
+        if (cudaMallocFromPoolAsync(&p_, bytes, pool, s) != cudaSuccess) {
+            cudaGetLastError();
+            p_ = nullptr;
+        }
+        s_ = s;
+        return p_;
+    }
+
+private:
+    void *p_ = nullptr;
+    cudaStream_t s_ = nullptr;
+};
+
 inline bool bad_shape(int log2n, int batch) {
     return log2n < 1 || log2n > BENES_MAX_LOG2N || batch < 1;
 }
@@ -410,11 +470,16 @@ int benes_release_workspace(void) {
     BENES_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kMaxDevices) return BENES_ERR_CUDA;
     std::lock_guard<std::mutex> lk(g_mu);
+    if (g_call_pool[dev]) {
+        BENES_CUDA_TRY(cudaDeviceSynchronize());
+        BENES_CUDA_TRY(cudaMemPoolTrimTo(g_call_pool[dev], 0));
+    }
     return drop_own(g_ws[dev], dev, false, nullptr);
 }
 
 // What splitting the levels of a few permutations of 2^12 .. 2^15 over the SMs takes on top of route_ws_bytes (which
-// is 0 there): only ever from a buffer of the library's own, and a call does without where there is none.
+// is 0 there): from the call itself (benes_route), from the part of the workspace that a call with buffers of its own
+// there has anyway, or from a plan; a call does without where there is none.
 static size_t peel_bytes(int n, size_t batch) {
     return n >= kPeelLog2 && n <= kFusedLog2M && 2 * batch <= size_t(sm_count()) ? 2 * align_up((batch << n) * 4) : 0;
 }
@@ -424,13 +489,13 @@ static bool caller_workspace() {
     std::lock_guard<std::mutex> lk(g_mu);
     return g_ws[dev].user != nullptr;
 }
-// the part of the workspace that benes_route uses inside a call that keeps buffers of its own behind it
+// the part of the workspace that the route uses inside a call that keeps buffers of its own behind it
 static size_t route_inner_bytes(int n, size_t batch) {
     const size_t need = route_ws_bytes(n, batch), more = need ? 0 : peel_bytes(n, batch);
     return align_up(need + (more && !caller_workspace() ? more : 0));
 }
 
-// benes_route on a given scratch buffer (`ws` may be null when route_ws_bytes is 0)
+// benes_route on a given scratch buffer of route_ws_bytes, or of peel_bytes where those are 0 (then it may be null)
 static int route_on(const uint32_t *perm, int n, int batch, uint32_t *switch_bits, char *ws, cudaStream_t s,
                     const Options &opt) {
     if (n <= kFusedLog2M) {
@@ -494,11 +559,12 @@ int benes_route(const uint32_t *perm, int log2n, int batch, uint32_t *switch_bit
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const Options opt = options();
     void *ws = nullptr;
+    CallScratch own;
     if (route_needs_ws(log2n, opt)) {
         int rc = get_workspace(route_ws_bytes(log2n, size_t(batch)), &ws, s);
         if (rc) return rc;
     } else if (const size_t more = peel_bytes(log2n, size_t(batch))) {
-        if (caller_workspace() || get_workspace(more, &ws, s)) ws = nullptr;
+        ws = own.take(more, s);
     }
     return route_on(perm, log2n, batch, switch_bits, static_cast<char *>(ws), s, opt);
 }
@@ -548,7 +614,7 @@ int benes_route_padded(const uint32_t *perm, size_t n_elems, int batch, uint32_t
     if (rc) return rc;
     uint32_t *padded = reinterpret_cast<uint32_t *>(static_cast<char *>(ws) + inner);
     if ((rc = launch_pad_perm(perm, padded, n_elems, n, size_t(batch), s))) return rc;
-    return benes_route(padded, n, batch, switch_bits, stream);
+    return route_on(padded, n, batch, switch_bits, inner ? static_cast<char *>(ws) : nullptr, s, options());
 }
 
 int benes_apply_padded(const uint32_t *switch_bits, const void *in, void *out, int elem_bytes,
@@ -610,7 +676,7 @@ int benes_route_host(const uint32_t *perm_host, int log2n, int batch, uint32_t *
         return fetch_redone_bits(*hp, d_bits, bits_bytes, s);
     }
     BENES_CUDA_TRY(cudaMemcpyAsync(d_perm, perm_host, perm_bytes, cudaMemcpyHostToDevice, s));
-    rc = benes_route(d_perm, log2n, batch, d_bits, stream);
+    rc = route_on(d_perm, n, batch, d_bits, inner ? base : nullptr, s, opt);
     if (rc) return rc;
     BENES_CUDA_TRY(cudaMemcpyAsync(switch_bits_host, d_bits, bits_bytes, cudaMemcpyDeviceToHost, s));
     BENES_CUDA_TRY(cudaStreamSynchronize(s));

@@ -24,7 +24,7 @@ constexpr int kListSmemLog2 = 14;
 constexpr uint32_t kUnowned = 0u;
 
 // Every kernel launch of the library goes through this counter.
-extern unsigned long long g_launches;
+extern std::atomic<unsigned long long> g_launches;
 
 #define BENES_CUDA_TRY(expr)                                   \
     do {                                                       \

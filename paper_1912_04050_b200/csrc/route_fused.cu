@@ -1160,17 +1160,25 @@ k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restri
 }
 
 template <int LOGC, int THREADS>
-int launch_one(const uint32_t *P, int records, size_t first, size_t end, uint32_t *bits, int log2n, int logs,
-               cudaStream_t s, const uint32_t *gate, const uint32_t *redone) {
+int configure_one() {
     using Cfg = FusedCfg<LOGC, THREADS>;
     static OncePerDevice configured;
-    const int rc = configured.run([]() -> int {
+    return configured.run([]() -> int {
         BENES_CUDA_TRY(cudaFuncSetAttribute(k_route_fused<LOGC, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             int(Cfg::kSmemBytes)));
         BENES_CUDA_TRY(cudaFuncSetAttribute(k_route_fused<LOGC, THREADS>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                             cudaSharedmemCarveoutMaxShared));
+        cudaFuncAttributes loaded;                             // (asking for them loads the kernel)
+        BENES_CUDA_TRY(cudaFuncGetAttributes(&loaded, k_route_fused<LOGC, THREADS>));
         return BENES_OK;
     });
+}
+
+template <int LOGC, int THREADS>
+int launch_one(const uint32_t *P, int records, size_t first, size_t end, uint32_t *bits, int log2n, int logs,
+               cudaStream_t s, const uint32_t *gate, const uint32_t *redone) {
+    using Cfg = FusedCfg<LOGC, THREADS>;
+    const int rc = configure_one<LOGC, THREADS>();
     if (rc) return rc;
     const size_t ctas = (end - first + Cfg::C - 1) >> LOGC;
     launch_kernel(k_route_fused<LOGC, THREADS>, unsigned(ctas), THREADS, Cfg::kSmemBytes, s, P, records, bits, log2n, logs, first, end,
@@ -1223,7 +1231,14 @@ int launch_fused(const void *Pv, int records, size_t total, int log2m, uint32_t 
     if (log2m == kClusterLog2M) return launch_cluster2(P, records, first_block, blocks, bits, log2n, s, gate, redone);
     const size_t first = first_block << log2m, end = first + (blocks << log2m);
     int m = log2m;
-    if (spare && first == 0 && end == total)
+    if (spare && first == 0 && end == total) {
+        // A call that splits whole permutations readies the kernel of a call that may not (a captured one) too, so that
+        // one ordinary call is enough before a capture.
+        if (log2m == log2n && m >= kPeelLog2 && 2 * (total >> m) <= size_t(sm_count())) {
+            const int rc = m == 15 ? configure_one<15, 1024>() : m == 14 ? configure_one<14, 1024>()
+                         : m == 13 ? configure_one<13, 1024>() : configure_one<12, 1024>();
+            if (rc) return rc;
+        }
         for (int i = 0; m >= kPeelLog2 && 2 * (total >> m) <= size_t(sm_count()); --m, i ^= 1) {
             const int rc = m == 15 ? launch_peel<15>(P, records, total, bits, log2n, spare[i], s, gate, redone)
                          : m == 14 ? launch_peel<14>(P, records, total, bits, log2n, spare[i], s, gate, redone)
@@ -1234,6 +1249,7 @@ int launch_fused(const void *Pv, int records, size_t total, int log2m, uint32_t 
             records = 0;
             gate = nullptr;
         }
+    }
     // blocks of up to 2^11 in a plain array, and not more switches than the GPU has threads
     if (records == 0 && !gate && m <= 11 && first == 0 && end / 2 <= size_t(sm_count()) * 2048) {
         const int logc = m > 8 ? m : 8;

@@ -26,7 +26,7 @@ BENES_GUARD_TU("route_levels.cu")
 
 namespace benes {
 
-unsigned long long g_launches = 0;
+std::atomic<unsigned long long> g_launches{0};
 
 int sm_count() {
     static std::atomic<int> cached[kMaxDevices] = {};

@@ -52,7 +52,7 @@ def test_sizing_helpers(lib):
     assert lib.benes_switch_words(8, 0) == 0
     m = lib.benes_fused_log2m()
     assert 8 <= m <= 16
-    assert lib.benes_route_workspace_bytes(m, 4) == 0          # fused path needs no scratch
+    assert lib.benes_route_workspace_bytes(m, 4) == 0          # whole permutations in their CTAs: nothing shared
     assert lib.benes_route_workspace_bytes(20, 1) >= 24 << 20  # P, P', Q, Q' and 64-bit words
     assert lib.benes_apply_workspace_bytes(8, 20, 1) == 8 << 20
     assert lib.benes_apply_workspace_bytes(3, 20, 1) == 0

@@ -63,8 +63,8 @@ def test_route_batched(n, batch):
 
 @pytest.mark.parametrize("n,batch", [(12, 1), (12, 37), (12, 75), (13, 3), (14, 1), (14, 19), (15, 1), (15, 5), (16, 3), (18, 1)])
 def test_route_levels_split_over_the_sms(n, batch):
-    """Few blocks: a level at a time on twice as many SMs, which takes scratch of the library's own; with a
-    caller's workspace too small for it the blocks stay in their CTAs.  Same bits."""
+    """Few blocks: a level at a time on twice as many SMs, which takes scratch of the call's own; with a
+    caller's workspace installed the blocks stay in their CTAs.  Same bits."""
     perm = inputs.random_perm_batch(n, batch, seed0=23 * n)
     want = oracle.route(perm, n)
     assert np.array_equal(gpu_route(perm, n), want)
@@ -77,6 +77,69 @@ def test_route_levels_split_over_the_sms(n, batch):
             assert np.array_equal(gpu_route(perm, n), want)
         finally:
             binding.benes_set_workspace(None)
+
+
+@pytest.mark.parametrize("n,batch", [(12, 9), (13, 8), (15, 3)])
+def test_routes_without_workspace_run_at_once(n, batch):
+    """Calls for which benes_route_workspace_bytes is 0 share nothing: two streams, first from one thread and then
+    from one each, route different permutations again and again without any ordering between them."""
+    import threading
+    assert binding.benes_route_workspace_bytes(n, batch) == 0
+    rounds, shape = 24, (batch, 2 * n - 1, (1 << n) // 64)
+    perms = [inputs.random_perm_batch(n, batch, seed0=61 * n + 1000 * k) for k in range(2)]
+    wants = [oracle.route(p, n) for p in perms]
+    d_perms = [dev(p) for p in perms]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    words = binding.benes_switch_words(n, batch)
+
+    def work(k, first, count, outs):
+        for i in range(first, first + count):
+            binding.benes_route(d_perms[k], n, batch, outs[k][i], streams[k].cuda_stream)
+
+    for threads in (False, True):
+        outs = [[torch.full((words,), -1, dtype=torch.int32, device="cuda") for _ in range(rounds)] for _ in range(2)]
+        torch.cuda.synchronize()
+        if threads:
+            both = [threading.Thread(target=work, args=(k, 0, rounds, outs)) for k in range(2)]
+            for t in both:
+                t.start()
+            for t in both:
+                t.join()
+        else:
+            for i in range(rounds):
+                for k in range(2):
+                    work(k, i, 1, outs)
+        torch.cuda.synchronize()
+        for k in range(2):
+            for o in outs[k]:
+                assert np.array_equal(host(o, np.uint32).reshape(shape), wants[k]), (threads, k)
+
+
+@pytest.mark.parametrize("n,batch", [(13, 3), (15, 1)])
+def test_a_captured_route_without_workspace_outlives_larger_calls(n, batch):
+    """A caller's own graph of a route that needs no workspace holds no buffer of the library: it is replayed after a
+    call that has replaced the workspace and after everything has been released."""
+    perms = [inputs.random_perm_batch(n, batch, seed0=71 * n + 100 * k) for k in range(2)]
+    wants = [oracle.route(p, n) for p in perms]
+    d_perm = dev(perms[0])
+    bits = torch.full((binding.benes_switch_words(n, batch),), -1, dtype=torch.int32, device="cuda")
+    side = torch.cuda.Stream()
+    binding.benes_release_workspace()
+    binding.benes_route(d_perm, n, batch, bits, side)                  # the one ordinary call before a capture
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        binding.benes_route(d_perm, n, batch, bits, torch.cuda.current_stream())
+    for k in (1, 0):
+        d_perm.copy_(dev(perms[k]))
+        bits.fill_(-1)
+        if k:
+            gpu_route(inputs.random_perm(20, 3), 20)
+        else:
+            binding.benes_release_workspace()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(host(bits, np.uint32).reshape(wants[k].shape), wants[k]), k
 
 
 @pytest.mark.parametrize("n,batch", [(1, 2049), (2, 1031), (3, 131), (4, 67), (5, 33), (6, 17), (6, 10007), (7, 2401), (8, 5),
