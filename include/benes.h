@@ -287,7 +287,7 @@ unsigned long long benes_launch_count(void);
  * for one kind, the launches and the summed device time since the last reset.
  * Kinds: 0 inverse scatter, 1 pointer jumping over all outputs (one launch for all
  * levels), 2 input-side bits + compaction, 3 fused in-CTA levels, 4 payload-apply
- * stage, 5 ruler walk, 6 unused (always 0), 7 walk over a contracted
+ * stage, 5 ruler walk, 6 none any more (always 0; the other numbers stay), 7 walk over a contracted
  * list, 8 in-CTA labelling of a contracted list, 9 labels back to a sampled
  * list, 10 colouring + output-side bits, 11 payload-apply over several stages.
  * BENES_PROFILE_KINDS = number of kinds.

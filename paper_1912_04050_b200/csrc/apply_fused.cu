@@ -385,7 +385,7 @@ k_apply_inner(const uint32_t *__restrict__ bits, const E *__restrict__ x, E *__r
 // chunk; output side (OUT = true): stages 2n-2-(l0+k-1) .. 2n-2-l0, chunk
 // gathered from its 2^k runs and written contiguously.
 template <typename E, int C, bool OUT>
-__global__ void __launch_bounds__(kApplyThreads<C>, (sizeof(E) == 8 ? (C == 13 ? 2 : 5) : 4))
+__global__ void __launch_bounds__(kApplyThreads<C>, (sizeof(E) == 8 ? 5 : 4))
 k_apply_outer(const uint32_t *__restrict__ bits, const E *__restrict__ x, E *__restrict__ y, int n,
               int l0, int k, uint32_t cta0) {
     after_previous_kernel();

@@ -278,9 +278,9 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
         BENES_CUDA_TRY(cudaMemcpyAsync(Pbuf[0], perm, T * 4, cudaMemcpyDeviceToDevice, s));
         perm = Pbuf[0];
     }
-    auto records = [&](int level, int buf) {
+    auto records = [&](int level, int buf) {                    // (with sampling)
         const bool packed = rec_is_packed(n - level, kappa);
-        return LevelRecords{kappa ? Sbuf[buf] : nullptr, packed ? nullptr : level ? Pbuf[buf] : const_cast<uint32_t *>(perm), packed};
+        return LevelRecords{Sbuf[buf], packed ? nullptr : level ? Pbuf[buf] : const_cast<uint32_t *>(perm), packed};
     };
     SampledScratch sc;
     int rc;

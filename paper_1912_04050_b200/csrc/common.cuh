@@ -148,7 +148,7 @@ int sm_count();
 
 // Optional event timing of a group of launches of one kind (see benes.h).
 enum ProfileKind {
-    kInverse = 0, kFullLabel, kSplit, kFused, kApply, kWalk, kCombine, kListWalk, kListLabel,
+    kInverse = 0, kFullLabel, kSplit, kFused, kApply, kWalk, kListWalk = 7, kListLabel,    // 6: no kernel any more
     kListResolve, kColour, kApplyFused
 };
 struct ProfileScope {
@@ -250,15 +250,15 @@ __device__ __forceinline__ unsigned long long claim_record(uint32_t t, uint32_t 
                                                          : ((unsigned long long)p0 | ((unsigned long long)p1 << 32));
 }
 // Two neighbouring switches t, t + 1 (t even) of a level: 16-byte stores.  A wide level gets its P
-// here too, unless P is null (level 0), and its claim records, unless S is null (no sampling).
+// here too, unless P is null (level 0).
 template <bool PACKED>
 __device__ __forceinline__ void rec_write2(void *S, uint32_t *P, size_t t, int m, uint4 p, int kappa, uint32_t salt) {
     if (PACKED) {
         static_cast<ulonglong2 *>(S)[t >> 1] = make_ulonglong2(packed_record(m, p.x, p.y), packed_record(m, p.z, p.w));
     } else {
         if (P) reinterpret_cast<uint4 *>(P)[t >> 1] = p;
-        if (S) static_cast<ulonglong2 *>(S)[t >> 1] = make_ulonglong2(claim_record(uint32_t(t), p.x, p.y, kappa, salt),
-                                                                      claim_record(uint32_t(t) + 1u, p.z, p.w, kappa, salt));
+        static_cast<ulonglong2 *>(S)[t >> 1] = make_ulonglong2(claim_record(uint32_t(t), p.x, p.y, kappa, salt),
+                                                               claim_record(uint32_t(t) + 1u, p.z, p.w, kappa, salt));
     }
 }
 template <bool PACKED>
@@ -267,7 +267,7 @@ __device__ __forceinline__ void rec_write(void *S, uint32_t *P, size_t t, int m,
         static_cast<unsigned long long *>(S)[t] = packed_record(m, p0, p1);
     } else {
         if (P) reinterpret_cast<uint2 *>(P)[t] = make_uint2(p0, p1);
-        if (S) static_cast<unsigned long long *>(S)[t] = claim_record(uint32_t(t), p0, p1, kappa, salt);
+        static_cast<unsigned long long *>(S)[t] = claim_record(uint32_t(t), p0, p1, kappa, salt);
     }
 }
 
@@ -288,8 +288,7 @@ inline uint32_t stream_rounds(size_t items, int threads) {
 
 // ---- per-level HBM path (route_levels.cu) ----------------------------------
 // total = batch * N flat elements (<= 2^30), all blocks of one level per launch.
-// The records of a level: packed, or wide (S = claim records, null without sampling; P = plain array,
-// null where it need not be written).
+// The records of a level: packed, or wide (S = claim records, P = plain array).
 struct LevelRecords {
     void *S;
     uint32_t *P;

@@ -32,7 +32,7 @@ cudaEvent_t take_event(int dev) {
 }
 
 const char *kNames[BENES_PROFILE_KINDS] = {"inverse", "full_label", "split", "fused", "apply", "walk",
-                                           "combine", "list_walk", "list_label", "list_resolve",
+                                           "unused", "list_walk", "list_label", "list_resolve",
                                            "colour", "apply_fused"};
 
 }  // namespace
