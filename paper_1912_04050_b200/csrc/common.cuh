@@ -298,8 +298,8 @@ struct LevelRecords {
 int launch_inverse(const uint32_t *perm, LevelRecords S, uint32_t *Q, size_t total, int log2m, int kappa,
                    cudaStream_t s);
 // The same for total >= 2^kInversePartitionMinLog2 in two streaming passes:
-// `pairs` = total x 8 bytes of scratch, `fill` = total >> 18 zero-initialised
-// counters (at most kInverseMaxBuckets).
+// `pairs` = total x 8 bytes of scratch, `fill` = kInverseMaxBuckets zero-initialised counters, one
+// per bucket (total >> 15 of them are used, or total >> 18 where that would be too many).
 constexpr int kInversePartitionMinLog2 = 22;
 constexpr int kInverseMaxBuckets = 4096;
 int launch_inverse_partitioned(const uint32_t *perm, LevelRecords S, uint32_t *Q, void *pairs,

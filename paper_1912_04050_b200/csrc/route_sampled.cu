@@ -30,9 +30,10 @@
 //      claimed lies on a loop without ruler; such loops are short
 //      (probability (1-1/k)^length) and the thread walks the cycle itself.
 //
-// Every walk gives up after `cap` hops and raises the level's gate; the gate
-// opens the full pointer-jumping kernel of route_levels.cu, which relabels the
-// level.  So the result never depends on the sampling.
+// Every walk gives up after `cap` hops and raises the gate, one word for the whole route.  What the
+// kernels after it then compute is discarded (they only have to stay in bounds and to end): behind the
+// last of these levels the gate opens the pointer-jumping kernel of route_levels.cu, which does all of
+// them again from the caller's permutation.  So the result never depends on the sampling.
 #include "common.cuh"
 
 BENES_GUARD_TU("route_sampled.cu")
@@ -148,7 +149,7 @@ k_walk(unsigned long long *__restrict__ S8, const uint32_t *__restrict__ P, cons
             }
         }
         if (W == 1 || (++rounds & 63u) == 0u) {
-            if (((W == 1 ? hops : rounds) & 63u) == 0u && gate_raised(gate)) break;      // the level is relabelled anyway
+            if (((W == 1 ? hops : rounds) & 63u) == 0u && gate_raised(gate)) break;      // the route is redone anyway
         }
         if (ends) {
             rec[rho] = make_uint2(least, peer);
@@ -454,8 +455,7 @@ __device__ __forceinline__ uint32_t owner_colour(const uint32_t *cb, uint32_t co
 // (owner reset).  A thread owns the neighbouring switches 2i and 2i+1: their
 // colour-0 outputs are neighbours in the upper half-block of the next level and
 // their colour-1 outputs in the lower one, i.e. the thread writes one whole
-// record of each.  If the gate is raised afterwards, the split kernel redoes
-// the records from the relabelled stage.
+// record of each.  (With the gate raised what it writes is never used.)
 template <bool PACKED, bool NEXT_PACKED>
 __global__ void __launch_bounds__(kThreads)
 k_colour(const void *__restrict__ S, const uint32_t *__restrict__ P, const uint32_t *__restrict__ Q,

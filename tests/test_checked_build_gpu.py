@@ -76,8 +76,8 @@ def test_no_guard_fires_for_any_ruler_spacing(kappa, options):
 
 @pytest.mark.parametrize("cap", [1, 3, 40])
 def test_no_guard_fires_when_walks_give_up(cap, options):
-    """Forced fallback: the walk records are then partly unused, the level is relabelled by
-    pointer jumping over all outputs."""
+    """Forced fallback: the walk records are then partly unused, the route is redone by pointer
+    jumping over all outputs."""
     binding.benes_set_option(binding.OPT_WALK_CAP, cap)
     for n in (16, 18):
         perm = inputs.random_perm(n, 900 + n)

@@ -279,8 +279,8 @@ def test_route_structured_in_clusters(n, kind, cluster_mode):
 
 @pytest.mark.parametrize("cap", [1, 3, 40])
 def test_route_walks_that_give_up_fall_back_to_full_pointer_jumping(cap, labelling_options):
-    """With a tiny hop limit almost every level raises its gate and is relabelled
-    by the full pointer-jumping kernels; the bits must not change."""
+    """With a tiny hop limit some walk of almost every level gives up, and the route is redone by
+    pointer jumping over all outputs; the bits must not change."""
     binding.benes_set_option(binding.OPT_WALK_CAP, cap)
     for n in (16, 18):
         for kind, perm in inputs.structured_perms(n).items():
@@ -591,7 +591,7 @@ def test_route_maximum_size_properties():
 @pytest.mark.parametrize("n,batch,pinned", [(15, 2, False), (17, 3, False), (18, 1, True), (23, 1, True), (23, 1, False)])
 def test_host_entry_points(n, batch, pinned):
     """Host buffers in and out; above the in-CTA size the copies are overlapped with
-    the levels (the permutation arrives in pieces from N = 2^23 on)."""
+    the levels (the permutation arrives in pieces from 2^22 elements on)."""
     perm = inputs.random_perm_batch(n, batch, seed0=5)
     bits = np.full((batch, 2 * n - 1, (1 << n) // 64), 0xAAAAAAAA, dtype=np.uint32)
     if pinned:
@@ -616,9 +616,8 @@ def test_host_entry_points(n, batch, pinned):
                                                      (23, 2, np.uint64, False), (18, 3, np.uint64, True),
                                                      (15, 2, np.uint32, False), (25, 1, np.uint64, True)])
 def test_route_apply_host_in_one_call(n, batch, dtype, want_bits):
-    """Permutation and payload in, routed payload (and, if wanted, the switch words) out; from
-    2^23 elements on the payload arrives while the levels run and the words never pass through
-    host memory."""
+    """Permutation and payload in, routed payload (and, if wanted, the switch words) out; the payload
+    arrives while the levels run (in parts from 8 MiB on) and the words never pass through host memory."""
     perm = inputs.random_perm_batch(n, batch, seed0=600 + n)
     x = inputs.payload_u64(batch << n, 8).reshape(batch, -1)
     if dtype == np.uint32:
@@ -653,7 +652,7 @@ def test_route_host_split_tail_matches_device_path():
 
 
 def test_apply_host_piped_u32():
-    """Payloads of 64 MiB and more go through benes_apply_host in parts (first pass
+    """Payloads of 8 MiB and more go through benes_apply_host in parts (first pass
     as the parts arrive, last pass handing finished parts to the copy stream)."""
     n = 24
     perm = inputs.random_perm(n, 13)
