@@ -46,11 +46,11 @@
  * which benes_route_workspace_bytes is 0 does not use it: such calls may run at
  * once, on several streams and from several threads.  Where splitting the levels
  * of a few permutations of 2^12 .. 2^15 over more SMs is faster, such a call takes
- * scratch of its own in stream order (at most 19 MiB, from a memory pool of the
- * library's own that keeps up to 32 MiB per device and gives them back in
- * benes_release_workspace); with a caller's workspace installed and inside a
- * capture it takes none and those levels stay in their CTAs (same result, up to
- * about twice the time; a plan has scratch of its own and splits them).
+ * one of up to four buffers (19 MiB at most) that the library keeps per device until
+ * benes_release_workspace, for itself until its kernels have ended.  While all
+ * four are in use, with a caller's workspace installed and inside a capture it
+ * takes none and those levels stay in their CTAs (same result, up to about twice
+ * the time; a plan has scratch of its own and splits them).
  */
 #ifndef BENES_H_
 #define BENES_H_
@@ -232,7 +232,7 @@ size_t benes_apply_workspace_bytes(int elem_bytes, int log2n, int batch);
  */
 int benes_set_workspace(void *dev_ptr, size_t bytes);
 
-/* Free the internal workspace of the current device and what the pool behind the calls without one has kept
+/* Free the internal workspace of the current device and the buffers of the calls that need none
  * (synchronises the device). */
 int benes_release_workspace(void);
 

@@ -128,12 +128,32 @@ int get_workspace(size_t bytes, void **out, cudaStream_t s) {
 
 // Scratch that belongs to one call.  A route of at most 2^15 needs no workspace, so such calls may run at once, on
 // several streams and from several threads; what one of them passes from launch to launch must not lie in the
-// workspace, which they would share.  It comes and goes in stream order from a memory pool of the library's own,
-// one per device, that keeps up to kCallPoolKeep bytes when it is idle (a call takes 19 MiB at most) and returns
-// them in benes_release_workspace.  (The device's default pool keeps nothing across a synchronisation unless the
-// program has changed that, and then an allocation takes longer than the route.)
-constexpr uint64_t kCallPoolKeep = uint64_t(32) << 20;
-cudaMemPool_t g_call_pool[kMaxDevices] = {};
+// workspace, which they would share.  It takes one of a few buffers per device: the one its stream used last (the
+// stream orders the two uses), else one whose last use has ended, by the event recorded behind it; grown where it
+// is too small.  While the host is inside a call, the buffer is that call's alone.  When all are in use the call does
+// without (it would split its levels over SMs that the others are using).  Four buffers of 19 MiB at most;
+// benes_release_workspace gives them back.
+// What it costs the host is 0.7 us a call.  Allocating from a memory pool of the library's own in every call took 3 us, and
+// 20-50 from three streams on; waiting for the event on the same stream too, 2 us on the device, since the first
+// kernel then cannot take its places before the one ahead of it has ended.
+constexpr int kCallSlots = 4;
+constexpr unsigned long long kNoStream = ~0ull;
+struct CallSlot {
+    void *p = nullptr;
+    size_t bytes = 0;
+    unsigned long long stream = kNoStream;      // id of the stream of the last use (a handle may be another one's later)
+    cudaEvent_t done = nullptr;          // recorded behind the last use
+    bool taken = false, pooled = false;
+};
+CallSlot g_call_slots[kMaxDevices][kCallSlots];
+
+// Calls that query or allocate are not allowed to other threads while somebody captures in the global mode, unless
+// they say that they mean no captured work.
+struct NoCapturedWork {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    NoCapturedWork() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~NoCapturedWork() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 
 class CallScratch {
 public:
@@ -141,49 +161,86 @@ public:
     CallScratch(const CallScratch &) = delete;
     CallScratch &operator=(const CallScratch &) = delete;
     ~CallScratch() {
-        if (p_ && cudaFreeAsync(p_, s_) != cudaSuccess) cudaGetLastError();
+        if (!slot_) return;
+        const bool recorded = cudaEventRecord(slot_->done, s_) == cudaSuccess;
+        if (!recorded) cudaGetLastError();
+        std::lock_guard<std::mutex> lk(g_mu);
+        slot_->stream = id_;
+        slot_->taken = !recorded;                              // (no event: nobody may use the buffer again)
     }
-    // Null where there is none to be had: with a caller's workspace no call allocates, and a graph must not hold
-    // memory of a call (an allocation in a capture would become part of the caller's graph).
+    // Null where there is none to be had: all taken; with a caller's workspace, when no call allocates; and in a
+    // capture, since a graph must not hold memory of a call.
     void *take(size_t bytes, cudaStream_t s) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
         int dev = 0;
         if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
-            cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+            cudaStreamGetId(s, &id_) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
             cudaGetLastError();
             return nullptr;
         }
-        cudaMemPool_t pool = nullptr;
-        {
-            std::lock_guard<std::mutex> lk(g_mu);
-            if (g_ws[dev].user || !pool_supported(dev)) return nullptr;
-            if (!g_call_pool[dev]) {
-                cudaMemPoolProps props = {};
-                props.allocType = cudaMemAllocationTypePinned;
-                props.location.type = cudaMemLocationTypeDevice;
-                props.location.id = dev;
-                uint64_t keep = kCallPoolKeep;
-                if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
-                    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-                    if (pool) cudaMemPoolDestroy(pool);
-                    cudaGetLastError();
-                    return nullptr;
-                }
-                g_call_pool[dev] = pool;
+        if (s == cudaStreamPerThread) id_ = kNoStream;         // one handle, many streams
+        NoCapturedWork relaxed;
+        std::lock_guard<std::mutex> lk(g_mu);
+        if (g_ws[dev].user) return nullptr;
+        CallSlot *slot = nullptr;
+        for (CallSlot &c : g_call_slots[dev])
+            if (!c.taken && c.p && id_ != kNoStream && c.stream == id_) { slot = &c; break; }
+        if (!slot) {
+            for (CallSlot &c : g_call_slots[dev]) {
+                if (c.taken) continue;
+                if (c.p && cudaEventQuery(c.done) != cudaSuccess) { cudaGetLastError(); continue; }
+                if (!slot || (c.bytes >= bytes && slot->bytes < bytes)) slot = &c;
             }
-            pool = g_call_pool[dev];
+            if (!slot) return nullptr;
         }
-        if (cudaMallocFromPoolAsync(&p_, bytes, pool, s) != cudaSuccess) {
-            cudaGetLastError();
-            p_ = nullptr;
-        }
+        if (!fit(*slot, bytes, dev, s)) return nullptr;
+        slot->taken = true;
+        slot_ = slot;
         s_ = s;
-        return p_;
+        return slot->p;
+    }
+    // Gives the buffers of the device back (g_mu held).
+    static int drop_all(int dev) {
+        for (CallSlot &c : g_call_slots[dev]) {
+            if (c.taken || !c.p) continue;
+            BENES_CUDA_TRY(cudaEventSynchronize(c.done));
+            if (c.pooled) {
+                BENES_CUDA_TRY(cudaFreeAsync(c.p, nullptr));
+                BENES_CUDA_TRY(cudaStreamSynchronize(nullptr));
+            } else {
+                BENES_CUDA_TRY(cudaFree(c.p));
+            }
+            c.p = nullptr;
+            c.bytes = 0;
+        }
+        return BENES_OK;
     }
 
 private:
-    void *p_ = nullptr;
+    // A buffer of at least `bytes` in a slot whose last use precedes what is enqueued on `s` from here on.
+    static bool fit(CallSlot &c, size_t bytes, int dev, cudaStream_t s) {
+        if (!c.done && cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming) != cudaSuccess) {
+            cudaGetLastError();
+            c.done = nullptr;
+            return false;
+        }
+        if (c.bytes >= bytes) return true;
+        const bool pool = pool_supported(dev);
+        if (c.p && (pool ? cudaFreeAsync(c.p, s) : cudaFree(c.p)) != cudaSuccess) { cudaGetLastError(); return false; }
+        c.p = nullptr;
+        c.bytes = 0;
+        if ((pool ? cudaMallocAsync(&c.p, bytes, s) : cudaMalloc(&c.p, bytes)) != cudaSuccess) {
+            cudaGetLastError();
+            c.p = nullptr;
+            return false;
+        }
+        c.bytes = bytes;
+        c.pooled = pool;
+        return true;
+    }
+    CallSlot *slot_ = nullptr;
     cudaStream_t s_ = nullptr;
+    unsigned long long id_ = kNoStream;
 };
 
 inline bool bad_shape(int log2n, int batch) {
@@ -470,10 +527,8 @@ int benes_release_workspace(void) {
     BENES_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kMaxDevices) return BENES_ERR_CUDA;
     std::lock_guard<std::mutex> lk(g_mu);
-    if (g_call_pool[dev]) {
-        BENES_CUDA_TRY(cudaDeviceSynchronize());
-        BENES_CUDA_TRY(cudaMemPoolTrimTo(g_call_pool[dev], 0));
-    }
+    const int rc = CallScratch::drop_all(dev);
+    if (rc) return rc;
     return drop_own(g_ws[dev], dev, false, nullptr);
 }
 

@@ -81,38 +81,47 @@ def test_route_levels_split_over_the_sms(n, batch):
 
 @pytest.mark.parametrize("n,batch", [(12, 9), (13, 8), (15, 3)])
 def test_routes_without_workspace_run_at_once(n, batch):
-    """Calls for which benes_route_workspace_bytes is 0 share nothing: two streams, first from one thread and then
-    from one each, route different permutations again and again without any ordering between them."""
+    """Calls for which benes_route_workspace_bytes is 0 share nothing: six streams (more than there are buffers for
+    splitting levels), first from one thread and then from one each, route different permutations again and again
+    without any ordering between them, in changing sizes of batch."""
     import threading
     assert binding.benes_route_workspace_bytes(n, batch) == 0
-    rounds, shape = 24, (batch, 2 * n - 1, (1 << n) // 64)
-    perms = [inputs.random_perm_batch(n, batch, seed0=61 * n + 1000 * k) for k in range(2)]
+    lanes, rounds, words = 6, 16, binding.benes_switch_words(n, 1)
+    counts = [batch + 2 * (k % 3) for k in range(lanes)]
+    perms = [inputs.random_perm_batch(n, counts[k], seed0=61 * n + 1000 * k) for k in range(lanes)]
     wants = [oracle.route(p, n) for p in perms]
     d_perms = [dev(p) for p in perms]
-    streams = [torch.cuda.Stream() for _ in range(2)]
-    words = binding.benes_switch_words(n, batch)
+    streams = [torch.cuda.Stream() for _ in range(lanes)]
 
-    def work(k, first, count, outs):
-        for i in range(first, first + count):
-            binding.benes_route(d_perms[k], n, batch, outs[k][i], streams[k].cuda_stream)
+    def work(k, i):
+        b = counts[k] - (i & 1)                                  # (not the whole batch every time)
+        binding.benes_route(d_perms[k], n, b, outs[k][i], streams[k].cuda_stream)
+
+    def lane(k):
+        for i in range(rounds):
+            work(k, i)
 
     for threads in (False, True):
-        outs = [[torch.full((words,), -1, dtype=torch.int32, device="cuda") for _ in range(rounds)] for _ in range(2)]
+        outs = [[torch.full((c * words,), -1, dtype=torch.int32, device="cuda") for _ in range(rounds)] for c in counts]
         torch.cuda.synchronize()
         if threads:
-            both = [threading.Thread(target=work, args=(k, 0, rounds, outs)) for k in range(2)]
-            for t in both:
+            together = [threading.Thread(target=lane, args=(k,)) for k in range(lanes)]
+            for t in together:
                 t.start()
-            for t in both:
+            for t in together:
                 t.join()
         else:
             for i in range(rounds):
-                for k in range(2):
-                    work(k, i, 1, outs)
+                for k in range(lanes):
+                    work(k, i)
         torch.cuda.synchronize()
-        for k in range(2):
-            for o in outs[k]:
-                assert np.array_equal(host(o, np.uint32).reshape(shape), wants[k]), (threads, k)
+        for k in range(lanes):
+            for i, o in enumerate(outs[k]):
+                b = counts[k] - (i & 1)
+                got = host(o, np.uint32).reshape(wants[k].shape)
+                assert np.array_equal(got[:b], wants[k][:b]), (threads, k, i)
+                assert (got[b:] == 0xFFFFFFFF).all()
+    binding.benes_release_workspace()
 
 
 @pytest.mark.parametrize("n,batch", [(13, 3), (15, 1)])
