@@ -400,7 +400,6 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     // Pointer jumping over all outputs, all levels: the whole labelling when sampling is off, otherwise gated
     // (returns at once unless some walk gave up).  Its sub-permutations go where the records were.
     uint32_t *const jump_p[2] = {static_cast<uint32_t *>(Sbuf[0]), static_cast<uint32_t *>(Sbuf[1])};
-    const uint32_t *redone = jump_p[(n - fused_m) & 1];
     {
         ProfileScope ps(kFullLabel, s);
         if ((rc = launch_route_jump(given, jump_p, Qbuf, Wd, T, n, fused_m, L, kappa ? gate : nullptr, s))) return rc;
@@ -412,10 +411,8 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
             if ((rc = copy_stage_rows(*hp, bits, n, batch, 2 * n - 2 - level, 1, s))) return rc;
         }
     }
-    const LevelRecords tail = records(n - fused_m, cur);
-    const void *tail_p = kappa == 0 ? redone : tail.packed ? tail.S : tail.P;
-    const int tail_format = kappa && tail.packed ? 1 : 0;
-    const uint32_t *tail_gate = kappa ? gate : nullptr;
+    // the in-CTA levels start from the inverses, which either labelling leaves in the same place
+    const uint32_t *tail = Qbuf[(n - fused_m) & 1];
     const size_t blocks = T >> fused_m;
     // the stages of the in-CTA levels are one run of rows in the middle
     const int first = n - fused_m, rows = 2 * fused_m - 1;
@@ -426,12 +423,12 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
         const size_t b1 = ((waves + 1) / 2) * kFusedSplitWave;
         {
             ProfileScope ps(kFused, s);
-            if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, 0, b1, tail_gate, redone))) return rc;
+            if ((rc = launch_fused(tail, true, T, fused_m, bits, n, s, 0, b1))) return rc;
         }
         BENES_CUDA_TRY(cudaEventRecord(hp->stage_ready[kMaxLevels - 2], s));
         {
             ProfileScope ps(kFused, s);
-            if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, b1, blocks - b1, tail_gate, redone))) return rc;
+            if ((rc = launch_fused(tail, true, T, fused_m, bits, n, s, b1, blocks - b1))) return rc;
         }
         // a block of 2^m outputs owns 2^(m-6) words of every stage
         const size_t w = stage_words(n) * 4, col1 = (b1 << (fused_m - 6)) * 4;
@@ -447,7 +444,7 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     }
     {
         ProfileScope ps(kFused, s);
-        if ((rc = launch_fused(tail_p, tail_format, T, fused_m, bits, n, s, 0, 0, tail_gate, redone, Qbuf))) return rc;
+        if ((rc = launch_fused(tail, true, T, fused_m, bits, n, s, 0, 0, jump_p))) return rc;
     }
     if (hp && hp->bits_host) {
         BENES_CUDA_TRY(cudaEventRecord(hp->stage_ready[kMaxLevels - 2], s));
@@ -561,8 +558,8 @@ static int route_on(const uint32_t *perm, int n, int batch, uint32_t *switch_bit
             size_t nb = size_t(batch) - b0 < max_ctas ? size_t(batch) - b0 : max_ctas;
             uint32_t *const spare[2] = {reinterpret_cast<uint32_t *>(ws),
                                         reinterpret_cast<uint32_t *>(ws + align_up((nb << n) * 4))};
-            int rc = launch_fused(perm + (b0 << n), 0, nb << n, n,
-                                  switch_bits + b0 * size_t(2 * n - 1) * stage_words(n), n, s, 0, 0, nullptr, nullptr,
+            int rc = launch_fused(perm + (b0 << n), false, nb << n, n,
+                                  switch_bits + b0 * size_t(2 * n - 1) * stage_words(n), n, s, 0, 0,
                                   ws ? spare : nullptr);
             if (rc) return rc;
         }
@@ -571,7 +568,7 @@ static int route_on(const uint32_t *perm, int n, int batch, uint32_t *switch_bit
     if (n == kFusedLog2M + 1 && opt.cluster) {
         // whole permutations of 2^16, one cluster of two CTAs each
         ProfileScope ps(kFused, s);
-        return launch_fused(perm, 0, size_t(batch) << n, n, switch_bits, n, s);
+        return launch_fused(perm, false, size_t(batch) << n, n, switch_bits, n, s);
     }
     const size_t chunk = level_chunk(n, size_t(batch), opt.chunk_log2);
     for (size_t b0 = 0; b0 < size_t(batch); b0 += chunk) {

@@ -339,12 +339,10 @@ size_t sampled_owner_bytes(const SampledScratch &sc, size_t total, int log2m, in
 // Finishes levels (n - log2m) .. n-1 of every block of size 2^log2m of the flat
 // level array (total elements), one CTA per block for log2m <= kFusedLog2M, one
 // cluster of two CTAs per block for log2m = kFusedLog2M + 1.
-// P is a plain uint32 array if records == 0, packed records if 1.
-// `blocks` blocks from `first_block` on (blocks = 0: all from first_block).  With a gate: if *gate is not 0, the
-// blocks are those of the plain array `redone`.
-int launch_fused(const void *P, int records, size_t total, int log2m, uint32_t *bits, int log2n,
-                 cudaStream_t s, size_t first_block = 0, size_t blocks = 0, const uint32_t *gate = nullptr,
-                 const uint32_t *redone = nullptr, uint32_t *const spare[2] = nullptr);
+// `src`: the blocks' values, local to their block: the permutation, or its inverse if `inverse`.
+// `blocks` blocks from `first_block` on (blocks = 0: all from first_block).
+int launch_fused(const uint32_t *src, bool inverse, size_t total, int log2m, uint32_t *bits, int log2n,
+                 cudaStream_t s, size_t first_block = 0, size_t blocks = 0, uint32_t *const spare[2] = nullptr);
 // With `spare` (two arrays of total words), blocks of 2^kPeelLog2 and more that leave at least half of the SMs without
 // one run a level at a time, on twice as many SMs each time.
 constexpr int kPeelLog2 = 12;

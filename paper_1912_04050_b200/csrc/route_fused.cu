@@ -5,40 +5,35 @@
 // permutations; a CTA holds one block, or several when the blocks are smaller
 // than 2^LOGC.
 //
-// A level works on sub-blocks of S = 2^logs outputs.  The kernel is bound by the
-// shared-memory wavefronts of its random 16-bit accesses (3-4 per warp access; about
-// 25 thousand per level of 2^15 outputs, of 34 thousand cycles) and by instruction
-// issue, hardly by memory, so the labelling changes with S:
+// A level works on sub-blocks of S = 2^logs outputs, and from its inverse Q alone.  The outputs a = Q[2s] and
+// b = Q[2s+1] of an input switch are each other's partners on the loop, so one pass over the input switches
+// scatters the successors, g(a ^ 1) = b and g(b ^ 1) = a: no gather forms them and no P is kept.  Behind the
+// colouring the same pass takes the colour of every input switch (a bit gathered through Q[2s]: the input-side
+// stage), forms the two half-blocks' inverses from pairs of neighbouring switches, and scatters their successors.
+// What bounds the kernel: the shared-memory wavefronts of these random accesses (3.5 per warp access) and, as close, the
+// integer pipe (64 lanes per clock and SM, so that two cycles go by with every instruction of a warp).  Hence one
+// scatter of all outputs and two gathers per switch in a level, nothing else at random but the walks, and little
+// arithmetic beside them.
 //
-//   S >= 256   16-bit entries.  One ruler switch per 8 switches; a walker per
-//              ruler output follows g, claims the switches it passes and stops where
-//              it meets the walker from the other end; the contracted list (S/8
-//              words of next and minimum) is labelled by in-place pointer jumping;
-//              a switch takes (parity of its owner's minimum) ^ side.  Switches
-//              nobody claimed (loops without ruler) walk their own cycle.
-//   S = 128..16  8-bit entries.  One THREAD runs the sequential looping algorithm on
-//              a sub-block: from the smallest switch not seen yet it follows the
-//              loop once, and every output it stands on goes up, which is the
-//              canonical colouring by construction (no minimum, no list).  S/2
-//              visits of about 17 instructions without divergence, against 5-7
-//              pointer-jumping passes over all outputs.
+//   S >= 512   16-bit entries (byte offsets in the CTA, so that an entry is an address).  One ruler INPUT switch
+//              per 8 G; a walker leaves it from either output, follows g, claims the output switches it stands on
+//              and stops where it meets the walker from the other end.  In place of the two successors that lead
+//              across a ruler switch lie the codes of the walkers beyond, so that a walker meets a ruler as it
+//              meets a walker.  The contracted list (next and minimum) is labelled by in-place pointer jumping; a
+//              switch takes (parity of its owner's minimum) ^ side.  Switches nobody claimed (loops without
+//              ruler) walk their own cycle.
+//   S = 256..16  8-bit entries.  One THREAD runs the sequential looping algorithm on a sub-block: from the
+//              smallest switch not seen yet it follows the loop; the output it started from goes up, which
+//              is the canonical colouring by construction (no minimum, no list).
 //   S = 8      the colours of 4 switches depend on the input switches of the first
 //              7 outputs only: 14 bits into a table.
 //   S = 4, 2   256-entry table: all three stages at once.
 //
-// Entries carry one bit beside the index: the parity of the input the value stood
-// for one level up.  The inverse scattered from such entries therefore holds, in
-// input order, the input-side bits of the level above (of every upper half-block:
-// an input switch is crossed iff its odd input goes up), which leave as bytes
-// without a gather.
-//
-// 16-bit entries (byte offsets, so that an entry is an address without a shift):
-//   P[i] = 2 (first output of the sub-block + value) | parity,  Q[..] = 2 i | parity
-// 8-bit entries:  value local to the sub-block | parity << 7.
-//
-// Measured on B200, before (walks and compaction on plain 16-bit indices at every level, warp
-// shuffles below 64) and after: 2048 blocks of 2^15 4.71 -> 2.40 ms, 4096 x 2^12 0.82 -> 0.37 ms,
-// 16384 x 2^8 0.117 -> 0.050 ms.
+// Measured on B200, before (P and Q kept, successors gathered through both; twice as many rulers; a look for
+// the next start with every hop at all 8-bit levels) and after: 2048 blocks of 2^15 2.38 -> 1.88 ms, 4096 x 2^14
+// 1.96 -> 1.58 ms, 4096 x 2^12 374 -> 314 us, 16384 x 2^8 53 -> 40 us.  Units of 8192 outputs inside a larger CTA with
+// barriers of their own, meant to fall out of step, took 2.04 and 1.90 ms for the first two: the CTA waits for
+// its last unit.
 #include "common.cuh"
 
 #include <cooperative_groups.h>
@@ -50,14 +45,11 @@ BENES_GUARD_TU("route_fused.cu")
 namespace benes {
 namespace {
 
-constexpr int kFKappa = 3;                     // ruler spacing (log2) inside a CTA
-constexpr int kFMinLogS = 8;                   // smallest sub-block labelled by ruler walks (16-bit entries)
-// Word of a switch in the successor array, two 16-bit halves.  Unclaimed: g(2t) and g(2t+1), each as
-// twice the output.  Claimed: the same code in both halves, bit 0 set, bit 1 the side of arrival,
-// bits 2-14 the walker (a ruler output), bit 15 set if the switch is a ruler switch (then the
-// walker is its even output).
-constexpr uint32_t kCodeRho = 0x7FFCu, kRulerFlag = 0x8000u;
-constexpr uint32_t kNone16 = 0xFFFFu;          // (two-CTA level) owner of a switch nobody claimed
+constexpr int kFMinLogS = 9;                   // smallest sub-block labelled by ruler walks (16-bit entries)
+// A half of the word of an output switch t in the successor array, at the place of output j = 2t or 2t + 1: the
+// successor of j as twice the output; or, bit 0 set, the walker (a ruler output, from bit 2 on: its byte offset in
+// the list) that owns the switch and stood on the OTHER output of it.
+constexpr uint32_t kCodeRho = 0xFFFCu;
 
 // ---- tables of the last levels ----------------------------------------------------
 // Colours of the four switches of a sub-block of 8: index = input switch (2 bits) of
@@ -128,28 +120,38 @@ constexpr FusedTables make_tables(std::integer_sequence<uint32_t, W...>) { retur
 __device__ const FusedTables g_fused_tables = make_tables(std::make_integer_sequence<uint32_t, kLut8Words + kLut4Words>());
 
 // ---- shared memory ------------------------------------------------------------------
-//   [0, 2C)    P (16 bit)      |  8 bit: P and the next level's P, C bytes each
-//   [2C, 4C)   Q (16 bit); once the successors are formed: walk records and list words
-//              (32 bit per ruler output), queue of unclaimed switches   |  8 bit: Q
-//   [4C, 6C)   successors / owners, a 32-bit word per switch   |  8 bit: the tables
-//   then the stage words of the level's output side and of the previous level's input side
-template <int LOGC, int THREADS>
+// A thread has 16 G inputs (8 G switches) of every level.
+//   [0, 2C)     successors / owners, 16 bit       |  8 bit: successors, the first half; then the tables
+//   kRec        walk records, contracted list, 32 bit per walker each  |  marks of the sub-blocks of 2^8, behind the tables
+//   kQ (2C)     inverse: pairs of 16-bit entries per input switch, as uint4 of four switches at a place of
+//               their thread's that makes reads and writes free of bank conflicts  |  8 bit: two buffers
+//   kCw (C/16)  colours of the level, kInw (C/16) input-side bits of small permutations
+// Bytes from the marks of a sub-block of 2^8 to the next one's: the lanes of a warp look at the same place of theirs.
+constexpr uint32_t kMarkStride = 128 + 8;
+
+template <int LOGC, int GROUPS>
 struct FusedCfg {
-    static constexpr int C = 1 << LOGC;
-    static constexpr int T = THREADS;
-    static constexpr int kRulers = C >> kFKappa;
-    static constexpr int kQ = 2 * C;
-    static constexpr int kRec = kQ;
-    static constexpr int kList = kRec + kRulers * 4;
-    static constexpr int kQueue = kList + kRulers * 4;         // 4 bytes (a list word of 0), then the entries
-    static constexpr int kN = 4 * C;
-    static constexpr int kLabelBytes = 2 * C > kLutBytes ? 2 * C : kLutBytes;
-    static constexpr int kCw = kN + kLabelBytes;
-    static constexpr int kInw = kCw + C / 16;
-    static constexpr int kCount = kInw + C / 16;               // entries of the queue
+    static constexpr int LOG = LOGC;
+    static constexpr uint32_t C = 1u << LOGC;
+    static constexpr uint32_t G = GROUPS;
+    static constexpr uint32_t T = C / (16 * G);
+    static constexpr int kSpacing = G == 2 ? 4 : 3;              // log2(input switches per ruler): one ruler per thread
+    static constexpr uint32_t R = C / (8 * G);                   // walkers = words of the contracted list, 2 per thread
+    static constexpr uint32_t kRec = 2 * C;
+    static constexpr uint32_t kList = kRec + 4 * R;
+    static constexpr uint32_t kLevelBytes = kList + 4 * R;
+    static constexpr uint32_t kTables = C;
+    static constexpr uint32_t kTablesEnd = kTables + uint32_t(kLutBytes);
+    static constexpr uint32_t kMarks = kTablesEnd;                 // marks of the sub-blocks of 2^8
+    static constexpr uint32_t kMarkBytes = C / 256 * kMarkStride;
+    static constexpr uint32_t kMarksEnd = kMarks + kMarkBytes;
+    static constexpr uint32_t kQ = ((kMarksEnd > kLevelBytes ? kMarksEnd : kLevelBytes) + 15u) & ~15u;
+    static constexpr uint32_t kCw = kQ + 2 * C;
+    static constexpr uint32_t kInw = kCw + C / 16;
+    static constexpr uint32_t kCount = kInw + C / 16;            // queued switches
     static constexpr size_t kSmemBytes = size_t(kCount) + 16;
     // CTAs per SM the register budget has to leave room for
-    static constexpr int kMinCtas = THREADS > C / 32 || LOGC >= 15 ? 1 : (LOGC == 14 ? 2 : (LOGC == 13 ? 4 : 8));
+    static constexpr int kMinCtas = G == 1 || T > 512 ? 1 : int(1024 / T) < 8 ? int(1024 / T) : 8;
 };
 
 template <class Tp>
@@ -157,9 +159,20 @@ __device__ __forceinline__ Tp &at(unsigned char *sm, uint32_t byte) {
     return *reinterpret_cast<Tp *>(sm + byte);
 }
 
+// The ruler switch of a group: top bits of a multiplicative hash
+template <int SPACING>
 __device__ __forceinline__ uint32_t fused_slot(uint32_t group, uint32_t salt) {
-    // top bits of a multiplicative hash
-    return ((group + salt * 0x632BE5ABu) * 0x9E3779B1u) >> (32 - kFKappa);
+    return ((group + salt * 0x632BE5ABu) * 0x9E3779B1u) >> (32 - SPACING);
+}
+
+// Place of the pair word of input switch s (the four from a multiple of 4 on are 16 bytes): the four switches `c` of
+// every thread side by side; the odd ones shifted by half of the banks, because neighbouring threads write them
+// together.
+template <class Cfg>
+__device__ __forceinline__ uint32_t q_place(uint32_t s) {
+    constexpr uint32_t G = Cfg::G;
+    const uint32_t i = s / (8 * G), c = (s / 4) % (2 * G);
+    return Cfg::kQ + (c * Cfg::T + (i ^ (c >= G ? 4u : 0u))) * 16u + (s & 3u) * 4u;
 }
 
 // Where the CTA's words go: flat output index of its first output, how many outputs
@@ -186,14 +199,6 @@ struct FusedOut {
         for (uint32_t k = 0; k < per && ((r * per + k) << n) < valid; ++k)
             bits[(perm0 + k) * size_t(2 * n - 1) + size_t(stage)] = (half >> (k * nb)) & ((1u << nb) - 1u);
     }
-    template <class Cfg>
-    __device__ __forceinline__ void store_row(unsigned char *sm, uint32_t row, int stage) const {
-        if (n >= 6) {
-            for (uint32_t w = threadIdx.x; w < valid >> 6; w += Cfg::T) *stage_word(stage, w) = at<uint32_t>(sm, row + w * 4);
-        } else {
-            for (uint32_t r = threadIdx.x; r < uint32_t(Cfg::C / 32); r += Cfg::T) store16(stage, r, at<uint16_t>(sm, row + r * 2));
-        }
-    }
 };
 
 // bits 7, 15, 23, 31 of w, in this order, as 4 bits
@@ -208,18 +213,36 @@ __device__ __forceinline__ uint32_t spread4(uint32_t c) {
 // 2-bit fields at the bottom of the four bytes -> 8 bits, byte 0 on top
 __device__ __forceinline__ uint32_t fields_of_bytes(uint32_t x) { return (x * 0x40100401u) >> 24; }
 
+// Byte `g` of a stage: the 8 switches of the CTA's outputs [16 g, 16 g + 16) (n >= 6).
+__device__ __forceinline__ uint8_t *stage_byte(const FusedOut &out, int stage, uint32_t g) {
+    return reinterpret_cast<uint8_t *>(out.stage_word(stage, g >> 2)) + (g & 3u);
+}
+
 // ---- a level with 16-bit entries -------------------------------------------------------
-// Input-side bits of the level above a level of sub-blocks of 2^logs: the parities in the upper half-blocks, in input order.
+// Pair words x = Q[2s] | Q[2s+1] << 16 scatter the successors of the outputs beside theirs.
 template <class Cfg>
-__device__ __forceinline__ void input_bits16(unsigned char *sm, int logs) {
-    constexpr uint32_t C = Cfg::C, T = Cfg::T;
-    for (uint32_t c = threadIdx.x; c < C / 16; c += T) {
-        const uint32_t i = ((c >> (logs - 3)) << (logs + 1)) + ((c & ((1u << (logs - 3)) - 1u)) << 3);
-        const uint4 q = at<uint4>(sm, Cfg::kQ + 2 * i);
-        const uint32_t x = (q.x & 0x00010001u) | ((q.y & 0x00010001u) << 2) | ((q.z & 0x00010001u) << 4) |
-                           ((q.w & 0x00010001u) << 6);
-        at<uint8_t>(sm, Cfg::kInw + c) = uint8_t(x | (x >> 15));
-    }
+__device__ __forceinline__ void scatter_successors(unsigned char *sm, uint32_t x) {
+    const uint32_t y = x ^ 0x00020002u;
+    at<uint16_t>(sm, y & 0xFFFFu) = uint16_t(x >> 16);
+    at<uint16_t>(sm, y >> 16) = uint16_t(x);
+}
+
+// The ruler of a thread: its group, and the pair of outputs its walkers start from.
+struct Ruler {
+    uint32_t group, pair;
+};
+
+// Puts the codes of the two walkers of ruler switch s in place of the successors across it; the calling thread
+// has written the pair word and those successors itself.
+template <class Cfg>
+__device__ __forceinline__ Ruler place_ruler(unsigned char *sm, uint32_t s) {
+    Ruler r;
+    r.group = s >> Cfg::kSpacing;
+    r.pair = at<uint32_t>(sm, q_place<Cfg>(s));
+    const uint32_t y = r.pair ^ 0x00020002u, code = (r.group << 3) | 1u;
+    at<uint16_t>(sm, y & 0xFFFFu) = uint16_t(code);
+    at<uint16_t>(sm, y >> 16) = uint16_t(code + 4u);
+    return r;
 }
 
 // Colour of output 2t of a switch nobody claimed: its g-cycle (at most S/2 outputs) from both ends;
@@ -229,381 +252,431 @@ __device__ __forceinline__ uint32_t loop_colour16(unsigned char *sm, uint32_t t,
     constexpr uint32_t kMask = 2u * Cfg::C - 2u;
     const uint32_t j0 = 4u * t;
     uint32_t f = j0, bk = j0, least = j0;
-    for (uint32_t hops = 0; hops < S; ++hops) {
-        const uint32_t nf = at<uint16_t>(sm, Cfg::kN + f) & kMask;
-        const uint32_t nb = at<uint16_t>(sm, Cfg::kN + (bk ^ 2u)) & kMask;
-        f = nf;
-        if (f == bk) break;
-        least = min(least, f);
-        bk = nb ^ 2u;
-        if (bk == f) break;
-        least = min(least, bk);
+    // (four hops per look at whether the two have met: on the way past each other they see what they know already)
+    for (uint32_t hops = 0; hops < S; hops += 4) {
+        bool met = false;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t nf = at<uint16_t>(sm, f) & kMask, nb = (at<uint16_t>(sm, bk ^ 2u) & kMask) ^ 2u;
+            met |= nf == bk || nf == nb;
+            f = nf;
+            bk = nb;
+            least = min(least, min(f, bk));
+        }
+        if (met) break;
     }
     return (least >> 1) & 1u;
 }
 
+// Labelling and colouring of a level; the colours go to kCw.
 template <class Cfg>
-__device__ __forceinline__ void level16(unsigned char *sm, const FusedOut &out, int logs, int level, bool first) {
-    constexpr uint32_t C = Cfg::C, T = Cfg::T, R = Cfg::kRulers;
-    constexpr uint32_t kMask = 2u * C - 2u;                     // a byte offset of an entry
-    constexpr int kGroups = int(C / 16 / T) > 0 ? int(C / 16 / T) : 1;     // ruler groups (8 switches) per thread
+__device__ __forceinline__ void colours16(unsigned char *sm, int logs, const Ruler &ruler) {
+    constexpr uint32_t T = Cfg::T, R = Cfg::R, G = Cfg::G;
     const uint32_t tid = threadIdx.x;
     const uint32_t S = 1u << logs;
 
-    if (!first) input_bits16<Cfg>(sm, logs);
-    // Successors g(j) = Q[P[j^1] ^ 1], so that a hop of a walk is one load: the gathers here run
-    // with all lanes, those of the walks with a quarter of them.  The word of a ruler switch is its
-    // code from the start; its thread keeps the successors, with which it starts the two walks.
-    uint32_t start[kGroups];
-#pragma unroll
-    for (int r = 0; r < kGroups; ++r) {
-        const uint32_t g = tid + uint32_t(r) * T;
-        start[r] = 0u;
-        if (g < C / 16) {
-            const uint4 pa = at<uint4>(sm, g * 32), pb = at<uint4>(sm, g * 32 + 16);
-            uint32_t w[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
-            const uint32_t slot = fused_slot(g, uint32_t(level));
-#pragma unroll
-            for (uint32_t k = 0; k < 8; ++k) {
-                const uint32_t g1 = at<uint16_t>(sm, Cfg::kQ + ((w[k] ^ 2u) & kMask));
-                const uint32_t g0 = at<uint16_t>(sm, Cfg::kQ + (((w[k] >> 16) ^ 2u) & kMask));
-                w[k] = (g0 | (g1 << 16)) & (kMask * 0x10001u);
-                if (k == slot) {
-                    start[r] = w[k];
-                    w[k] = (kRulerFlag | (g << 3) | 1u) * 0x10001u;
-                }
-            }
-            at<uint4>(sm, Cfg::kN + g * 32) = make_uint4(w[0], w[1], w[2], w[3]);
-            at<uint4>(sm, Cfg::kN + g * 32 + 16) = make_uint4(w[4], w[5], w[6], w[7]);
-        }
-    }
-    __syncthreads();
-
-    // Walks from the ruler outputs; the two of a segment meet in the middle.  A claim needs no
-    // atomic.  Only the two walkers of this segment ever reach switch t, from opposite ends.  If both
-    // find it free at the same moment, both write (either code is a valid owner: the two stand for
-    // mirror cycles and arrive on opposite sides, so the colour comes out the same), both go on, and
+    // Walks from the ruler outputs; the two of a segment meet in the middle.  A claim needs no atomic.  Only the
+    // two walkers of this segment ever reach a switch, from opposite ends, and each looks at the half the
+    // other one writes.  If both find it free at the same moment, both write (either code is a valid owner: the two
+    // stand for mirror cycles and on opposite outputs, so the colour comes out the same), both go on, and
     // each stops at the next switch, which the other has claimed; minima are taken over one switch
     // more, which changes nothing.  A walker keeps one minimum: the outputs on the far side of its
     // switches are the ones it stood on with the last bit flipped, and so is their minimum.
-    // A thread has the walks of its own rulers; walks differ in length, so a lane goes on to its
-    // next walk every four hops instead of waiting for the longest walk of the warp.
-    if (tid < C / 16) {
-        const uint32_t walks = 2u * min(uint32_t(kGroups), (C / 16 - tid + T - 1) / T);
-        uint32_t k = 0, g = tid, rho = 2u * g;
-        uint32_t least = 4u * ((g << kFKappa) | fused_slot(g, uint32_t(level))), j = start[0] & 0xFFFFu;
-        uint32_t code = ((rho << 2) | 1u) * 0x10001u;
+    // Walks differ in length, so a lane goes on to its next one every few hops instead of waiting for the longest walk of
+    // the warp.  (Successors that form no cycles, of an input that is no permutation, end with the rounds.)
+    {
+        uint32_t rounds = S + 8u;
+        uint32_t code = (ruler.group << 3) | 1u, j = ruler.pair & 0xFFFFu, least = j;
         for (;;) {
             // (no branches: a lane that has met somebody reads the same code again)
             bool met = false;
             uint32_t v = 0;
 #pragma unroll
             for (int hop = 0; hop < 4; ++hop) {
-                v = at<volatile uint16_t>(sm, Cfg::kN + j);
+                v = at<volatile uint16_t>(sm, j);
                 met = (v & 1u) != 0u;
-                if (!met) at<volatile uint32_t>(sm, Cfg::kN + (j & ~3u)) = code + (j & 2u) * 0x10001u;
+                if (!met) at<volatile uint16_t>(sm, j ^ 2u) = uint16_t(code);
                 least = met ? least : min(least, j);
                 j = met ? j : v;
             }
-            if (met) {
-                // a ruler switch (its code names its even output), or one the other walker owns
-                const uint32_t peer4 = (v & kCodeRho) ^ ((v & kRulerFlag) ? ((~j & 2u) << 1) : 0u);
-                at<uint32_t>(sm, Cfg::kRec + rho * 4) = (least << 16) | peer4;
-                if (++k == walks) break;
-                g = tid + (k >> 1) * T;
-                rho = 2u * g + (k & 1u);
-                least = 4u * ((g << kFKappa) | fused_slot(g, uint32_t(level))) + 2u * (k & 1u);
-                uint32_t st = start[0];
-#pragma unroll
-                for (int r = 1; r < kGroups; ++r) st = (k >> 1) == uint32_t(r) ? start[r] : st;
-                j = (k & 1u) ? st >> 16 : st & 0xFFFFu;
-                code = ((rho << 2) | 1u) * 0x10001u;
+            if (met || --rounds == 0u) {
+                at<uint32_t>(sm, Cfg::kRec + code - 1u) = (least << 16) | (v & kCodeRho);
+                if ((code & 4u) || rounds == 0u) break;
+                code += 4u;
+                j = ruler.pair >> 16;
+                least = j;
             }
         }
-    }
-    if (tid == 0) {
-        at<uint32_t>(sm, Cfg::kQueue) = 0u;
-        at<uint32_t>(sm, Cfg::kCount) = 0u;
     }
     __syncthreads();
 
     // Contracted list: next = peer ^ 1.  What the other walker of my ruler switch has seen, with the last bit
     // flipped, lies on my cycle too, and every segment of a cycle has both of its walkers in such pairs of the cycle:
-    // no need to fetch the minimum of the peer.
-    constexpr int kPer = int(R / T) > 0 ? int(R / T) : 1;
-    uint32_t w[kPer];
+    // no need to fetch the minimum of the peer.  In-place pointer jumping, own words in registers; a cycle of the list
+    // has at most half of the walkers of its sub-block.
+    uint32_t w[2];
 #pragma unroll
-    for (int r = 0; r < kPer; ++r) {
-        const uint32_t rho = tid + uint32_t(r) * T;
-        if (rho < R) {
-            const uint32_t a = at<uint32_t>(sm, Cfg::kRec + rho * 4), b = at<uint32_t>(sm, Cfg::kRec + (rho ^ 1u) * 4);
-            w[r] = ((a & (R * 4u - 4u)) ^ 4u) | min(a & 0xFFFF0000u, (b ^ 0x00020000u) & 0xFFFF0000u);
-            at<uint32_t>(sm, Cfg::kList + rho * 4) = w[r];
-        }
+    for (int r = 0; r < 2; ++r) {
+        const uint32_t o = (tid + uint32_t(r) * T) * 4u;
+        const uint32_t a = at<uint32_t>(sm, Cfg::kRec + o), b = at<uint32_t>(sm, Cfg::kRec + (o ^ 4u));
+        w[r] = ((a & (R * 4u - 4u)) ^ 4u) | (min(a, b ^ 0x00020000u) & 0xFFFF0000u);
+        at<uint32_t>(sm, Cfg::kList + o) = w[r];
     }
-    // Switches nobody claimed lie on loops without ruler.  A few of them in a group queue up, so that
-    // one thread takes one; a group full of them (permutations made of short loops) stays with
-    // its thread.
-    uint32_t dense[kGroups];                                     // free switches | their colours << 8
-#pragma unroll
-    for (int r = 0; r < kGroups; ++r) {
-        const uint32_t g = tid + uint32_t(r) * T;
-        dense[r] = 0u;
-        if (g < C / 16) {
-            const uint4 a = at<uint4>(sm, Cfg::kN + g * 32), b = at<uint4>(sm, Cfg::kN + g * 32 + 16);
-            uint32_t free_ = (~a.x & 1u) | ((~a.y & 1u) << 1) | ((~a.z & 1u) << 2) | ((~a.w & 1u) << 3) |
-                             ((~b.x & 1u) << 4) | ((~b.y & 1u) << 5) | ((~b.z & 1u) << 6) | ((~b.w & 1u) << 7);
-            const uint32_t count = uint32_t(__popc(free_));
-            if (count > 3u) {
-                dense[r] = free_;
-            } else if (free_) {
-                uint32_t pos = atomicAdd(&at<uint32_t>(sm, Cfg::kCount), count);
-                while (free_) {
-                    const uint32_t k = uint32_t(__ffs(int(free_))) - 1u;
-                    free_ &= free_ - 1u;
-                    at<uint16_t>(sm, Cfg::kQueue + 4u + 2u * pos++) = uint16_t(8u * g + k);
-                }
-            }
-        }
-    }
-    if (!first) out.store_row<Cfg>(sm, Cfg::kInw, level - 1);
+    if (tid == 0u) at<uint32_t>(sm, Cfg::kCount) = 0u;
     __syncthreads();
-
-    // In-place pointer jumping, own words in registers; a cycle of the list has at most S/16 words
-    // (half of the ruler outputs of its sub-block): logs - 4 passes, at least 4.  The queue rides
-    // along: colours before the first barrier, codes (list word R, which is 0, and the colour as the
-    // side) after it, when no walk reads successors any more.
-    constexpr uint32_t resolved = (R << 2) | 1u;
-    const uint32_t queued = at<uint32_t>(sm, Cfg::kCount);
-    for (uint32_t e = tid; e < queued; e += T) {
-        const uint32_t t = at<uint16_t>(sm, Cfg::kQueue + 4u + 2u * e);
-        at<uint16_t>(sm, Cfg::kQueue + 4u + 2u * e) = uint16_t(t | (loop_colour16<Cfg>(sm, t, S) << 15));
-    }
+    for (int pass = 0; pass < logs - Cfg::kSpacing - 1; ++pass) {
 #pragma unroll
-    for (int r = 0; r < kGroups; ++r)
-        for (uint32_t left = dense[r]; left; left &= left - 1u) {
-            const uint32_t k = uint32_t(__ffs(int(left))) - 1u;
-            dense[r] |= loop_colour16<Cfg>(sm, 8u * (tid + uint32_t(r) * T) + k, S) << (8u + k);
-        }
-    for (int pass = 0; pass < logs - kFKappa - 1; ++pass) {
-#pragma unroll
-        for (int r = 0; r < kPer; ++r) {
-            const uint32_t rho = tid + uint32_t(r) * T;
-            if (rho < R) {
-                const uint32_t v = at<volatile uint32_t>(sm, Cfg::kList + (w[r] & 0xFFFFu));
-                w[r] = (v & 0xFFFFu) | min(w[r] & 0xFFFF0000u, v & 0xFFFF0000u);
-                at<volatile uint32_t>(sm, Cfg::kList + rho * 4) = w[r];
-            }
+        for (int r = 0; r < 2; ++r) {
+            const uint32_t v = at<volatile uint32_t>(sm, Cfg::kList + (w[r] & 0xFFFFu));
+            w[r] = (v & 0xFFFFu) | (min(w[r], v) & 0xFFFF0000u);
+            at<volatile uint32_t>(sm, Cfg::kList + (tid + uint32_t(r) * T) * 4u) = w[r];
         }
         __syncthreads();
-        if (pass == 0) {
-            for (uint32_t e = tid; e < queued; e += T) {
-                const uint32_t x = at<uint16_t>(sm, Cfg::kQueue + 4u + 2u * e);
-                at<uint32_t>(sm, Cfg::kN + 4u * (x & 0x7FFFu)) = resolved | ((x >> 14) & 2u);
-            }
-        }
     }
 
-    // Colours of 8 switches (a ruler group) per round, and the next level's entries of their 16
-    // outputs, which stay in registers until everybody has read this level's.
-    uint32_t u[kGroups][4], l[kGroups][4];
-    const bool wide_next = logs - 1 >= kFMinLogS;
+    // Switches nobody claimed lie on loops without ruler.  They queue up over the walk records, so that one thread takes
+    // one; where the queue is full (permutations made of short loops) they stay with their thread.
+    // Colours of 8 switches per round.  A half with a code names the owner, who stood on the output of the other half.
+    constexpr uint32_t kQueue = 2u * R;
+    const uint32_t h = (tid >> 2) & 1u;                             // (lanes 4 apart would meet in a bank)
 #pragma unroll
-    for (int r = 0; r < kGroups; ++r) {
-        const uint32_t g = tid + uint32_t(r) * T;
-        if (g < C / 16) {
-            const uint4 na = at<uint4>(sm, Cfg::kN + g * 32), nb = at<uint4>(sm, Cfg::kN + g * 32 + 16);
-            uint32_t code[8] = {na.x, na.y, na.z, na.w, nb.x, nb.y, nb.z, nb.w};
-            uint32_t c[8], byte = 0;
-            if (dense[r]) {
+    for (uint32_t r = 0; r < G; ++r) {
+        const uint32_t g = tid + r * T;
+        const uint4 first = at<uint4>(sm, g * 32u + h * 16u), second = at<uint4>(sm, g * 32u + (h ^ 1u) * 16u);
+        const uint32_t n8[8] = {first.x, first.y, first.z, first.w, second.x, second.y, second.z, second.w};
+        uint32_t bits = 0, free_ = 0;
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if ((dense[r] >> k) & 1u) code[k] = resolved | (((dense[r] >> (8 + k)) & 1u) << 1);
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                c[k] = ((at<uint32_t>(sm, Cfg::kList + (code[k] & kCodeRho)) >> 17) ^ (code[k] >> 1)) & 1u;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) byte |= c[k] << k;
-            at<uint8_t>(sm, Cfg::kCw + g) = uint8_t(byte);
-            const uint4 pa = at<uint4>(sm, g * 32), pb = at<uint4>(sm, g * 32 + 16);
-            uint32_t y[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
-            const uint32_t sb = (16u * g) & ~(S - 1u);
-            if (wide_next) {
-                const uint32_t vmask = (S - 1u) * 0x10001u, up = (2u * sb) * 0x10001u, low = S * 0x10001u;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) y[k] = ((y[k] >> 1) & vmask) | up;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint32_t sel = 0x5410u | (c[2 * k] * 0x22u) | (c[2 * k + 1] * 0x2200u);
-                    // (0x5410 and 0x2222 share no set bit, so | adds them)
-                    u[r][k] = __byte_perm(y[2 * k], y[2 * k + 1], sel);
-                    l[r][k] = __byte_perm(y[2 * k], y[2 * k + 1], sel ^ 0x2222u) | low;
-                }
-            } else {
-                // to 8-bit entries: value (v >> 1) with the parity in bit 7, from 2 (base + v) | parity
-#pragma unroll
-                for (int k = 0; k < 8; ++k) y[k] = ((y[k] >> 2) & 0x007F007Fu) | ((y[k] << 6) & 0x00800080u);
-                uint32_t hu[4], hl[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint32_t sel = 0x40u | (c[2 * k] * 0x02u) | (c[2 * k + 1] * 0x20u);
-                    hu[k] = __byte_perm(y[2 * k], y[2 * k + 1], sel);
-                    hl[k] = __byte_perm(y[2 * k], y[2 * k + 1], sel ^ 0x22u);
-                }
-                u[r][0] = __byte_perm(hu[0], hu[1], 0x5410); u[r][1] = __byte_perm(hu[2], hu[3], 0x5410);
-                l[r][0] = __byte_perm(hl[0], hl[1], 0x5410); l[r][1] = __byte_perm(hl[2], hl[3], 0x5410);
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t lo = n8[k] & 1u, code = lo ? n8[k] : n8[k] >> 16;
+            const uint32_t c = (at<uint32_t>(sm, Cfg::kList + (code & (R * 4u - 4u))) >> 17) ^ lo;
+            bits |= (c & 1u) << k;
+            free_ |= (~code & 1u) << k;
+        }
+        bits &= ~free_;
+        if (free_) {
+            uint32_t pos = atomicAdd(&at<uint32_t>(sm, Cfg::kCount), uint32_t(__popc(free_)));
+            for (uint32_t left = free_; left; left &= left - 1u, ++pos) {
+                const uint32_t k = uint32_t(__ffs(int(left))) - 1u, t = 8u * g + (k ^ (h << 2));
+                if (pos < kQueue) at<uint16_t>(sm, Cfg::kRec + 2u * pos) = uint16_t(t);
+                else bits |= loop_colour16<Cfg>(sm, t, S) << k;
             }
         }
+        at<uint8_t>(sm, Cfg::kCw + g) = uint8_t(h ? (bits >> 4) | (bits << 4) : bits);
     }
     __syncthreads();
-    // the next level's entries and their inverse
-    const uint32_t H = S >> 1;
-#pragma unroll
-    for (int r = 0; r < kGroups; ++r) {
-        const uint32_t g = tid + uint32_t(r) * T;
-        if (g < C / 16) {
-            const uint32_t sb = (16u * g) & ~(S - 1u), tl = (16u * g - sb) >> 1;
-            if (wide_next) {
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const uint32_t i = sb + tl + (half ? H : 0u);
-                    const uint32_t *e = half ? l[r] : u[r];
-                    at<uint4>(sm, 2u * i) = make_uint4(e[0], e[1], e[2], e[3]);
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const uint32_t x = (k & 1) ? e[k >> 1] >> 16 : e[k >> 1];
-                        at<uint16_t>(sm, Cfg::kQ + (x & 0xFFFEu)) = uint16_t((x & 1u) | (2u * (i + uint32_t(k))));
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const uint32_t base = sb + (half ? H : 0u);
-                    const uint32_t *e = half ? l[r] : u[r];
-                    at<uint2>(sm, base + tl) = make_uint2(e[0], e[1]);
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const uint32_t x = e[k >> 2] >> (8 * (k & 3));
-                        at<uint8_t>(sm, Cfg::kQ + base + (x & 0x7Fu)) = uint8_t((x & 0x80u) | (tl + uint32_t(k)));
-                    }
-                }
-            }
+    const uint32_t queued = min(at<uint32_t>(sm, Cfg::kCount), kQueue);
+    if (queued) {                                                   // (same value for all threads)
+        for (uint32_t e = tid; e < queued; e += T) {
+            const uint32_t t = at<uint16_t>(sm, Cfg::kRec + 2u * e);
+            if (loop_colour16<Cfg>(sm, t, S)) atomicOr(&at<uint32_t>(sm, Cfg::kCw + ((t >> 3) & ~3u)), 1u << (t & 31u));
         }
+        __syncthreads();
     }
-    out.store_row<Cfg>(sm, Cfg::kCw, 2 * out.n - 2 - level);
-    __syncthreads();
 }
 
-// ---- a level with 8-bit entries ----------------------------------------------------------
-// The looping algorithm on the 2^LOGREG outputs from byte `rb` on (one sub-block, or the two
-// sub-blocks of 16 of a region of 32): ascending start switches, one visit per switch.
-template <int LOGREG>
-__device__ __forceinline__ void loop_region(const unsigned char *P, const unsigned char *Q, uint32_t smask,
-                                            uint32_t *col) {
-    constexpr uint32_t kReg = 1u << LOGREG, kSw = kReg / 2;
-    constexpr int kWords = kSw > 32 ? int(kSw / 32) : 1;
-    uint32_t seen[kWords];
+// Input side of the thread's 8 G switches and the next level's entries: u[], l[] = pairs of the upper and the lower
+// half-block, as they are stored (16-bit entries), or, if the next level has 8-bit entries, words of four of them.
+template <class Cfg>
+__device__ __forceinline__ void split16(unsigned char *sm, const FusedOut &out, int logs, int level, bool wide_next,
+                                        uint32_t u[4 * Cfg::G], uint32_t l[4 * Cfg::G]) {
+    constexpr uint32_t G = Cfg::G;
+    const uint32_t tid = threadIdx.x;
+    const uint32_t S = 1u << logs, sb = (16u * G * tid) & ~(S - 1u);
+    const uint32_t vmask = (S - 1u) * 0x10001u, up = (2u * sb) * 0x10001u, low = S * 0x10001u;
+    uint32_t in = 0;
 #pragma unroll
-    for (int w = 0; w < kWords; ++w) seen[w] = col[w] = 0u;
-    uint32_t j = 0, start = 0;                 // j goes up; the loop being walked began at output `start`
-#pragma unroll 4
-    for (uint32_t it = 0; it < kSw; ++it) {
-        const uint32_t sb = LOGREG == 5 ? (j & ~smask & (kReg - 1u)) : 0u;
-        const uint32_t x = ((uint32_t(P[j]) & smask) ^ 1u) | sb;
-        const uint32_t next = ((uint32_t(Q[x]) & smask) ^ 1u) | sb;
-        const uint32_t bit = 1u << ((j >> 1) & 31u), odd = (j & 1u) ? bit : 0u;
-        uint32_t fresh;                        // smallest switch not seen
-        if (kWords == 1) {
-            seen[0] |= bit;
-            col[0] |= odd;
-            fresh = uint32_t(__ffs(int(~seen[0]))) - 1u;
-        } else {
-            const bool hi = j >= 64u;
-            seen[0] |= hi ? 0u : bit; seen[kWords - 1] |= hi ? bit : 0u;
-            col[0] |= hi ? 0u : odd; col[kWords - 1] |= hi ? odd : 0u;
-            fresh = ~seen[0] ? uint32_t(__ffs(int(~seen[0]))) - 1u : 31u + uint32_t(__ffs(int(~seen[kWords - 1])));
+    for (uint32_t q = 0; q < 2 * G; ++q) {
+        const uint4 w4 = at<uint4>(sm, q_place<Cfg>(8u * G * tid + 4u * q));
+        uint32_t y[4] = {w4.x, w4.y, w4.z, w4.w}, c[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            // output 2 t + side is entry 4 t + 2 side; its switch is bit t
+            const uint32_t word = at<uint32_t>(sm, Cfg::kCw + ((y[k] >> 5) & (Cfg::C / 16 - 4)));
+            c[k] = (__funnelshift_r(word, word, y[k] >> 2) ^ (y[k] >> 1)) & 1u;
+            in |= c[k] << (4u * q + uint32_t(k));
         }
-        const bool closed = next == start;
-        start = closed ? (2u * fresh) & (kReg - 1u) : start;
-        j = closed ? start : next;
+        if (wide_next) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) y[k] = ((y[k] >> 1) & vmask & 0xFFFEFFFEu) | up;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                // (0x5410 and 0x2222 share no set bit, so | adds them)
+                const uint32_t sel = 0x5410u | (c[2 * k] * 0x22u) | (c[2 * k + 1] * 0x2200u);
+                u[2 * q + k] = __byte_perm(y[2 * k], y[2 * k + 1], sel);
+                l[2 * q + k] = __byte_perm(y[2 * k], y[2 * k + 1], sel ^ 0x2222u) | low;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) y[k] = (y[k] >> 2) & 0x00FF00FFu;
+            uint32_t hu[2], hl[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const uint32_t sel = 0x40u | (c[2 * k] * 0x02u) | (c[2 * k + 1] * 0x20u);
+                hu[k] = __byte_perm(y[2 * k], y[2 * k + 1], sel);
+                hl[k] = __byte_perm(y[2 * k], y[2 * k + 1], sel ^ 0x22u);
+            }
+            u[q] = __byte_perm(hu[0], hu[1], 0x5410);
+            l[q] = __byte_perm(hl[0], hl[1], 0x5410);
+        }
+    }
+    if (16u * G * tid < out.valid) {
+        uint8_t *to_in = stage_byte(out, level, G * tid), *to_out = stage_byte(out, 2 * out.n - 2 - level, G * tid);
+        if (G == 1) {
+            *to_in = uint8_t(in);
+            *to_out = at<uint8_t>(sm, Cfg::kCw + tid);
+        } else {
+            *reinterpret_cast<uint16_t *>(to_in) = uint16_t(in);
+            *reinterpret_cast<uint16_t *>(to_out) = at<uint16_t>(sm, Cfg::kCw + 2u * tid);
+        }
+    }
+}
+
+// Successors of four 8-bit pairs (words e0, e1 = eight entries in input order), local to a sub-block that starts at byte n8
+__device__ __forceinline__ void scatter_successors8(unsigned char *sm, uint32_t n8, uint32_t e0, uint32_t e1) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t e = (k < 2 ? e0 : e1) >> (16 * (k & 1)), a = e & 0xFFu, b = (e >> 8) & 0xFFu;
+        at<uint8_t>(sm, n8 + a) = uint8_t(b ^ 1u);
+        at<uint8_t>(sm, n8 + b) = uint8_t(a ^ 1u);
     }
 }
 
 template <class Cfg>
-__device__ __forceinline__ void level8(unsigned char *sm, const FusedOut &out, int logs, int level, bool first,
-                                       uint32_t pcur) {
-    constexpr uint32_t C = Cfg::C, T = Cfg::T;
+__device__ __forceinline__ void clear_marks(unsigned char *sm) {
+    for (uint32_t o = 8u * threadIdx.x; o < Cfg::kMarkBytes; o += 8u * Cfg::T) at<uint2>(sm, Cfg::kMarks + o) = make_uint2(0, 0);
+}
+
+// One level of 16-bit entries after another, down to sub-blocks of 2^8 (whose entries are then in place).
+template <class Cfg>
+__device__ __forceinline__ void levels16(unsigned char *sm, const FusedOut &out, int logs, Ruler &ruler) {
+    constexpr uint32_t G = Cfg::G;
     const uint32_t tid = threadIdx.x;
-    const uint32_t S = 1u << logs, smask = S - 1u, H = S >> 1;
-    if (!first) {
-        for (uint32_t c = tid; c < C / 16; c += T) {
-            const uint32_t i = ((c >> (logs - 3)) << (logs + 1)) + ((c & ((S >> 3) - 1u)) << 3);
-            const uint2 q = at<uint2>(sm, Cfg::kQ + i);
-            at<uint8_t>(sm, Cfg::kInw + c) = uint8_t(tops_of_bytes(q.x) | (tops_of_bytes(q.y) << 4));
+    for (;; --logs) {
+        const int level = out.n - logs;
+        const uint32_t S = 1u << logs;
+        colours16<Cfg>(sm, logs, ruler);
+        uint32_t u[4 * G], l[4 * G];
+        const bool wide_next = logs - 1 >= kFMinLogS;
+        split16<Cfg>(sm, out, logs, level, wide_next, u, l);
+        __syncthreads();
+        const uint32_t sb = (16u * G * tid) & ~(S - 1u), tl = (16u * G * tid - sb) >> 1, H = S >> 1;
+        if (!wide_next) {
+            clear_marks<Cfg>(sm);
+#pragma unroll
+            for (uint32_t q = 0; q < G; ++q) {
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    const uint32_t *e = half ? l : u;
+                    const uint32_t base = sb + (half ? H : 0u);
+                    at<uint2>(sm, Cfg::kQ + base + tl + 8u * q) = make_uint2(e[2 * q], e[2 * q + 1]);
+                    scatter_successors8(sm, base, e[2 * q], e[2 * q + 1]);
+                }
+            }
+            __syncthreads();
+            return;
         }
+        // positions (in switches) of the thread's first pair in either half-block
+        const uint32_t su = (sb + tl) >> 1, sl = su + (H >> 1);
+#pragma unroll
+        for (uint32_t q = 0; q < G; ++q) {
+            at<uint4>(sm, q_place<Cfg>(su + 4u * q)) = make_uint4(u[4 * q], u[4 * q + 1], u[4 * q + 2], u[4 * q + 3]);
+            at<uint4>(sm, q_place<Cfg>(sl + 4u * q)) = make_uint4(l[4 * q], l[4 * q + 1], l[4 * q + 2], l[4 * q + 3]);
+        }
+#pragma unroll
+        for (uint32_t k = 0; k < 4 * G; ++k) {
+            scatter_successors<Cfg>(sm, u[k]);
+            scatter_successors<Cfg>(sm, l[k]);
+        }
+        // a group is the upper or the lower switches of two threads: one of them takes its ruler in the upper one,
+        // the other in the lower one
+        const uint32_t slot = fused_slot<Cfg::kSpacing>(tid >> 1, uint32_t(level) + 1u);
+        ruler = place_ruler<Cfg>(sm, (((slot / (4 * G)) ^ tid) & 1u ? sl : su) + slot % (4 * G));
+        __syncthreads();
     }
-    if (logs == 7) {
-        for (uint32_t r = tid; r < C / 128; r += T) {
-            uint32_t col[2];
-            loop_region<7>(sm + pcur + 128 * r, sm + Cfg::kQ + 128 * r, smask, col);
-            at<uint2>(sm, Cfg::kCw + 8 * r) = make_uint2(col[0], col[1]);
+}
+
+// ---- a level with 8-bit entries ----------------------------------------------------------
+// The looping algorithm: ascending start switches, every output it stands on goes up.  In sub-blocks of 2^7 and 2^8 hops
+// come in rounds, and only at the end of one a lane whose loop has closed goes on with the next (it went round its
+// loop again meanwhile and noted what it had noted): what is done once a round need not be done with every hop.
+constexpr int kLoopHops = 3;
+
+// The 2^8 outputs whose successors start at N.  The mark of a switch, 2 + the colour of its even output, says that it has
+// been seen; marks are clear at first.  The next start, the smallest switch without a mark, is looked up eight marks at a
+// time beside the hops of a round, and not taken if this round has seen it.  A hop is a load, a store and
+// eight instructions (with the set of seen switches and its smallest gap in registers it was 36, and they, not the
+// load, were what a hop took: 114 cycles alone and 186 with two warps on a scheduler, now 88).
+__device__ __forceinline__ void loop_marks(const unsigned char *N, unsigned char *marks) {
+    constexpr uint32_t kSw = 128;
+    uint32_t j = 0, start = 0, from = 0, seen = 0;
+    bool idle = false;                         // the loop has closed, and there was no next one to take
+    for (uint32_t round = 0; round < 3u * kSw; ++round) {
+        uint32_t t[kLoopHops];
+        bool closed = idle;
+        uint2 x;
+#pragma unroll
+        for (int k = 0; k < kLoopHops; ++k) {
+            const uint32_t next = N[j];
+            t[k] = j >> 1;
+            marks[t[k]] = uint8_t(2u + (j & 1u));
+            if (k == 0) x = *reinterpret_cast<const uint2 *>(marks + from);
+            seen += closed ? 0u : 1u;
+            closed |= next == start;
+            j = next;
         }
-    } else if (logs == 6) {
-        for (uint32_t r = tid; r < C / 64; r += T) {
-            uint32_t col[1];
-            loop_region<6>(sm + pcur + 64 * r, sm + Cfg::kQ + 64 * r, smask, col);
-            at<uint32_t>(sm, Cfg::kCw + 4 * r) = col[0];
+        const uint32_t y0 = ~x.x & 0x02020202u, y1 = ~x.y & 0x02020202u, y = y0 ? y0 : y1;
+        const uint32_t fresh = from + (y0 ? 0u : 4u) + (uint32_t(__ffs(int(y))) >> 3);
+        bool take = closed && y != 0u;
+#pragma unroll
+        for (int k = 1; k < kLoopHops; ++k) take = take && t[k] != fresh;
+        idle = closed && !take;
+        from = y ? from : min(from + 8u, kSw - 8u);
+        start = take ? 2u * fresh : start;
+        j = take ? 2u * fresh : j;
+        if (__all_sync(~0u, seen >= kSw)) break;
+    }
+}
+
+// A sub-block of 2^7.  Bit sets run from the top bit down, so that the smallest gap is one count of leading ones.
+__device__ __forceinline__ uint2 loop_128(const unsigned char *N) {
+    uint32_t seen0 = 0, seen1 = 0, col0 = 0, col1 = 0, j = 0, start = 0;
+    for (uint32_t round = 0; round < 64u; ++round) {
+        bool closed = false;
+#pragma unroll
+        for (int k = 0; k < kLoopHops; ++k) {
+            const uint32_t next = N[j] & 127u;                 // (places that nobody has written)
+            const uint32_t bit = 0x80000000u >> ((j >> 1) & 31u), odd = (j & 1u) ? bit : 0u;
+            if (j >= 64u) {
+                seen1 |= bit;
+                col1 |= odd;
+            } else {
+                seen0 |= bit;
+                col0 |= odd;
+            }
+            closed |= next == start;
+            j = next;
         }
-    } else {
-        for (uint32_t r = tid; r < C / 32; r += T) {
-            uint32_t col[1];
-            loop_region<5>(sm + pcur + 32 * r, sm + Cfg::kQ + 32 * r, smask, col);
-            at<uint16_t>(sm, Cfg::kCw + 2 * r) = uint16_t(col[0]);
+        const bool full0 = seen0 == ~0u;
+        if (closed) start = j = ((full0 ? 64u : 0u) + 2u * uint32_t(__clz(int(~(full0 ? seen1 : seen0))))) & 127u;
+        if (__all_sync(~0u, (seen0 & seen1) == ~0u)) break;
+    }
+    return make_uint2(__brev(col0), __brev(col1));
+}
+
+// The 2^LOGREG outputs whose successors start at N: a sub-block of 2^6 or 2^5, or the two sub-blocks of 16 of a region
+// of 32.  One visit per switch: a look for the next start with every hop costs less than the hops that rounds waste here.
+template <int LOGREG>
+__device__ __forceinline__ uint32_t loop_region(const unsigned char *N, uint32_t smask) {
+    constexpr uint32_t kReg = 1u << LOGREG, kSw = kReg / 2;
+    uint32_t seen = 0, col = 0, j = 0, start = 0;
+#pragma unroll 4
+    for (uint32_t it = 0; it < kSw; ++it) {
+        uint32_t next = N[j] & smask;
+        if (LOGREG == 5) next |= j & ~smask;                   // (entries are local to sub-blocks of 16 or 32)
+        const uint32_t bit = 0x80000000u >> (j >> 1);
+        seen |= bit;
+        col |= (j & 1u) ? bit : 0u;
+        const bool closed = next == start;
+        start = closed ? (2u * uint32_t(__clz(int(~seen)))) & (kReg - 1u) : start;
+        j = closed ? start : next;
+    }
+    return __brev(col);
+}
+
+// `q8` is the buffer (0 or 1) of the inverse; the next level's goes to the other one, or, below 16, its P.
+template <class Cfg, int LOGS>
+__device__ __forceinline__ void level8(unsigned char *sm, const FusedOut &out, uint32_t q8) {
+    constexpr uint32_t C = Cfg::C, T = Cfg::T, S = 1u << LOGS, H = S >> 1;
+    constexpr int kReg = LOGS > 5 ? LOGS : 5;
+    const uint32_t tid = threadIdx.x;
+    const int level = out.n - LOGS;
+    constexpr uint32_t kRegions = C >> kReg;
+    const uint32_t q_from = Cfg::kQ + q8 * C, q_to = Cfg::kQ + (q8 ^ 1u) * C;
+    // (whole warps: lanes without a sub-block repeat the last one.  With few sub-blocks it is the first warps that have one:
+    // an SM's warps are bound to its four schedulers, warp w of its k-th CTA to scheduler (w + k) % 4)
+    for (uint32_t r0 = tid & ~31u; r0 < kRegions; r0 += T) {
+        const uint32_t r = min(r0 + tid % 32u, kRegions - 1u);
+        if (LOGS == 8) {
+            loop_marks(sm + (r << kReg), sm + Cfg::kMarks + r * kMarkStride);
+            continue;
         }
+        if (LOGS == 7) {
+            at<uint2>(sm, Cfg::kCw + 8u * r) = loop_128(sm + (r << kReg));
+            continue;
+        }
+        const uint32_t col = loop_region<LOGS == 6 ? 6 : 5>(sm + (r << kReg), S - 1u);
+        if (LOGS == 6) at<uint32_t>(sm, Cfg::kCw + 4u * r) = col;
+        else at<uint16_t>(sm, Cfg::kCw + 2u * r) = uint16_t(col);
     }
     __syncthreads();
-    // next level's entries and, unless the tables take over, their inverse
-    const uint32_t pnext = pcur ^ C;
-    const uint32_t vmask = (H - 1u) * 0x01010101u;
-    const bool inverse = logs - 1 >= 4;
     for (uint32_t g = tid; g < C / 16; g += T) {
-        const uint4 p4 = at<uint4>(sm, pcur + 16 * g);
-        uint32_t y[4] = {p4.x, p4.y, p4.z, p4.w};
-        const uint32_t byte = at<uint8_t>(sm, Cfg::kCw + g);
+        const uint4 q4 = at<uint4>(sm, q_from + 16u * g);
+        const uint32_t q[4] = {q4.x, q4.y, q4.z, q4.w};
+        const uint32_t sb = (16u * g) & ~(S - 1u), tl = (16u * g - sb) >> 1;
+        const uint32_t own = Cfg::kMarks + (g >> 4) * kMarkStride;
+        uint32_t in = 0, out8, y[4], word = 0;
+        if (LOGS <= 6) word = at<uint32_t>(sm, Cfg::kCw + ((sb >> 4) & ~3u)) >> ((sb >> 1) & 31u);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) y[k] = ((y[k] >> 1) & vmask) | ((y[k] << 7) & 0x80808080u);
-        const uint32_t s0 = 0x6420u | spread4(byte & 15u), s1 = 0x6420u | spread4(byte >> 4);
-        const uint32_t sb = (16u * g) & ~smask, tl = (16u * g - sb) >> 1;
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t v = q[k >> 1] >> (16 * (k & 1));              // Q[2 s] in the low byte
+            if (LOGS == 8) {
+                in |= ((at<uint8_t>(sm, own + ((v >> 1) & 127u)) ^ v) & 1u) << k;
+            } else {
+                if (LOGS > 6) word = at<uint32_t>(sm, Cfg::kCw + (sb >> 4) + ((v >> 4) & (S / 16 - 4)));
+                in |= ((__funnelshift_r(word, word, v >> 1) ^ v) & 1u) << k;
+            }
+        }
+        if (LOGS == 8) {
+            const uint2 m8 = at<uint2>(sm, own + tl);
+            out8 = tops_of_bytes(m8.x << 7) | (tops_of_bytes(m8.y << 7) << 4);
+        } else {
+            out8 = at<uint8_t>(sm, Cfg::kCw + g);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) y[k] = (q[k] >> 1) & ((H - 1u) * 0x01010101u);
+        const uint32_t s0 = 0x6420u | spread4(in & 15u), s1 = 0x6420u | spread4(in >> 4);
         const uint32_t e[2][2] = {{__byte_perm(y[0], y[1], s0), __byte_perm(y[2], y[3], s1)},
                                   {__byte_perm(y[0], y[1], s0 ^ 0x1111u), __byte_perm(y[2], y[3], s1 ^ 0x1111u)}};
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
             const uint32_t base = sb + (half ? H : 0u);
-            at<uint2>(sm, pnext + base + tl) = make_uint2(e[half][0], e[half][1]);
-            if (inverse) {
+            if (LOGS > 4) {
+                at<uint2>(sm, q_to + base + tl) = make_uint2(e[half][0], e[half][1]);
+                scatter_successors8(sm, base, e[half][0], e[half][1]);
+            } else {
+                // the tables want P
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const uint32_t x = e[half][k >> 2] >> (8 * (k & 3));
-                    at<uint8_t>(sm, Cfg::kQ + base + (x & (H - 1u))) = uint8_t((x & 0x80u) | (tl + uint32_t(k)));
-                }
+                for (int k = 0; k < 8; ++k)
+                    at<uint8_t>(sm, q_to + base + ((e[half][k >> 2] >> (8 * (k & 3))) & 7u)) = uint8_t(k);
             }
         }
+        if (out.n >= 6) {
+            if (16u * g < out.valid) {
+                *stage_byte(out, level, g) = uint8_t(in);
+                *stage_byte(out, 2 * out.n - 2 - level, g) = uint8_t(out8);
+            }
+        } else {
+            at<uint8_t>(sm, Cfg::kInw + g) = uint8_t(in);
+        }
     }
-    if (!first) out.store_row<Cfg>(sm, Cfg::kInw, level - 1);
-    out.store_row<Cfg>(sm, Cfg::kCw, 2 * out.n - 2 - level);
     __syncthreads();
+    if (out.n < 6) {
+        for (uint32_t r = tid; r < C / 32; r += T) {
+            out.store16(level, r, at<uint16_t>(sm, Cfg::kInw + 2u * r));
+            out.store16(2 * out.n - 2 - level, r, at<uint16_t>(sm, Cfg::kCw + 2u * r));
+        }
+        __syncthreads();
+    }
 }
 
 // ---- sub-blocks of 8 and less: 32 outputs (16 switches of every stage) per thread ----------
 template <class Cfg>
-__device__ __forceinline__ void last_levels(unsigned char *sm, const FusedOut &out, int logs, uint32_t pcur,
-                                            bool first) {
-    constexpr uint32_t C = Cfg::C, T = Cfg::T;
+__device__ __forceinline__ void last_levels(unsigned char *sm, const FusedOut &out, int logs, uint32_t q8) {
     const int n = out.n;
-    const uint32_t *lut8 = &at<uint32_t>(sm, Cfg::kN), *lut4 = lut8 + kLut8Words;
-    for (uint32_t r = threadIdx.x; r < C / 32; r += T) {
-        const uint4 a = at<uint4>(sm, pcur + 32 * r), b = at<uint4>(sm, pcur + 32 * r + 16);
+    const uint32_t p8 = Cfg::kQ + q8 * Cfg::C;
+    const uint32_t *lut8 = &at<uint32_t>(sm, Cfg::kTables), *lut4 = lut8 + kLut8Words;
+    for (uint32_t r = threadIdx.x; r < Cfg::C / 32; r += Cfg::T) {
+        const uint4 a = at<uint4>(sm, p8 + 32 * r), b = at<uint4>(sm, p8 + 32 * r + 16);
         const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
         if (logs == 1) {
             uint32_t mid = 0;
@@ -619,18 +692,10 @@ __device__ __forceinline__ void last_levels(unsigned char *sm, const FusedOut &o
                 z4[k] = (lut4[fields_of_bytes(w[2 * k] & 0x03030303u)] >> 16) |
                         ((lut4[fields_of_bytes(w[2 * k + 1] & 0x03030303u)] >> 16) << 2);
         } else {
-            uint32_t in16 = 0, out8 = 0, in8 = 0;
+            uint32_t out8 = 0, in8 = 0;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const uint32_t w0 = w[2 * k], w1 = w[2 * k + 1];
-                if ((k & 1) == 0 && !first) {
-                    // input side of the level of 16: parity at the place of the value
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const uint32_t x = (e < 4 ? w0 : w1) >> (8 * (e & 3));
-                        in16 |= ((x >> 7) & 1u) << ((x & 7u) + 4u * uint32_t(k));
-                    }
-                }
                 const uint32_t x0 = (w0 >> 1) & 0x03030303u, x1 = (w1 >> 1) & 0x03030303u;
                 const uint32_t idx = (fields_of_bytes(x0) << 6) | (fields_of_bytes(x1) >> 2);
                 const uint32_t c = (lut8[idx >> 3] >> (4u * (idx & 7u))) & 15u;
@@ -643,7 +708,6 @@ __device__ __forceinline__ void last_levels(unsigned char *sm, const FusedOut &o
                 in8 |= tops_of_bytes(__byte_perm(up, 0u, eu & 0x3333u)) << (4 * k);
                 z4[k] = (eu >> 16) | ((el >> 16) << 2);
             }
-            if (!first) out.store16(n - 4, r, in16);
             out.store16(2 * n - 2 - (n - 3), r, out8);
             out.store16(n - 3, r, in8);
         }
@@ -660,34 +724,41 @@ __device__ __forceinline__ void last_levels(unsigned char *sm, const FusedOut &o
     }
 }
 
-// Levels n - logs .. n - 1 of the CTA's outputs; P and Q of the first of them are in place.
+// The 8-bit levels from sub-blocks of 2^logs on; their entries (P, for sub-blocks of 8 and less) are in place.
 template <class Cfg>
-__device__ __forceinline__ void fused_levels(unsigned char *sm, const FusedOut &out, int logs0) {
-    const int n = out.n;
-    int logs = logs0;
-    for (; logs >= kFMinLogS; --logs) level16<Cfg>(sm, out, logs, n - logs, logs == logs0);
-    for (uint32_t i = threadIdx.x; i < uint32_t(kLutBytes / 16); i += Cfg::T)
-        at<uint4>(sm, Cfg::kN + 16 * i) = __ldg(reinterpret_cast<const uint4 *>(&g_fused_tables) + i);
-    uint32_t pcur = 0;
-    for (; logs >= 4; --logs) {
-        level8<Cfg>(sm, out, logs, n - logs, logs == logs0, pcur);
-        pcur ^= uint32_t(Cfg::C);
-    }
-    if (logs == logs0) __syncthreads();        // no level above the tables: they have just been copied
-    last_levels<Cfg>(sm, out, logs, pcur, logs == logs0);
+__device__ __forceinline__ void levels8(unsigned char *sm, const FusedOut &out, int logs) {
+    uint32_t q8 = 0;
+    if (logs == 8) { level8<Cfg, 8>(sm, out, q8); q8 ^= 1u; --logs; }
+    if (logs == 7) { level8<Cfg, 7>(sm, out, q8); q8 ^= 1u; --logs; }
+    if (logs == 6) { level8<Cfg, 6>(sm, out, q8); q8 ^= 1u; --logs; }
+    if (logs == 5) { level8<Cfg, 5>(sm, out, q8); q8 ^= 1u; --logs; }
+    if (logs == 4) { level8<Cfg, 4>(sm, out, q8); q8 ^= 1u; --logs; }
+    last_levels<Cfg>(sm, out, logs, q8);
 }
 
-// P and Q of the first level from four neighbouring values, local to their sub-block
 template <class Cfg>
-__device__ __forceinline__ void fused_enter4(unsigned char *sm, uint32_t i4, const uint32_t v[4], int logs) {
-    const uint32_t smask = (1u << logs) - 1u;
+__device__ __forceinline__ void copy_tables(unsigned char *sm) {
+    for (uint32_t i = threadIdx.x; i < uint32_t(kLutBytes / 16); i += Cfg::T)
+        at<uint4>(sm, Cfg::kTables + 16 * i) = __ldg(reinterpret_cast<const uint4 *>(&g_fused_tables) + i);
+}
+
+// Four neighbouring values: 16-bit entries of the inverse in input order at the start of the shared memory, 8-bit ones
+// in the first buffer (of the permutation, for sub-blocks of 8 and less).
+template <class Cfg>
+__device__ __forceinline__ void enter4(unsigned char *sm, uint32_t i4, const uint32_t v[4], bool inverse, int logs) {
+    const uint32_t smask = (1u << logs) - 1u, sb = (4u * i4) & ~smask;
     if (logs >= kFMinLogS) {
-        const uint32_t sb = (4u * i4) & ~smask;
-        at<uint2>(sm, 8 * i4) = make_uint2(2u * (sb + v[0]) | (2u * (sb + v[1]) << 16), 2u * (sb + v[2]) | (2u * (sb + v[3]) << 16));
+        if (inverse) {
+            at<uint2>(sm, 8u * i4) = make_uint2(2u * (sb + v[0]) | (2u * (sb + v[1]) << 16), 2u * (sb + v[2]) | (2u * (sb + v[3]) << 16));
+        } else {
 #pragma unroll
-        for (uint32_t k = 0; k < 4; ++k) at<uint16_t>(sm, Cfg::kQ + 2u * (sb + v[k])) = uint16_t(2u * (4u * i4 + k));
+            for (uint32_t k = 0; k < 4; ++k) at<uint16_t>(sm, 2u * (sb + v[k])) = uint16_t(2u * (4u * i4 + k));
+        }
+        return;
+    }
+    if (logs < 4) {
+        at<uint32_t>(sm, Cfg::kQ + 4u * i4) = v[0] | (v[1] << 8) | (v[2] << 16) | (v[3] << 24);
     } else {
-        at<uint32_t>(sm, 4 * i4) = v[0] | (v[1] << 8) | (v[2] << 16) | (v[3] << 24);
 #pragma unroll
         for (uint32_t k = 0; k < 4; ++k) {
             const uint32_t i = 4u * i4 + k;
@@ -696,52 +767,106 @@ __device__ __forceinline__ void fused_enter4(unsigned char *sm, uint32_t i4, con
     }
 }
 
-// The CTA's blocks of 2^logs outputs from a plain array (records = 0) or from packed records
-// P[2t] | P[2t+1] << logs | ... (1), four entries per load, four loads of a thread under way together.
+// The first level's entries from an array of 32-bit values of the CTA's blocks, local to their blocks of 2^logs: the
+// permutation, or its inverse.  Four values per load, four loads of a thread under way together.
 template <class Cfg>
-__device__ __forceinline__ void fused_load(unsigned char *sm, const FusedOut &out, const uint32_t *P, int records, int logs) {
-    constexpr uint32_t T = Cfg::T, kItems = Cfg::C / 4, kBatch = kItems / T >= 4 ? 4 : 1;
+__device__ __forceinline__ void fused_load(unsigned char *sm, const FusedOut &out, const uint32_t *src, bool inverse, int logs) {
+    constexpr uint32_t T = Cfg::T, kItems = Cfg::C / 4, kBatch = 4;
     const uint32_t smask = (1u << logs) - 1u;
-    const bool aligned = (reinterpret_cast<uintptr_t>(P) & 15u) == 0;
+    const bool aligned = (reinterpret_cast<uintptr_t>(src) & 15u) == 0;
+    if (!inverse && logs >= kFMinLogS) {
+        // (an input that is no permutation leaves places nobody writes; from here on the successor array holds
+        // nothing but places in it and codes)
+        for (uint32_t i = threadIdx.x; i < Cfg::C / 8; i += T) at<uint4>(sm, 16u * i) = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+    }
     for (uint32_t i0 = threadIdx.x; i0 < kItems; i0 += kBatch * T) {
         uint32_t v[kBatch][4];
 #pragma unroll
         for (uint32_t r = 0; r < kBatch; ++r) {
             const uint32_t i4 = i0 + r * T;
             const size_t f = out.flat0 + 4u * i4;
-            if (4u * i4 + 4u <= out.valid && (records != 0 || aligned)) {
-                if (records == 0) {
-                    const uint4 p = __ldcs(reinterpret_cast<const uint4 *>(P + f));
-                    v[r][0] = p.x; v[r][1] = p.y; v[r][2] = p.z; v[r][3] = p.w;
-                } else {
-                    const ulonglong2 p = __ldcs(reinterpret_cast<const ulonglong2 *>(P) + (f >> 2));
-                    v[r][0] = uint32_t(p.x) & smask; v[r][1] = uint32_t(p.x >> logs) & smask;
-                    v[r][2] = uint32_t(p.y) & smask; v[r][3] = uint32_t(p.y >> logs) & smask;
-                }
+            if (4u * i4 + 4u <= out.valid && aligned) {
+                const uint4 p = __ldcs(reinterpret_cast<const uint4 *>(src + f));
+                v[r][0] = p.x; v[r][1] = p.y; v[r][2] = p.z; v[r][3] = p.w;
             } else {
                 // a permutation that does not start on 16 bytes, the end of a batch of permutations of 2,
                 // or padding: the identity
 #pragma unroll
-                for (uint32_t k = 0; k < 4; ++k)
-                    v[r][k] = (records == 0 && 4u * i4 + k < out.valid) ? P[f + k] : (4u * i4 + k) & smask;
+                for (uint32_t k = 0; k < 4; ++k) v[r][k] = 4u * i4 + k < out.valid ? src[f + k] : (4u * i4 + k) & smask;
             }
         }
 #pragma unroll
         for (uint32_t r = 0; r < kBatch; ++r) {
 #pragma unroll
             for (uint32_t k = 0; k < 4; ++k) v[r][k] = BENES_GUARD(v[r][k], smask);
-            fused_enter4<Cfg>(sm, i0 + r * T, v[r], logs);
+            enter4<Cfg>(sm, i0 + r * T, v[r], inverse, logs);
         }
     }
     __syncthreads();
 }
 
-template <int LOGC, int THREADS>
-__global__ void __launch_bounds__(THREADS, (FusedCfg<LOGC, THREADS>::kMinCtas))
-k_route_fused(const uint32_t *__restrict__ P, int records, uint32_t *__restrict__ bits, int log2n, int logs,
-              size_t first, size_t end, const uint32_t *__restrict__ gate, const uint32_t *__restrict__ redone) {
+// From the entries of enter4 (complete: a barrier lies between) to the places and successors of the first level.
+template <class Cfg>
+__device__ __forceinline__ void start16(unsigned char *sm, int logs, int level, Ruler &ruler) {
+    constexpr uint32_t G = Cfg::G;
+    const uint32_t tid = threadIdx.x, first = 8u * G * tid;
+    // (whatever the entries of an input that is no permutation hold: they stay in their block)
+    const uint32_t local = (2u << logs) - 2u, keep = local * 0x10001u, base = ((32u * G * tid) & ~(local + 1u)) * 0x10001u;
+    uint32_t x[8 * G];
+#pragma unroll
+    for (uint32_t q = 0; q < 2 * G; ++q) {
+        const uint4 w = at<uint4>(sm, 4u * first + 16u * q);
+        x[4 * q] = w.x; x[4 * q + 1] = w.y; x[4 * q + 2] = w.z; x[4 * q + 3] = w.w;
+    }
+    __syncthreads();
+#pragma unroll
+    for (uint32_t k = 0; k < 8 * G; ++k) x[k] = (x[k] & keep) | base;
+#pragma unroll
+    for (uint32_t q = 0; q < 2 * G; ++q)
+        at<uint4>(sm, q_place<Cfg>(first + 4u * q)) = make_uint4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
+#pragma unroll
+    for (uint32_t k = 0; k < 8 * G; ++k) scatter_successors<Cfg>(sm, x[k]);
+    ruler = place_ruler<Cfg>(sm, first + fused_slot<Cfg::kSpacing>(tid, uint32_t(level)));
+    __syncthreads();
+}
+template <class Cfg>
+__device__ __forceinline__ void start8(unsigned char *sm, int logs) {
+    const uint32_t smask = (1u << logs) - 1u;
+    if (logs == 8) clear_marks<Cfg>(sm);
+    for (uint32_t g = threadIdx.x; g < Cfg::C / 16; g += Cfg::T) {
+        uint4 q = at<uint4>(sm, Cfg::kQ + 16u * g);
+        const uint32_t keep = smask * 0x01010101u;
+        q.x &= keep; q.y &= keep; q.z &= keep; q.w &= keep;
+        at<uint4>(sm, Cfg::kQ + 16u * g) = q;
+        const uint32_t n8 = (16u * g) & ~smask;
+        scatter_successors8(sm, n8, q.x, q.y);
+        scatter_successors8(sm, n8, q.z, q.w);
+    }
+    __syncthreads();
+}
+
+// All levels of the CTA's blocks of 2^logs outputs; enter4 has been called for every entry, and a barrier passed.
+template <class Cfg>
+__device__ __forceinline__ void fused_levels(unsigned char *sm, const FusedOut &out, int logs) {
+    if (logs >= kFMinLogS) {
+        Ruler ruler;
+        start16<Cfg>(sm, logs, out.n - logs, ruler);
+        levels16<Cfg>(sm, out, logs, ruler);
+        logs = kFMinLogS - 1;
+    } else if (logs >= 4) {
+        start8<Cfg>(sm, logs);
+    }
+    copy_tables<Cfg>(sm);
+    if (logs < 4) __syncthreads();
+    levels8<Cfg>(sm, out, logs);
+}
+
+template <class Cfg>
+__global__ void __launch_bounds__(Cfg::T, Cfg::kMinCtas)
+k_route_fused(const uint32_t *__restrict__ src, bool inverse, uint32_t *__restrict__ bits, int log2n, int logs,
+              size_t first, size_t end) {
     after_previous_kernel();
-    using Cfg = FusedCfg<LOGC, THREADS>;
     constexpr uint32_t C = Cfg::C;
     extern __shared__ __align__(16) unsigned char sm[];
     FusedOut out;
@@ -749,41 +874,44 @@ k_route_fused(const uint32_t *__restrict__ P, int records, uint32_t *__restrict_
     out.n = log2n;
     out.flat0 = first + size_t(blockIdx.x) * C;
     out.valid = uint32_t(end - out.flat0 < size_t(C) ? end - out.flat0 : size_t(C));
-    const bool redo = gate && *gate != 0u;
-    fused_load<Cfg>(sm, out, redo ? redone : P, redo ? 0 : records, logs);
+    fused_load<Cfg>(sm, out, src, inverse, logs);
     fused_levels<Cfg>(sm, out, logs);
 }
 
-// One level of one block of 2^LOGC outputs per CTA; the two half-blocks go to `next` (a plain array), where the
+// One level of one block of 2^LOGC outputs per CTA; the inverses of the two half-blocks go to `next`, where the
 // next launch finds them with twice as many CTAs.  While more than half of the SMs would have no block, that is how the
 // in-CTA levels run: a level takes a time in proportion to the CTA's outputs, so halving the block with every level
 // costs about two levels of the first block instead of one for each (one block of 2^15: 172 -> 82 us,
 // 2^13: 51 -> 37; the route of 2^16: 206 -> 140, of 2^20: 545 -> 497).
-template <int LOGC, int THREADS>
-__global__ void __launch_bounds__(THREADS)
-k_route_peel(const uint32_t *__restrict__ P, int records, uint32_t *__restrict__ bits, int log2n,
-             uint32_t *__restrict__ next, const uint32_t *__restrict__ gate, const uint32_t *__restrict__ redone) {
+template <class Cfg>
+__global__ void __launch_bounds__(Cfg::T, 1)
+k_route_peel(const uint32_t *__restrict__ src, bool inverse, uint32_t *__restrict__ bits, int log2n, uint32_t *__restrict__ next) {
     after_previous_kernel();
-    using Cfg = FusedCfg<LOGC, THREADS>;
-    constexpr uint32_t C = Cfg::C, T = Cfg::T, H = C / 2;
+    constexpr uint32_t C = Cfg::C, G = Cfg::G, H = C / 2;
+    constexpr int logs = Cfg::LOG;
     extern __shared__ __align__(16) unsigned char sm[];
     FusedOut out;
     out.bits = bits;
     out.n = log2n;
     out.flat0 = size_t(blockIdx.x) * C;
     out.valid = C;
-    const bool redo = gate && *gate != 0u;
-    fused_load<Cfg>(sm, out, redo ? redone : P, redo ? 0 : records, LOGC);
-    level16<Cfg>(sm, out, LOGC, log2n - LOGC, true);
-    // entries 2 (base of the half + value) | parity -> values; input-side bits from the inverse of the upper half
-    for (uint32_t i4 = threadIdx.x; i4 < C / 4; i4 += T) {
-        const uint2 e = at<uint2>(sm, 8 * i4);
-        const uint32_t x = (e.x >> 1) & ((H - 1u) * 0x10001u), y = (e.y >> 1) & ((H - 1u) * 0x10001u);
-        *reinterpret_cast<uint4 *>(next + out.flat0 + 4u * i4) = make_uint4(x & 0xFFFFu, x >> 16, y & 0xFFFFu, y >> 16);
+    fused_load<Cfg>(sm, out, src, inverse, logs);
+    Ruler ruler;
+    start16<Cfg>(sm, logs, log2n - logs, ruler);
+    colours16<Cfg>(sm, logs, ruler);
+    uint32_t u[4 * G], l[4 * G];
+    split16<Cfg>(sm, out, logs, log2n - logs, true, u, l);
+    // pairs of entries 2 (half-block + value) -> values
+#pragma unroll
+    for (uint32_t q = 0; q < 2 * G; ++q) {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const uint32_t *e = half ? l : u;
+            const uint32_t x = (e[2 * q] >> 1) & ((H - 1u) * 0x10001u), y = (e[2 * q + 1] >> 1) & ((H - 1u) * 0x10001u);
+            *reinterpret_cast<uint4 *>(next + out.flat0 + half * H + 8u * G * threadIdx.x + 4u * q) =
+                make_uint4(x & 0xFFFFu, x >> 16, y & 0xFFFFu, y >> 16);
+        }
     }
-    input_bits16<Cfg>(sm, LOGC - 1);
-    __syncthreads();
-    out.store_row<Cfg>(sm, Cfg::kInw, log2n - LOGC);
 }
 
 // ---- few outputs in all ---------------------------------------------------------------------
@@ -839,7 +967,7 @@ __device__ __forceinline__ void few_tail32(uint32_t p, uint32_t r, uint16_t *Q, 
 
 template <int LOGC>
 __global__ void __launch_bounds__((1 << LOGC) / 2)
-k_route_few(const uint32_t *__restrict__ P, uint32_t *__restrict__ bits, int n, int logs, size_t total) {
+k_route_few(const uint32_t *__restrict__ src, bool inverse, uint32_t *__restrict__ bits, int n, int logs, size_t total) {
     after_previous_kernel();
     constexpr uint32_t C = 1u << LOGC, kAll = 0xFFFFFFFFu;
     __shared__ uint32_t W[C];                  // (minimum << 16 | next) of every output
@@ -855,8 +983,17 @@ k_route_few(const uint32_t *__restrict__ P, uint32_t *__restrict__ bits, int n, 
     const uint32_t block = (1u << logs) - 1u;
     uint32_t p0 = j & block, p1 = (j + 1u) & block;            // padding: the identity
     if (j < out.valid) {                                       // (valid is even)
-        p0 = BENES_GUARD(P[out.flat0 + j], block);
-        p1 = BENES_GUARD(P[out.flat0 + j + 1], block);
+        p0 = BENES_GUARD(src[out.flat0 + j], block);
+        p1 = BENES_GUARD(src[out.flat0 + j + 1], block);
+    }
+    if (inverse) {                             // (blocks of 2^11 that k_route_peel has made)
+        const uint32_t sb = j & ~block;
+        Pn[sb + p0] = uint16_t(j & block);
+        Pn[sb + p1] = uint16_t((j + 1u) & block);
+        __syncthreads();
+        const uint32_t pp = Pn32[t];
+        p0 = pp & block;
+        p1 = (pp >> 16) & block;
     }
     for (; logs > 6; --logs) {
         const int level = n - logs;
@@ -934,8 +1071,8 @@ k_route_few(const uint32_t *__restrict__ P, uint32_t *__restrict__ bits, int n, 
 }
 
 template <int LOGC>
-int launch_few(const uint32_t *P, size_t total, uint32_t *bits, int n, int logs, cudaStream_t s) {
-    launch_kernel(k_route_few<LOGC>, unsigned((total + (size_t(1) << LOGC) - 1) >> LOGC), (1 << LOGC) / 2, 0, s, P, bits, n, logs, total);
+int launch_few(const uint32_t *src, bool inverse, size_t total, uint32_t *bits, int n, int logs, cudaStream_t s) {
+    launch_kernel(k_route_few<LOGC>, unsigned((total + (size_t(1) << LOGC) - 1) >> LOGC), (1 << LOGC) / 2, 0, s, src, inverse, bits, n, logs, total);
     return launch_status();
 }
 
@@ -960,24 +1097,21 @@ struct Pair2 {                       // the same array in the two CTAs of the cl
 
 // The layout of the level that spans both CTAs (P 2M, Q 2M, colour words, the next P 2M + the
 // part of the scratch that does not fit there); the levels below use FusedCfg's.
-using ClusterTailCfg = FusedCfg<kFusedLog2M, 1024>;
-constexpr size_t kClusterTopBytes = size_t(ClusterTailCfg::C) * 6 + ClusterTailCfg::C / 16 + size_t(ClusterTailCfg::kRulers) * 2 + 16;
+using ClusterTailCfg = FusedCfg<kFusedLog2M, 2>;
+constexpr int kClusterKappa = 3;                // ruler spacing (log2) of that level
+constexpr uint32_t kNone16 = 0xFFFFu;          // owner of a switch nobody claimed
+constexpr size_t kClusterTopBytes = size_t(ClusterTailCfg::C) * 6 + ClusterTailCfg::C / 16 + (size_t(ClusterTailCfg::C) >> kClusterKappa) * 2 + 16;
 constexpr size_t kClusterSmemBytes = kClusterTopBytes > ClusterTailCfg::kSmemBytes ? kClusterTopBytes : ClusterTailCfg::kSmemBytes;
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(ClusterTailCfg::T)
-k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restrict__ bits, int log2n,
-                 uint32_t block0, const uint32_t *__restrict__ gate, const uint32_t *__restrict__ redone) {
+k_route_cluster2(const uint32_t *__restrict__ src, bool inverse, uint32_t *__restrict__ bits, int log2n, uint32_t block0) {
     after_previous_kernel();
-    if (gate && *gate != 0u) {
-        P = redone;
-        records = 0;
-    }
     constexpr int LOGM = kFusedLog2M;           // per CTA
     using Cfg = ClusterTailCfg;
-    constexpr int M = Cfg::C;                      // outputs per CTA
-    constexpr int T = Cfg::T;
-    constexpr int R = Cfg::kRulers;                // ruler outputs per CTA
-    constexpr int LOGR = LOGM - kFKappa;
+    constexpr int M = int(Cfg::C);                      // outputs per CTA
+    constexpr int T = int(Cfg::T);
+    constexpr int R = M >> kClusterKappa;        // ruler outputs per CTA
+    constexpr int LOGR = LOGM - kClusterKappa;
     constexpr uint32_t kInCta = uint32_t(M) - 1u, kSwInCta = uint32_t(M / 2) - 1u, kRInCta = uint32_t(R) - 1u;
     constexpr uint32_t kWordsPerCta = M / 64;    // colour words per CTA
     constexpr uint32_t kBoth = 2u * uint32_t(M) - 1u;
@@ -1019,23 +1153,16 @@ k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restri
     // this CTA's half of the block's words of a stage
     uint32_t *my_bits = bits + perm * size_t(2 * n - 1) * stage_w + (local_first_switch >> 5) + rank * kWordsPerCta;
 
-    for (int j = tid; j < M; j += T) {
-        const size_t f = flat0 + rank * uint32_t(M) + j;
-        uint32_t v;
-        if (records) {
-            const unsigned long long w = reinterpret_cast<const unsigned long long *>(P)[f >> 1];
-            v = uint32_t(w >> ((f & 1) ? kClusterLog2M : 0)) & kBoth;
-        } else {
-            v = P[f];
-        }
-        Pa[j] = uint16_t(BENES_GUARD(v, kBoth));
-    }
+    // what is given stays with the CTA: the permutation, or its inverse
+    uint16_t *const given = inverse ? Q : Pa;
+    const Pair2<uint16_t> &other = inverse ? Pa2 : Q2;
+    for (int j = tid; j < M; j += T) given[j] = uint16_t(BENES_GUARD(src[flat0 + rank * uint32_t(M) + j], kBoth));
     for (int t = tid; t < M / 2; t += T) own[t] = uint16_t(kNone16);
     cluster.sync();           // both CTAs are running (and loaded) before either touches the other's memory
-    // a1: the inverse goes to the CTA that keeps that input
+    // a1: its inverse goes to the CTA that keeps that place
     for (int j = tid; j < M; j += T) {
-        const uint32_t v = Pa[j];
-        Q2.of(v >> LOGM)[v & kInCta] = uint16_t(rank * uint32_t(M) + j);
+        const uint32_t v = given[j];
+        other.of(v >> LOGM)[v & kInCta] = uint16_t(rank * uint32_t(M) + j);
     }
     cluster.sync();
 
@@ -1044,7 +1171,7 @@ k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restri
     for (int rl = tid; rl < R; rl += T) {
         const uint32_t rho = rank * uint32_t(R) + rl;
         const uint32_t group = rho >> 1, side0 = rho & 1u;
-        const uint32_t t0 = (group << kFKappa) | fused_slot(group, uint32_t(level));
+        const uint32_t t0 = (group << kClusterKappa) | fused_slot<kClusterKappa>(group, uint32_t(level));
         uint32_t j = 2u * t0 + side0;
         uint32_t fwd = j, part = kNone16, pr = rho ^ 1u;
         if (!side0) own[t0 & kSwInCta] = uint16_t(rho << 1);
@@ -1053,8 +1180,8 @@ k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restri
         uint32_t q = Q2.of((p ^ 1u) >> LOGM)[(p ^ 1u) & kInCta];
         for (uint32_t hops = 0; hops <= kBoth; ++hops) {                 // a walk claims < 2^15 switches
             j = q;
-            const uint32_t t = j >> 1, side = j & 1u, g = t >> kFKappa;
-            if ((t & ((1u << kFKappa) - 1u)) == fused_slot(g, uint32_t(level))) {
+            const uint32_t t = j >> 1, side = j & 1u, g = t >> kClusterKappa;
+            if ((t & ((1u << kClusterKappa) - 1u)) == fused_slot<kClusterKappa>(g, uint32_t(level))) {
                 pr = (2u * g + side) ^ 1u;                               // reached the next ruler
                 break;
             }
@@ -1085,7 +1212,7 @@ k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restri
     }
     cluster.sync();
     // in-place pointer jumping; a cycle of the list has at most 2^12 words (half of the ruler outputs)
-    for (int r = 0; r < kClusterLog2M - kFKappa - 1; ++r) {
+    for (int r = 0; r < kClusterLog2M - kClusterKappa - 1; ++r) {
         for (int e = tid; e < R; e += T) {
             const uint32_t w = list[e], nx = w & 0xFFFFu;
             const uint32_t v = list2.of((nx >> LOGR) & 1u)[nx & kRInCta];
@@ -1149,7 +1276,7 @@ k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restri
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kEnter; ++r) fused_enter4<Cfg>(smem_raw, uint32_t(tid + r * T), v[r], LOGM);
+    for (int r = 0; r < kEnter; ++r) enter4<Cfg>(smem_raw, uint32_t(tid + r * T), v[r], false, LOGM);
     __syncthreads();
     FusedOut out;
     out.bits = bits;
@@ -1159,51 +1286,41 @@ k_route_cluster2(const uint32_t *__restrict__ P, int records, uint32_t *__restri
     fused_levels<Cfg>(smem_raw, out, LOGM);
 }
 
-template <int LOGC, int THREADS>
-int configure_one() {
-    using Cfg = FusedCfg<LOGC, THREADS>;
+template <class Cfg>
+int configure_fused() {
     static OncePerDevice configured;
     return configured.run([]() -> int {
-        BENES_CUDA_TRY(cudaFuncSetAttribute(k_route_fused<LOGC, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            int(Cfg::kSmemBytes)));
-        BENES_CUDA_TRY(cudaFuncSetAttribute(k_route_fused<LOGC, THREADS>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        BENES_CUDA_TRY(cudaFuncSetAttribute(k_route_fused<Cfg>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Cfg::kSmemBytes)));
+        BENES_CUDA_TRY(cudaFuncSetAttribute(k_route_fused<Cfg>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                             cudaSharedmemCarveoutMaxShared));
         cudaFuncAttributes loaded;                             // (asking for them loads the kernel)
-        BENES_CUDA_TRY(cudaFuncGetAttributes(&loaded, k_route_fused<LOGC, THREADS>));
+        BENES_CUDA_TRY(cudaFuncGetAttributes(&loaded, k_route_fused<Cfg>));
         return BENES_OK;
     });
 }
 
-template <int LOGC, int THREADS>
-int launch_one(const uint32_t *P, int records, size_t first, size_t end, uint32_t *bits, int log2n, int logs,
-               cudaStream_t s, const uint32_t *gate, const uint32_t *redone) {
-    using Cfg = FusedCfg<LOGC, THREADS>;
-    const int rc = configure_one<LOGC, THREADS>();
+template <class Cfg>
+int launch_one(const uint32_t *src, bool inverse, size_t first, size_t end, uint32_t *bits, int log2n, int logs, cudaStream_t s) {
+    const int rc = configure_fused<Cfg>();
     if (rc) return rc;
-    const size_t ctas = (end - first + Cfg::C - 1) >> LOGC;
-    launch_kernel(k_route_fused<LOGC, THREADS>, unsigned(ctas), THREADS, Cfg::kSmemBytes, s, P, records, bits, log2n, logs, first, end,
-                  gate, redone);
+    const size_t ctas = (end - first + Cfg::C - 1) >> Cfg::LOG;
+    launch_kernel(k_route_fused<Cfg>, unsigned(ctas), Cfg::T, Cfg::kSmemBytes, s, src, inverse, bits, log2n, logs, first, end);
     return launch_status();
 }
 
-template <int LOGC>
-int launch_peel(const uint32_t *P, int records, size_t total, uint32_t *bits, int log2n, uint32_t *next, cudaStream_t s,
-                const uint32_t *gate, const uint32_t *redone) {
-    constexpr int T = 1024;
-    using Cfg = FusedCfg<LOGC, T>;
+template <class Cfg>
+int launch_peel(const uint32_t *src, bool inverse, size_t total, uint32_t *bits, int log2n, uint32_t *next, cudaStream_t s) {
     static OncePerDevice configured;
     const int rc = configured.run([]() -> int {
-        BENES_CUDA_TRY(cudaFuncSetAttribute(k_route_peel<LOGC, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            int(Cfg::kSmemBytes)));
+        BENES_CUDA_TRY(cudaFuncSetAttribute(k_route_peel<Cfg>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Cfg::kSmemBytes)));
         return BENES_OK;
     });
     if (rc) return rc;
-    launch_kernel(k_route_peel<LOGC, T>, unsigned(total >> LOGC), T, Cfg::kSmemBytes, s, P, records, bits, log2n, next, gate, redone);
+    launch_kernel(k_route_peel<Cfg>, unsigned(total >> Cfg::LOG), Cfg::T, Cfg::kSmemBytes, s, src, inverse, bits, log2n, next);
     return launch_status();
 }
 
-int launch_cluster2(const uint32_t *P, int records, size_t first_block, size_t blocks, uint32_t *bits,
-                    int log2n, cudaStream_t s, const uint32_t *gate, const uint32_t *redone) {
+int launch_cluster2(const uint32_t *src, bool inverse, size_t first_block, size_t blocks, uint32_t *bits, int log2n, cudaStream_t s) {
     static OncePerDevice configured;
     const int rc = configured.run([]() -> int {
         BENES_CUDA_TRY(cudaFuncSetAttribute(k_route_cluster2, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1214,47 +1331,44 @@ int launch_cluster2(const uint32_t *P, int records, size_t first_block, size_t b
     });
     if (rc) return rc;
     // two CTAs per block (the cluster size is part of the kernel)
-    launch_kernel(k_route_cluster2, unsigned(2 * blocks), ClusterTailCfg::T, kClusterSmemBytes, s, P, records, bits, log2n,
-                  uint32_t(first_block), gate, redone);
+    launch_kernel(k_route_cluster2, unsigned(2 * blocks), ClusterTailCfg::T, kClusterSmemBytes, s, src, inverse, bits, log2n,
+                  uint32_t(first_block));
     return launch_status();
 }
 
 }  // namespace
 
-int launch_fused(const void *Pv, int records, size_t total, int log2m, uint32_t *bits, int log2n,
-                 cudaStream_t s, size_t first_block, size_t blocks, const uint32_t *gate, const uint32_t *redone,
-                 uint32_t *const spare[2]) {
-    const uint32_t *P = static_cast<const uint32_t *>(Pv);
+int launch_fused(const uint32_t *src, bool inverse, size_t total, int log2m, uint32_t *bits, int log2n,
+                 cudaStream_t s, size_t first_block, size_t blocks, uint32_t *const spare[2]) {
     if (log2m < 1 || log2m > kClusterLog2M) return BENES_ERR_BADARG;
     if (blocks == 0) blocks = (total >> log2m) - first_block;        // all the rest
     if (first_block + blocks > (total >> log2m)) return BENES_ERR_BADARG;
-    if (log2m == kClusterLog2M) return launch_cluster2(P, records, first_block, blocks, bits, log2n, s, gate, redone);
+    if (log2m == kClusterLog2M) return launch_cluster2(src, inverse, first_block, blocks, bits, log2n, s);
     const size_t first = first_block << log2m, end = first + (blocks << log2m);
     int m = log2m;
     if (spare && first == 0 && end == total) {
         // A call that splits whole permutations readies the kernel of a call that may not (a captured one) too, so that
         // one ordinary call is enough before a capture.
         if (log2m == log2n && m >= kPeelLog2 && 2 * (total >> m) <= size_t(sm_count())) {
-            const int rc = m == 15 ? configure_one<15, 1024>() : m == 14 ? configure_one<14, 1024>()
-                         : m == 13 ? configure_one<13, 1024>() : configure_one<12, 1024>();
+            const int rc = m == 15 ? configure_fused<FusedCfg<15, 2>>() : m == 14 ? configure_fused<FusedCfg<14, 1>>()
+                         : m == 13 ? configure_fused<FusedCfg<13, 1>>() : configure_fused<FusedCfg<12, 1>>();
             if (rc) return rc;
         }
         for (int i = 0; m >= kPeelLog2 && 2 * (total >> m) <= size_t(sm_count()); --m, i ^= 1) {
-            const int rc = m == 15 ? launch_peel<15>(P, records, total, bits, log2n, spare[i], s, gate, redone)
-                         : m == 14 ? launch_peel<14>(P, records, total, bits, log2n, spare[i], s, gate, redone)
-                         : m == 13 ? launch_peel<13>(P, records, total, bits, log2n, spare[i], s, gate, redone)
-                                   : launch_peel<12>(P, records, total, bits, log2n, spare[i], s, gate, redone);
+            const int rc = m == 15 ? launch_peel<FusedCfg<15, 2>>(src, inverse, total, bits, log2n, spare[i], s)
+                         : m == 14 ? launch_peel<FusedCfg<14, 1>>(src, inverse, total, bits, log2n, spare[i], s)
+                         : m == 13 ? launch_peel<FusedCfg<13, 1>>(src, inverse, total, bits, log2n, spare[i], s)
+                                   : launch_peel<FusedCfg<12, 1>>(src, inverse, total, bits, log2n, spare[i], s);
             if (rc) return rc;
-            P = spare[i];
-            records = 0;
-            gate = nullptr;
+            src = spare[i];
+            inverse = true;
         }
     }
-    // blocks of up to 2^11 in a plain array, and not more switches than the GPU has threads
-    if (records == 0 && !gate && m <= 11 && first == 0 && end / 2 <= size_t(sm_count()) * 2048) {
+    // blocks of up to 2^11, and not more switches than the GPU has threads
+    if (m <= 11 && first == 0 && end / 2 <= size_t(sm_count()) * 2048) {
         const int logc = m > 8 ? m : 8;
-        return logc == 8 ? launch_few<8>(P, end, bits, log2n, m, s) : logc == 9 ? launch_few<9>(P, end, bits, log2n, m, s)
-             : logc == 10 ? launch_few<10>(P, end, bits, log2n, m, s) : launch_few<11>(P, end, bits, log2n, m, s);
+        return logc == 8 ? launch_few<8>(src, inverse, end, bits, log2n, m, s) : logc == 9 ? launch_few<9>(src, inverse, end, bits, log2n, m, s)
+             : logc == 10 ? launch_few<10>(src, inverse, end, bits, log2n, m, s) : launch_few<11>(src, inverse, end, bits, log2n, m, s);
     }
     // Small blocks share a CTA: a thread of the 8-bit levels takes a whole sub-block, so the more
     // sub-blocks a CTA holds, the fuller its warps.  Up to 2^13 outputs per CTA, as long as
@@ -1264,14 +1378,14 @@ int launch_fused(const void *Pv, int records, size_t total, int log2m, uint32_t 
     // CTAs that have an SM to themselves get more threads: their time is a chain of short
     // phases, not the instructions they issue.
     const bool alone = ((end - first + (size_t(1) << logc) - 1) >> logc) <= size_t(sm_count());
-#define BENES_FUSED(LC, T) return launch_one<LC, T>(P, records, first, end, bits, log2n, m, s, gate, redone)
+#define BENES_FUSED(LC, G) return launch_one<FusedCfg<LC, G>>(src, inverse, first, end, bits, log2n, m, s)
     switch (logc) {
-        case 10: if (alone) BENES_FUSED(10, 256); BENES_FUSED(10, 32);
-        case 11: if (alone) BENES_FUSED(11, 512); BENES_FUSED(11, 64);
-        case 12: if (alone) BENES_FUSED(12, 1024); BENES_FUSED(12, 128);
-        case 13: if (alone) BENES_FUSED(13, 1024); BENES_FUSED(13, 256);
-        case 14: if (alone) BENES_FUSED(14, 1024); BENES_FUSED(14, 512);
-        default: BENES_FUSED(15, 1024);
+        case 10: if (alone) BENES_FUSED(10, 1); BENES_FUSED(10, 2);
+        case 11: if (alone) BENES_FUSED(11, 1); BENES_FUSED(11, 2);
+        case 12: if (alone) BENES_FUSED(12, 1); BENES_FUSED(12, 2);
+        case 13: if (alone) BENES_FUSED(13, 1); BENES_FUSED(13, 2);
+        case 14: if (alone) BENES_FUSED(14, 1); BENES_FUSED(14, 2);
+        default: BENES_FUSED(15, 2);
     }
 #undef BENES_FUSED
 }

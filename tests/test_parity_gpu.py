@@ -173,6 +173,25 @@ def test_route_structured(n, kind):
     assert np.array_equal(gpu_route(perm, n), oracle.route(perm, n))
 
 
+def loops_of_few_switches(n: int, group: int, seed: int) -> np.ndarray:
+    """Outputs shuffled among `group` neighbours: every loop stays within `group` / 2 switches at the outermost level."""
+    rng = np.random.default_rng(seed)
+    p = np.arange(1 << n, dtype=np.uint32).reshape(-1, min(group, 1 << n))
+    return rng.permuted(p, axis=1).reshape(-1)
+
+
+@pytest.mark.parametrize("n,batch", [(4, 700), (5, 333), (7, 2500), (8, 1300), (9, 700), (10, 650), (12, 160), (13, 160), (14, 40),
+                                     (14, 160), (15, 90), (15, 150)])
+@pytest.mark.parametrize("group", [2, 16, 512])
+def test_route_loops_without_ruler_inside_a_cta(n, batch, group):
+    """Loops too short for a ruler switch: few enough to queue up, or so many that the queue of the CTA overflows."""
+    perm = np.stack([loops_of_few_switches(n, group, s % 3) for s in range(batch)])
+    want = np.stack([oracle.route(perm[s], n) for s in range(3)])
+    got = gpu_route(perm, n)
+    for s in range(batch):
+        assert np.array_equal(got[s], want[s % 3]), s
+
+
 def test_route_exhaustive_n8():
     """All 40320 permutations of N = 8 in one batched call."""
     import itertools
