@@ -251,7 +251,9 @@ template <class Cfg>
 __device__ __forceinline__ uint32_t loop_colour16(unsigned char *sm, uint32_t t, uint32_t S) {
     constexpr uint32_t kMask = 2u * Cfg::C - 2u;
     const uint32_t j0 = 4u * t;
-    uint32_t f = j0, bk = j0, least = j0;
+    uint32_t f = at<uint16_t>(sm, j0) & kMask, bk = (at<uint16_t>(sm, j0 ^ 2u) & kMask) ^ 2u, least = min(j0, f);
+    if (f == bk) return (least >> 1) & 1u;     // (one switch or two)
+    least = min(least, bk);
     // (four hops per look at whether the two have met: on the way past each other they see what they know already)
     for (uint32_t hops = 0; hops < S; hops += 4) {
         bool met = false;
@@ -353,6 +355,17 @@ __device__ __forceinline__ void colours16(unsigned char *sm, int logs, const Rul
             free_ |= (~code & 1u) << k;
         }
         bits &= ~free_;
+        if (__popc(free_) > 4) {
+            // a permutation made of short loops: those of one switch or two at once, by one load each
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const uint32_t j = 4u * (8u * g + (uint32_t(k) ^ (h << 2))), f = n8[k] & (2u * Cfg::C - 2u);
+                if (((free_ >> k) & 1u) && (at<uint16_t>(sm, f) & (2u * Cfg::C - 2u)) == j) {
+                    free_ &= ~(1u << k);
+                    bits |= ((min(j, f) >> 1) & 1u) << k;
+                }
+            }
+        }
         if (free_) {
             uint32_t pos = atomicAdd(&at<uint32_t>(sm, Cfg::kCount), uint32_t(__popc(free_)));
             for (uint32_t left = free_; left; left &= left - 1u, ++pos) {
@@ -501,6 +514,25 @@ __device__ __forceinline__ void levels16(unsigned char *sm, const FusedOut &out,
 // loop again meanwhile and noted what it had noted): what is done once a round need not be done with every hop.
 constexpr int kLoopHops = 3;
 
+// Marks the switches on loops of one or two.
+__device__ __forceinline__ uint32_t mark_short_loops(const unsigned char *N, unsigned char *marks) {
+    uint32_t seen = 0;
+    for (uint32_t i = 0; i < 32; ++i) {
+        const uint32_t t0 = 4u * ((i + threadIdx.x) & 31u);    // (lanes side by side would meet in a bank)
+        const uint2 n = *reinterpret_cast<const uint2 *>(N + 2u * t0);
+        const uint32_t f[4] = {n.x & 255u, (n.x >> 16) & 255u, n.y & 255u, (n.y >> 16) & 255u};
+        uint32_t m = *reinterpret_cast<const uint32_t *>(marks + t0);
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) {
+            const uint32_t j = 2u * (t0 + k);
+            if (N[f[k]] == j) m |= (2u + (min(j, f[k]) & 1u)) << (8u * k);
+        }
+        *reinterpret_cast<uint32_t *>(marks + t0) = m;
+        seen += uint32_t(__popc(m & 0x02020202u));
+    }
+    return seen;
+}
+
 // The 2^8 outputs whose successors start at N.  The mark of a switch, 2 + the colour of its even output, says that it has
 // been seen; marks are clear at first.  The next start, the smallest switch without a mark, is looked up eight marks at a
 // time beside the hops of a round, and not taken if this round has seen it.  A hop is a load, a store and
@@ -534,16 +566,24 @@ __device__ __forceinline__ void loop_marks(const unsigned char *N, unsigned char
         start = take ? 2u * fresh : start;
         j = take ? 2u * fresh : j;
         if (__all_sync(~0u, seen >= kSw)) break;
+        // Loop after loop that ends within a round, in most lanes: the short ones together first.  (What is left of the
+        // loop at hand is then not short, unless it has not been begun.)
+        if (round == 3u && __popc(__ballot_sync(~0u, seen <= 8u)) > 16) {
+            seen = mark_short_loops(N, marks);
+            idle = idle || (j == start && marks[j >> 1] != 0);
+        }
     }
 }
 
 // A sub-block of 2^7.  Bit sets run from the top bit down, so that the smallest gap is one count of leading ones.
 __device__ __forceinline__ uint2 loop_128(const unsigned char *N) {
     uint32_t seen0 = 0, seen1 = 0, col0 = 0, col1 = 0, j = 0, start = 0;
+    bool full = false, quick = false;          // all switches seen; all lanes' loops closed in the last round
     for (uint32_t round = 0; round < 64u; ++round) {
-        bool closed = false;
+        bool closed = full;
 #pragma unroll
         for (int k = 0; k < kLoopHops; ++k) {
+            if (k == 1 && quick && __all_sync(~0u, closed)) break;
             const uint32_t next = N[j] & 127u;                 // (places that nobody has written)
             const uint32_t bit = 0x80000000u >> ((j >> 1) & 31u), odd = (j & 1u) ? bit : 0u;
             if (j >= 64u) {
@@ -557,8 +597,10 @@ __device__ __forceinline__ uint2 loop_128(const unsigned char *N) {
             j = next;
         }
         const bool full0 = seen0 == ~0u;
+        full = full0 && seen1 == ~0u;
         if (closed) start = j = ((full0 ? 64u : 0u) + 2u * uint32_t(__clz(int(~(full0 ? seen1 : seen0))))) & 127u;
-        if (__all_sync(~0u, (seen0 & seen1) == ~0u)) break;
+        quick = __all_sync(~0u, closed);
+        if (quick && __all_sync(~0u, full)) break;
     }
     return make_uint2(__brev(col0), __brev(col1));
 }
