@@ -324,8 +324,9 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     uint32_t *fill = reinterpret_cast<uint32_t *>(ws + off); off += align_up(kInverseMaxBuckets * 4);
     char *sampled = ws + off;
     // Small inputs are bound by the longest walk of a level, not by throughput:
-    // closer rulers (shorter walks) pay there although the lists get longer.
-    const int kappa = (opt.kappa > 3 && T <= (size_t(1) << 22)) ? 3 : opt.kappa;
+    // closer rulers (shorter walks) pay there although the lists get longer.  Where walks are chained (2^16 .. 2^20), one
+    // ruler per 4 switches instead of 8: 2^18 203 -> 195 us, 2^19 293 -> 284, but 2^20 400 -> 407.
+    const int kappa = opt.kappa > 3 && T <= (size_t(1) << 22) ? (2 * T <= kChainMaxTotal ? 2 : 3) : opt.kappa;
     const uint32_t cap = uint32_t(opt.walk_cap);
     // Level 0: P is the caller's permutation, which nobody writes.  The kernels of the sampled levels load it 16 bytes at
     // a time, from a copy where it does not start on 16 bytes.  The copy lasts as long as level 0 only (level 2
@@ -335,7 +336,10 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
         BENES_CUDA_TRY(cudaMemcpyAsync(Pbuf[0], perm, T * 4, cudaMemcpyDeviceToDevice, s));
         perm = Pbuf[0];
     }
+    const bool chained = kappa && T <= kChainMaxTotal;
+    uint32_t *const G = static_cast<uint32_t *>(Sbuf[0]), *const owner = static_cast<uint32_t *>(Sbuf[1]);    // (if chained)
     auto records = [&](int level, int buf) {                    // (with sampling)
+        if (chained) return LevelRecords{nullptr, nullptr, true};
         const bool packed = rec_is_packed(n - level, kappa);
         return LevelRecords{Sbuf[buf], packed ? nullptr : level ? Pbuf[buf] : const_cast<uint32_t *>(perm), packed};
     };
@@ -373,20 +377,22 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
                           : launch_inverse(perm, S0, Qbuf[0], T, n, kappa, s);
         }
         if (rc) return rc;
+        if (chained && (rc = launch_chain_start(perm, Qbuf[0], G, owner, T, n, s))) return rc;
     }
     const int fused_m = opt.cluster ? kFusedLog2M + 1 : kFusedLog2M;
     int cur = 0;
     for (int level = 0; kappa && n - level > fused_m; ++level) {
         const int m = n - level;
         const int out_stage = 2 * n - 2 - level;
-        const LevelRecords S = records(level, cur), Sn = records(level + 1, cur ^ 1);
+        const LevelRecords S = records(level, cur), Sn = m - 1 > fused_m ? records(level + 1, cur ^ 1) : LevelRecords{nullptr, nullptr, true};
         uint32_t *Q = Qbuf[cur];
         // ruler-sampled labelling; raises the gate if a walk had to give up
-        if ((rc = sampled_label(S, Q, Sn, sc, T, m, kappa, uint32_t(level), cap, opt.walk_pairs, L, out_stage, gate, s)))
-            return rc;
+        rc = chained ? chain_label(G, owner, sc, T, m, kappa, uint32_t(level), cap, L, out_stage, gate, s)
+                     : sampled_label(S, Q, Sn, sc, T, m, kappa, uint32_t(level), cap, opt.walk_pairs, L, out_stage, gate, s);
+        if (rc) return rc;
         {
             ProfileScope ps(kSplit, s);
-            if ((rc = launch_split(Q, Qbuf[cur ^ 1], T, m, L, level, out_stage, s))) return rc;
+            if ((rc = launch_split(Q, Qbuf[cur ^ 1], T, m, L, level, out_stage, s, chained && m - 1 > fused_m ? G : nullptr))) return rc;
         }
         cur ^= 1;
         if (hp && hp->bits_host) {

@@ -294,7 +294,7 @@ struct LevelRecords {
     uint32_t *P;
     bool packed;
 };
-// Level 0: records from the caller's permutation (rulers of salt 0), and Q[P[j]] = j.
+// Level 0: records from the caller's permutation (rulers of salt 0; none if S.S is null), and Q[P[j]] = j.
 int launch_inverse(const uint32_t *perm, LevelRecords S, uint32_t *Q, size_t total, int log2m, int kappa,
                    cudaStream_t s);
 // The same for total >= 2^kInversePartitionMinLog2 in two streaming passes:
@@ -313,9 +313,9 @@ int launch_inverse_scatter(const void *pairs, uint32_t *Q, size_t total, int log
 // blocks of 2^last_m are left in P[(log2n - last_m) & 1].
 int launch_route_jump(const uint32_t *perm, uint32_t *const P[2], uint32_t *const Q[2], unsigned long long *Wd,
                       size_t total, int log2n, int last_m, BitsLayout L, const uint32_t *gate, cudaStream_t s);
-// Input-side bits + next level's inverses.
+// Input-side bits + next level's inverses; its successors too, if G is not null (chained levels).
 int launch_split(const uint32_t *Q, uint32_t *Qn, size_t total, int log2m, BitsLayout L, int in_stage, int out_stage,
-                 cudaStream_t s);
+                 cudaStream_t s, uint32_t *G = nullptr);
 
 // ---- ruler-sampled loop labelling (route_sampled.cu) --------------------------
 struct SampledScratch {
@@ -327,10 +327,21 @@ struct SampledScratch {
 size_t sampled_scratch_bytes(size_t total, int kappa);
 void sampled_scratch_carve(char *base, size_t total, int kappa, SampledScratch *out);
 // Labels every loop of the level, writes the output-side stage and the next
-// level's records Sn; raises *gate if some walk exceeded `cap` hops (the route must then be
+// level's records Sn (none if Sn.S is null); raises *gate if some walk exceeded `cap` hops (the route must then be
 // redone by launch_route_jump).
 int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const SampledScratch &sc, size_t total,
                   int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage, uint32_t *gate, cudaStream_t s);
+// Chained levels: the successors themselves in an array, G[j] = g(j), local to the block (two per 8 bytes), and the owners
+// of the switches beside them (`owner`, one word per switch, all kUnowned between levels).  A hop then waits for one load,
+// G[j], and its claim, which are under way together.  Total elements up to which the sampled levels run that way: where a
+// level lasts as long as its longest chain, not where the GPU is full of them, because a successor costs the level above a
+// random store and the walks a second table (records -> chained: 2^20 417 -> 394 us, 2^21 593 -> 597, 3 x 2^20 612 -> 625,
+// 2^22 946 -> 981, 2^24 3.35 -> 3.76 ms).
+constexpr size_t kChainMaxTotal = size_t(1) << 20;
+int launch_chain_start(const uint32_t *perm, const uint32_t *Q, uint32_t *G, uint32_t *owner, size_t total, int log2m, cudaStream_t s);
+// Labels every loop of a chained level and writes the output-side stage.
+int chain_label(const uint32_t *G, uint32_t *owner, const SampledScratch &sc, size_t total, int log2m, int kappa, uint32_t salt,
+                uint32_t cap, BitsLayout L, int out_stage, uint32_t *gate, cudaStream_t s);
 // The bytes from the start of the scratch that have to be zero (owners kUnowned) before the first sampled_label of a
 // route (log2m of the first level).
 size_t sampled_owner_bytes(const SampledScratch &sc, size_t total, int log2m, int kappa);

@@ -68,7 +68,7 @@ k_inverse(const uint4 *__restrict__ P4, void *__restrict__ S, uint32_t *__restri
         size_t j = i * 4;
         size_t base = j & ~size_t(mmask);
         uint32_t jl = uint32_t(j) & mmask;
-        rec_write2<PACKED>(S, nullptr, 2 * i, m, p, kappa, 0u);
+        if (S) rec_write2<PACKED>(S, nullptr, 2 * i, m, p, kappa, 0u);
         Q[base + p.x] = jl;
         Q[base + p.y] = jl + 1;
         Q[base + p.z] = jl + 2;
@@ -126,7 +126,7 @@ k_inverse_partition(const uint32_t *__restrict__ P, void *__restrict__ S, uint2 
         const size_t j = j0 + 2 * (size_t(i / 2) * kPartThreads + tid);
         const uint2 p = __ldcs(reinterpret_cast<const uint2 *>(P + j));
         const uint32_t px = BENES_GUARD(p.x, mmask), py = BENES_GUARD(p.y, mmask);
-        rec_write<PACKED>(S, nullptr, j >> 1, m, px, py, kappa, 0u);
+        if (S) rec_write<PACKED>(S, nullptr, j >> 1, m, px, py, kappa, 0u);
         const uint32_t base = uint32_t(j) & ~mmask;
         dest[i] = base + px;
         dest[i + 1] = base + py;
@@ -320,10 +320,13 @@ k_route_jump(JumpArrays a, uint32_t total, int log2n, int last_m, BitsLayout L, 
     }
 }
 
-// in-side half of a5 + a6: input-side stage word and Q' (the colouring kernel has written the next level's records).
+// in-side half of a5 + a6: input-side stage word and Q' (the colouring kernel has written the next level's records, or,
+// with SUCC, this one scatters its successors: the outputs a and b of an input switch are each other's partners on the
+// loop, so g(a ^ 1) = b and g(b ^ 1) = a).
+template <bool SUCC>
 __global__ void __launch_bounds__(kThreads, 8)
 k_split(const uint4 *__restrict__ Q4, uint32_t *__restrict__ Qn, uint32_t pairs, int m,
-        BitsLayout L, int in_stage, int out_stage, uint32_t rounds) {
+        BitsLayout L, int in_stage, int out_stage, uint32_t rounds, uint32_t *__restrict__ G) {
     after_previous_kernel();
     const uint32_t mmask = (1u << m) - 1u;
     // a CTA takes `rounds` consecutive groups of blockDim.x pairs: the colour
@@ -351,10 +354,16 @@ k_split(const uint4 *__restrict__ Q4, uint32_t *__restrict__ Qn, uint32_t pairs,
         const uint32_t cin1 = ((colours[q.z >> 6] >> ((q.z >> 1) & 31u)) ^ q.z) & 1u;
         store_stage_bits64(L.bits + L.word32(in_stage, (t - 2u * (threadIdx.x & 31u)) >> 5), cin0, cin1);
         // positions tl, tl+1 of the two half-blocks
-        *reinterpret_cast<uint2 *>(Qn + base + tl) =
-            make_uint2((cin0 ? q.y : q.x) >> 1, (cin1 ? q.w : q.z) >> 1);
-        *reinterpret_cast<uint2 *>(Qn + base + H + tl) =
-            make_uint2((cin0 ? q.x : q.y) >> 1, (cin1 ? q.z : q.w) >> 1);
+        const uint2 up = make_uint2((cin0 ? q.y : q.x) >> 1, (cin1 ? q.w : q.z) >> 1);
+        const uint2 low = make_uint2((cin0 ? q.x : q.y) >> 1, (cin1 ? q.z : q.w) >> 1);
+        *reinterpret_cast<uint2 *>(Qn + base + tl) = up;
+        *reinterpret_cast<uint2 *>(Qn + base + H + tl) = low;
+        if (SUCC) {
+            __stcg(G + base + (up.x ^ 1u), up.y);
+            __stcg(G + base + (up.y ^ 1u), up.x);
+            __stcg(G + base + H + (low.x ^ 1u), low.y);
+            __stcg(G + base + H + (low.y ^ 1u), low.x);
+        }
         q = qn;
         i = inext;
     }
@@ -470,7 +479,7 @@ int launch_route_jump(const uint32_t *perm, uint32_t *const P[2], uint32_t *cons
 }
 
 int launch_split(const uint32_t *Q, uint32_t *Qn, size_t total, int log2m, BitsLayout L, int in_stage, int out_stage,
-                 cudaStream_t s) {
+                 cudaStream_t s, uint32_t *G) {
     const uint32_t pairs = uint32_t(total / 4);                  // two switches per thread
     const uint4 *Q4 = reinterpret_cast<const uint4 *>(Q);
     // Colour words are gathered at random from the block's row of the output-side stage (2^(m-1) bits).  Rows of 32
@@ -480,7 +489,8 @@ int launch_split(const uint32_t *Q, uint32_t *Qn, size_t total, int log2m, BitsL
     // of 2^24 outputs 37.6 instead of 35.7 and 37.2 instead of 39.1.
     const uint32_t rounds = stream_rounds(pairs, kThreads);
     const unsigned grid = unsigned((size_t(pairs) + size_t(kThreads) * rounds - 1) / (size_t(kThreads) * rounds));
-    launch_kernel(k_split, grid, kThreads, 0, s, Q4, Qn, pairs, log2m, L, in_stage, out_stage, rounds);
+    if (G) launch_kernel(k_split<true>, grid, kThreads, 0, s, Q4, Qn, pairs, log2m, L, in_stage, out_stage, rounds, G);
+    else launch_kernel(k_split<false>, grid, kThreads, 0, s, Q4, Qn, pairs, log2m, L, in_stage, out_stage, rounds, G);
     return launch_status();
 }
 

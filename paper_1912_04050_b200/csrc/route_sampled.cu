@@ -51,6 +51,12 @@ __device__ __forceinline__ bool gate_raised(const uint32_t *gate) {
     return *reinterpret_cast<const volatile uint32_t *>(gate) != 0u;
 }
 
+// colour of output 2t from the owner of switch t
+__device__ __forceinline__ uint32_t owner_colour(const uint32_t *cb, uint32_t code, uint32_t rulers) {
+    const uint32_t rho = BENES_GUARD_BELOW(code >> 1, rulers, 0u);
+    return ((__ldg(cb + (rho >> 5)) >> (rho & 31u)) ^ code) & 1u;
+}
+
 // Step 2.  W walks per thread, one after another, launched in index order so that the blocks being
 // walked at any moment are neighbours in memory.
 //
@@ -163,6 +169,98 @@ k_walk(unsigned long long *__restrict__ S8, const uint32_t *__restrict__ P, cons
             least = 2u * (((rho >> 1) << kappa) | ruler_slot(rho >> 1, salt, kmask)) + (rho & 1u);
         }
     }
+}
+
+// ---- chained levels ---------------------------------------------------------------------
+// Where a level lasts as long as its longest walk, what counts is what a hop waits for.  Here that is one access: the
+// successor G[j] and the claim of its switch (a compare-and-swap on the owner's word) are under way together.  On
+// records a hop waits for an atomic and then for a gather.  One permutation, walks of a level and the whole route, on
+// records and chained: 2^20 30.5 -> 22.5 and 417 -> 394 us, 2^18 30 -> 21.5 and 231 -> 198 us (with twice as many
+// rulers; 203 without).  A switch that the two walkers of a segment claim at the same time may be counted by both.
+// (Behind a raised gate, or an input that is no permutation, some successors are left over from other levels: they are
+// masked into the block.)
+__global__ void __launch_bounds__(kWalkThreads)
+k_chain_walk(const uint32_t *__restrict__ G, uint32_t *__restrict__ owner, uint2 *__restrict__ rec, uint32_t rulers, int m,
+             int kappa, uint32_t salt, uint32_t cap, uint32_t *__restrict__ gate) {
+    after_previous_kernel();
+    const uint32_t rho = blockIdx.x * kWalkThreads + threadIdx.x;
+    if (rho >= rulers) return;
+    const uint32_t mmask = (1u << m) - 1u, kmask = (1u << kappa) - 1u;
+    const uint32_t t0 = ((rho >> 1) << kappa) | ruler_slot(rho >> 1, salt, kmask);
+    const uint32_t base = (2u * t0) & ~mmask;
+    if (!(rho & 1u)) owner[t0] = ~(rho << 1);                       // the ruler switch belongs to its even walker
+    uint32_t least = 2u * t0 + (rho & 1u), peer = rho ^ 1u, hops = 0;
+    uint32_t j = base + (__ldcg(G + least) & mmask);
+    for (;;) {
+        const uint32_t t = j >> 1, side = j & 1u, g = t >> kappa;
+        if ((t & kmask) == ruler_slot(g, salt, kmask)) {
+            peer = (2u * g + side) ^ 1u;
+            break;
+        }
+        if (++hops > cap) *gate = 1u;
+        if (hops > cap || ((hops & 63u) == 0u && gate_raised(gate))) break;
+        const uint32_t next = __ldcg(G + j);
+        const uint32_t met = atomicCAS(owner + t, kUnowned, ~((rho << 1) | side));
+        least = min(least, j);
+        if (met != kUnowned) {
+            peer = ~met >> 1;
+            break;
+        }
+        j = base + (next & mmask);
+    }
+    rec[rho] = make_uint2(least, peer);
+}
+
+// The successors of the first level: g(j) = Q[P[j ^ 1] ^ 1].  Two switches per thread.
+__global__ void __launch_bounds__(kThreads)
+k_chain_start(const uint4 *__restrict__ P4, const uint32_t *__restrict__ Q, uint4 *__restrict__ G4, uint2 *__restrict__ owner2,
+              uint32_t quads, int m) {
+    after_previous_kernel();
+    const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
+    if (i >= quads) return;
+    const uint32_t mmask = (1u << m) - 1u;
+    const uint32_t *Qb = Q + ((4u * i) & ~mmask);
+    const uint4 p = __ldcs(P4 + i);
+    G4[i] = make_uint4(Qb[BENES_GUARD(p.y, mmask) ^ 1u], Qb[BENES_GUARD(p.x, mmask) ^ 1u], Qb[BENES_GUARD(p.w, mmask) ^ 1u],
+                       Qb[BENES_GUARD(p.z, mmask) ^ 1u]);
+    owner2[i] = make_uint2(kUnowned, kUnowned);
+}
+
+// A switch on a loop without ruler: the minimum of the g-cycle of output 2t, from both ends (see loop_colour).
+__device__ __forceinline__ uint32_t chain_loop_colour(const uint32_t *G, uint32_t t, uint32_t base, uint32_t mmask, uint32_t cap,
+                                                      uint32_t *gate) {
+    const uint32_t j0 = 2u * t;
+    uint32_t f = j0, bk = j0, mn = j0, hops = 0;
+    for (;;) {
+        const uint32_t nf = base + (__ldg(G + f) & mmask), nb = (base + (__ldg(G + (bk ^ 1u)) & mmask)) ^ 1u;
+        f = nf;
+        if (f == bk) break;
+        mn = min(mn, f);
+        bk = nb;
+        if (bk == f) break;
+        mn = min(mn, bk);
+        if (++hops > cap) {
+            *gate = 1u;
+            break;
+        }
+        if ((hops & 63u) == 0u && gate_raised(gate)) break;
+    }
+    return mn & 1u;
+}
+
+// Output side of a chained level; hands the owners back as kUnowned.  Two switches per thread.
+__global__ void __launch_bounds__(kThreads)
+k_chain_colour(const uint32_t *__restrict__ G, uint2 *__restrict__ owner2, const uint32_t *__restrict__ cb, uint32_t pairs,
+               uint32_t rulers, int m, BitsLayout L, int out_stage, uint32_t cap, uint32_t *__restrict__ gate) {
+    after_previous_kernel();
+    const uint32_t i = blockIdx.x * kThreads + threadIdx.x;         // pairs is a multiple of 32
+    if (i >= pairs) return;
+    const uint32_t mmask = (1u << m) - 1u, t = 2u * i, base = (2u * t) & ~mmask;
+    const uint2 o = owner2[i];
+    owner2[i] = make_uint2(kUnowned, kUnowned);
+    const uint32_t c0 = o.x != kUnowned ? owner_colour(cb, ~o.x, rulers) : chain_loop_colour(G, t, base, mmask, cap, gate);
+    const uint32_t c1 = o.y != kUnowned ? owner_colour(cb, ~o.y, rulers) : chain_loop_colour(G, t + 1u, base, mmask, cap, gate);
+    store_stage_bits64(L.bits + L.word32(out_stage, (t - 2u * (threadIdx.x & 31u)) >> 5), c0, c1);
 }
 
 // Step 3, the contracted list.  It needs no pass of its own.  The segment of walker rho ends at ruler output
@@ -445,18 +543,14 @@ __device__ __forceinline__ uint32_t loop_colour(const void *S, const uint32_t *P
     return mn & 1u;
 }
 
-// colour of output 2t from the owner of switch t
-__device__ __forceinline__ uint32_t owner_colour(const uint32_t *cb, uint32_t code, uint32_t rulers) {
-    const uint32_t rho = BENES_GUARD_BELOW(code >> 1, rulers, 0u);
-    return ((__ldg(cb + (rho >> 5)) >> (rho & 31u)) ^ code) & 1u;
-}
-
 // Step 5 + output side of the level's switches + the next level's records
 // (owner reset).  A thread owns the neighbouring switches 2i and 2i+1: their
 // colour-0 outputs are neighbours in the upper half-block of the next level and
 // their colour-1 outputs in the lower one, i.e. the thread writes one whole
-// record of each.  (With the gate raised what it writes is never used.)
-template <bool PACKED, bool NEXT_PACKED>
+// record of each.  (With the gate raised what it writes is never used.)  The last level writes none: the in-CTA levels
+// start from the inverses (256 x 2^16: 921 -> 907 us, 2^24: 3.40 -> 3.38 ms).
+enum NextRecords { kNextWide, kNextPacked, kNextNone };
+template <bool PACKED, NextRecords NEXT>
 __global__ void __launch_bounds__(kThreads)
 k_colour(const void *__restrict__ S, const uint32_t *__restrict__ P, const uint32_t *__restrict__ Q,
          const uint32_t *__restrict__ cb, void *__restrict__ Sn, uint32_t *__restrict__ Pn, uint32_t salt_next, uint32_t pairs,
@@ -520,11 +614,11 @@ k_colour(const void *__restrict__ S, const uint32_t *__restrict__ P, const uint3
         const uint32_t r = (base >> 1) + (((t - (base >> 1)) >> 1));   // record of the upper half
         const uint32_t u0 = (c0 ? py0 : px0) >> 1, u1 = (c1 ? py1 : px1) >> 1;     // upper half-block
         const uint32_t d0 = (c0 ? px0 : py0) >> 1, d1 = (c1 ? px1 : py1) >> 1;     // lower half-block
-        if (NEXT_PACKED) {
+        if (NEXT == kNextPacked) {
             uint2 *Sn8 = static_cast<uint2 *>(Sn);
             Sn8[r] = make_uint2(u0 | (u1 << (m - 1)) | ones_lo, (u1 >> (33 - m)) | ones_hi);
             Sn8[r + (H >> 1)] = make_uint2(d0 | (d1 << (m - 1)) | ones_lo, (d1 >> (33 - m)) | ones_hi);
-        } else {
+        } else if (NEXT == kNextWide) {
             rec_write<false>(Sn, Pn, r, m - 1, u0, u1, kappa, salt_next);
             rec_write<false>(Sn, Pn, r + (H >> 1), m - 1, d0, d1, kappa, salt_next);
         }
@@ -588,30 +682,10 @@ size_t sampled_owner_bytes(const SampledScratch &sc, size_t total, int log2m, in
     return bytes;
 }
 
-int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const SampledScratch &sc, size_t total,
-                  int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage,
-                  uint32_t *gate, cudaStream_t s) {
-    const uint32_t R = uint32_t(total >> kappa);
-    {
-        ProfileScope ps(kWalk, s);
-        // Two walks per thread pay once half of the threads still fills the GPU (2^26, levels 0-3:
-        // 2.05 / 1.70 / 1.20 / 0.70 -> 1.98 / 1.62 / 1.08 / 0.67 ms, cache-resident levels 0.62 -> 0.53);
-        // below that the launch lasts as long as its longest thread and one walk per thread is
-        // faster.  More are slower: the rulers that are being walked at any moment then
-        // spread over more blocks than the L2 holds (four: 0.95 ms per cache-resident level, eight: 1.6).
-        const bool two = walk_pairs == 2 || (walk_pairs == 1 && size_t(R >> 1) >= size_t(sm_count()) * 2048);
-#define BENES_WALK(PACKED, W)                                                                            \
-    launch_kernel(k_walk<PACKED, W>, (R / W + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s, \
-        static_cast<unsigned long long *>(S.S), S.P, Q, sc.rec[0], R, log2m, kappa, salt, cap, gate)
-        if (S.packed) { if (two) BENES_WALK(true, 2); else BENES_WALK(true, 1); }
-        else { if (two) BENES_WALK(false, 2); else BENES_WALK(false, 1); }
-#undef BENES_WALK
-        int rc = launch_status();
-        if (rc) return rc;
-    }
-    uint32_t *cb = sc.bits[0];
+// The parities of the minima of the walk records in sc.rec[0] (R words, 2^beta per block), to sc.bits[0].
+static int label_lists(const SampledScratch &sc, uint32_t R, int beta, uint32_t salt, uint32_t cap, uint32_t *gate, cudaStream_t s) {
     // label the contracted list: sample it until a block's list fits one CTA
-    int beta = log2m - kappa, depth = 0;
+    int depth = 0;
     if (beta < 7) return BENES_ERR_BADARG;                     // (a CTA labels 2^7 words at least)
     uint32_t counts[kMaxLists + 1] = {R};
     for (int sp; (sp = list_spacing(beta)) != 0; ++depth) {
@@ -640,22 +714,71 @@ int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const Samp
         int rc = launch_status();
         if (rc) return rc;
     }
+    return BENES_OK;
+}
+
+int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const SampledScratch &sc, size_t total,
+                  int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage,
+                  uint32_t *gate, cudaStream_t s) {
+    const uint32_t R = uint32_t(total >> kappa);
+    {
+        ProfileScope ps(kWalk, s);
+        // Two walks per thread pay once half of the threads still fills the GPU (2^26, levels 0-3:
+        // 2.05 / 1.70 / 1.20 / 0.70 -> 1.98 / 1.62 / 1.08 / 0.67 ms, cache-resident levels 0.62 -> 0.53);
+        // below that the launch lasts as long as its longest thread and one walk per thread is
+        // faster.  More are slower: the rulers that are being walked at any moment then
+        // spread over more blocks than the L2 holds (four: 0.95 ms per cache-resident level, eight: 1.6).
+        const bool two = walk_pairs == 2 || (walk_pairs == 1 && size_t(R >> 1) >= size_t(sm_count()) * 2048);
+#define BENES_WALK(PACKED, W)                                                                            \
+    launch_kernel(k_walk<PACKED, W>, (R / W + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s, \
+        static_cast<unsigned long long *>(S.S), S.P, Q, sc.rec[0], R, log2m, kappa, salt, cap, gate)
+        if (S.packed) { if (two) BENES_WALK(true, 2); else BENES_WALK(true, 1); }
+        else { if (two) BENES_WALK(false, 2); else BENES_WALK(false, 1); }
+#undef BENES_WALK
+        int rc = launch_status();
+        if (rc) return rc;
+    }
+    const uint32_t *cb = sc.bits[0];
+    if (const int rc = label_lists(sc, R, log2m - kappa, salt, cap, gate, s)) return rc;
     {
         ProfileScope ps(kColour, s);
         const uint32_t switches = uint32_t(total / 4);           // pairs of switches, one per thread
         const uint32_t rounds = stream_rounds(switches, kThreads);
         const unsigned grid = unsigned((size_t(switches) + size_t(kThreads) * rounds - 1) / (size_t(kThreads) * rounds));
-        if (S.packed)        // a packed level is followed by packed levels only
-            launch_kernel(k_colour<true, true>, grid, kThreads, 0, s, S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
-                          out_stage, cap, gate, rounds);
-        else if (Sn.packed)
-            launch_kernel(k_colour<false, true>, grid, kThreads, 0, s, S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
-                          out_stage, cap, gate, rounds);
-        else
-            launch_kernel(k_colour<false, false>, grid, kThreads, 0, s, S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L,
-                          out_stage, cap, gate, rounds);
+#define BENES_COLOUR(PACKED, NEXT)                                                                                        \
+    launch_kernel(k_colour<PACKED, NEXT>, grid, kThreads, 0, s, S.S, S.P, Q, cb, Sn.S, Sn.P, salt + 1u, switches, R, log2m, kappa, L, \
+                  out_stage, cap, gate, rounds)
+        // (a packed level is followed by packed levels only, and so is the last one)
+        if (S.packed) { if (Sn.S) BENES_COLOUR(true, kNextPacked); else BENES_COLOUR(true, kNextNone); }
+        else if (Sn.packed) BENES_COLOUR(false, kNextPacked);
+        else BENES_COLOUR(false, kNextWide);
+#undef BENES_COLOUR
         return launch_status();
     }
+}
+
+int launch_chain_start(const uint32_t *perm, const uint32_t *Q, uint32_t *G, uint32_t *owner, size_t total, int log2m, cudaStream_t s) {
+    const uint32_t quads = uint32_t(total / 4);
+    launch_kernel(k_chain_start, (quads + kThreads - 1) / kThreads, kThreads, 0, s, reinterpret_cast<const uint4 *>(perm), Q,
+                  reinterpret_cast<uint4 *>(G), reinterpret_cast<uint2 *>(owner), quads, log2m);
+    return launch_status();
+}
+
+int chain_label(const uint32_t *G, uint32_t *owner, const SampledScratch &sc, size_t total, int log2m, int kappa, uint32_t salt,
+                uint32_t cap, BitsLayout L, int out_stage, uint32_t *gate, cudaStream_t s) {
+    const uint32_t R = uint32_t(total >> kappa), pairs = uint32_t(total / 4);
+    int rc;
+    {
+        ProfileScope ps(kWalk, s);
+        launch_kernel(k_chain_walk, (R + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0, s, G, owner, sc.rec[0], R, log2m, kappa,
+                      salt, cap, gate);
+        if ((rc = launch_status())) return rc;
+    }
+    if ((rc = label_lists(sc, R, log2m - kappa, salt, cap, gate, s))) return rc;
+    ProfileScope ps(kColour, s);
+    launch_kernel(k_chain_colour, (pairs + kThreads - 1) / kThreads, kThreads, 0, s, G, reinterpret_cast<uint2 *>(owner), sc.bits[0],
+                  pairs, R, log2m, L, out_stage, cap, gate);
+    return launch_status();
 }
 
 }  // namespace benes

@@ -369,6 +369,22 @@ def test_route_batch_not_a_power_of_two_with_resampled_lists(n, batch, kappa, ca
     assert np.array_equal(gpu_route(perm, n), oracle.route(perm, n))
 
 
+@pytest.mark.parametrize("kappa", [None, 2, 3])
+@pytest.mark.parametrize("n,batch", [(16, 7), (16, 8), (16, 9), (16, 16), (16, 17), (19, 2), (20, 1)])
+@pytest.mark.parametrize("kind", ["random", "sattolo", "short loops"])
+def test_route_chained_levels_and_levels_on_records(n, batch, kappa, kind, labelling_options):
+    """Up to 2^20 outputs in all the levels above a CTA are chained, with closer rulers up to 2^19; above, on records."""
+    if kappa is not None:
+        binding.benes_set_option(binding.OPT_SAMPLE_LOG2K, kappa)
+    make = {"random": lambda s: inputs.random_perm(n, 900 + s), "sattolo": lambda s: inputs.sattolo_perm(n, s),
+            "short loops": lambda s: loops_of_few_switches(n, 32, s)}[kind]
+    few = [make(s) for s in range(min(batch, 3))]
+    want = [oracle.route(p, n) for p in few]
+    got = gpu_route(np.stack([few[b % len(few)] for b in range(batch)]), n)
+    for b in range(batch):
+        assert np.array_equal(got[b], want[b % len(few)]), b
+
+
 @pytest.mark.parametrize("n,batch", [(22, 1), (16, 64), (17, 64), (23, 1), (16, 65)])
 def test_route_bucketed_inverse(n, batch):
     """batch * N >= 2^22 in whole multiples of 2^18 takes the two-pass inverse at
