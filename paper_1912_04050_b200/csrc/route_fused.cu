@@ -125,7 +125,7 @@ __device__ const FusedTables g_fused_tables = make_tables(std::make_integer_sequ
 //   kRec        walk records, contracted list, 32 bit per walker each  |  marks of the sub-blocks of 2^8, behind the tables
 //   kQ (2C)     inverse: pairs of 16-bit entries per input switch, as uint4 of four switches at a place of
 //               their thread's that makes reads and writes free of bank conflicts  |  8 bit: two buffers
-//   kCw (C/16)  colours of the level, kInw (C/16) input-side bits of small permutations
+//   kCw (C/16)  colours of the level
 // Bytes from the marks of a sub-block of 2^8 to the next one's: the lanes of a warp look at the same place of theirs.
 constexpr uint32_t kMarkStride = 128 + 8;
 
@@ -147,8 +147,7 @@ struct FusedCfg {
     static constexpr uint32_t kMarksEnd = kMarks + kMarkBytes;
     static constexpr uint32_t kQ = ((kMarksEnd > kLevelBytes ? kMarksEnd : kLevelBytes) + 15u) & ~15u;
     static constexpr uint32_t kCw = kQ + 2 * C;
-    static constexpr uint32_t kInw = kCw + C / 16;
-    static constexpr uint32_t kCount = kInw + C / 16;            // queued switches
+    static constexpr uint32_t kCount = kCw + C / 16;            // queued switches
     static constexpr size_t kSmemBytes = size_t(kCount) + 16;
     // CTAs per SM the register budget has to leave room for
     static constexpr int kMinCtas = G == 1 || T > 512 ? 1 : int(1024 / T) < 8 ? int(1024 / T) : 8;
@@ -509,9 +508,9 @@ __device__ __forceinline__ void levels16(unsigned char *sm, const FusedOut &out,
 }
 
 // ---- a level with 8-bit entries ----------------------------------------------------------
-// The looping algorithm: ascending start switches, every output it stands on goes up.  In sub-blocks of 2^7 and 2^8 hops
-// come in rounds, and only at the end of one a lane whose loop has closed goes on with the next (it went round its
-// loop again meanwhile and noted what it had noted): what is done once a round need not be done with every hop.
+// The looping algorithm: ascending start switches, every output it stands on goes up.  In sub-blocks of 2^8 hops come in
+// rounds, and only at the end of one a lane whose loop has closed goes on with the next (it went round its loop again
+// meanwhile and noted what it had noted): what is done once a round need not be done with every hop.
 constexpr int kLoopHops = 3;
 
 // Marks the switches on loops of one or two.
@@ -538,6 +537,7 @@ __device__ __forceinline__ uint32_t mark_short_loops(const unsigned char *N, uns
 // time beside the hops of a round, and not taken if this round has seen it.  A hop is a load, a store and
 // eight instructions (with the set of seen switches and its smallest gap in registers it was 36, and they, not the
 // load, were what a hop took: 114 cycles alone and 186 with two warps on a scheduler, now 88).
+template <uint32_t LANES>
 __device__ __forceinline__ void loop_marks(const unsigned char *N, unsigned char *marks) {
     constexpr uint32_t kSw = 128;
     uint32_t j = 0, start = 0, from = 0, seen = 0;
@@ -568,7 +568,7 @@ __device__ __forceinline__ void loop_marks(const unsigned char *N, unsigned char
         if (__all_sync(~0u, seen >= kSw)) break;
         // Loop after loop that ends within a round, in most lanes: the short ones together first.  (What is left of the
         // loop at hand is then not short, unless it has not been begun.)
-        if (round == 3u && __popc(__ballot_sync(~0u, seen <= 8u)) > 16) {
+        if (round == 3u && 2 * __popc(__ballot_sync(~0u, seen <= 8u) & LANES) > __popc(LANES)) {
             seen = mark_short_loops(N, marks);
             idle = idle || (j == start && marks[j >> 1] != 0);
         }
@@ -578,29 +578,21 @@ __device__ __forceinline__ void loop_marks(const unsigned char *N, unsigned char
 // A sub-block of 2^7.  Bit sets run from the top bit down, so that the smallest gap is one count of leading ones.
 __device__ __forceinline__ uint2 loop_128(const unsigned char *N) {
     uint32_t seen0 = 0, seen1 = 0, col0 = 0, col1 = 0, j = 0, start = 0;
-    bool full = false, quick = false;          // all switches seen; all lanes' loops closed in the last round
-    for (uint32_t round = 0; round < 64u; ++round) {
-        bool closed = full;
-#pragma unroll
-        for (int k = 0; k < kLoopHops; ++k) {
-            if (k == 1 && quick && __all_sync(~0u, closed)) break;
-            const uint32_t next = N[j] & 127u;                 // (places that nobody has written)
-            const uint32_t bit = 0x80000000u >> ((j >> 1) & 31u), odd = (j & 1u) ? bit : 0u;
-            if (j >= 64u) {
-                seen1 |= bit;
-                col1 |= odd;
-            } else {
-                seen0 |= bit;
-                col0 |= odd;
-            }
-            closed |= next == start;
-            j = next;
+#pragma unroll 4
+    for (uint32_t it = 0; it < 64u; ++it) {
+        const uint32_t next = N[j] & 127u;                     // (places that nobody has written)
+        const uint32_t bit = 0x80000000u >> ((j >> 1) & 31u), odd = (j & 1u) ? bit : 0u;
+        if (j >= 64u) {
+            seen1 |= bit;
+            col1 |= odd;
+        } else {
+            seen0 |= bit;
+            col0 |= odd;
         }
-        const bool full0 = seen0 == ~0u;
-        full = full0 && seen1 == ~0u;
-        if (closed) start = j = ((full0 ? 64u : 0u) + 2u * uint32_t(__clz(int(~(full0 ? seen1 : seen0))))) & 127u;
-        quick = __all_sync(~0u, closed);
-        if (quick && __all_sync(~0u, full)) break;
+        const bool full0 = seen0 == ~0u, closed = next == start;
+        const uint32_t fresh = ((full0 ? 64u : 0u) + 2u * uint32_t(__clz(int(~(full0 ? seen1 : seen0))))) & 127u;
+        start = closed ? fresh : start;
+        j = closed ? fresh : next;
     }
     return make_uint2(__brev(col0), __brev(col1));
 }
@@ -634,12 +626,13 @@ __device__ __forceinline__ void level8(unsigned char *sm, const FusedOut &out, u
     const int level = out.n - LOGS;
     constexpr uint32_t kRegions = C >> kReg;
     const uint32_t q_from = Cfg::kQ + q8 * C, q_to = Cfg::kQ + (q8 ^ 1u) * C;
-    // (whole warps: lanes without a sub-block repeat the last one.  With few sub-blocks it is the first warps that have one:
-    // an SM's warps are bound to its four schedulers, warp w of its k-th CTA to scheduler (w + k) % 4)
+    // (whole warps: lanes without a sub-block repeat the last one.  With few sub-blocks it is the first warps that have one: an SM's warps are bound to its four schedulers, warp w of
+    // its k-th CTA to scheduler (w + k) % 4)
+    constexpr uint32_t kLanes = kRegions < 32u ? (1u << (kRegions & 31u)) - 1u : ~0u;     // of a warp that has some
     for (uint32_t r0 = tid & ~31u; r0 < kRegions; r0 += T) {
         const uint32_t r = min(r0 + tid % 32u, kRegions - 1u);
         if (LOGS == 8) {
-            loop_marks(sm + (r << kReg), sm + Cfg::kMarks + r * kMarkStride);
+            loop_marks<kLanes>(sm + (r << kReg), sm + Cfg::kMarks + r * kMarkStride);
             continue;
         }
         if (LOGS == 7) {
@@ -698,17 +691,17 @@ __device__ __forceinline__ void level8(unsigned char *sm, const FusedOut &out, u
                 *stage_byte(out, 2 * out.n - 2 - level, g) = uint8_t(out8);
             }
         } else {
-            at<uint8_t>(sm, Cfg::kInw + g) = uint8_t(in);
+            // permutations of 2^5 (two threads) or 2^4: a word per stage
+            const uint32_t in2 = __shfl_xor_sync(~0u, in, 1), out2 = __shfl_xor_sync(~0u, out8, 1);
+            uint32_t *row = out.bits + ((out.flat0 + 16u * g) >> out.n) * size_t(2 * out.n - 1);
+            const bool first = !(g & 1u);
+            if (16u * g < out.valid) {
+                if (out.n == 4 || first) row[level] = out.n == 4 ? in : in | (in2 << 8);
+                if (out.n == 4 || !first) row[2 * out.n - 2 - level] = out.n == 4 ? out8 : out2 | (out8 << 8);
+            }
         }
     }
     __syncthreads();
-    if (out.n < 6) {
-        for (uint32_t r = tid; r < C / 32; r += T) {
-            out.store16(level, r, at<uint16_t>(sm, Cfg::kInw + 2u * r));
-            out.store16(2 * out.n - 2 - level, r, at<uint16_t>(sm, Cfg::kCw + 2u * r));
-        }
-        __syncthreads();
-    }
 }
 
 // ---- sub-blocks of 8 and less: 32 outputs (16 switches of every stage) per thread ----------
@@ -1414,9 +1407,11 @@ int launch_fused(const uint32_t *src, bool inverse, size_t total, int log2m, uin
     }
     // Small blocks share a CTA: a thread of the 8-bit levels takes a whole sub-block, so the more
     // sub-blocks a CTA holds, the fuller its warps.  Up to 2^13 outputs per CTA, as long as
-    // every SM still gets a few CTAs.
+    // every SM still gets a few CTAs: up to five, so that the warps that walk the sub-blocks of 2^8 (one of every CTA) have
+    // a scheduler to themselves, or nearly (up to four against five against eight: 707 x 2^12 91 / 68 / 68 us,
+    // 10000 x 2^8 48 / 33 / 33, 7094 x 2^8 33 / 33 / 50).
     int logc = m > 10 ? m : 10;
-    while (logc < 13 && ((end - first) >> logc) > 4 * size_t(sm_count())) ++logc;
+    while (logc < 13 && ((end - first) >> logc) > 5 * size_t(sm_count())) ++logc;
     // CTAs that have an SM to themselves get more threads: their time is a chain of short
     // phases, not the instructions they issue.
     const bool alone = ((end - first + (size_t(1) << logc) - 1) >> logc) <= size_t(sm_count());
