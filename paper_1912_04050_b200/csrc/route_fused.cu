@@ -1021,7 +1021,7 @@ k_route_few(const uint32_t *__restrict__ src, bool inverse, uint32_t *__restrict
         p0 = BENES_GUARD(src[out.flat0 + j], block);
         p1 = BENES_GUARD(src[out.flat0 + j + 1], block);
     }
-    if (inverse) {                             // (blocks of 2^11 that k_route_peel has made)
+    if (LOGC == 11 && inverse) {               // (blocks of 2^11 that k_route_peel has made)
         const uint32_t sb = j & ~block;
         Pn[sb + p0] = uint16_t(j & block);
         Pn[sb + p1] = uint16_t((j + 1u) & block);
