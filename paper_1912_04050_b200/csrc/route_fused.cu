@@ -1406,12 +1406,14 @@ int launch_fused(const uint32_t *src, bool inverse, size_t total, int log2m, uin
              : logc == 10 ? launch_few<10>(src, inverse, end, bits, log2n, m, s) : launch_few<11>(src, inverse, end, bits, log2n, m, s);
     }
     // Small blocks share a CTA: a thread of the 8-bit levels takes a whole sub-block, so the more
-    // sub-blocks a CTA holds, the fuller its warps.  Up to 2^13 outputs per CTA, as long as
+    // sub-blocks a CTA holds, the fuller its warps.  Up to 2^13 outputs per CTA (2^12 for blocks of 2^4 .. 2^9, whose time is
+    // the walks': eight CTAs per SM instead of four, 22230 x 2^8 72 -> 61 us, 32768 x 2^7 32 -> 28, 600000 x 2^5 69 -> 65;
+    // with 2^11 98, 36 and 72; 16384 x 2^10 232 -> 236, a million of 2^3 33 -> 34), as long as
     // every SM still gets a few CTAs: up to five, so that the warps that walk the sub-blocks of 2^8 (one of every CTA) have
     // a scheduler to themselves, or nearly (up to four against five against eight: 707 x 2^12 91 / 68 / 68 us,
     // 10000 x 2^8 48 / 33 / 33, 7094 x 2^8 33 / 33 / 50).
     int logc = m > 10 ? m : 10;
-    while (logc < 13 && ((end - first) >> logc) > 5 * size_t(sm_count())) ++logc;
+    while (logc < (m >= 4 && m <= 9 ? 12 : 13) && ((end - first) >> logc) > 5 * size_t(sm_count())) ++logc;
     // CTAs that have an SM to themselves get more threads: their time is a chain of short
     // phases, not the instructions they issue.
     const bool alone = ((end - first + (size_t(1) << logc) - 1) >> logc) <= size_t(sm_count());
