@@ -310,7 +310,7 @@ int launch_inverse_partition_piece(const uint32_t *perm, LevelRecords S, void *p
 int launch_inverse_scatter(const void *pairs, uint32_t *Q, size_t total, int log2m, cudaStream_t s);
 // Levels of blocks of 2^log2n .. 2^(last_m + 1) by pointer jumping over all outputs, in ONE cooperative launch;
 // `gate` (may be null) is a device word: the kernel returns at once while it is 0.  P[], Q[]: total words each; the
-// blocks of 2^last_m are left in P[(log2n - last_m) & 1].
+// blocks of 2^last_m are left in P[(log2n - last_m) & 1], their inverses, where the in-CTA levels start, in Q[ditto].
 int launch_route_jump(const uint32_t *perm, uint32_t *const P[2], uint32_t *const Q[2], unsigned long long *Wd,
                       size_t total, int log2n, int last_m, BitsLayout L, const uint32_t *gate, cudaStream_t s);
 // Input-side bits + next level's inverses; its successors too, if G is not null (chained levels).

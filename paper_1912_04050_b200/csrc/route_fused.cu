@@ -30,8 +30,8 @@
 //   S = 4, 2   256-entry table: all three stages at once.
 //
 // Measured on B200, before (P and Q kept, successors gathered through both; twice as many rulers; a look for
-// the next start with every hop at all 8-bit levels) and after: 2048 blocks of 2^15 2.38 -> 1.88 ms, 4096 x 2^14
-// 1.96 -> 1.58 ms, 4096 x 2^12 374 -> 314 us, 16384 x 2^8 53 -> 40 us.  Units of 8192 outputs inside a larger CTA with
+// the next start with every hop in sub-blocks of 2^8 too, by register sets from the low bit up) and after: 2048 blocks of 2^15 2.38 -> 1.87 ms, 4096 x 2^14
+// 1.96 -> 1.61 ms, 4096 x 2^12 374 -> 318 us, 16384 x 2^8 53 -> 40 us.  Units of 8192 outputs inside a larger CTA with
 // barriers of their own, meant to fall out of step, took 2.04 and 1.90 ms for the first two: the CTA waits for
 // its last unit.
 #include "common.cuh"
