@@ -38,13 +38,11 @@ __device__ __forceinline__ uint32_t mark_short_loops(const unsigned char *N, uns
 // time beside the hops of a round, and not taken if this round has seen it.  A hop is a load, a store and
 // eight instructions (with the set of seen switches and its smallest gap in registers it was 36, and they, not the
 // load, were what a hop took: 114 cycles alone and 186 with two warps on a scheduler, now 88).
-// LANES: the lanes that have a sub-block.  The others vote as finished and store nothing: only a vote keeps lanes together,
-// and one that repeated another's walk could show it marks that it is not to know yet, and so a start that is not the
-// smallest of its loop.
-template <uint32_t LANES>
-__device__ __forceinline__ void loop_marks(const unsigned char *N, unsigned char *marks) {
+// `mine`: the lane has a sub-block.  The others vote as finished and store nothing: only a vote keeps lanes together, and one
+// that repeated another's walk could show it marks that it is not to know yet, and so a start that is not the smallest of
+// its loop; and one that walked padding, the identity, would take three times as long as those beside it.
+__device__ __forceinline__ void loop_marks(const unsigned char *N, unsigned char *marks, bool mine) {
     constexpr uint32_t kSw = 128;
-    const bool mine = LANES == ~0u || ((LANES >> (threadIdx.x & 31u)) & 1u) != 0u;
     uint32_t j = 0, start = 0, from = 0, seen = mine ? 0u : kSw;
     bool idle = !mine;                         // the loop has closed, and there was no next one to take
     for (uint32_t round = 0; round < 3u * kSw; ++round) {
@@ -73,7 +71,7 @@ __device__ __forceinline__ void loop_marks(const unsigned char *N, unsigned char
         if (__all_sync(~0u, seen >= kSw)) break;
         // Loop after loop that ends within a round, in most lanes: the short ones together first.  (What is left of the
         // loop at hand is then not short, unless it has not been begun.)
-        if (round == 3u && 2 * __popc(__ballot_sync(~0u, seen <= 8u)) > __popc(LANES)) {
+        if (round == 3u && 2 * __popc(__ballot_sync(~0u, seen <= 8u)) > __popc(__ballot_sync(~0u, mine))) {
             if (mine) seen = mark_short_loops(N, marks);
             idle = idle || (j == start && marks[j >> 1] != 0);
         }

@@ -518,12 +518,14 @@ __device__ __forceinline__ void level8(unsigned char *sm, const FusedOut &out, u
     // (whole warps: lanes without a sub-block follow the last one's successors and store nothing.  With few sub-blocks it
     // is the first warps that have one: an SM's warps are bound to its four schedulers, warp w of its k-th CTA to
     // scheduler (w + k) % 4)
-    constexpr uint32_t kLanes = kRegions < 32u ? (1u << (kRegions & 31u)) - 1u : ~0u;     // of a warp that has some
     for (uint32_t r0 = tid & ~31u; r0 < kRegions; r0 += T) {
         const uint32_t r = min(r0 + tid % 32u, kRegions - 1u);
-        const bool mine = r == r0 + tid % 32u;
+        const bool mine = kRegions >= 32u || r == r0 + tid % 32u;
         if (LOGS == 8) {
-            loop_marks<kLanes>(sm + (r << kReg), sm + Cfg::kMarks + r * kMarkStride);
+            // (sub-blocks of padding, the identity, are coloured as they are: all marks clear.  Loop after loop of one switch
+            // takes three times as long as one loop, so the last CTA kept the call waiting: 9741 x 2^8 42 -> 31 us, 2435 x 2^8
+            // 35 -> 23, 1722 x 2^10 50 -> 39.  CTAs above 2^13 have no padding)
+            loop_marks(sm + (r << kReg), sm + Cfg::kMarks + r * kMarkStride, mine && (Cfg::LOG > 13 || (r << kReg) < out.valid));
             continue;
         }
         if (LOGS == 7) {

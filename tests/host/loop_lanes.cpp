@@ -51,25 +51,23 @@ namespace {
 struct Job {
     const unsigned char *N;
     unsigned char *marks;
-    uint32_t regions;
+    uint32_t regions, valid;
 } g_job;
 
-template <uint32_t REGIONS>
 void lane_main() {
-    // (the pointers level8 gives: a lane without a sub-block has the last one's)
-    const uint32_t lane = threadIdx.x, r = min(lane, REGIONS - 1u);
-    constexpr uint32_t kLanes = REGIONS < 32u ? (1u << (REGIONS & 31u)) - 1u : ~0u;
-    benes::loop_marks<kLanes>(g_job.N + 256u * r, g_job.marks + benes::kMarkStride * r);
+    // (the pointers level8 gives: a lane behind the CTA's last sub-block has that one's)
+    const uint32_t lane = threadIdx.x, r = min(lane, g_job.regions - 1u);
+    benes::loop_marks(g_job.N + 256u * r, g_job.marks + benes::kMarkStride * r, lane < g_job.valid);
     g_done[lane] = true;
     swapcontext(&g_lane[lane], &g_scheduler);
 }
 }  // namespace
 
-// `order`: 0 = lanes ascending, 1 = descending, otherwise the seed of an order drawn anew after every vote.  Returns 0,
-// or -1 where some lanes ended while others wait for a vote.
-extern "C" int play_loop_marks(uint32_t regions, const unsigned char *N, unsigned char *marks, uint32_t order) {
-    void (*const body)() = regions == 4 ? lane_main<4> : regions == 8 ? lane_main<8> : regions == 16 ? lane_main<16> : lane_main<32>;
-    g_job = Job{N, marks, regions};
+// `regions` sub-blocks, of which those from `valid` on are padding.  `order`: 0 = lanes ascending, 1 = descending, otherwise
+// the seed of an order drawn anew after every vote.  Returns the number of votes, or -1 where some lanes ended while others
+// wait for one.
+extern "C" int play_loop_marks(uint32_t regions, uint32_t valid, const unsigned char *N, unsigned char *marks, uint32_t order) {
+    g_job = Job{N, marks, regions, valid};
     std::vector<std::vector<char>> stacks(kWarp, std::vector<char>(1 << 16));
     std::vector<int> turn(kWarp);
     for (int i = 0; i < kWarp; ++i) {
@@ -79,10 +77,10 @@ extern "C" int play_loop_marks(uint32_t regions, const unsigned char *N, unsigne
         g_lane[i].uc_stack.ss_sp = stacks[i].data();
         g_lane[i].uc_stack.ss_size = stacks[i].size();
         g_lane[i].uc_link = &g_scheduler;
-        makecontext(&g_lane[i], body, 0);
+        makecontext(&g_lane[i], lane_main, 0);
     }
     std::mt19937 rng(order);
-    for (;;) {
+    for (int votes = 0;; ++votes) {
         if (order > 1) std::shuffle(turn.begin(), turn.end(), rng);
         for (int lane : turn) {
             threadIdx.x = uint32_t(lane);
@@ -94,7 +92,7 @@ extern "C" int play_loop_marks(uint32_t regions, const unsigned char *N, unsigne
             ballot |= g_vote[i] << i;
             done += g_done[i];
         }
-        if (done == kWarp) return 0;
+        if (done == kWarp) return votes;
         if (done) return -1;
         g_ballot = ballot;
     }

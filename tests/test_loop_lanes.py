@@ -32,8 +32,8 @@ def permutation(kind, rng):
     return p
 
 
-def marks_of(lanes, perms, order):
-    """The marks as the lanes leave them, one row per sub-block."""
+def play(lanes, perms, order, valid=None):
+    """The marks as the lanes leave them, one row per sub-block, and the number of votes."""
     succ = np.empty((len(perms), N), np.uint8)
     j = np.arange(N)
     for r, p in enumerate(perms):
@@ -42,8 +42,14 @@ def marks_of(lanes, perms, order):
         succ[r] = inv[p[j ^ 1] ^ 1]
     marks = np.zeros((len(perms), MARK_STRIDE), np.uint8)
     ptr = [a.ctypes.data_as(ctypes.c_void_p) for a in (succ, marks)]
-    assert lanes.play_loop_marks(len(perms), *ptr, order) == 0
-    return marks[:, :N // 2]
+    votes = lanes.play_loop_marks(len(perms), len(perms) if valid is None else valid, *ptr, order)
+    assert votes > 0
+    return marks[:, :N // 2], votes
+
+
+def marks_wanted(p):
+    words = oracle.route(p.astype(np.uint32), 8)[14]          # the output side of the first level
+    return 2 + ((np.repeat(words, 32) >> np.tile(np.arange(32, dtype=np.uint32), 4)) & 1)
 
 
 @pytest.mark.parametrize("kind", ["random", "identity", "shift1", "transpose", "sattolo"])
@@ -54,8 +60,18 @@ def test_marks_of_sub_blocks_do_not_depend_on_the_order_of_the_lanes(lanes, regi
     rng = np.random.default_rng(regions)
     for order in range(400 if kind == "random" else 40):
         perms = [permutation(kind, rng) for _ in range(regions)]
-        marks = marks_of(lanes, perms, order)
+        marks, _ = play(lanes, perms, order)
         for r, p in enumerate(perms):
-            words = oracle.route(p.astype(np.uint32), 8)[14]  # the output side of the first level
-            colours = (np.repeat(words, 32) >> np.tile(np.arange(32, dtype=np.uint32), 4)) & 1
-            assert np.array_equal(marks[r], 2 + colours), (kind, r, order)
+            assert np.array_equal(marks[r], marks_wanted(p)), (kind, r, order)
+
+
+@pytest.mark.parametrize("regions,valid", [(16, 1), (16, 5), (16, 16), (32, 31)])
+def test_padding_gets_no_marks_and_takes_no_rounds(lanes, regions, valid):
+    """Sub-blocks of padding, the identity, beside random ones: 128 loops of one switch each would keep the others waiting."""
+    rng = np.random.default_rng(100 * regions + valid)
+    perms = [rng.permutation(N) for _ in range(valid)] + [np.arange(N)] * (regions - valid)
+    marks, votes = play(lanes, perms, 2, valid)
+    for r in range(valid):
+        assert np.array_equal(marks[r], marks_wanted(perms[r])), r
+    assert not marks[valid:].any()
+    assert votes == play(lanes, perms[:valid], 2)[1]
