@@ -75,3 +75,19 @@ def test_padding_gets_no_marks_and_takes_no_rounds(lanes, regions, valid):
         assert np.array_equal(marks[r], marks_wanted(perms[r])), r
     assert not marks[valid:].any()
     assert votes == play(lanes, perms[:valid], 2)[1]
+
+
+@pytest.mark.parametrize("kind", ["identity", "transpose", "bitrev"])
+@pytest.mark.parametrize("short", [1, 5, 15])
+def test_sub_blocks_of_short_loops_beside_random_ones(lanes, short, kind):
+    """A lane whose loops all end within a round keeps the others waiting: its loops are marked without walks, however few
+    such lanes there are.  (Round by round they take 64 to 128 votes; a random one has 128 hops, three to a round, a
+    hop or two of every loop lost: 48 to 60.)"""
+    rng = np.random.default_rng(short)
+    perms = [rng.permutation(N) for _ in range(16)]
+    for r in rng.permutation(16)[:short]:
+        perms[r] = inputs.structured_perms(8)[kind].astype(np.int64)
+    marks, votes = play(lanes, perms, 2)
+    for r, p in enumerate(perms):
+        assert np.array_equal(marks[r], marks_wanted(p)), r
+    assert votes < 62
