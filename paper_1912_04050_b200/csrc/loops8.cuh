@@ -69,12 +69,14 @@ __device__ __forceinline__ void loop_marks(const unsigned char *N, unsigned char
         start = take ? 2u * fresh : start;
         j = take ? 2u * fresh : j;
         if (__all_sync(~0u, seen >= kSw)) break;
-        // Loop after loop that ends within a round, in any lane: the short ones together first, which adds 2 us to the walk of
-        // the others, where 128 loops of one take 11 us longer than a long one.  (8 of 12 hops or less: one sub-block in 5000
-        // of random permutations.  When most lanes had to be that slow, 12000 x 2^8 took 46 us instead of 36 with a quarter
-        // of them the identity, 9741 x 2^9 shift 105 instead of 81.  What is left of the loop at hand is then not short,
-        // unless it has not been begun.)
-        if (round == 3u && __any_sync(~0u, seen <= 8u)) {
+        // Loop after loop that ends within a round: the short ones together first, which adds 2 us to the walk of the others,
+        // where 128 loops of one take 11 us longer than a long one.  Loops of one in any lane do (when most lanes had to
+        // have short ones, 12000 x 2^8 took 46 us instead of 36 with a quarter of them the identity, 9741 x 2^9 shift 105
+        // instead of 81), loops of two, 70 rounds instead of 48 to 60, in most.  (A lane has seen 7 of 12 switches or
+        // less in no random permutation of 200000, 8 in one of 5000; in any lane 8 and less made 128 x 2^13 50.3 us
+        // instead of 48.6.  What is left of the loop at hand is then not short, unless it has not been begun.)
+        if (round == 3u && (__any_sync(~0u, seen <= 7u) ||
+                            2 * __popc(__ballot_sync(~0u, seen <= 8u)) > __popc(__ballot_sync(~0u, mine)))) {
             if (mine) seen = mark_short_loops(N, marks);
             idle = idle || (j == start && marks[j >> 1] != 0);
         }

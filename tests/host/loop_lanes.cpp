@@ -43,6 +43,7 @@ uint32_t vote(bool v) {
 }
 }  // namespace
 static inline int __all_sync(uint32_t, bool v) { return vote(v) == ~0u; }
+static inline uint32_t __ballot_sync(uint32_t, bool v) { return vote(v); }
 static inline int __any_sync(uint32_t, bool v) { return vote(v) != 0u; }
 
 #include "loops8.cuh"

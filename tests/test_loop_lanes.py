@@ -77,12 +77,12 @@ def test_padding_gets_no_marks_and_takes_no_rounds(lanes, regions, valid):
     assert votes == play(lanes, perms[:valid], 2)[1]
 
 
-@pytest.mark.parametrize("kind", ["identity", "transpose", "bitrev"])
-@pytest.mark.parametrize("short", [1, 5, 15])
-def test_sub_blocks_of_short_loops_beside_random_ones(lanes, short, kind):
-    """A lane whose loops all end within a round keeps the others waiting: its loops are marked without walks, however few
-    such lanes there are.  (Round by round they take 64 to 128 votes; a random one has 128 hops, three to a round, a
-    hop or two of every loop lost: 48 to 60.)"""
+@pytest.mark.parametrize("short,kind,most", [(1, "identity", 64), (5, "identity", 64), (15, "identity", 64),
+                                             (9, "transpose", 64), (15, "bitrev", 64)])
+def test_sub_blocks_of_short_loops_beside_random_ones(lanes, short, kind, most):
+    """A lane whose loops all end within a round keeps the others waiting: loops of one switch are marked without walks
+    however few such lanes there are, loops of two where most are such.  (Round by round they take 128 and 70 votes; a
+    random permutation has 128 hops, three to a round, a hop or two of every loop lost: 48 to 60.)"""
     rng = np.random.default_rng(short)
     perms = [rng.permutation(N) for _ in range(16)]
     for r in rng.permutation(16)[:short]:
@@ -90,4 +90,5 @@ def test_sub_blocks_of_short_loops_beside_random_ones(lanes, short, kind):
     marks, votes = play(lanes, perms, 2)
     for r, p in enumerate(perms):
         assert np.array_equal(marks[r], marks_wanted(p)), r
-    assert votes < 62
+    assert votes <= most, votes
+
