@@ -1300,15 +1300,19 @@ int launch_fused(const uint32_t *src, bool inverse, size_t total, int log2m, uin
         return logc == 8 ? launch_few<8>(src, inverse, end, bits, log2n, m, s) : logc == 9 ? launch_few<9>(src, inverse, end, bits, log2n, m, s)
              : logc == 10 ? launch_few<10>(src, inverse, end, bits, log2n, m, s) : launch_few<11>(src, inverse, end, bits, log2n, m, s);
     }
-    // Small blocks share a CTA: a thread of the 8-bit levels takes a whole sub-block, so the more
-    // sub-blocks a CTA holds, the fuller its warps.  Up to 2^13 outputs per CTA (2^12 for blocks of 2^4 .. 2^9, whose time is
-    // the walks': eight CTAs per SM instead of four, 22230 x 2^8 72 -> 61 us, 32768 x 2^7 32 -> 28, 600000 x 2^5 69 -> 65;
-    // with 2^11 98, 36 and 72; 16384 x 2^10 232 -> 236, a million of 2^3 33 -> 34), as long as
-    // every SM still gets a few CTAs: up to five, so that the warps that walk the sub-blocks of 2^8 (one of every CTA) have
-    // a scheduler to themselves, or nearly (up to four against five against eight: 707 x 2^12 91 / 68 / 68 us,
-    // 10000 x 2^8 48 / 33 / 33, 7094 x 2^8 33 / 33 / 50).
+    // Small blocks share a CTA: a thread of the 8-bit levels takes a whole sub-block, so the more sub-blocks a CTA holds, the
+    // fuller its warps, and every CTA copies 9 KiB of tables; but it takes its phases one after the other, and smaller ones
+    // run side by side.  Up to CTAs of 2^12, of which an SM holds eight: as soon as there are more CTAs than SMs for
+    // blocks of 2^6 and less (against up to five per SM 22708 x 2^5 9.2 -> 7.1 us, 9741 x 2^6 10.6 -> 8.9), above three per SM
+    // up to 2^9 (4915 x 2^8 27.6 -> 25.2, 2896 x 2^9 34.4 -> 32.2; as soon as there are more than SMs 6888 x 2^7 shift 13.4 ->
+    // 14.1), above four from there on (1448 x 2^10 40.9 -> 38.7; above three 1024 x 2^10 34.2 -> 35.3).  CTAs of 2^13 pay
+    // where those of 2^12 do not run all at once (1024 x 2^12 84 us in CTAs of 2^12 and 95 in larger ones, 2048 x 2^11 72 and
+    // 82; blocks of 2^3 and less already above five per SM: 440871 x 2^3 14.6 and 13.4), and never for blocks of 2^4 to 2^9
+    // (22230 x 2^8 61 and 72, 32768 x 2^7 28 and 32; CTAs of 2^11 98 and 36).
     int logc = m > 10 ? m : 10;
-    while (logc < (m >= 4 && m <= 9 ? 12 : 13) && ((end - first) >> logc) > 5 * size_t(sm_count())) ++logc;
+    const int most = m >= 4 && m <= 9 ? 12 : 13;
+    auto per_sm = [m](int lc) { return size_t(lc < 12 ? (m <= 6 ? 1 : m <= 9 ? 3 : 4) : (m <= 3 ? 5 : 8)); };
+    while (logc < most && ((end - first) >> logc) > per_sm(logc) * size_t(sm_count())) ++logc;
     // CTAs that have an SM to themselves get more threads: their time is a chain of short
     // phases, not the instructions they issue.
     const bool alone = ((end - first + (size_t(1) << logc) - 1) >> logc) <= size_t(sm_count());
