@@ -849,8 +849,8 @@ k_route_peel(const uint32_t *__restrict__ src, bool inverse, uint32_t *__restric
 // steps, and the labelling with the shortest one is pointer jumping over all outputs: one thread per
 // switch, one barrier per pass, and from sub-blocks of 64 down a warp in registers (a switch, then an output,
 // per lane; jumps by shuffle).  One permutation of 2^10: 22.8 -> 10.5 us; 32 of 2^6:
-// 8.7 -> 4 us; 290 of 2^10 (half of the GPU's threads): 43 -> 17 us.  From about twice the GPU's threads on the
-// kernels above are faster, which issue fewer instructions (5000 of 2^8: 37 us either way).
+// 8.7 -> 4 us; 290 of 2^10 (half of the GPU's threads): 30 us by the kernels above, 14 here.  Where they take over, because they
+// issue fewer instructions: see launch_fused.
 
 // The levels of sub-blocks of 2^ls0 <= 32 outputs and less of 32 neighbouring outputs: p = the lane's entry, gathers
 // by shuffle, the inverse through the group's 32 entries of Q, which only this warp touches.  r = index of the
@@ -1294,8 +1294,14 @@ int launch_fused(const uint32_t *src, bool inverse, size_t total, int log2m, uin
             inverse = true;
         }
     }
-    // blocks of up to 2^11, and not more switches than the GPU has threads
-    if (m <= 11 && first == 0 && end / 2 <= size_t(sm_count()) * 2048) {
+    // Blocks of up to 2^11 and few switches: k_route_few.  A thread of it goes through every level of its switch, which costs
+    // the same at every size; the kernels below have tables and one thread per sub-block for the last levels, so
+    // the smaller the blocks, the earlier they are faster.  Limits in outputs per SM (a GPU full of threads has 4096), either
+    // side of the line: 2^5 2^17.0 outputs 4.8 and 5.7 us, 2^17.5 5.3 and 5.0; 2^6 2^18 6.2 and 6.4, 2^18.5 8.0 and 6.6;
+    // 2^7 2^18.75 11.5 and 13.0, 2^19 13.0 and 11.4; 2^8 2^19 15.8 and 19.2, 2^20 29 and 21; 2^11 2^19 33 and 36, 2^19.25 49 and 38.
+    // (Up to 4096 for all of them, 17912 x 2^5 took 12.4 us and 25171 x 2^5 7.6.)
+    const size_t few_per_sm = 1024 * size_t(m <= 5 ? 1 : m <= 8 ? m - 4 : 4);
+    if (m <= 11 && first == 0 && end <= few_per_sm * size_t(sm_count())) {
         const int logc = m > 8 ? m : 8;
         return logc == 8 ? launch_few<8>(src, inverse, end, bits, log2n, m, s) : logc == 9 ? launch_few<9>(src, inverse, end, bits, log2n, m, s)
              : logc == 10 ? launch_few<10>(src, inverse, end, bits, log2n, m, s) : launch_few<11>(src, inverse, end, bits, log2n, m, s);

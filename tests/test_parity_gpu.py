@@ -153,6 +153,7 @@ def test_a_captured_route_without_workspace_outlives_larger_calls(n, batch):
 
 @pytest.mark.parametrize("n,batch", [(1, 2049), (2, 1031), (3, 131), (4, 67), (5, 33), (6, 17), (6, 10007), (7, 2401), (8, 5),
                                      (8, 601), (9, 1201), (10, 149), (10, 593), (11, 297), (12, 149), (13, 149), (14, 149),
+                                     (1, 80273), (2, 40135), (3, 20069), (4, 10035), (5, 4737), (5, 17912), (6, 5017), (7, 3589),
                                      (1, 440871), (3, 220435), (5, 22707), (6, 19483), (7, 6889), (8, 4915), (9, 2895),
                                      (10, 1449), (10, 3443), (11, 1723), (12, 1187)])
 def test_route_blocks_that_share_a_cta(n, batch):
