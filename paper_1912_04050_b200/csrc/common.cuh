@@ -99,7 +99,6 @@ struct OncePerDevice {
 // benes_debug_guard_hits adds the words up.  It stands in for a memory checker
 // where none can be run.
 //   BENES_GUARD(v, mask)          v & mask, v expected to be <= mask already
-//   BENES_GUARD16(v, mask)        the same for the low 16 bits of v (the rest is other data)
 //   BENES_GUARD_BELOW(v, n, alt)  v < n ? v : alt, v expected to be < n
 #ifdef BENES_DEBUG
 static __device__ unsigned int t_guard_words[2];         // hits, line of the last one
@@ -119,7 +118,6 @@ __device__ __forceinline__ uint32_t guard_below(uint32_t v, uint32_t n, uint32_t
     return v;
 }
 #define BENES_GUARD(v, mask) ::benes::guard_mask((v), (mask), __LINE__)
-#define BENES_GUARD16(v, mask) ::benes::guard_mask((v) & 0xFFFFu, (mask), __LINE__)
 #define BENES_GUARD_BELOW(v, n, alt) ::benes::guard_below((v), (n), (alt), __LINE__)
 // Every translation unit with kernels registers a reader of its own words.
 using GuardReader = int (*)(unsigned int out[2], int clear);
@@ -138,7 +136,6 @@ void guard_register(GuardReader reader, const char *file);
     }
 #else
 #define BENES_GUARD(v, mask) ((v) & (mask))
-#define BENES_GUARD16(v, mask) ((v) & (mask))
 #define BENES_GUARD_BELOW(v, n, alt) ((v) < (n) ? (v) : (alt))
 #define BENES_GUARD_TU(name)
 #endif

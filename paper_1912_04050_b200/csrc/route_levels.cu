@@ -126,7 +126,7 @@ k_inverse_partition(const uint32_t *__restrict__ P, void *__restrict__ S, uint2 
         const size_t j = j0 + 2 * (size_t(i / 2) * kPartThreads + tid);
         const uint2 p = __ldcs(reinterpret_cast<const uint2 *>(P + j));
         const uint32_t px = BENES_GUARD(p.x, mmask), py = BENES_GUARD(p.y, mmask);
-        if (S) rec_write<PACKED>(S, nullptr, j >> 1, m, px, py, kappa, 0u);
+        rec_write<PACKED>(S, nullptr, j >> 1, m, px, py, kappa, 0u);
         const uint32_t base = uint32_t(j) & ~mmask;
         dest[i] = base + px;
         dest[i + 1] = base + py;
