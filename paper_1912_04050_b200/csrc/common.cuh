@@ -90,14 +90,15 @@ struct OncePerDevice {
 };
 
 // ---- index guards ---------------------------------------------------------------
-// Every index a kernel forms from data is forced into range with a mask or a
-// clamp, so that an input that is not a permutation cannot cause an access out
-// of bounds.  On a permutation no guard ever changes the value it is given.  A
-// build with -DBENES_DEBUG checks exactly that: a guard that has to change its
-// value counts the event in a device word of its translation unit and keeps the
-// source line (no trap, no printf; the access itself is still the guarded one).
-// benes_debug_guard_hits adds the words up.  It stands in for a memory checker
-// where none can be run.
+// Every index a kernel forms from data stays in range, so that an input that is not a permutation cannot cause an access
+// out of bounds.  What comes from global memory (permutations, inverses, owners, next words) passes a guard, a mask or a
+// clamp that on a permutation never changes its value.  A build with -DBENES_DEBUG checks exactly that: a guard that has to
+// change its value counts the event in a device word of its translation unit and keeps the source line (no trap, no
+// printf; the access itself is still the guarded one).  benes_debug_guard_hits adds the words up.  It stands in for a
+// memory checker where none can be run.  What it does not see: the fields of packed records, which cannot exceed their
+// mask; the successors of chained levels, masked without a count, because behind a raised gate some are left over from
+// other levels, rightly out of range; and successors, codes and list words in shared memory (k_list_label, in-CTA levels),
+// which have plain masks, or none where everything that writes them keeps them in their array.
 //   BENES_GUARD(v, mask)          v & mask, v expected to be <= mask already
 //   BENES_GUARD_BELOW(v, n, alt)  v < n ? v : alt, v expected to be < n
 #ifdef BENES_DEBUG
