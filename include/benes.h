@@ -247,9 +247,9 @@ int benes_validate_perm(const uint32_t *perm, int log2n, int batch, benes_stream
  *   BENES_OPT_SAMPLE_LOG2K : 0 = label every loop by pointer jumping over all
  *       outputs; kappa in 2..8 (default 4) = label only one sampled "ruler"
  *       switch per 2^kappa switches by pointer jumping and reach the rest by
- *       sequential walks between rulers (for batch * N <= 2^22 at most 2^3: short
- *       walks matter more than short lists there).  The result is identical
- *       either way.
+ *       sequential walks between rulers (a value above 3 counts as 3 for
+ *       batch * N <= 2^22 and as 2 for batch * N <= 2^19: short walks matter
+ *       more than short lists there).  The result is identical either way.
  *   BENES_OPT_WALK_CAP : hops (1 .. 2^24, default 2^14) after which a walk gives
  *       up; a route in which that happens is redone by full pointer jumping.
  *   BENES_OPT_APPLY_FUSED : 1 (default) = benes_apply / benes_apply_ex run up to
@@ -269,7 +269,9 @@ int benes_validate_perm(const uint32_t *perm, int log2n, int batch, benes_stream
  *       1.06, 2^26 17.2 instead of 15.7).
  *   BENES_OPT_WALK_PAIRS : a thread can take both walks that leave one ruler switch, one
  *       after the other.  0 = never, 1 (default) = where the halved number of threads
- *       still fills the GPU, 2 = at every level.  Same result.
+ *       still fills the GPU, 2 = at every level above a CTA.  No effect for batch * N <=
+ *       2^20 (chunks that small included): a level lasts as long as its longest walk
+ *       there, and every walk has a thread.  Same result.
  * benes_set_option returns BENES_OK or BENES_ERR_BADARG; benes_get_option
  * returns the value, or BENES_ERR_BADARG for an unknown key.
  */
@@ -338,9 +340,9 @@ int benes_probe_random_access(void *table, int log2_records, int record_bytes, i
                               uint32_t *sink, benes_stream_t stream);
 
 /*
- * Checked build.  Every index a kernel forms from data is forced into range (a
- * mask or a clamp), which is what keeps a non-permutation input memory-safe; on a
- * permutation no such guard ever changes its value.  The library built with
+ * Checked build.  Every index a kernel forms from data stays in range, which is what
+ * keeps a non-permutation input memory-safe: mostly by a guard, a mask or a clamp,
+ * and on a permutation no such guard ever changes its value.  The library built with
  * -DBENES_DEBUG (libbenes_debug.so, same ABI) counts, in device words, every guard
  * that did change a value, and remembers the source line of one of them.  Nothing
  * traps and nothing is printed.  benes_debug_build returns 1 for that build, 0
