@@ -149,7 +149,11 @@ k_walk(unsigned long long *__restrict__ S8, const uint32_t *__restrict__ P, cons
             }
         }
         if (W == 1 || (++rounds & 63u) == 0u) {
-            if (((W == 1 ? hops : rounds) & 63u) == 0u && gate_raised(gate)) break;      // the route is redone anyway
+            if (((W == 1 ? hops : rounds) & 63u) == 0u && gate_raised(gate)) {           // the route is redone anyway
+                // (what an earlier route left in the records could name words beyond this one's lists)
+                do rec[rho] = make_uint2(least, rho ^ 1u), ++rho; while (W > 1 && ++walk < uint32_t(W));
+                break;
+            }
         }
         if (ends) {
             rec[rho] = make_uint2(least, peer);

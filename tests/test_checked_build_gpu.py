@@ -108,6 +108,23 @@ def test_no_guard_fires_with_resampled_lists_bucketed_inverse_and_clusters(optio
         assert_clean("two walks per thread n=%d" % n)
 
 
+@pytest.mark.parametrize("kappa,cap,walks", [(None, None, 0), (None, None, 2), (2, None, 1), (3, 1, 2), (None, 3, 0), (None, 40, 2),
+                                             (5, None, 2), (8, None, 0)])
+def test_no_guard_fires_on_record_levels(kappa, cap, walks, options, known_route):
+    """More than 2^20 outputs (2^22 for the wider spacings): the walks, lists and colouring on records, lists sampled again,
+    batches that are no power of two, one and two walks per thread, and walks that give up."""
+    binding.benes_set_option(binding.OPT_WALK_PAIRS, walks)
+    if kappa is not None:
+        binding.benes_set_option(binding.OPT_SAMPLE_LOG2K, kappa)
+    if cap is not None:
+        binding.benes_set_option(binding.OPT_WALK_CAP, cap)
+    for kind, n, batch in [("random", 20, 5), ("shift1", 20, 5)] if kappa and kappa > 3 else \
+            [("random", 21, 1), ("random", 19, 3), ("shift1", 21, 1), ("transpose", 21, 1)]:
+        perm, want = known_route(kind, n, batch)
+        assert np.array_equal(route(perm, n), want), (kind, n, batch)
+        assert_clean("%s %d x 2^%d" % (kind, batch, n))
+
+
 @pytest.mark.parametrize("n", [6, 14, 17, 22])
 def test_guards_fire_on_an_input_that_is_not_a_permutation(n):
     """Values out of range: the guards must catch them (and the call must stay in bounds:
