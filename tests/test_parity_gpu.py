@@ -388,6 +388,53 @@ def test_route_chained_levels_and_levels_on_records(n, batch, kappa, kind, label
         assert np.array_equal(got[b], want[b % len(few)]), b
 
 
+# Levels on records: more than 2^20 outputs in all (below, the levels above a CTA are chained).  Ruler spacings above 2^3
+# take effect from more than 2^22 on.
+RECORD_INPUTS = [("random", 21, 1), ("random", 19, 3), ("sattolo", 21, 1), ("shift1", 21, 1), ("bitrev", 21, 1), ("transpose", 21, 1)]
+WIDE_SPACING_INPUTS = [("random", 20, 5), ("shift1", 20, 5)]
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2])
+@pytest.mark.parametrize("kappa,cap", [(None, None), (2, None), (None, 3), (3, 40), (None, 1), (5, None), (8, None), (6, 100)])
+def test_route_record_levels_with_any_option_of_the_walks(mode, kappa, cap, labelling_options, known_route):
+    """One or two walks per thread, every spacing and hop limit, where they change the kernels that run."""
+    w0 = binding.benes_get_option(binding.OPT_WALK_PAIRS)
+    binding.benes_set_option(binding.OPT_WALK_PAIRS, mode)
+    try:
+        if kappa is not None:
+            binding.benes_set_option(binding.OPT_SAMPLE_LOG2K, kappa)
+        if cap is not None:
+            binding.benes_set_option(binding.OPT_WALK_CAP, cap)
+        for kind, n, batch in WIDE_SPACING_INPUTS if kappa and kappa > 3 else RECORD_INPUTS:
+            perm, want = known_route(kind, n, batch)
+            assert np.array_equal(gpu_route(perm, n), want), (kind, n, batch)
+    finally:
+        binding.benes_set_option(binding.OPT_WALK_PAIRS, w0)
+
+
+def test_route_random_option_combinations_on_record_levels(labelling_options, known_route):
+    """As above, with inputs that are large enough for records (chunked or not)."""
+    rng = np.random.default_rng(2025)
+    keys = (binding.OPT_WALK_PAIRS, binding.OPT_CLUSTER, binding.OPT_INVERSE_PARTITIONED, binding.OPT_CHUNK_LOG2)
+    old = [binding.benes_get_option(k) for k in keys]
+    try:
+        for trial in range(48):
+            kind, n, batch = (RECORD_INPUTS + WIDE_SPACING_INPUTS + [("random", 17, 33)])[int(rng.integers(0, 9))]
+            opts = {binding.OPT_SAMPLE_LOG2K: int(rng.choice([2, 3, 4, 4, 5, 6, 8])),
+                    binding.OPT_WALK_CAP: int(rng.choice([1, 7, 100, 1 << 14, 1 << 14])),
+                    binding.OPT_WALK_PAIRS: int(rng.integers(0, 3)),
+                    binding.OPT_CLUSTER: int(rng.integers(0, 2)),
+                    binding.OPT_INVERSE_PARTITIONED: int(rng.integers(0, 2)),
+                    binding.OPT_CHUNK_LOG2: int(rng.choice([30, 30, 21, 22]))}
+            for k, v in opts.items():
+                binding.benes_set_option(k, v)
+            perm, want = known_route(kind, n, batch)
+            assert np.array_equal(gpu_route(perm, n), want), (trial, n, batch, kind, opts)
+    finally:
+        for k, v in zip(keys, old):
+            binding.benes_set_option(k, v)
+
+
 @pytest.mark.parametrize("n,batch", [(22, 1), (16, 64), (17, 64), (23, 1), (16, 65)])
 def test_route_bucketed_inverse(n, batch):
     """batch * N >= 2^22 in whole multiples of 2^18 takes the two-pass inverse at
