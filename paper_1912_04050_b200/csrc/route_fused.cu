@@ -31,7 +31,7 @@
 //
 // Measured on B200, before (P and Q kept, successors gathered through both; twice as many rulers; a look for
 // the next start with every hop in sub-blocks of 2^8 too, by register sets from the low bit up) and after: 2048 blocks of 2^15 2.38 -> 1.87 ms, 4096 x 2^14
-// 1.96 -> 1.61 ms, 4096 x 2^12 374 -> 318 us, 16384 x 2^8 53 -> 40 us.  Units of 8192 outputs inside a larger CTA with
+// 1.96 -> 1.61 ms, 4096 x 2^12 374 -> 316 us, 16384 x 2^8 53 -> 38 us.  Units of 8192 outputs inside a larger CTA with
 // barriers of their own, meant to fall out of step, took 2.04 and 1.90 ms for the first two: the CTA waits for
 // its last unit.
 #include "common.cuh"
@@ -811,8 +811,8 @@ k_route_fused(const uint32_t *__restrict__ src, bool inverse, uint32_t *__restri
 // One level of one block of 2^LOGC outputs per CTA; the inverses of the two half-blocks go to `next`, where the
 // next launch finds them with twice as many CTAs.  While more than half of the SMs would have no block, that is how the
 // in-CTA levels run: a level takes a time in proportion to the CTA's outputs, so halving the block with every level
-// costs about two levels of the first block instead of one for each (one block of 2^15: 172 -> 82 us,
-// 2^13: 51 -> 37; the route of 2^16: 206 -> 140, of 2^20: 545 -> 497).
+// costs about two levels of the first block instead of one for each (all levels in one launch -> this: one block of 2^15
+// 134 -> 68 us, 2^13 47 -> 32, 37 of 2^12 34 -> 24; the route of 2^16 175 -> 109, of 2^20 441 -> 388).
 template <class Cfg>
 __global__ void __launch_bounds__(Cfg::T, 1)
 k_route_peel(const uint32_t *__restrict__ src, bool inverse, uint32_t *__restrict__ bits, int log2n, uint32_t *__restrict__ next) {
@@ -848,8 +848,8 @@ k_route_peel(const uint32_t *__restrict__ src, bool inverse, uint32_t *__restric
 // When every thread of the GPU could have a switch to itself, the time of a call is its chain of dependent
 // steps, and the labelling with the shortest one is pointer jumping over all outputs: one thread per
 // switch, one barrier per pass, and from sub-blocks of 64 down a warp in registers (a switch, then an output,
-// per lane; jumps by shuffle).  One permutation of 2^10: 22.8 -> 10.5 us; 32 of 2^6:
-// 8.7 -> 4 us; 290 of 2^10 (half of the GPU's threads): 30 us by the kernels above, 14 here.  Where they take over, because they
+// per lane; jumps by shuffle).  Up to 64 of 2^10: 23.9 -> 8.6 us; 32 of
+// 2^6: 6.6 -> 3.3; 290 of 2^10 (half of the GPU's threads): 30 -> 14.  Where the kernels above take over, because they
 // issue fewer instructions: see launch_fused.
 
 // The levels of sub-blocks of 2^ls0 <= 32 outputs and less of 32 neighbouring outputs: p = the lane's entry, gathers

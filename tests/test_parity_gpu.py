@@ -238,8 +238,8 @@ def test_route_every_ruler_spacing(kappa, labelling_options):
 @pytest.mark.parametrize("mode", [0, 2])
 @pytest.mark.parametrize("kappa,cap", [(None, None), (2, None), (5, None), (None, 3)])
 def test_route_one_or_two_walks_per_thread(mode, kappa, cap, labelling_options):
-    """At packed levels a thread advances one walk or the two walks of a ruler switch
-    (the default picks by size; both forced here at sizes that take either)."""
+    """At levels on records a thread advances one walk or the two walks of a ruler switch (the default picks by
+    size).  Of these inputs 5 x 2^19 has such levels; the option must not change the others, whose levels are chained."""
     w0 = binding.benes_get_option(binding.OPT_WALK_PAIRS)
     binding.benes_set_option(binding.OPT_WALK_PAIRS, mode)
     try:
@@ -259,7 +259,7 @@ def test_route_one_or_two_walks_per_thread(mode, kappa, cap, labelling_options):
 def test_route_random_option_combinations(labelling_options):
     """Seeded draws over sizes, batches, input kinds and every option that changes the path
     (ruler spacing, hop limit, walks per thread, clusters, inverse form, chunking): the bits never
-    depend on the path."""
+    depend on the path.  Mostly inputs of up to 2^20 outputs, chained."""
     rng = np.random.default_rng(2024)
     keys = (binding.OPT_WALK_PAIRS, binding.OPT_CLUSTER, binding.OPT_INVERSE_PARTITIONED, binding.OPT_CHUNK_LOG2)
     old = [binding.benes_get_option(k) for k in keys]
@@ -310,8 +310,8 @@ def test_route_structured_in_clusters(n, kind, cluster_mode):
 
 @pytest.mark.parametrize("cap", [1, 3, 40])
 def test_route_walks_that_give_up_fall_back_to_full_pointer_jumping(cap, labelling_options):
-    """With a tiny hop limit some walk of almost every level gives up, and the route is redone by
-    pointer jumping over all outputs; the bits must not change."""
+    """With a tiny hop limit some walk of almost every level (chained, at these sizes) gives up, and the route is
+    redone by pointer jumping over all outputs; the bits must not change."""
     binding.benes_set_option(binding.OPT_WALK_CAP, cap)
     for n in (16, 18):
         for kind, perm in inputs.structured_perms(n).items():
