@@ -325,7 +325,7 @@ struct SampledScratch {
 size_t sampled_scratch_bytes(size_t total, int kappa);
 void sampled_scratch_carve(char *base, size_t total, int kappa, SampledScratch *out);
 // Labels every loop of the level, writes the output-side stage and the next
-// level's records Sn (none if Sn.S is null); raises *gate if some walk exceeded `cap` hops (the route must then be
+// level's records Sn (none if Sn.S is null, behind packed records S only); raises *gate if some walk exceeded `cap` hops (the route must then be
 // redone by launch_route_jump).
 int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const SampledScratch &sc, size_t total,
                   int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage, uint32_t *gate, cudaStream_t s);
@@ -348,7 +348,7 @@ size_t sampled_owner_bytes(const SampledScratch &sc, size_t total, int log2m, in
 // Finishes levels (n - log2m) .. n-1 of every block of size 2^log2m of the flat
 // level array (total elements), one CTA per block for log2m <= kFusedLog2M, one
 // cluster of two CTAs per block for log2m = kFusedLog2M + 1.
-// `src`: the blocks' values, local to their block: the permutation, or its inverse if `inverse`.
+// `src`: the blocks' values, local to their block: the permutation, or its inverse if `inverse` (blocks of 2^11 and more).
 // `blocks` blocks from `first_block` on (blocks = 0: all from first_block).
 int launch_fused(const uint32_t *src, bool inverse, size_t total, int log2m, uint32_t *bits, int log2n,
                  cudaStream_t s, size_t first_block = 0, size_t blocks = 0, uint32_t *const spare[2] = nullptr);

@@ -1000,6 +1000,8 @@ k_route_few(const uint32_t *__restrict__ src, bool inverse, uint32_t *__restrict
     }
 }
 
+constexpr int kMinInverseLog2 = 11;            // (see k_route_few: from the inverse in blocks of 2^11 only)
+
 template <int LOGC>
 int launch_few(const uint32_t *src, bool inverse, size_t total, uint32_t *bits, int n, int logs, cudaStream_t s) {
     launch_kernel(k_route_few<LOGC>, unsigned((total + (size_t(1) << LOGC) - 1) >> LOGC), (1 << LOGC) / 2, 0, s, src, inverse, bits, n, logs, total);
@@ -1271,6 +1273,9 @@ int launch_cluster2(const uint32_t *src, bool inverse, size_t first_block, size_
 int launch_fused(const uint32_t *src, bool inverse, size_t total, int log2m, uint32_t *bits, int log2n,
                  cudaStream_t s, size_t first_block, size_t blocks, uint32_t *const spare[2]) {
     if (log2m < 1 || log2m > kClusterLog2M) return BENES_ERR_BADARG;
+    // Inverses are taken where every kernel below does (and k_route_peel leaves them): k_route_few of 2^11, 16-bit entries.
+    static_assert(kPeelLog2 - 1 >= kMinInverseLog2 && kMinInverseLog2 >= kFMinLogS, "");
+    if (inverse && log2m < kMinInverseLog2) return BENES_ERR_BADARG;
     if (blocks == 0) blocks = (total >> log2m) - first_block;        // all the rest
     if (first_block + blocks > (total >> log2m)) return BENES_ERR_BADARG;
     if (log2m == kClusterLog2M) return launch_cluster2(src, inverse, first_block, blocks, bits, log2n, s);

@@ -727,6 +727,7 @@ static int label_lists(const SampledScratch &sc, uint32_t R, int beta, uint32_t 
 int sampled_label(LevelRecords S, const uint32_t *Q, LevelRecords Sn, const SampledScratch &sc, size_t total,
                   int log2m, int kappa, uint32_t salt, uint32_t cap, int walk_pairs, BitsLayout L, int out_stage,
                   uint32_t *gate, cudaStream_t s) {
+    if (!S.packed && !Sn.S) return BENES_ERR_BADARG;           // (no k_colour for a last level on wide records)
     const uint32_t R = uint32_t(total >> kappa);
     {
         ProfileScope ps(kWalk, s);

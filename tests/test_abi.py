@@ -3,6 +3,7 @@ host-side argument checks and sizing helpers (no GPU work is launched)."""
 import ctypes
 import os
 import re
+import subprocess
 
 import pytest
 
@@ -74,6 +75,43 @@ def test_argument_errors_are_reported_on_the_host(lib):
     assert lib.benes_apply_host(one, one, one, 5, 10, 1, None) == binding.BENES_ERR_BADARG
     assert lib.benes_set_workspace(ctypes.c_void_p(256), 0) == binding.BENES_ERR_BADARG
     assert lib.benes_set_workspace(ctypes.c_void_p(100), 1024) == binding.BENES_ERR_BADARG  # alignment
+
+
+def _internal(lib_path, name):
+    """The one C++ function benes::`name` of the library."""
+    names = subprocess.check_output(["nm", "-D", "--defined-only", lib_path], text=True).split()
+    found = [s for s in names if s.startswith("_ZN5benes%d%sE" % (len(name), name))]
+    assert len(found) == 1, found
+    return getattr(ctypes.CDLL(lib_path), found[0])
+
+
+@pytest.mark.parametrize("debug", [False, True])
+def test_launches_refuse_what_no_kernel_takes(debug):
+    """The in-CTA levels start from an inverse in blocks of 2^11 and more only, and the levels on wide records are never the
+    last: an error on the host, nothing is launched.  (With no blocks at all a launch that went ahead would end in another
+    error, or in none.)"""
+    path = build.build(debug=debug)
+    u64, i32, ptr = ctypes.c_size_t, ctypes.c_int, ctypes.c_void_p
+    fused = _internal(path, "launch_fused")
+    fused.argtypes = [ptr, ctypes.c_bool, u64, i32, ptr, i32, ptr, u64, u64, ptr]
+    for m in range(1, 11):
+        assert fused(None, True, 0, m, None, m, None, 0, 0, None) == binding.BENES_ERR_BADARG, m
+
+    class Records(ctypes.Structure):
+        _fields_ = [("S", ptr), ("P", ptr), ("packed", ctypes.c_bool)]
+
+    class Layout(ctypes.Structure):
+        _fields_ = [("bits", ptr), ("log2n", i32), ("log2w", i32)]
+
+    class Scratch(ctypes.Structure):
+        _fields_ = [("rec", ptr * 5), ("owner", ptr * 5), ("bits", ptr * 5)]
+
+    label = _internal(path, "sampled_label")
+    label.argtypes = [Records, ptr, Records, ctypes.POINTER(Scratch), u64, i32, i32, ctypes.c_uint32, ctypes.c_uint32, i32,
+                      Layout, i32, ptr, ptr]
+    wide, none = Records(256, 256, False), Records(None, None, True)
+    assert label(wide, None, none, ctypes.byref(Scratch()), 0, 23, 4, 0, 1 << 14, 1, Layout(None, 23, 17), 44, None, None) \
+        == binding.BENES_ERR_BADARG
 
 
 def test_options_are_validated(lib):
