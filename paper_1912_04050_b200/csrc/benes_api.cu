@@ -324,8 +324,8 @@ int route_levels(const uint32_t *perm, int n, size_t batch, uint32_t *bits, char
     uint32_t *fill = reinterpret_cast<uint32_t *>(ws + off); off += align_up(kInverseMaxBuckets * 4);
     char *sampled = ws + off;
     // Small inputs are bound by the longest walk of a level, not by throughput:
-    // closer rulers (shorter walks) pay there although the lists get longer.  Where walks are chained (2^16 .. 2^20), one
-    // ruler per 4 switches instead of 8: 2^18 203 -> 195 us, 2^19 293 -> 284, but 2^20 400 -> 407.
+    // closer rulers (shorter walks) pay there although the lists get longer.  Where walks are chained, one ruler per 4
+    // switches instead of 8 up to 2^19 outputs: 2^18 203 -> 195 us, 2^19 293 -> 284, but 2^20 400 -> 407.
     const int kappa = opt.kappa > 3 && T <= (size_t(1) << 22) ? (2 * T <= kChainMaxTotal ? 2 : 3) : opt.kappa;
     const uint32_t cap = uint32_t(opt.walk_cap);
     // Level 0: P is the caller's permutation, which nobody writes.  The kernels of the sampled levels load it 16 bytes at

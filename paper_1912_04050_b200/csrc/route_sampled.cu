@@ -172,9 +172,9 @@ k_walk(unsigned long long *__restrict__ S8, const uint32_t *__restrict__ P, cons
 // ---- chained levels ---------------------------------------------------------------------
 // Where a level lasts as long as its longest walk, what counts is what a hop waits for.  Here that is one access: the
 // successor G[j] and the claim of its switch (a compare-and-swap on the owner's word) are under way together.  On
-// records a hop waits for an atomic and then for a gather.  One permutation, walks of a level and the whole route, on
-// records and chained: 2^20 30.5 -> 22.5 and 417 -> 394 us, 2^18 30 -> 21.5 and 231 -> 198 us (with twice as many
-// rulers; 203 without).  A switch that the two walkers of a segment claim at the same time may be counted by both.
+// records a hop waits for an atomic and then for a gather.  One permutation, on
+// records and chained, with the same rulers: 2^20 walks of a level 30.5 -> 22.5 us, route 417 -> 394; 2^18 route 231 ->
+// 203.  A switch that the two walkers of a segment claim at the same time may be counted by both.
 // (Behind a raised gate, or an input that is no permutation, some successors are left over from other levels: they are
 // masked into the block.)
 __global__ void __launch_bounds__(kWalkThreads)

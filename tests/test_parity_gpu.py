@@ -195,6 +195,19 @@ def test_route_loops_without_ruler_inside_a_cta(n, batch, group):
         assert np.array_equal(got[s], want[s % 3]), s
 
 
+@pytest.mark.parametrize("n,batch", [(8, 1300), (8, 12000), (10, 1449), (12, 601)])
+def test_route_short_loops_beside_long_ones(n, batch):
+    """Sub-blocks of 2^8 whose loops have one switch or two, alone and many among random ones of the same warp."""
+    kinds = [inputs.random_perm(n, 61), inputs.random_perm(n, 62), loops_of_few_switches(n, 2, 0), np.arange(1 << n, dtype=np.uint32),
+             inputs.structured_perms(n)["transpose"]]
+    rng = np.random.default_rng(n)
+    want = [oracle.route(p, n) for p in kinds]
+    for short in (1 / 40, 1 / 2, 39 / 40):
+        pick = np.where(rng.random(batch) < short, rng.integers(2, 5, batch), rng.integers(0, 2, batch))
+        got = gpu_route(np.stack(kinds)[pick], n)
+        assert np.array_equal(got, np.stack(want)[pick]), short
+
+
 def test_route_exhaustive_n8():
     """All 40320 permutations of N = 8 in one batched call."""
     import itertools
